@@ -82,6 +82,18 @@ size_t emul_workspace_bytes(emul_handle_t handle);
 int emul_schedule(int slices, int k, int wide, int level_sums, int threshold, int* sweeps, int cap_sweeps,
                   unsigned char* table, int cap_table, int* meta);
 
+/* The same for the kernel's CTA-pair variant (more than 128 rows): sweeps of up
+ * to four jobs.  slices_a, slices_b: slices of A and B whose pairs are kept;
+ * threshold = 0: max + 1.  Needs no GPU.
+ *   sweeps  out, cap_sweeps rows of EMUL_PAIR_SWEEP_INTS ints: k0c, k1c, njobs,
+ *           final job (-1: none), nplanes, kcs, then L, pb, pe of four jobs
+ *   meta    out, 3 ints: nsweeps; 1 (64-bit state) or 2 (its 16 low bits are put
+ *           aside after a job); that job's number within the tile (-1: none)
+ * Returns EMUL_OK, or EMUL_INVALID_ARG (no such schedule: meta[0] = 0; or a
+ * capacity too small). */
+#define EMUL_PAIR_SWEEP_INTS 18
+int emul_schedule_pair(int slices_a, int slices_b, int k, int threshold, int* sweeps, int cap_sweeps, int* meta);
+
 /* ---------------------------------------------------------------- steps --
  * Exposed individually so each step of the method can be checked bit for bit.
  */

@@ -31,6 +31,7 @@ SIGNATURES = {
     "emul_sync_status": (_c_int, [_vp]),
     "emul_workspace_bytes": (ctypes.c_size_t, [_vp]),
     "emul_schedule": (_c_int, [_c_int, _c_int, _c_int, _c_int, _c_int, _vp, _c_int, _vp, _c_int, _vp]),
+    "emul_schedule_pair": (_c_int, [_c_int, _c_int, _c_int, _c_int, _vp, _c_int, _vp]),
     "emul_split": (_c_int, [_vp, _c_int, _c_int, _vp, _c_long, _c_long, _c_int, _vp, _vp, _c_long]),
     "emul_level_sums": (_c_int, [_vp, _c_int, _c_int, _c_int, _vp, _c_int, _vp, _c_int, _c_int, _vp, _c_int,
                                  _c_long]),
@@ -361,6 +362,28 @@ def schedule(slices, k, wide=False, level_sums=False, t=0):
     sweeps = [dict(zip(SWEEP_FIELDS, sw[i * n:(i + 1) * n])) for i in range(meta[0])]
     info = {"nsweeps": meta[0], "njobs": meta[1], "t0": meta[2], "period": meta[3], "table_bytes": meta[4]}
     return sweeps, bytes(tab[:meta[4]]), info
+
+
+def schedule_pair(slices_a, slices_b, k, t=0):
+    """The CTA-pair variant's schedule from emul_schedule_pair (host only): (list
+    of sweep dicts, kind 1 or 2, job after which the low bits are put aside),
+    or None when the variant does not apply."""
+    L = load()
+    meta = (ctypes.c_int * 3)()
+    L.emul_schedule_pair(slices_a, slices_b, k, t, None, 0, meta)
+    if meta[0] == 0:
+        return None
+    n = 18
+    sw = (ctypes.c_int * (meta[0] * n))()
+    rc = L.emul_schedule_pair(slices_a, slices_b, k, t, sw, meta[0], meta)
+    if rc != 0:
+        raise EmulError(f"emul_schedule_pair failed ({rc})")
+    out = []
+    for i in range(meta[0]):
+        r = sw[i * n:(i + 1) * n]
+        out.append({"k0c": r[0], "k1c": r[1], "final": r[3], "nplanes": r[4], "kcs": r[5],
+                    "jobs": [tuple(r[6 + 3 * j:9 + 3 * j]) for j in range(r[2])]})
+    return out, meta[1], meta[2]
 
 
 def lib():

@@ -47,25 +47,27 @@ long double exact_sum_bound_per_k(const PairSet& ps, int last) {
 int seg_chunks(int n) { return n > 0 ? kExactBudget / (n * kBK) : 0; }
 
 struct Job {
-  int L, pb, pe, c0, c1, flags;
+  int L, pb, pe, c0, c1;
+  bool fin;   // completes and rounds the sum
 };
 
-Job make_job(const PairSet& ps, int L, int c0, int c1, int flags) {
-  return Job{L, ps.lo(L), ps.hi(L), c0, c1, flags};
+Job make_job(const PairSet& ps, int L, int c0, int c1, bool fin) {
+  return Job{L, ps.lo(L), ps.hi(L), c0, c1, fin};
 }
 
-void push_sweep(std::vector<Sweep>& out, const Job& a, const Job* b) {
+// A sweep of jobs over one K range, in the order given.
+void push_sweep(std::vector<Sweep>& out, const std::vector<Job>& jobs) {
   Sweep sw{};
-  sw.k0c = static_cast<int16_t>(a.c0);
-  sw.k1c = static_cast<int16_t>(a.c1);
-  const Job* js[2] = {&a, b};
+  sw.k0c = static_cast<int16_t>(jobs[0].c0);
+  sw.k1c = static_cast<int16_t>(jobs[0].c1);
+  sw.njobs = static_cast<int8_t>(jobs.size());
   int np = 0;
-  for (int j = 0; j < 2 && js[j]; ++j) {
-    sw.L[j] = static_cast<int8_t>(js[j]->L);
-    sw.pb[j] = static_cast<int8_t>(js[j]->pb);
-    sw.pe[j] = static_cast<int8_t>(js[j]->pe);
-    sw.flags[j] = static_cast<int8_t>(js[j]->flags);
-    const int pj = js[j]->pe > js[j]->L - js[j]->pb ? js[j]->pe : js[j]->L - js[j]->pb;
+  for (size_t j = 0; j < jobs.size(); ++j) {
+    const Job& q = jobs[j];
+    sw.L[j] = static_cast<int8_t>(q.L);
+    sw.pp[j] = static_cast<uint8_t>(q.pb | (q.pe << 4));
+    if (q.fin) sw.final_mask = static_cast<int8_t>(sw.final_mask | (1 << j));
+    const int pj = q.pe > q.L - q.pb ? q.pe : q.L - q.pb;
     np = np > pj ? np : pj;
   }
   sw.nplanes = static_cast<int8_t>(np);
@@ -115,7 +117,7 @@ bool build_banded(const PairSet& ps, int t, int nch, bool wide, std::vector<Swee
       const int size = (nch + G - 1) / G;
       for (int g = 0; g < G; ++g) {
         const int c0 = g * size, c1 = c0 + size < nch ? c0 + size : nch;
-        push_sweep(out, make_job(ps, L, c0, c1, (!wide && L == 2) ? kFinal : 0), nullptr);
+        push_sweep(out, {make_job(ps, L, c0, c1, !wide && L == 2)});
       }
     } else {
       const int a = seg_chunks(ps.count(L)), b = seg_chunks(ps.count(L + 1));
@@ -123,8 +125,7 @@ bool build_banded(const PairSet& ps, int t, int nch, bool wide, std::vector<Swee
       const int size = (nch + G - 1) / G;
       for (int g = 0; g < G; ++g) {
         const int c0 = g * size, c1 = c0 + size < nch ? c0 + size : nch;
-        const Job j1 = make_job(ps, L + 1, c0, c1, 0);
-        push_sweep(out, make_job(ps, L, c0, c1, 0), &j1);
+        push_sweep(out, {make_job(ps, L, c0, c1, false), make_job(ps, L + 1, c0, c1, false)});
       }
     }
   }
@@ -144,7 +145,7 @@ bool build_levelwise(const PairSet& ps, int t, int nch, bool wide, std::vector<S
     const int pb = ps.lo(L);
     const int pe = ps.hi(L);
     const int n = pe - pb + 1;
-    const int fin = (!wide && L == 2) ? kFinal : 0;
+    const bool fin = !wide && L == 2;
     if (n * kc <= kExactBudget) {
       jobs.push_back(Job{L, pb, pe, 0, nch, fin});
     } else if (!wide) {
@@ -152,21 +153,21 @@ bool build_levelwise(const PairSet& ps, int t, int nch, bool wide, std::vector<S
       const int per = kExactBudget / kc;          // pairs per job
       if (per < 1) return false;
       for (int p = pb; p <= pe; p += per)
-        jobs.push_back(Job{L, p, p + per - 1 < pe ? p + per - 1 : pe, 0, nch, 0});
+        jobs.push_back(Job{L, p, p + per - 1 < pe ? p + per - 1 : pe, 0, nch, false});
     } else {
       int cm = kExactBudget / (kBK * n);
       if (cm < 1) cm = 1;
-      for (int c0 = 0; c0 < nch; c0 += cm) jobs.push_back(Job{L, pb, pe, c0, c0 + cm < nch ? c0 + cm : nch, 0});
+      for (int c0 = 0; c0 < nch; c0 += cm) jobs.push_back(Job{L, pb, pe, c0, c0 + cm < nch ? c0 + cm : nch, false});
     }
   }
   for (size_t i = 0; i < jobs.size();) {
     // the final job stays alone in its sweep
-    if (i + 1 < jobs.size() && !(jobs[i + 1].flags & kFinal) && jobs[i + 1].c0 == jobs[i].c0 &&
+    if (i + 1 < jobs.size() && !jobs[i + 1].fin && jobs[i + 1].c0 == jobs[i].c0 &&
         jobs[i + 1].c1 == jobs[i].c1) {
-      push_sweep(out, jobs[i], &jobs[i + 1]);
+      push_sweep(out, {jobs[i], jobs[i + 1]});
       i += 2;
     } else {
-      push_sweep(out, jobs[i], nullptr);
+      push_sweep(out, {jobs[i]});
       i += 1;
     }
   }
@@ -185,7 +186,7 @@ bool plan_slots(const std::vector<Sweep>& sw, std::vector<uint8_t>& tab, int& nj
   std::vector<int> first_of_job;
   for (const Sweep& w : sw) {
     const int first = static_cast<int>(first_of_job.size());
-    for (int j = 0; j < 2 && w.L[j]; ++j) first_of_job.push_back(first);
+    for (int j = 0; j < w.njobs; ++j) first_of_job.push_back(first);
   }
   njobs = static_cast<int>(first_of_job.size());
   if (njobs == 0) return false;
@@ -256,6 +257,138 @@ bool build_schedule(int s, int nch, bool wide, bool mode1, std::vector<Sweep>& o
   return true;
 }
 
+// Schedule of the CTA-pair kernel.  Its single issuing warp takes a job's slot
+// only before the job's own first MMA, so a sweep may hold as many jobs as
+// there are slots: bands of up to four adjacent levels share every staged
+// chunk.  At s = 7 the bands {8,7,6,5} and {4,3,2} stage 10 planes per chunk,
+// bands of two levels 16, and the staged bytes set the pace (12 KB per plane
+// and chunk against 64 cycles per MMA: with 16 planes the copies alone need
+// 1.0 of the MMAs' time at 54 bytes per clock, with 10 planes 0.65).  The bands
+// minimise the staged planes (dynamic programme over the levels), then the
+// jobs; they are issued from the highest level down, and so are the jobs of a
+// sweep, each sweep's longest MMA job first.  A band runs in K groups that
+// keep every job inside the exactness budget; the last job of all, level 2's
+// last group, completes the sum.
+bool build_pair(const PairSet& ps, int t, int nch, std::vector<Sweep>& out) {
+  out.clear();
+  constexpr long kInf = 1l << 40;
+  std::vector<long> cost(t + 6, kInf);
+  std::vector<int> choice(t + 6, 0);
+  cost[t + 1] = 0;
+  auto seg_of = [&](int L, int b) {   // chunks per group of the band L .. L+b-1
+    int seg = nch;
+    for (int l = L; l < L + b; ++l) {
+      const int n = ps.count(l);
+      if (n > 0 && seg_chunks(n) < seg) seg = seg_chunks(n);
+    }
+    return seg;
+  };
+  auto planes_of = [&](int L, int b) {
+    int np = 0;
+    for (int l = L; l < L + b; ++l) np = ps.planes(l) > np ? ps.planes(l) : np;
+    return np;
+  };
+  for (int L = t; L >= 2; --L)
+    for (int b = 1; b <= kSweepJobs && L + b <= t + 1; ++b) {
+      const int seg = seg_of(L, b);
+      if (seg < 1 || cost[L + b] >= kInf) continue;
+      const long jobs = static_cast<long>((nch + seg - 1) / seg) * b;
+      const long c = cost[L + b] + static_cast<long>(planes_of(L, b)) * nch * 64 + jobs;
+      if (c < cost[L]) {
+        cost[L] = c;
+        choice[L] = b;
+      }
+    }
+  if (cost[2] >= kInf) return false;
+  std::vector<std::pair<int, int>> bands;
+  for (int L = 2; L <= t; L += choice[L]) bands.push_back({L, choice[L]});
+  for (auto it = bands.rbegin(); it != bands.rend(); ++it) {
+    const int seg = seg_of(it->first, it->second);
+    const int G = (nch + seg - 1) / seg, size = (nch + G - 1) / G;
+    for (int c0 = 0; c0 < nch; c0 += size) {
+      const int c1 = c0 + size < nch ? c0 + size : nch;
+      std::vector<Job> jobs;
+      for (int L = it->first + it->second - 1; L >= it->first; --L)
+        if (ps.count(L) > 0) jobs.push_back(make_job(ps, L, c0, c1, L == 2 && c1 == nch));
+      push_sweep(out, jobs);
+    }
+  }
+  return true;
+}
+
+// Which CTA-pair variant sums the levels 2..t exactly: 0 none, 1 the 64-bit
+// state, 2 the 64-bit state with the 16 low bits put aside.  R is the state
+// before the final job's term; it must stay below 2^61 (the term is tested in
+// the kernel).  The low bits are put aside after the first band: what follows
+// has to weigh at least 2^16 (levels t-3 and down: 2^21 after a band of three),
+// and what came before has to fit in 64 bits.
+int pair_plan(int s, int t, int nch, int sa, int sb, std::vector<Sweep>* sweeps, int* stash_job) {
+  const PairSet ps{sa, sb};
+  std::vector<Sweep> sw;
+  if (!build_pair(ps, t, nch, sw)) return 0;
+  set_chunks_per_stage(s, sw);
+  const long double kk = static_cast<long double>(nch * kBK) * 127.0L * 127.0L;
+  const long double lim = 2305843009213693952.0L;   // 2^61
+  // everything but the final job's term, which is the last group of level 2
+  const Sweep& last = sw.back();
+  long double all = 0.0L;
+  for (int L = 2; L <= t; ++L) all += ps.count(L) * kk * powl(2.0L, 7.0L * (t - L));
+  const long double fin =
+      static_cast<long double>((last.k1c - last.k0c) * kBK) * 127.0L * 127.0L * powl(2.0L, 7.0L * (t - 2));
+  const long double r = all - fin;
+  int kind = 0, stash = -1;
+  if (r < lim) {
+    kind = 1;
+  } else {
+    // jobs of the first band
+    const int top = sw[0].L[0], bottom = sw[0].L[sw[0].njobs - 1];
+    int jobs = 0;
+    size_t i = 0;
+    for (; i < sw.size() && sw[i].L[0] == top; ++i) jobs += sw[i].njobs;
+    long double before = 0.0L;
+    for (int L = bottom; L <= t; ++L) before += ps.count(L) * kk * powl(2.0L, 7.0L * (t - L));
+    if (i < sw.size() && bottom > 2 && 7 * (t - bottom + 1) >= 16 && before < lim && r / 65536.0L < lim &&
+        fin / 65536.0L < 2.0L * lim) {
+      kind = 2;
+      stash = jobs - 1;
+    }
+  }
+  if (kind && sweeps) {
+    *sweeps = sw;
+    *stash_job = stash;
+  }
+  return kind;
+}
+
+// The constants that the kernel's drains leave in the 64-bit state, negated:
+// kMagicPair per unit of weight for two adjacent levels drained together,
+// kMagicBits for a job drained alone, in the units of the state before and
+// after the low bits were put aside.
+DrainConstants drained_constants(const std::vector<Sweep>& sw, int t, int stash_job) {
+  DrainConstants d{stash_job, 0, 0};
+  uint64_t sum[2] = {0, 0};
+  int jj = 0;
+  for (const Sweep& w : sw)
+    for (int j = 0; j < w.njobs;) {
+      const bool after = stash_job >= 0 && jj > stash_job;
+      const int units = after ? 16 : 0;
+      const int d1 = j + 1 < w.njobs ? w.L[j + 1] - w.L[j] : 0;
+      if ((d1 == 1 || d1 == -1) && !((w.final_mask >> j) & 1) && !((w.final_mask >> (j + 1)) & 1)) {
+        const int L = w.L[j] > w.L[j + 1] ? w.L[j] : w.L[j + 1];
+        sum[after] += static_cast<uint64_t>(static_cast<int64_t>(kMagicPair)) << (7 * (t - L) - units);
+        j += 2;
+        jj += 2;
+      } else {
+        sum[after] += static_cast<uint64_t>(kMagicBits) << (7 * (t - w.L[j]) - units);
+        j += 1;
+        jj += 1;
+      }
+    }
+  d.r_init = static_cast<long long>(0 - sum[0]);
+  d.r_init2 = static_cast<long long>(0 - sum[1]);
+  return d;
+}
+
 // The narrow variant keeps the state R in int64 and completes T = R + I_2 2^(7(t-2))
 // in its final job (in 64 bits when the warp's terms allow, else in 128): it
 // needs level 2 in one job and the sum of the other levels inside int64.
@@ -285,40 +418,37 @@ bool wide_ok(int s, int t, int k, int sa = 0, int sb = 0) {
   return exact_sum_bound_per_k(PairSet{sa ? sa : s, sb ? sb : s}, t) * static_cast<long double>(nch * kBK) < 8.5e37L;
 }
 
-// Device copy of a schedule: the sweeps, then the slot table (16-byte aligned).
-size_t schedule_bytes(size_t nsweeps, size_t ntab) { return nsweeps * sizeof(Sweep) + 16 + ntab; }
-
-int get_schedule(emul_handle_t h, int s, int t, int nch, bool wide, bool mode1, Sweep** dptr, int* count,
-                 SlotPlan* plan, int sa, int sb) {
-  const uint64_t key = (static_cast<uint64_t>(sa) << 40) | (static_cast<uint64_t>(sb) << 32) |
-                       (static_cast<uint64_t>(s) << 24) | (static_cast<uint64_t>(wide) << 23) |
-                       (static_cast<uint64_t>(mode1) << 22) | (static_cast<uint64_t>(t) << 13) |
-                       static_cast<uint64_t>(nch);   // nch < 2^13 (k <= 65536)
+int get_schedule(emul_handle_t h, int s, int t, int nch, bool wide, bool pair, bool mode1, Sweep** dptr, int* count,
+                 DrainConstants* drains, int sa, int sb) {
+  const uint64_t key = (static_cast<uint64_t>(pair) << 48) | (static_cast<uint64_t>(sa) << 40) |
+                       (static_cast<uint64_t>(sb) << 32) | (static_cast<uint64_t>(s) << 24) |
+                       (static_cast<uint64_t>(wide) << 23) | (static_cast<uint64_t>(mode1) << 22) |
+                       (static_cast<uint64_t>(t) << 13) | static_cast<uint64_t>(nch);   // nch < 2^13 (k <= 65536)
   auto it = h->sched_cache.find(key);
   if (it != h->sched_cache.end()) {
     *dptr = it->second.sched;
     *count = it->second.nsweeps;
-    *plan = it->second.plan;
+    *drains = it->second.drains;
     return EMUL_OK;
   }
   std::vector<Sweep> v;
   std::vector<uint8_t> tab;
-  SlotPlan sp{};
-  if (!build_schedule(s, nch, wide, mode1, v, tab, sp.njobs, sp.t0, sp.period, t, sa, sb))
+  int njobs, t0, period, stash = -1;
+  if (pair ? pair_plan(s, t, nch, sa, sb, &v, &stash) == 0
+           : !build_schedule(s, nch, wide, mode1, v, tab, njobs, t0, period, t, sa, sb))
     return set_error(h, EMUL_INVALID_ARG, "no schedule for this slice count / k");
-  const size_t off_tab = (v.size() * sizeof(Sweep) + 15) / 16 * 16;
-  std::vector<uint8_t> blob(off_tab + tab.size(), 0);
-  std::memcpy(blob.data(), v.data(), v.size() * sizeof(Sweep));
-  std::memcpy(blob.data() + off_tab, tab.data(), tab.size());
-  uint8_t* d = nullptr;
-  if (cudaMalloc(&d, blob.size()) != cudaSuccess) return set_error(h, EMUL_NO_WORKSPACE, "schedule allocation failed");
-  if (cudaMemcpy(d, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+  const DrainConstants dc = drained_constants(v, t, stash);
+  Sweep* d = nullptr;
+  if (cudaMalloc(&d, v.size() * sizeof(Sweep)) != cudaSuccess)
+    return set_error(h, EMUL_NO_WORKSPACE, "schedule allocation failed");
+  if (cudaMemcpy(d, v.data(), v.size() * sizeof(Sweep), cudaMemcpyHostToDevice) != cudaSuccess) {
+    cudaFree(d);
     return set_error(h, EMUL_CUDA_ERROR, "schedule upload failed");
-  sp.tab = d + off_tab;
-  h->sched_cache[key] = emul_handle_s::SchedEntry{reinterpret_cast<Sweep*>(d), static_cast<int>(v.size()), sp};
-  *dptr = reinterpret_cast<Sweep*>(d);
+  }
+  h->sched_cache[key] = emul_handle_s::SchedEntry{d, static_cast<int>(v.size()), dc};
+  *dptr = d;
   *count = static_cast<int>(v.size());
-  *plan = sp;
+  *drains = dc;
   return EMUL_OK;
 }
 
@@ -454,30 +584,38 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
     rc = check_cuda(h, cudaGetLastError(), "zero levels");
     if (rc) return rc;
   }
-  // the narrow test plans a schedule; it is made once per (s, t, K chunks)
+  const int nch = (k + kBK - 1) / kBK;
+  // the variant tests plan a schedule; they are made once per (s, t, K chunks)
   const uint64_t nkey = (static_cast<uint64_t>(s_a) << 48) | (static_cast<uint64_t>(s_b) << 40) |
-                        (static_cast<uint64_t>(s) << 32) | (static_cast<uint64_t>(t) << 16) |
-                        static_cast<uint64_t>((k + kBK - 1) / kBK);
+                        (static_cast<uint64_t>(s) << 32) | (static_cast<uint64_t>(t) << 16) | static_cast<uint64_t>(nch);
   auto nit = h->narrow_cache.find(nkey);
-  if (nit == h->narrow_cache.end()) nit = h->narrow_cache.emplace(nkey, narrow_ok(s, k, t, s_a, s_b)).first;
-  const bool wide = !nit->second;
+  if (nit == h->narrow_cache.end()) {
+    const int kinds = (narrow_ok(s, k, t, s_a, s_b) ? 4 : 0) |
+                      pair_plan(s, t, nch, s_a, s_b, nullptr, nullptr);
+    nit = h->narrow_cache.emplace(nkey, kinds).first;
+  }
+  // CTA pairs (cta_group::2) once there are two 128-row tiles: each SM stages
+  // half of B, a quarter less than alone
+  GemmConfig cfg{Variant::kWide, 64, false};
+  const int pair_kind = nit->second & 3;
+  if (pair_kind && m > 128 && h->nsm >= 2) {
+    GemmConfig c{Variant::kPair, 128, pair_kind == 2};
+    const long tiles = static_cast<long>((m + 255) / 256) * ((n + 127) / 128);
+    if (!lower && tiles < h->nsm / 2) c.bn = 64;
+    size_t smem_pair = 0;
+    if (gemm_stages(c, s, &smem_pair) >= 2 && gemm_pair_capacity(smem_pair) >= 1) cfg = c;   // else one CTA per tile
+  }
+  const bool pair = cfg.var == Variant::kPair;
+  if (!pair && (nit->second & 4)) cfg = GemmConfig{Variant::kNarrow, 128, false};
+  const bool wide = cfg.var == Variant::kWide;
   if (wide && mode == 0 && !wide_ok(s, t, k, s_a, s_b))
     return set_error(h, EMUL_NOT_SUPPORTED, "threshold too high for this k: the 128-bit exact sum could overflow");
-  const int nch = (k + kBK - 1) / kBK;
   Sweep* sched = nullptr;
   int nsweeps = 0;
-  SlotPlan plan{};
-  rc = get_schedule(h, s, t, nch, wide, mode == 1, &sched, &nsweeps, &plan, s_a, s_b);
+  DrainConstants drains{};
+  rc = get_schedule(h, s, t, nch, wide, pair, mode == 1, &sched, &nsweeps, &drains, s_a, s_b);
   if (rc) return rc;
-  const int BN = wide ? 64 : 128;
-  // CTA pairs (cta_group::2) for the 128-column tile once there are two
-  // 128-row tiles: each SM stages half of B, a quarter less than alone
-  bool pair = !wide && m > 128 && h->nsm >= 2;
-  if (pair) {
-    size_t smem_pair = 0;
-    gemm_stages(false, s, true, &smem_pair);
-    pair = gemm_pair_capacity(smem_pair) >= 1;   // else one CTA per tile
-  }
+  const int BN = cfg.bn;
   CUtensorMap tmA, tmB;
   rc = encode_slices_map(h, &tmA, sa, m, k, kp, s, 128);
   if (rc) return rc;
@@ -498,7 +636,9 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
   a.fb = fb;
   a.sched = sched;
   a.nsweeps = nsweeps;
-  a.slots = plan;
+  a.stash_job = drains.stash_job;
+  a.r_init = drains.r_init;
+  a.r_init2 = drains.r_init2;
   a.tiles_m = pair ? (m + 255) / 256 : (m + 127) / 128;
   a.tiles_n = (n + BN - 1) / BN;
   a.lower = lower ? 1 : 0;
@@ -517,7 +657,7 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
   a.wait_limit = h->wait_limit;
 
   size_t smem = 0;
-  const int stages = gemm_stages(wide, s, pair, &smem);
+  const int stages = gemm_stages(cfg, s, &smem);
   if (stages < 2) return set_error(h, EMUL_NOT_SUPPORTED, "slice tiles do not fit in shared memory");
   const int units = pair ? h->nsm / 2 : h->nsm;   // CTAs, or CTA pairs
   const int grid = (a.ntiles < units ? a.ntiles : units) * (pair ? 2 : 1);
@@ -541,7 +681,7 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
     rec.bytes = cells * (beta != 0.0 ? 16.0 : 8.0) + static_cast<double>(s) * 2.0 * k * (m + (same ? 0 : n));
     cudaEventRecord(rec.e0, h->stream);
   }
-  rc = check_cuda(h, launch_gemm(h->stream, wide, pair, tmA, tmB, a, grid, stages, smem), "gemm kernel");
+  rc = check_cuda(h, launch_gemm(h->stream, cfg, tmA, tmB, a, grid, stages, smem), "gemm kernel");
   h->launches++;
   if (h->prof) {
     cudaEventRecord(rec.e1, h->stream);
@@ -720,11 +860,50 @@ int emul_schedule(int slices, int k, int wide, int level_sums, int threshold, in
     return EMUL_INVALID_ARG;
   for (size_t i = 0; i < v.size(); ++i) {
     const Sweep& w = v[i];
-    const int row[EMUL_SWEEP_INTS] = {w.k0c,   w.k1c,      w.L[0],     w.L[1],    w.pb[0], w.pb[1],
-                                      w.pe[0], w.pe[1],    w.flags[0], w.flags[1], w.nplanes, w.kcs};
+    const int row[EMUL_SWEEP_INTS] = {w.k0c,        w.k1c,        w.L[0],           w.L[1],
+                                      w.pp[0] & 15, w.pp[1] & 15, w.pp[0] >> 4,     w.pp[1] >> 4,
+                                      w.final_mask & 1, w.final_mask >> 1, w.nplanes, w.kcs};
     for (int j = 0; j < EMUL_SWEEP_INTS; ++j) sweeps[i * EMUL_SWEEP_INTS + j] = row[j];
   }
   std::memcpy(table, tab.data(), tab.size());
+  return EMUL_OK;
+}
+
+int emul_schedule_pair(int slices_a, int slices_b, int k, int threshold, int* sweeps, int cap_sweeps, int* meta) {
+  using namespace emul;
+  if (!meta) return EMUL_INVALID_ARG;
+  meta[0] = meta[1] = 0;
+  meta[2] = -1;
+  const int s = slices_a > slices_b ? slices_a : slices_b;
+  if (slices_a < 1 || slices_b < 1 || s > kMaxSlices || k < 1 || k > 16384 * 4 ||
+      (threshold != 0 && (threshold < 2 || threshold > slices_a + slices_b)))
+    return EMUL_INVALID_ARG;
+  std::vector<Sweep> v;
+  int stash = -1;
+  const int kind = pair_plan(s, threshold ? threshold : s + 1, (k + kBK - 1) / kBK, slices_a, slices_b, &v, &stash);
+  if (!kind) return EMUL_INVALID_ARG;
+  meta[0] = static_cast<int>(v.size());
+  meta[1] = kind;
+  meta[2] = stash;
+  if (!sweeps || cap_sweeps < static_cast<int>(v.size())) return EMUL_INVALID_ARG;
+  for (size_t i = 0; i < v.size(); ++i) {
+    const Sweep& w = v[i];
+    int* r = sweeps + i * EMUL_PAIR_SWEEP_INTS;
+    int fin = -1;
+    for (int j = 0; j < w.njobs; ++j)
+      if ((w.final_mask >> j) & 1) fin = j;
+    r[0] = w.k0c;
+    r[1] = w.k1c;
+    r[2] = w.njobs;
+    r[3] = fin;
+    r[4] = w.nplanes;
+    r[5] = w.kcs;
+    for (int j = 0; j < kSweepJobs; ++j) {
+      r[6 + 3 * j] = w.L[j];
+      r[7 + 3 * j] = w.pp[j] & 15;
+      r[8 + 3 * j] = w.pp[j] >> 4;
+    }
+  }
   return EMUL_OK;
 }
 
@@ -795,7 +974,7 @@ namespace emul {
 namespace {
 
 constexpr size_t kNoAllocScratchBytes = size_t(16) << 20;   // 16 MiB
-constexpr size_t kNoAllocSchedBytes = 16384;                // sweeps (16 B each) and the slot table
+constexpr size_t kNoAllocSchedBytes = 16384;                // sweeps (16 B each); the slot plan counts towards the limit
 constexpr int kNoAllocMaxDevices = 64;
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
@@ -889,17 +1068,13 @@ extern "C" int emul_dgemm_noalloc(void* stream, int m, int n, int k, double alph
   const int nch = (k + kBK - 1) / kBK;
   std::vector<Sweep> v;
   std::vector<uint8_t> tab;
-  SlotPlan plan{};
-  if (!build_schedule(slices, nch, wide, false, v, tab, plan.njobs, plan.t0, plan.period)) return EMUL_INVALID_ARG;
-  const size_t off_tab = (v.size() * sizeof(Sweep) + 15) / 16 * 16;
-  if (off_tab + tab.size() > kNoAllocSchedBytes) return EMUL_NO_WORKSPACE;
-  std::vector<uint8_t> blob(off_tab + tab.size(), 0);
-  std::memcpy(blob.data(), v.data(), v.size() * sizeof(Sweep));
-  std::memcpy(blob.data() + off_tab, tab.data(), tab.size());
-  plan.tab = reinterpret_cast<const uint8_t*>(sched) + off_tab;
+  int njobs, t0, period;
+  if (!build_schedule(slices, nch, wide, false, v, tab, njobs, t0, period)) return EMUL_INVALID_ARG;
+  if (v.size() * sizeof(Sweep) + tab.size() > kNoAllocSchedBytes) return EMUL_NO_WORKSPACE;
+  const DrainConstants drains = drained_constants(v, slices + 1, -1);
   // the status word must start at zero; the rest is fully rewritten by this call
   if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return EMUL_CUDA_ERROR;
-  if (cudaMemcpyAsync(sched, blob.data(), blob.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
+  if (cudaMemcpyAsync(sched, v.data(), v.size() * sizeof(Sweep), cudaMemcpyHostToDevice, st) != cudaSuccess)
     return EMUL_CUDA_ERROR;
   if (launch_split(st, m, k, A, 1, lda, slices, ea, sa, kp) != cudaSuccess) return EMUL_CUDA_ERROR;
   if (launch_split(st, n, k, B, ldb, 1, slices, fb, sb, kp) != cudaSuccess) return EMUL_CUDA_ERROR;
@@ -923,17 +1098,18 @@ extern "C" int emul_dgemm_noalloc(void* stream, int m, int n, int k, double alph
   a.fb = fb;
   a.sched = sched;
   a.nsweeps = static_cast<int>(v.size());
-  a.slots = plan;
+  a.stash_job = drains.stash_job;
+  a.r_init = drains.r_init;
+  a.r_init2 = drains.r_init2;
   a.tiles_m = (m + 127) / 128;
   a.tiles_n = (n + BN - 1) / BN;
   a.ntiles = a.tiles_m * a.tiles_n;
   a.status = status;
   a.wait_limit = 2000000000LL;
-  const size_t stage = gemm_stage_bytes(wide, slices, false);
-  int stages = static_cast<int>((232448 - 1024 - 2048) / stage);
-  if (stages > kMaxStagesCfg) stages = kMaxStagesCfg;
+  const GemmConfig cfg = wide ? GemmConfig{Variant::kWide, 64, false} : GemmConfig{Variant::kNarrow, 128, false};
+  size_t smem = 0;
+  const int stages = gemm_stages(cfg, slices, &smem);
   if (stages < 2) return EMUL_NOT_SUPPORTED;
   const int grid = a.ntiles < d->nsm ? a.ntiles : d->nsm;
-  return launch_gemm(st, wide, false, tmA, tmB, a, grid, stages, stages * stage + 1024) == cudaSuccess ? EMUL_OK
-                                                                                             : EMUL_CUDA_ERROR;
+  return launch_gemm(st, cfg, tmA, tmB, a, grid, stages, smem) == cudaSuccess ? EMUL_OK : EMUL_CUDA_ERROR;
 }

@@ -12,29 +12,35 @@ constexpr int kBK = 32;                  // K elements per staged chunk (64 B of
 constexpr int kMaxStagesCfg = 8;         // deepest ring of staged chunks
 constexpr int kExactBudget = 1040;       // k * pairs per accumulator: 1040 * 127^2 < 2^24
 
-// One sweep of the product schedule: one or two accumulator jobs over the K
+// One sweep of the product schedule: up to four accumulator jobs over the K
 // chunks [k0c, k1c), sharing the staged slice tiles of each chunk.  A job
 // sums the slice pairs (p, L-p), p = pb..pe, of one level L into one TMEM slot.
 // The epilogue takes the jobs in schedule order and adds each job's sum with
-// its weight into the state, R += I 2^(7(t-L)); a job flagged kFinal (the last
-// job of the 64-bit variant) completes T = R + I 2^(7(t-L)), rounds it and
+// its weight into the state, R += I 2^(7(t-L)); the job in final_mask (the last
+// job of the 64-bit variants) completes T = R + I 2^(7(t-L)), rounds it and
 // updates C.
-enum JobFlag : int8_t { kFinal = 1 };
+constexpr int kSweepJobs = 4;
 struct Sweep {
-  int16_t k0c, k1c;    // chunk range
-  int8_t L[2];         // job levels (L[1] = 0: one job)
-  int8_t pb[2], pe[2]; // pair ranges
-  int8_t flags[2];     // JobFlag bits of the two jobs
-  int8_t nplanes;      // slice planes 1..nplanes of A and of B are staged
-  int8_t kcs;          // K chunks per stage (kcs * nplanes <= s tiles of A and of B)
+  int16_t k0c, k1c;       // chunk range
+  int8_t L[kSweepJobs];   // job levels (0: no job)
+  uint8_t pp[kSweepJobs]; // pair ranges, pb | pe << 4
+  int8_t nplanes;         // slice planes 1..nplanes of A and of B are staged
+  int8_t kcs;             // K chunks per stage (kcs * nplanes <= s tiles of A and of B)
+  int8_t njobs;
+  int8_t final_mask;      // bit j: job j completes and rounds the sum
 };
+static_assert(sizeof(Sweep) == 16, "a sweep is one 16-byte record");
 
-// Slot assignment of the jobs: TMEM slot (bits 0-1) and the parity of the
-// slot's use count (bit 2) for job j of the tile-phase ph, at tab[ph * njobs + j];
-// the i-th tile of a CTA uses phase i (i < t0) or t0 + (i - t0) % period.
-struct SlotPlan {
-  const uint8_t* tab;
-  int njobs, t0, period;
+// Constants that the drains of the 64-bit state leave in it (gemm_kernel.cuh):
+// kMagicBits per unit of weight for a job drained alone, kMagicPair for two
+// adjacent levels drained together (129 kMagicBits modulo 2^32, signed).
+constexpr int kMagicBits = 0x4B400000;
+constexpr long long kMagicPair = -348127232;
+
+// Where the low bits are put aside and what the state starts from (GemmArgs).
+struct DrainConstants {
+  int stash_job;            // job of the tile after which the low bits are put aside (-1: never)
+  long long r_init, r_init2;
 };
 
 struct GemmArgs {
@@ -47,7 +53,9 @@ struct GemmArgs {
   const int32_t* fb;        // column scales of B [N]
   const Sweep* sched;       // device array
   int nsweeps;
-  SlotPlan slots;           // TMEM slot of every job (device table)
+  int stash_job;            // job of the tile after which the low bits are put aside (STASH variants)
+  long long r_init;         // the state's start: minus the drains' constants (64-bit variants, mode 0)
+  long long r_init2;        // the same for the jobs after stash_job, in the units of the state then
   int tiles_m, tiles_n, ntiles;
   int lower;                // 1: only entries with row >= col are written
   int tri;                  // 1: tiles enumerated over the lower triangle (square tiles)
@@ -61,14 +69,30 @@ struct GemmArgs {
 cudaError_t launch_split(cudaStream_t st, int rows, int k, const double* X, long rs, long cs, int s, int32_t* exps,
                          uint16_t* out, long ldk);
 
-// BN = 128 with an int64 state (wide = false) or BN = 64 with a 128-bit state
-// (wide = true).  pair (128-column tile only): clusters of two CTAs, tiles of
-// 256 rows (args.tiles_m counts them), tmB staged BN/2 rows per CTA, grid even.
-cudaError_t launch_gemm(cudaStream_t st, bool wide, bool pair, const CUtensorMap& tmA, const CUtensorMap& tmB,
+// The product kernel's variants.  kWide: 64-column tiles, 128-bit state, one CTA
+// per tile.  kNarrow: 128-column tiles, 64-bit state, one CTA per tile.  kPair:
+// clusters of two CTAs, tiles of 256 rows (args.tiles_m counts them) x bn
+// columns (tmB stages bn / 2 rows per CTA, grid even), 64-bit state, with the
+// 16 low bits of the sum put aside in shared memory if `stash`.
+enum class Variant { kWide, kNarrow, kPair };
+struct GemmConfig {
+  Variant var;
+  int bn;                   // tile columns: 64 (kWide), 128 (kNarrow), 128 or 64 (kPair)
+  bool stash;               // kPair only
+};
+
+cudaError_t launch_gemm(cudaStream_t st, const GemmConfig& cfg, const CUtensorMap& tmA, const CUtensorMap& tmB,
                         const GemmArgs& args, int grid, int stages, size_t smem_bytes);
-size_t gemm_stage_bytes(bool wide, int s, bool pair);
+// The update modes of C, each compiled in a source file of its own.
+cudaError_t launch_gemm_sub(cudaStream_t st, const GemmConfig& cfg, const CUtensorMap& tmA, const CUtensorMap& tmB,
+                            const GemmArgs& args, int grid, int stages, size_t smem_bytes);
+cudaError_t launch_gemm_set(cudaStream_t st, const GemmConfig& cfg, const CUtensorMap& tmA, const CUtensorMap& tmB,
+                            const GemmArgs& args, int grid, int stages, size_t smem_bytes);
+cudaError_t launch_gemm_general(cudaStream_t st, const GemmConfig& cfg, const CUtensorMap& tmA,
+                                const CUtensorMap& tmB, const GemmArgs& args, int grid, int stages,
+                                size_t smem_bytes);
 // Ring stages of a launch and its shared-memory bytes.
-int gemm_stages(bool wide, int s, bool pair, size_t* smem_bytes);
+int gemm_stages(const GemmConfig& cfg, int s, size_t* smem_bytes);
 // CTA pairs that can be resident at once with this much shared memory.
 int gemm_pair_capacity(size_t smem_bytes);
 

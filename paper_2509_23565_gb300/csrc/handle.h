@@ -20,12 +20,13 @@ struct emul_handle_s {
   void* ws = nullptr;               // workspace (device)
   size_t ws_bytes = 0;
   struct SchedEntry {
-    emul::Sweep* sched;             // device: sweeps, then the slot table
+    emul::Sweep* sched;             // device
     int nsweeps;
-    emul::SlotPlan plan;
+    emul::DrainConstants drains;
   };
   std::map<uint64_t, SchedEntry> sched_cache;   // (slices of A / B, s, wide, level-sum mode, threshold, chunks) -> device schedule
-  std::map<uint64_t, bool> narrow_cache;        // (s, t, chunks) -> the 128-column variant applies
+  std::map<uint64_t, int> narrow_cache;         // (s, t, chunks) -> variants that apply: bit 2 one CTA per
+                                                // 128-column tile, bits 0-1 CTA pairs (1, or 2 with low bits aside)
   std::string last_error;
   void* encode_fn = nullptr;        // cuTensorMapEncodeTiled
   long long wait_limit = 2000000000LL;

@@ -82,16 +82,32 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint6
           d_tmem),
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
 }
-// The same MMA issued by one elected lane of a converged warp.  The whole warp
-// runs the issuing loop, so every operand is warp-uniform and stays in the
-// uniform datapath; one thread alone recomputing descriptors issues an MMA
-// only every ~84 cycles, short of the 64 a 128 x 128 x 16 MMA takes.
-__device__ __forceinline__ void mma_bf16_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                               uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred e, p;\nelect.sync _|e, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+// Both K = 16 MMAs of a staged K chunk of 32 (64-byte rows: the second one reads
+// 32 bytes, two descriptor units, further), issued by one elected lane of a
+// converged warp.  The whole warp runs the issuing loop, so every operand is
+// warp-uniform and stays in the uniform datapath; one thread alone recomputing
+// descriptors issues an MMA only every ~84 cycles, short of the 64 a 128 x 128
+// x 16 MMA takes.  Descriptors come as their low word (the start address, the
+// only part that changes) and high word.
+template <bool PAIR>
+__device__ __forceinline__ void mma_bf16_k32_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                                   uint32_t idesc, uint32_t accumulate) {
+  if constexpr (PAIR)
+    asm volatile(
+        "{\n.reg .pred e, p;\n.reg .b32 a1, b1;\n.reg .b64 da, db, dc, dd;\nelect.sync _|e, 0xffffffff;\n"
+        "setp.ne.b32 p, %5, 0;\nadd.u32 a1, %1, 2;\nadd.u32 b1, %2, 2;\n"
+        "mov.b64 da, {%1, %3};\nmov.b64 db, {%2, %3};\nmov.b64 dc, {a1, %3};\nmov.b64 dd, {b1, %3};\n"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], dc, dd, %4, 1;\n}\n" ::"r"(d_tmem),
+        "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate));
+  else
+    asm volatile(
+        "{\n.reg .pred e, p;\n.reg .b32 a1, b1;\n.reg .b64 da, db, dc, dd;\nelect.sync _|e, 0xffffffff;\n"
+        "setp.ne.b32 p, %5, 0;\nadd.u32 a1, %1, 2;\nadd.u32 b1, %2, 2;\n"
+        "mov.b64 da, {%1, %3};\nmov.b64 db, {%2, %3};\nmov.b64 dc, {a1, %3};\nmov.b64 dd, {b1, %3};\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], dc, dd, %4, 1;\n}\n" ::"r"(d_tmem),
+        "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate));
 }
 // tcgen05.commit from one elected lane of a converged warp.
 __device__ __forceinline__ void mma_commit_elect(uint64_t* bar) {
@@ -155,14 +171,6 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem, uint32_t nco
 }
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
-}
-// M = 256 MMA over the pair, issued by one elected lane of rank 0.
-__device__ __forceinline__ void mma_bf16_pair_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                                    uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred e, p;\nelect.sync _|e, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
 }
 // Commit of the pair's MMAs arriving on `bar` at the same offset in both CTAs.
 __device__ __forceinline__ void mma_commit_pair_both_elect(uint64_t* bar) {
