@@ -536,6 +536,68 @@ size_t gemm_workspace_bytes(int m, int n, int k, int s, bool same_operand) {
   return b + kAlign;
 }
 
+namespace {
+
+// Event bracket of one product launch while profiling is enabled.
+int prof_begin(emul_handle_t h, emul_handle_s::ProfRec* rec, int m, int n, int k, int s, int t, int s_a, int s_b,
+               bool lower, double beta, bool same) {
+  if (!h->prof) return EMUL_OK;
+  for (int i = 0; i < 2; ++i) {
+    cudaEvent_t ev;
+    if (!h->event_pool.empty()) {
+      ev = h->event_pool.back();
+      h->event_pool.pop_back();
+    } else if (cudaEventCreate(&ev) != cudaSuccess) {
+      return set_error(h, EMUL_CUDA_ERROR, "event creation failed");
+    }
+    (i == 0 ? rec->e0 : rec->e1) = ev;
+  }
+  // slice pairs kept: those of the levels L = 2..t (s(s+1)/2 at t = s + 1)
+  double P = 0.0;
+  for (int L = 2; L <= t; ++L) P += PairSet{s_a, s_b}.count(L);
+  const double cells = lower ? 0.5 * m * (double)n : static_cast<double>(m) * n;
+  rec->flops = 2.0 * cells * k * P;
+  rec->bytes = cells * (beta != 0.0 ? 16.0 : 8.0) + static_cast<double>(s) * 2.0 * k * (m + (same ? 0 : n));
+  cudaEventRecord(rec->e0, h->stream);
+  return EMUL_OK;
+}
+
+void prof_end(emul_handle_t h, const emul_handle_s::ProfRec& rec) {
+  if (!h->prof) return;
+  cudaEventRecord(rec.e1, h->stream);
+  h->recs.push_back(rec);
+}
+
+// Whether the m x n block C (ldc) and the rows x k operand X share an entry.
+// Blocks of different leading dimensions whose address ranges meet count as
+// sharing one.
+bool blocks_meet(const double* C, long ldc, int m, int n, const Operand& X, int rows, int k) {
+  const bool by_rows = X.rs == 1;
+  const long ld = by_rows ? X.cs : X.rs, xr = by_rows ? rows : k, xc = by_rows ? k : rows;
+  const long c_len = (n - 1) * ldc + m, x_len = (xc - 1) * ld + xr;
+  const long d = X.ptr - C;                 // of X's first entry from C's
+  if (d >= c_len || -d >= x_len) return false;
+  if (ld != ldc || xr > ld || m > ldc) return true;
+  // position of X's first entry in C's columns: row r0 in (-ld, ld), for both columns it may be counted in
+  const long q = d >= 0 ? d / ld : -((-d + ld - 1) / ld);
+  const long r = d - q * ld;                // 0 <= r < ld
+  auto meet = [&](long r0, long c0) { return r0 < m && r0 + xr > 0 && c0 < n && c0 + xc > 0; };
+  return meet(r, q) || meet(r - ld, q + 1);
+}
+
+// The one-launch product reads its operands while other blocks write C, where
+// the sliced product reads all of both first.  C may lie over an operand only
+// when each block alone reads what it overwrites: over B with one row of tiles,
+// entry for entry, or over A with one column of tiles.
+bool small_product_alias_ok(int m, int n, int k, const Operand& A, const Operand& B, const double* C, long ldc) {
+  const bool one_row = m <= 128, one_col = n <= 32;
+  if (blocks_meet(C, ldc, m, n, A, m, k) && !(one_col && (one_row || (A.ptr == C && A.rs == 1 && A.cs == ldc)))) return false;
+  if (blocks_meet(C, ldc, m, n, B, n, k) && !(one_row && (one_col || (B.ptr == C && B.cs == 1 && B.rs == ldc)))) return false;
+  return true;
+}
+
+}  // namespace
+
 int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Operand B, double beta, double* C,
              long ldc, int s, bool lower, int mode, int32_t* levels, long ldl, long ldl_plane, size_t ws_offset,
              int t, int s_a, int s_b) {
@@ -554,6 +616,16 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
     return check_cuda(h, cudaGetLastError(), "scale C");
   }
   const bool same = (A.ptr == B.ptr && A.rs == B.rs && A.cs == B.cs && m == n);
+  if (mode == 0 && !lower && t == s + 1 && s_a == s_b && small_product_fits(m, n, k, s, h->nsm) &&
+      small_product_alias_ok(m, n, k, A, B, C, ldc)) {
+    emul_handle_s::ProfRec rec{};
+    if (int pe = prof_begin(h, &rec, m, n, k, s, t, s_a, s_b, false, beta, same)) return pe;
+    const int rc_small = check_cuda(h, launch_small_product(h->stream, m, n, k, alpha, A.ptr, A.rs, A.cs, B.ptr, B.rs, B.cs, beta,
+                                                  C, ldc, s, h->d_status, h->wait_limit), "small product");
+    h->launches++;
+    prof_end(h, rec);
+    return rc_small;
+  }
   const size_t need = ws_offset + gemm_workspace_bytes(m, n, k, s, same);
   int rc = reserve_workspace(h, need);
   if (rc) return rc;
@@ -570,14 +642,11 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
     w += align_up(static_cast<size_t>(s) * n * kp * 2);
     fb = reinterpret_cast<int32_t*>(w);
   }
-  rc = check_cuda(h, launch_split(h->stream, m, k, A.ptr, A.rs, A.cs, s, ea, sa, kp), "split A");
+  rc = check_cuda(h, same ? launch_split(h->stream, m, k, A.ptr, A.rs, A.cs, s, ea, sa, kp)
+                          : launch_split2(h->stream, k, s, kp, m, A.ptr, A.rs, A.cs, ea, sa, n, B.ptr, B.rs, B.cs, fb, sb),
+                  "split");
   if (rc) return rc;
   h->launches++;
-  if (!same) {
-    rc = check_cuda(h, launch_split(h->stream, n, k, B.ptr, B.rs, B.cs, s, fb, sb, kp), "split B");
-    if (rc) return rc;
-    h->launches++;
-  }
   if (mode == 1) {
     h->launches++;
     zero_levels_kernel<<<256, 256, 0, h->stream>>>(m, n, s, levels, ldl, ldl_plane);
@@ -662,31 +731,11 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
   const int units = pair ? h->nsm / 2 : h->nsm;   // CTAs, or CTA pairs
   const int grid = (a.ntiles < units ? a.ntiles : units) * (pair ? 2 : 1);
   emul_handle_s::ProfRec rec{};
-  if (h->prof) {
-    for (int i = 0; i < 2; ++i) {
-      cudaEvent_t ev;
-      if (!h->event_pool.empty()) {
-        ev = h->event_pool.back();
-        h->event_pool.pop_back();
-      } else if (cudaEventCreate(&ev) != cudaSuccess) {
-        return set_error(h, EMUL_CUDA_ERROR, "event creation failed");
-      }
-      (i == 0 ? rec.e0 : rec.e1) = ev;
-    }
-    // slice pairs kept: those of the levels L = 2..t (s(s+1)/2 at t = s + 1)
-    double P = 0.0;
-    for (int L = 2; L <= t; ++L) P += PairSet{s_a, s_b}.count(L);
-    const double cells = lower ? 0.5 * m * (double)n : static_cast<double>(m) * n;
-    rec.flops = 2.0 * cells * k * P;
-    rec.bytes = cells * (beta != 0.0 ? 16.0 : 8.0) + static_cast<double>(s) * 2.0 * k * (m + (same ? 0 : n));
-    cudaEventRecord(rec.e0, h->stream);
-  }
+  rc = prof_begin(h, &rec, m, n, k, s, t, s_a, s_b, lower, beta, same);
+  if (rc) return rc;
   rc = check_cuda(h, launch_gemm(h->stream, cfg, tmA, tmB, a, grid, stages, smem), "gemm kernel");
   h->launches++;
-  if (h->prof) {
-    cudaEventRecord(rec.e1, h->stream);
-    h->recs.push_back(rec);
-  }
+  prof_end(h, rec);
   return rc;
 }
 
@@ -1076,8 +1125,8 @@ extern "C" int emul_dgemm_noalloc(void* stream, int m, int n, int k, double alph
   if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return EMUL_CUDA_ERROR;
   if (cudaMemcpyAsync(sched, v.data(), v.size() * sizeof(Sweep), cudaMemcpyHostToDevice, st) != cudaSuccess)
     return EMUL_CUDA_ERROR;
-  if (launch_split(st, m, k, A, 1, lda, slices, ea, sa, kp) != cudaSuccess) return EMUL_CUDA_ERROR;
-  if (launch_split(st, n, k, B, ldb, 1, slices, fb, sb, kp) != cudaSuccess) return EMUL_CUDA_ERROR;
+  if (launch_split2(st, k, slices, kp, m, A, 1, lda, ea, sa, n, B, ldb, 1, fb, sb) != cudaSuccess)
+    return EMUL_CUDA_ERROR;
   const int BN = wide ? 64 : 128;
   CUtensorMap tmA, tmB;
   rc = noalloc_map(&tmA, sa, m, k, kp, slices, 128);

@@ -69,6 +69,17 @@ struct GemmArgs {
 cudaError_t launch_split(cudaStream_t st, int rows, int k, const double* X, long rs, long cs, int s, int32_t* exps,
                          uint16_t* out, long ldk);
 
+// Both operands of a product in one launch (same k, s and ldk).
+cudaError_t launch_split2(cudaStream_t st, int k, int s, long ldk, int rows_a, const double* A, long ars, long acs,
+                          int32_t* ea, uint16_t* sa, int rows_b, const double* B, long brs, long bcs, int32_t* fb,
+                          uint16_t* sb);
+
+// One-launch product for short K and few tiles (gemm_small.cu).
+bool small_product_fits(int m, int n, int k, int s, int nsm);
+cudaError_t launch_small_product(cudaStream_t st, int m, int n, int k, double alpha, const double* A, long ars,
+                                 long acs, const double* B, long brs, long bcs, double beta, double* C, long ldc,
+                                 int s, int* status, long long wait_limit);
+
 // The product kernel's variants.  kWide: 64-column tiles, 128-bit state, one CTA
 // per tile.  kNarrow: 128-column tiles, 64-bit state, one CTA per tile.  kPair:
 // clusters of two CTAs, tiles of 256 rows (args.tiles_m counts them) x bn

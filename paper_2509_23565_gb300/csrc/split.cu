@@ -1,4 +1,4 @@
-// Scale extraction and slicing of a GEMM operand (arXiv 2509.23565, Section 2,
+// Scale extraction and slicing of GEMM operands (arXiv 2509.23565, Section 2,
 // Eq. 1-4): per row r of a rows x k operand,
 //   e_r = smallest e with max_c |x(r,c)| < 2^e   (0 for a zero row, NONFINITE for Inf/NaN),
 //   N   = trunc(x * 2^(7s - e_r)),  |N| < 2^(7s),
@@ -9,163 +9,161 @@
 //   out[(p*rows + r)*ldk + c], the layout the TMA loads of the product read.
 #include <cstdint>
 #include <cuda_runtime.h>
-#include <cuda_bf16.h>
 
 #include "emul_internal.h"
+#include "slice.cuh"
 
 namespace emul {
+namespace {
 
-__device__ __forceinline__ int exponent_of_maxbits(uint64_t u) {
-  if (u >= 0x7FF0000000000000ull) return kNonFinite;
-  if (u == 0) return 0;
-  const int E = static_cast<int>(u >> 52);
-  if (E > 0) return E - 1022;                      // |x| in [2^(E-1023), 2^(E-1022))
-  return -1010 - __clzll(static_cast<long long>(u));  // subnormal: |x| = u * 2^-1074
-}
+constexpr int kSplitThreads = 256;
+constexpr int kSplitRows = 8;            // rows per block
 
-// |N| = trunc(|x| * 2^(W - e)) for |x| < 2^e; u = |x| bit pattern.
-__device__ __forceinline__ uint64_t scaled_magnitude(uint64_t u, int e, int W) {
-  const int E = static_cast<int>(u >> 52);
-  const uint64_t M = (u & 0xFFFFFFFFFFFFFull) | (E ? (1ull << 52) : 0ull);
-  const int sh = (E ? E : 1) - 1075 + W - e;      // x = M * 2^((E?E:1) - 1075)
-  if (sh >= 0) return M << sh;                     // sh <= W - 53 <= 3
-  const int r = -sh;
-  return r >= 64 ? 0ull : (M >> r);
-}
+struct SplitArgs {
+  const double* X;
+  long rs, cs;
+  int rows, k;
+  int32_t* exps;
+  uint16_t* out;
+  long ldk;
+  int blocks;       // blocks of this operand
+};
 
-__device__ __forceinline__ uint16_t digit_bf16(const uint16_t* lut, uint64_t mag, bool neg, int shift) {
-  const int d = static_cast<int>((mag >> shift) & 127ull);
-  return lut[neg ? 127 - d : 127 + d];
-}
-
-__device__ void fill_lut(uint16_t* lut) {
-  for (int i = threadIdx.x; i < 255; i += blockDim.x)
-    lut[i] = __bfloat16_as_ushort(__float2bfloat16_rn(static_cast<float>(i - 127)));
-}
-
-// Rows contiguous (rs == 1): tile of 64 rows per block, transposed through shared memory.
-__global__ void __launch_bounds__(256) split_rowcontig_kernel(int rows, int k, const double* __restrict__ X,
-                                                              long cs, int s, int32_t* __restrict__ exps,
-                                                              uint16_t* __restrict__ out, long ldk) {
-  __shared__ uint16_t lut[256];
-  __shared__ uint64_t red[4][64];
-  __shared__ int e_s[64];
-  __shared__ uint64_t tile[64][65];
-  fill_lut(lut);
-  const int tid = threadIdx.x;
-  const int r0 = blockIdx.x * 64;
-  const uint64_t* Xb = reinterpret_cast<const uint64_t*>(X);
-  {
-    const int r = tid & 63, part = tid >> 6;
-    uint64_t mx = 0;
-    if (r0 + r < rows)
-      for (int c = part; c < k; c += 4) {
-        const uint64_t u = __ldg(Xb + (r0 + r) + static_cast<long>(c) * cs) & 0x7FFFFFFFFFFFFFFFull;
-        mx = u > mx ? u : mx;
-      }
-    red[part][r] = mx;
-  }
-  __syncthreads();
-  if (tid < 64) {
-    uint64_t mx = red[0][tid];
-    for (int p = 1; p < 4; ++p) mx = red[p][tid] > mx ? red[p][tid] : mx;
-    const int e = exponent_of_maxbits(mx);
-    e_s[tid] = e;
-    if (r0 + tid < rows) exps[r0 + tid] = e;
-  }
-  __syncthreads();
-  const int W = 7 * s;
-  for (int c0 = 0; c0 < ldk; c0 += 64) {
-    for (int i = tid; i < 64 * 64; i += 256) {
-      const int r = i & 63, c = i >> 6;
-      uint64_t u = 0;
-      if (r0 + r < rows && c0 + c < k) u = __ldg(Xb + (r0 + r) + static_cast<long>(c0 + c) * cs);
-      tile[r][c] = u;
-    }
-    __syncthreads();
-    for (int item = tid; item < 64 * 8; item += 256) {
-      const int r = item >> 3, ch = item & 7;
-      const int c = c0 + ch * 8;
-      if (r0 + r >= rows || c >= ldk) continue;
-      const int e = e_s[r];
-      uint64_t mag[8];
-      bool neg[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint64_t u = tile[r][ch * 8 + j];
-        neg[j] = (u >> 63) != 0;
-        mag[j] = (e == kNonFinite) ? 0ull : scaled_magnitude(u & 0x7FFFFFFFFFFFFFFFull, e, W);
-      }
-      for (int p = 0; p < s; ++p) {
-        const int shift = 7 * (s - 1 - p);
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          w[j] = static_cast<uint32_t>(digit_bf16(lut, mag[2 * j], neg[2 * j], shift)) |
-                 (static_cast<uint32_t>(digit_bf16(lut, mag[2 * j + 1], neg[2 * j + 1], shift)) << 16);
-        *reinterpret_cast<uint4*>(out + (static_cast<long>(p) * rows + (r0 + r)) * ldk + c) =
-            make_uint4(w[0], w[1], w[2], w[3]);
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// k contiguous (cs == 1): one warp per row.
-__global__ void __launch_bounds__(256) split_kcontig_kernel(int rows, int k, const double* __restrict__ X, long rs,
-                                                            int s, int32_t* __restrict__ exps,
-                                                            uint16_t* __restrict__ out, long ldk) {
-  __shared__ uint16_t lut[256];
-  fill_lut(lut);
-  __syncthreads();
+// One block slices eight rows.  Rows contiguous in memory (rs = 1): a warp
+// covers the 8 rows x 4 groups of eight k, so a column of the tile is one 64-byte
+// piece and the four groups of a row are 64 bytes of a plane; k contiguous: a
+// warp takes one row, 32 groups at a time.  KEEP: all of K fits in one pass, the elements
+// stay in registers between the maximum and the digits; otherwise the second
+// pass reads them again (from L2).  Bound by memory for tall operands
+// (8 B read, 2s B written per element), by latency for small ones; the blocks
+// are small so that a 256-row operand already fills 32 SMs, and both operands
+// of a product go in one launch.
+template <int S, bool KEEP>
+__global__ void __launch_bounds__(kSplitThreads) split_kernel(const SplitArgs a0, const SplitArgs a1) {
+  __shared__ uint32_t up_s[kSplitThreads / 32][kSplitRows];
+  __shared__ unsigned long long full_s[kSplitRows];
+  const bool second = static_cast<int>(blockIdx.x) >= a0.blocks;
+  const SplitArgs& a = second ? a1 : a0;
+  const int r0 = (static_cast<int>(blockIdx.x) - (second ? a0.blocks : 0)) * kSplitRows;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * 8 + warp;
-  if (r >= rows) return;
-  const uint64_t* xr = reinterpret_cast<const uint64_t*>(X) + static_cast<long>(r) * rs;
-  uint64_t mx = 0;
-  for (int c = lane; c < k; c += 32) {
-    const uint64_t u = __ldg(xr + c) & 0x7FFFFFFFFFFFFFFFull;
-    mx = u > mx ? u : mx;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t v = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
-    mx = v > mx ? v : mx;
-  }
-  const int e = exponent_of_maxbits(mx);
-  if (lane == 0) exps[r] = e;
-  const int W = 7 * s;
-  for (int c = lane * 8; c < ldk; c += 256) {
-    uint64_t mag[8];
-    bool neg[8];
+  const bool by_rows = a.rs == 1;
+  const int rl = by_rows ? lane & 7 : warp;                       // row within the block
+  const int g0 = by_rows ? warp * 4 + (lane >> 3) : lane;         // first K group of this thread
+  constexpr int gstep = 32;
+  const int groups = static_cast<int>(a.ldk >> 3);
+  const int r = r0 + rl;
+  const bool row_ok = r < a.rows;
+  const uint64_t* row = reinterpret_cast<const uint64_t*>(a.X) + r * a.rs;
+  auto load = [&](int g, uint64_t (&u)[8]) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const uint64_t u = (c + j < k) ? __ldg(xr + c + j) : 0ull;
-      neg[j] = (u >> 63) != 0;
-      mag[j] = (e == kNonFinite) ? 0ull : scaled_magnitude(u & 0x7FFFFFFFFFFFFFFFull, e, W);
+      const int c = 8 * g + j;
+      u[j] = row_ok && c < a.k ? __ldg(row + c * a.cs) : 0ull;
     }
-    for (int p = 0; p < s; ++p) {
-      const int shift = 7 * (s - 1 - p);
-      uint32_t w[4];
+  };
+  // the maximum over the threads that share a row: lanes 8 and 16 apart, then
+  // the warps (rows contiguous), or the warp (k contiguous)
+  uint64_t u[8];
+  uint32_t up = 0;
+  if (KEEP) {
+    load(g0, u);
+    up = max_upper8(u);
+  } else {
+    for (int g = g0; g < groups; g += gstep) {
+      load(g, u);
+      up = max(up, max_upper8(u));
+    }
+  }
+  if (by_rows) {
+    up = max(up, __shfl_xor_sync(0xFFFFFFFFu, up, 8));
+    up = max(up, __shfl_xor_sync(0xFFFFFFFFu, up, 16));
+    if (lane < kSplitRows) up_s[warp][lane] = up;
+  } else {
+    up = __reduce_max_sync(0xFFFFFFFFu, up);
+  }
+  if (threadIdx.x < kSplitRows) full_s[threadIdx.x] = 0;
+  __syncthreads();
+  if (by_rows) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        w[j] = static_cast<uint32_t>(digit_bf16(lut, mag[2 * j], neg[2 * j], shift)) |
-               (static_cast<uint32_t>(digit_bf16(lut, mag[2 * j + 1], neg[2 * j + 1], shift)) << 16);
-      *reinterpret_cast<uint4*>(out + (static_cast<long>(p) * rows + r) * ldk + c) =
-          make_uint4(w[0], w[1], w[2], w[3]);
+    for (int w = 0; w < kSplitThreads / 32; ++w) up = max(up, up_s[w][rl]);
+  }
+  int e = exponent_of_upper(up);
+  if (__syncthreads_or(row_ok && needs_full_max(up))) {
+    // some row is all zeros and subnormals: the full patterns decide
+    if (row_ok && needs_full_max(up)) {
+      uint64_t mx = 0;
+      if (KEEP) {
+        mx = max_bits8(u);
+      } else {
+        for (int g = g0; g < groups; g += gstep) {
+          load(g, u);
+          const uint64_t v = max_bits8(u);
+          mx = v > mx ? v : mx;
+        }
+      }
+      atomicMax(&full_s[rl], static_cast<unsigned long long>(mx));
+    }
+    __syncthreads();
+    if (needs_full_max(up)) e = exponent_of_maxbits(full_s[rl]);
+  }
+  if (!row_ok) return;
+  if (g0 == 0) a.exps[r] = e;
+  if (KEEP) {
+    if (g0 < groups)
+      slice8<S>(u, e, [&](int p, uint4 w) {
+        *reinterpret_cast<uint4*>(a.out + (static_cast<long>(p) * a.rows + r) * a.ldk + 8 * g0) = w;
+      });
+  } else {
+    for (int g = g0; g < groups; g += gstep) {
+      load(g, u);
+      slice8<S>(u, e, [&](int p, uint4 w) {
+        *reinterpret_cast<uint4*>(a.out + (static_cast<long>(p) * a.rows + r) * a.ldk + 8 * g) = w;
+      });
     }
   }
 }
+
+template <int S>
+cudaError_t launch_s(cudaStream_t st, const SplitArgs& a, const SplitArgs& b) {
+  const int grid = a.blocks + b.blocks;
+  const long ldk = a.ldk > b.ldk ? a.ldk : b.ldk;
+  if (ldk <= 256)
+    split_kernel<S, true><<<grid, kSplitThreads, 0, st>>>(a, b);
+  else
+    split_kernel<S, false><<<grid, kSplitThreads, 0, st>>>(a, b);
+  return cudaGetLastError();
+}
+
+SplitArgs make_args(int rows, int k, const double* X, long rs, long cs, int32_t* exps, uint16_t* out, long ldk) {
+  return SplitArgs{X, rs, cs, rows, k, exps, out, ldk, rows > 0 ? (rows + kSplitRows - 1) / kSplitRows : 0};
+}
+
+cudaError_t dispatch(cudaStream_t st, int s, const SplitArgs& a, const SplitArgs& b) {
+  if (a.blocks + b.blocks == 0) return cudaSuccess;
+  switch (s) {
+    case 1: return launch_s<1>(st, a, b);
+    case 2: return launch_s<2>(st, a, b);
+    case 3: return launch_s<3>(st, a, b);
+    case 4: return launch_s<4>(st, a, b);
+    case 5: return launch_s<5>(st, a, b);
+    case 6: return launch_s<6>(st, a, b);
+    case 7: return launch_s<7>(st, a, b);
+    case 8: return launch_s<8>(st, a, b);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
 
 cudaError_t launch_split(cudaStream_t st, int rows, int k, const double* X, long rs, long cs, int s, int32_t* exps,
                          uint16_t* out, long ldk) {
-  if (rows <= 0) return cudaSuccess;
-  if (rs == 1) {
-    split_rowcontig_kernel<<<(rows + 63) / 64, 256, 0, st>>>(rows, k, X, cs, s, exps, out, ldk);
-  } else {
-    split_kcontig_kernel<<<(rows + 7) / 8, 256, 0, st>>>(rows, k, X, rs, s, exps, out, ldk);
-  }
-  return cudaGetLastError();
+  return dispatch(st, s, make_args(rows, k, X, rs, cs, exps, out, ldk), make_args(0, k, X, rs, cs, exps, out, 0));
+}
+
+cudaError_t launch_split2(cudaStream_t st, int k, int s, long ldk, int rows_a, const double* A, long ars, long acs,
+                          int32_t* ea, uint16_t* sa, int rows_b, const double* B, long brs, long bcs, int32_t* fb,
+                          uint16_t* sb) {
+  return dispatch(st, s, make_args(rows_a, k, A, ars, acs, ea, sa, ldk), make_args(rows_b, k, B, brs, bcs, fb, sb, ldk));
 }
 
 }  // namespace emul
