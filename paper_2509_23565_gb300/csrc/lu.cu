@@ -16,6 +16,7 @@
 // with one slice set serving both operands.
 #include <cmath>
 #include <cstdio>
+#include <map>
 #include <mutex>
 #include <set>
 #include <utility>
@@ -23,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include "handle.h"
+#include "ptx.cuh"
 
 namespace emul {
 
@@ -345,6 +347,195 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
   }
   for (int c = 0; c < w; ++c)
     for (int lr = tid; lr < rcount; lr += blockDim.x) A[(d0 + r0 + lr) + static_cast<long>(d0 + c) * lda] = P[c * R + lr];
+}
+
+// The same leaf on one thread-block cluster, for panels of at most
+// kClusterRows rows: the exchange of a column goes through distributed shared
+// memory instead of L2.  Each CTA stores its candidate (|value|, row) and the
+// candidate's row into every CTA of the cluster with st.async, which counts the
+// bytes on the receiver's barrier, so one trip of a few hundred cycles replaces
+// three through L2 (records out, records in, the winner's row), and the pivot
+// row is at hand once the winner is known.  Row c is sent along by its owner.
+// A column then costs one search, one exchange, one division and the rank-1
+// update of R = ceil(rows / CTAs) rows, bound by FP64 (1.68 FMA per clock per
+// SM; a warp's DFMA occupies its sub-partition for 64-76 cycles), so the rows
+// are spread over up to 16 SMs.  The arithmetic is that of getf2_leaf_kernel,
+// operation for operation.
+//
+// Buffers are double-buffered by column parity: a CTA sends column c + 2 only
+// after it has received column c + 1 from every CTA, which each sends after it
+// has used column c.
+constexpr int kClusterMax = 16;
+constexpr int kClusterR = 128;                        // rows per CTA at most
+constexpr int kClusterRows = kClusterMax * kClusterR;
+__global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, long lda, int n, int d0, int w, int R,
+                                                                    int pc0, int pc1, int32_t* ipiv, int32_t* info,
+                                                                    int* status, long long limit) {
+  extern __shared__ double P[];   // P[c*R + lr]
+  __shared__ double crow[2][kClusterMax][kLeaf], drow[2][kLeaf], prow[2][kLeaf];
+  __shared__ uint64_t rec[2][kClusterMax][2];
+  __shared__ __align__(8) uint64_t full[2];
+  __shared__ double rcp_s;
+  __shared__ uint64_t red_v[kClusterR / 32];
+  __shared__ int red_r[kClusterR / 32];
+  __shared__ int win_s, ok_s;
+  const int G = static_cast<int>(cluster_size()), b = static_cast<int>(cluster_rank());
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kLeafThreads / 32;
+  const int mp = n - d0;
+  const int r0 = b * R;
+  const int rcount = mp - r0 < R ? (mp - r0 > 0 ? mp - r0 : 0) : R;
+  const int nleft = d0 - pc0;
+  const int nout = nleft + (pc1 - d0 - w);
+  const int q = tid * G + b;      // outside column of this thread (as in getf2_leaf_kernel)
+  double* ocol = q < nout ? A + static_cast<long>(q < nleft ? pc0 + q : d0 + w + (q - nleft)) * lda : nullptr;
+  long sw_c = -1, sw_p = -1;
+  double sw_xc = 0.0, sw_xp = 0.0;
+  bool pend = false;
+  // deferred updates: warps 1..7 share the row groups of 32, and the columns of each
+  const int rgroups = (R + 31) / 32;
+  const int cstep = (kWarps - 1) / rgroups;
+  const int dgrp = warp >= 1 ? (warp - 1) % rgroups : 0, doff = warp >= 1 ? (warp - 1) / rgroups : cstep;
+  const int dlr = dgrp * 32 + lane;
+  if (tid < 2) mbar_init(&full[tid], 1);
+  if (tid == 0) fence_mbar_init();
+  for (int lr = tid & (kClusterR - 1), half = tid / kClusterR; lr < rcount; lr += kClusterR) {
+    // 16 columns per half of the block, their loads in flight together
+    const double* src = A + (d0 + r0 + lr) + static_cast<long>(d0) * lda;
+    double v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = half * 16 + j < w ? src[static_cast<long>(half * 16 + j) * lda] : 0.0;
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (half * 16 + j < w) P[(half * 16 + j) * R + lr] = v[j];
+  }
+  __syncthreads();
+  cluster_sync();               // every CTA's barriers are initialised
+
+  for (int c = 0; c < w; ++c) {
+    const int par = c & 1;
+    const double* pv = prow[par ^ 1];   // pivot row of column c-1
+    if (tid == 0) mbar_arrive_expect_tx(&full[par], static_cast<uint32_t>(G * (16 + 8 * w) + 8 * w));
+    // (1) candidate of the own rows: largest |value|, then the smallest row
+    if (warp < kClusterR / 32) {
+      const int pr = r0 + tid;
+      const bool in = tid < rcount && pr >= c;
+      const uint64_t v = in ? absbits(P[c * R + tid]) : 0ull;
+      const uint32_t hi = static_cast<uint32_t>(v >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+      const uint32_t lo = hi == mh ? static_cast<uint32_t>(v) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
+      const bool top = in && hi == mh && static_cast<uint32_t>(v) == ml;
+      const int mr = __reduce_min_sync(0xFFFFFFFFu, top ? pr : 0x7FFFFFFF);
+      if (lane == 0) {
+        red_v[warp] = (static_cast<uint64_t>(mh) << 32) | ml;
+        red_r[warp] = mr;
+      }
+    }
+    __syncthreads();
+    uint64_t bv = red_v[0];
+    int br = red_r[0];
+#pragma unroll
+    for (int i = 1; i < kClusterR / 32; ++i)
+      if (better(red_v[i], red_r[i], bv, br)) {
+        bv = red_v[i];
+        br = red_r[i];
+      }
+    // (2) candidate, its row and row c (current through pivot c-1) to every CTA
+    {
+      const bool own_c = c >= r0 && c < r0 + rcount;
+      double v = 0.0, dv = 0.0;
+      if (lane < w) {
+        if (br != 0x7FFFFFFF) {
+          v = P[lane * R + (br - r0)];
+          if (pend && lane > c) v = fma(-P[(c - 1) * R + (br - r0)], pv[lane], v);
+        }
+        if (own_c) {
+          dv = P[lane * R + (c - r0)];
+          if (pend && lane > c) dv = fma(-P[(c - 1) * R + (c - r0)], pv[lane], dv);
+        }
+      }
+      for (int t = warp; t < G; t += kWarps) {
+        const uint32_t bar = mapa_addr(smem_u32(&full[par]), t);
+        if (lane < w) {
+          st_async_b64(mapa_addr(smem_u32(&crow[par][b][lane]), t), static_cast<uint64_t>(__double_as_longlong(v)), bar);
+          if (own_c)
+            st_async_b64(mapa_addr(smem_u32(&drow[par][lane]), t), static_cast<uint64_t>(__double_as_longlong(dv)), bar);
+        }
+        if (lane < 2)
+          st_async_b64(mapa_addr(smem_u32(&rec[par][b][lane]), t), lane == 0 ? bv : static_cast<uint64_t>(br), bar);
+      }
+    }
+    __syncthreads();
+    // (3) winner, its row and the reciprocal (warp 0); deferred update of pivot c-1
+    if (warp == 0) {
+      const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(&full[par], (c >> 1) & 1, limit));
+      const uint64_t v = lane < G ? rec[par][lane][0] : 0ull;
+      const int r = lane < G ? static_cast<int>(rec[par][lane][1]) : 0x7FFFFFFF;
+      const uint32_t hi = static_cast<uint32_t>(v >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+      const uint32_t lo = hi == mh ? static_cast<uint32_t>(v) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
+      const bool top = lane < G && hi == mh && static_cast<uint32_t>(v) == ml;
+      const int gr = __reduce_min_sync(0xFFFFFFFFu, top ? r : 0x7FFFFFFF);
+      const int src = __ffs(__ballot_sync(0xFFFFFFFFu, top && r == gr)) - 1;
+      if (lane < w) {
+        const double x = crow[par][src][lane];
+        prow[par][lane] = x;
+        if (lane == c) rcp_s = 1.0 / x;
+      }
+      if (lane == 0) {
+        win_s = gr;
+        ok_s = ok;
+        if (!ok) atomicExch(status, kStatusTimeout);
+        if (ok && b == 0) {
+          ipiv[d0 + c] = d0 + gr + 1;
+          if (mh == 0 && ml == 0) atomicCAS(info, 0, d0 + c + 1);
+        }
+      }
+    } else if (pend && doff < cstep && dlr < rcount && r0 + dlr > c - 1) {
+      const double l = P[(c - 1) * R + dlr];
+      for (int cc = c + 1 + doff; cc < w; cc += cstep) P[cc * R + dlr] = fma(-l, pv[cc], P[cc * R + dlr]);
+    }
+    __syncthreads();
+    if (!ok_s) break;
+    const int p = win_s;
+    if (ocol) {
+      if (sw_c >= 0) {
+        ocol[sw_c] = sw_xp;
+        ocol[sw_p] = sw_xc;
+        sw_c = -1;
+      }
+      if (p != c) {
+        sw_c = d0 + c;
+        sw_p = d0 + p;
+        sw_xc = ocol[sw_c];
+        sw_xp = ocol[sw_p];
+      }
+    }
+    const double piv = prow[par][c];
+    pend = piv != 0.0;
+    if (pend) {
+      // (4) interchange rows c and p (both current through pivot c-1)
+      if (p != c) {
+        if (tid < w && c >= r0 && c < r0 + rcount) P[tid * R + (c - r0)] = prow[par][tid];
+        if (tid < w && p >= r0 && p < r0 + rcount) P[tid * R + (p - r0)] = drow[par][tid];
+      }
+      __syncthreads();
+      // (5) multipliers of column c, update of column c+1
+      if (tid < rcount && r0 + tid > c) {
+        const double l = fabs(piv) >= 2.2250738585072014e-308 ? P[c * R + tid] * rcp_s : P[c * R + tid] / piv;
+        P[c * R + tid] = l;
+        if (c + 1 < w) P[(c + 1) * R + tid] = fma(-l, prow[par][c + 1], P[(c + 1) * R + tid]);
+      }
+    }
+  }
+  if (sw_c >= 0) {
+    ocol[sw_c] = sw_xp;
+    ocol[sw_p] = sw_xc;
+  }
+  __syncthreads();
+  for (int e = tid; e < w * kClusterR; e += blockDim.x) {
+    const int lr = e & (kClusterR - 1), c = e / kClusterR;
+    if (lr < rcount) A[(d0 + r0 + lr) + static_cast<long>(d0 + c) * lda] = P[c * R + lr];
+  }
+  cluster_sync();               // no CTA leaves while another may still store into it
 }
 
 // Row interchanges ipiv[k1..k2) (1-based global rows, ipiv[k]-1 >= k) resolved
@@ -1010,9 +1201,67 @@ LuBufs carve(emul_handle_t h, size_t off, int nb) {
   return b;
 }
 
+// Largest cluster (16, 8, or 0: none) that the device can hold for the cluster
+// leaf; queried once per device.
+int leaf_cluster_max() {
+  static std::mutex mu;
+  static std::map<int, int> cache;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = cache.find(dev);
+  if (it != cache.end()) return it->second;
+  int best = 0;
+  const int smem = kClusterR * kLeaf * 8;
+  if (cudaFuncSetAttribute(getf2_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+      cudaFuncSetAttribute(getf2_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    for (int cs = kClusterMax; cs >= 8 && !best; cs /= 2) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(cs);
+      cfg.blockDim = dim3(kLeafThreads);
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = cs;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int num = 0;
+      if (cudaOccupancyMaxActiveClusters(&num, getf2_cluster_kernel, &cfg) == cudaSuccess && num >= 1) best = cs;
+    }
+  }
+  cudaGetLastError();   // a failed query leaves no error behind
+  cache[dev] = best;
+  return best;
+}
+
 int launch_leaf(emul_handle_t h, double* A, long lda, int n, int d0, int w, int pc0, int pc1, int32_t* ipiv,
                 int32_t* info, const LuBufs& B) {
   const int mp = n - d0;
+  const int cmax = mp <= kClusterRows ? leaf_cluster_max() : 0;
+  if (cmax > 0 && mp <= cmax * kClusterR) {
+    // as many CTAs as keep 32 rows each
+    int cs = 1;
+    while (cs < cmax && cs * 32 < mp) cs *= 2;
+    const int R = (mp + cs - 1) / cs;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cs);
+    cfg.blockDim = dim3(kLeafThreads);
+    cfg.dynamicSmemBytes = static_cast<size_t>(R) * w * 8;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    h->launches++;
+    return check_cuda(h, cudaLaunchKernelEx(&cfg, getf2_cluster_kernel, A, lda, n, d0, w, R, pc0, pc1, ipiv, info,
+                                            h->d_status, h->wait_limit),
+                      "panel leaf");
+  }
   int G = (mp + 127) / 128;   // 128 rows per block: the per-column FP64 work of a block overlaps the exchange
   const int smem_rows_cap = 200 * 1024 / (w * 8);
   if ((mp + G - 1) / G > smem_rows_cap) G = (mp + smem_rows_cap - 1) / smem_rows_cap;
