@@ -42,9 +42,10 @@ inline size_t al(size_t x) { return (x + kAl - 1) / kAl * kAl; }
 // a word also sees that word's payload, and no fence or counter is needed.
 // Record of block b for column parity par: words [0, 4) = |value| low and high
 // halves, candidate row, unused; words [4, 4 + 2w) = the candidate row, each
-// double as its low and high halves.  Epoch = salt * 32 + column (salt > 0,
+// double as its low and high halves; words [4 + 2 kLeaf, 6 + 2 kLeaf) = the
+// reciprocal of the candidate.  Epoch = salt * 32 + column (salt > 0,
 // distinct per leaf launch, records cleared before a factorization).
-constexpr int kRecWords = 4 + 2 * kLeaf;
+constexpr int kRecWords = 4 + 2 * kLeaf + 2;
 
 __device__ __forceinline__ void put_word(uint64_t* p, uint32_t payload, uint32_t epoch) {
   *reinterpret_cast<volatile uint64_t*>(p) = (static_cast<uint64_t>(epoch) << 32) | payload;
@@ -81,6 +82,31 @@ __device__ __forceinline__ bool better(uint64_t v1, int r1, uint64_t v2, int r2)
   return v1 > v2 || (v1 == v2 && r1 < r2);
 }
 
+// A column outside the leaf that follows its interchanges in global memory.  One
+// thread owns it for the whole launch, so successive interchanges of one element
+// stay in program order; the stores of an interchange are put off to the next
+// one, when its loads have long arrived.
+struct OutsideColumn {
+  double* col;
+  long r0 = -1, r1 = -1;
+  double x0 = 0.0, x1 = 0.0;
+  __device__ __forceinline__ void flush() {
+    if (col && r0 >= 0) {
+      col[r0] = x1;
+      col[r1] = x0;
+      r0 = -1;
+    }
+  }
+  __device__ __forceinline__ void swap(long a, long b) {
+    if (!col) return;
+    flush();
+    r0 = a;
+    r1 = b;
+    x0 = col[a];
+    x1 = col[b];
+  }
+};
+
 // Leaf panel: rows d0..n-1, columns d0..d0+w-1 of A, factored in place with
 // partial pivoting.  Block b keeps panel rows [b*R, b*R+R) in shared memory.
 //
@@ -116,7 +142,8 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
   __shared__ uint64_t red_v[kLeafThreads / 32];
   __shared__ int red_r[kLeafThreads / 32];
   __shared__ int win_s, ok_s, ok7_s;
-  constexpr int kRowTid = kLeafThreads - 32;   // first lane of the last warp: row-c reader
+  constexpr int kRowTid = kLeafThreads - 32;   // first lane of the last warp: publisher, row-c reader
+  constexpr int kRcpTid = kLeafThreads - 64;   // first lane of warp 6: the candidate's reciprocal
   const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
   const int mp = n - d0;
@@ -124,11 +151,11 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
   const int rcount = mp - r0 < R ? (mp - r0 > 0 ? mp - r0 : 0) : R;
   const int nleft = d0 - pc0;
   const int nout = nleft + (pc1 - d0 - w);
-  const int ot = (tid == 0 || tid == kRowTid) ? -1 : tid - 1 - (tid > kRowTid ? 1 : 0);
+  // outside columns go to the threads of warps 1-6 first: warps 0 and 7 run the exchange
+  const int ot = tid >= 32 && tid < kRowTid ? tid - 32 : (tid < 32 ? kLeafThreads - 64 + tid : tid);
   const int q = ot * G + b;
-  double* ocol = ot >= 0 && q < nout ? A + static_cast<long>(q < nleft ? pc0 + q : d0 + w + (q - nleft)) * lda : nullptr;
-  long sw_c = -1, sw_p = -1;   // pending interchange of this thread's outside column
-  double sw_xc = 0.0, sw_xp = 0.0;
+  OutsideColumn out{q < nout ? A + static_cast<long>(q < nleft ? pc0 + q : d0 + w + (q - nleft)) * lda : nullptr};
+  int p_last = -1;             // pivot row of column c-1
   bool pend = false;           // pivot c-1 was nonzero: its update of columns > c is pending
   // stage the rows: 16 loads in flight per thread before their stores
   for (int lr = tid; lr < rcount; lr += blockDim.x) {
@@ -163,35 +190,33 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
         br = pr;
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const uint64_t v2 = __shfl_xor_sync(0xFFFFFFFFu, bv, o);
-      const int r2 = __shfl_xor_sync(0xFFFFFFFFu, br, o);
-      if (better(v2, r2, bv, br)) {
-        bv = v2;
-        br = r2;
+    {
+      const uint32_t hi = static_cast<uint32_t>(bv >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+      const uint32_t lo = hi == mh ? static_cast<uint32_t>(bv) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
+      const bool top = hi == mh && static_cast<uint32_t>(bv) == ml;
+      const int mr = __reduce_min_sync(0xFFFFFFFFu, top ? br : 0x7FFFFFFF);
+      if (lane == 0) {
+        red_v[warp] = (static_cast<uint64_t>(mh) << 32) | ml;
+        red_r[warp] = mr;
       }
     }
-    if (lane == 0) {
-      red_v[warp] = bv;
-      red_r[warp] = br;
-    }
     __syncthreads();
-    if (tid == 0) {
-      for (int i = 1; i < static_cast<int>(blockDim.x / 32); ++i)
-        if (better(red_v[i], red_r[i], bv, br)) {
-          bv = red_v[i];
-          br = red_r[i];
-        }
+    bv = red_v[0];
+    br = red_r[0];
+#pragma unroll
+    for (int i = 1; i < kLeafThreads / 32; ++i)
+      if (better(red_v[i], red_r[i], bv, br)) {
+        bv = red_v[i];
+        br = red_r[i];
+      }
+    if (tid == kRowTid) {
       put_word(my + 0, static_cast<uint32_t>(bv), ep);
       put_word(my + 1, static_cast<uint32_t>(bv >> 32), ep);
       put_word(my + 2, static_cast<uint32_t>(br), ep);
-      win_s = br;
     }
-    __syncthreads();
     // (2) publish the candidate row and row c, current through pivot c-1
     {
-      const int pr = win_s;
+      const int pr = br;
       if (tid < 2 * w) {
         const int cc = tid >> 1;
         if (pr != 0x7FFFFFFF) {
@@ -254,22 +279,25 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
           gbk = lane + 32 * k;
         }
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const uint64_t v2 = __shfl_xor_sync(0xFFFFFFFFu, gv, o);
-        const int r2 = __shfl_xor_sync(0xFFFFFFFFu, gr, o);
-        const int b2 = __shfl_xor_sync(0xFFFFFFFFu, gbk, o);
-        if (better(v2, r2, gv, gr)) {
-          gv = v2;
-          gr = r2;
-          gbk = b2;
-        }
+      {
+        const uint32_t hi = static_cast<uint32_t>(gv >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+        const uint32_t lo = hi == mh ? static_cast<uint32_t>(gv) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
+        const bool top = hi == mh && static_cast<uint32_t>(gv) == ml;
+        const int mr = __reduce_min_sync(0xFFFFFFFFu, top ? gr : 0x7FFFFFFF);
+        const int src = __ffs(__ballot_sync(0xFFFFFFFFu, top && gr == mr)) - 1;
+        gbk = __shfl_sync(0xFFFFFFFFu, gbk, src);
+        gv = (static_cast<uint64_t>(mh) << 32) | ml;
+        gr = mr;
       }
       if (ok && lane < w) {
         double pvv = 0.0;
         ok = wait_pair(rec_all + static_cast<long>(gbk) * kRecWords + 4 + 2 * lane, ep, pvv, limit);
         prow[par][lane] = pvv;
-        if (lane == c) rcp_s = 1.0 / pvv;
+      }
+      if (ok && lane == 0) {
+        double r = 0.0;
+        ok = wait_pair(rec_all + static_cast<long>(gbk) * kRecWords + 4 + 2 * kLeaf, ep, r, limit);
+        rcp_s = r;
       }
       ok = __all_sync(0xFFFFFFFFu, ok);
       if (lane == 0) {
@@ -293,32 +321,32 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
         ok7_s = ok;
         if (!ok) atomicExch(status, kStatusTimeout);
       }
-    } else if (pend && c + 1 < w) {
+    } else {
+      if (tid == kRcpTid) {
+        // the block's candidate is the pivot of the whole panel for one block:
+        // its reciprocal is ready when the winner is known
+        const double r = br != 0x7FFFFFFF ? 1.0 / P[c * R + (br - r0)] : 0.0;
+        const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(r));
+        put_word(my + 4 + 2 * kLeaf, static_cast<uint32_t>(bits), ep);
+        put_word(my + 5 + 2 * kLeaf, static_cast<uint32_t>(bits >> 32), ep);
+      }
+      if (c > 0 && p_last != c - 1) out.swap(d0 + c - 1, d0 + p_last);
+      if (pend && c + 1 < w) {
       constexpr int kUpd = kLeafThreads - 64;   // warps 1-6
       for (int lr = tid - 32; lr < rcount; lr += kUpd) {
         if (r0 + lr <= c - 1) continue;
         const double l = P[(c - 1) * R + lr];
         for (int cc = c + 1; cc < w; ++cc) P[cc * R + lr] = fma(-l, pv[cc], P[cc * R + lr]);
       }
+      }
     }
+    if ((warp == 0 || warp == kLeafThreads / 32 - 1) && c > 0 && p_last != c - 1) out.swap(d0 + c - 1, d0 + p_last);
     __syncthreads();
     if (!ok_s || !ok7_s) return;
     const int p = win_s;
-    if (ocol) {
-      if (sw_c >= 0) {
-        ocol[sw_c] = sw_xp;
-        ocol[sw_p] = sw_xc;
-        sw_c = -1;
-      }
-      if (p != c) {
-        sw_c = d0 + c;
-        sw_p = d0 + p;
-        sw_xc = ocol[sw_c];
-        sw_xp = ocol[sw_p];
-      }
-    }
+    p_last = p;
     const double piv = prow[par][c];
-    pend = piv != 0.0;
+    pend = absbits(piv) != 0;           // (an FP64 comparison takes 64 cycles)
     if (pend) {
       // (4) interchange rows c and p (both current through pivot c-1)
       if (p != c) {
@@ -329,7 +357,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
       }
       __syncthreads();
       // (5) multipliers of column c, update of column c+1
-      const bool use_rcp = fabs(piv) >= 2.2250738585072014e-308;
+      const bool use_rcp = absbits(piv) >= 0x0010000000000000ull;
       const double rcp = rcp_s;
       const double u1 = c + 1 < w ? prow[par][c + 1] : 0.0;
       for (int lr = tid; lr < rcount; lr += blockDim.x) {
@@ -341,10 +369,8 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
     }
     __syncthreads();
   }
-  if (sw_c >= 0) {
-    ocol[sw_c] = sw_xp;
-    ocol[sw_p] = sw_xc;
-  }
+  if (p_last != w - 1 && p_last >= 0) out.swap(d0 + w - 1, d0 + p_last);
+  out.flush();
   for (int c = 0; c < w; ++c)
     for (int lr = tid; lr < rcount; lr += blockDim.x) A[(d0 + r0 + lr) + static_cast<long>(d0 + c) * lda] = P[c * R + lr];
 }
@@ -368,12 +394,14 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
 constexpr int kClusterMax = 16;
 constexpr int kClusterR = 128;                        // rows per CTA at most
 constexpr int kClusterRows = kClusterMax * kClusterR;
+constexpr int kPushWarps = 4;
 __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, long lda, int n, int d0, int w, int R,
                                                                     int pc0, int pc1, int32_t* ipiv, int32_t* info,
                                                                     int* status, long long limit) {
   extern __shared__ double P[];   // P[c*R + lr]
   __shared__ double crow[2][kClusterMax][kLeaf], drow[2][kLeaf], prow[2][kLeaf];
   __shared__ uint64_t rec[2][kClusterMax][2];
+  __shared__ double rcps[2][kClusterMax];
   __shared__ __align__(8) uint64_t full[2];
   __shared__ double rcp_s;
   __shared__ uint64_t red_v[kClusterR / 32];
@@ -387,10 +415,10 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
   const int rcount = mp - r0 < R ? (mp - r0 > 0 ? mp - r0 : 0) : R;
   const int nleft = d0 - pc0;
   const int nout = nleft + (pc1 - d0 - w);
-  const int q = tid * G + b;      // outside column of this thread (as in getf2_leaf_kernel)
-  double* ocol = q < nout ? A + static_cast<long>(q < nleft ? pc0 + q : d0 + w + (q - nleft)) * lda : nullptr;
-  long sw_c = -1, sw_p = -1;
-  double sw_xc = 0.0, sw_xp = 0.0;
+  const int q = (tid - 32) * G + b;      // outside column of this thread (as in getf2_leaf_kernel); none in warp 0
+  double* ocol = tid >= 32 && q < nout ? A + static_cast<long>(q < nleft ? pc0 + q : d0 + w + (q - nleft)) * lda : nullptr;
+  OutsideColumn out{ocol};
+  int p_last = -1;                // pivot row of column c-1
   bool pend = false;
   // deferred updates: warps 1..7 share the row groups of 32, and the columns of each
   const int rgroups = (R + 31) / 32;
@@ -415,7 +443,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
   for (int c = 0; c < w; ++c) {
     const int par = c & 1;
     const double* pv = prow[par ^ 1];   // pivot row of column c-1
-    if (tid == 0) mbar_arrive_expect_tx(&full[par], static_cast<uint32_t>(G * (16 + 8 * w) + 8 * w));
+    if (tid == 0) mbar_arrive_expect_tx(&full[par], static_cast<uint32_t>(G * (24 + 8 * w) + 8 * w));
     // (1) candidate of the own rows: largest |value|, then the smallest row
     if (warp < kClusterR / 32) {
       const int pr = r0 + tid;
@@ -440,7 +468,9 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
         br = red_r[i];
       }
     // (2) candidate, its row and row c (current through pivot c-1) to every CTA
-    {
+    // from warps 0-3, one per sub-partition; the candidate's reciprocal, whose
+    // division takes as long as the exchange, follows from warp 4
+    if (warp < kPushWarps) {
       const bool own_c = c >= r0 && c < r0 + rcount;
       double v = 0.0, dv = 0.0;
       if (lane < w) {
@@ -453,15 +483,21 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
           if (pend && lane > c) dv = fma(-P[(c - 1) * R + (c - r0)], pv[lane], dv);
         }
       }
-      for (int t = warp; t < G; t += kWarps) {
+      for (int t = warp; t < G; t += kPushWarps) {
         const uint32_t bar = mapa_addr(smem_u32(&full[par]), t);
+        const uint32_t to = bar - smem_u32(&full[par]);   // from an address here to the same one in CTA t
         if (lane < w) {
-          st_async_b64(mapa_addr(smem_u32(&crow[par][b][lane]), t), static_cast<uint64_t>(__double_as_longlong(v)), bar);
-          if (own_c)
-            st_async_b64(mapa_addr(smem_u32(&drow[par][lane]), t), static_cast<uint64_t>(__double_as_longlong(dv)), bar);
+          st_async_b64(to + smem_u32(&crow[par][b][lane]), static_cast<uint64_t>(__double_as_longlong(v)), bar);
+          if (own_c) st_async_b64(to + smem_u32(&drow[par][lane]), static_cast<uint64_t>(__double_as_longlong(dv)), bar);
         }
-        if (lane < 2)
-          st_async_b64(mapa_addr(smem_u32(&rec[par][b][lane]), t), lane == 0 ? bv : static_cast<uint64_t>(br), bar);
+        if (lane < 2) st_async_b64(to + smem_u32(&rec[par][b][lane]), lane == 0 ? bv : static_cast<uint64_t>(br), bar);
+      }
+    } else if (warp == kPushWarps) {
+      const double r = br != 0x7FFFFFFF ? 1.0 / P[c * R + (br - r0)] : 0.0;
+      if (lane < G) {
+        const uint32_t bar = mapa_addr(smem_u32(&full[par]), lane);
+        st_async_b64(bar - smem_u32(&full[par]) + smem_u32(&rcps[par][b]),
+                     static_cast<uint64_t>(__double_as_longlong(r)), bar);
       }
     }
     __syncthreads();
@@ -478,9 +514,9 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
       if (lane < w) {
         const double x = crow[par][src][lane];
         prow[par][lane] = x;
-        if (lane == c) rcp_s = 1.0 / x;
       }
       if (lane == 0) {
+        rcp_s = rcps[par][src];
         win_s = gr;
         ok_s = ok;
         if (!ok) atomicExch(status, kStatusTimeout);
@@ -489,28 +525,19 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
           if (mh == 0 && ml == 0) atomicCAS(info, 0, d0 + c + 1);
         }
       }
-    } else if (pend && doff < cstep && dlr < rcount && r0 + dlr > c - 1) {
-      const double l = P[(c - 1) * R + dlr];
-      for (int cc = c + 1 + doff; cc < w; cc += cstep) P[cc * R + dlr] = fma(-l, pv[cc], P[cc * R + dlr]);
+    } else {
+      if (c > 0 && p_last != c - 1) out.swap(d0 + c - 1, d0 + p_last);
+      if (pend && doff < cstep && dlr < rcount && r0 + dlr > c - 1) {
+        const double l = P[(c - 1) * R + dlr];
+        for (int cc = c + 1 + doff; cc < w; cc += cstep) P[cc * R + dlr] = fma(-l, pv[cc], P[cc * R + dlr]);
+      }
     }
     __syncthreads();
     if (!ok_s) break;
     const int p = win_s;
-    if (ocol) {
-      if (sw_c >= 0) {
-        ocol[sw_c] = sw_xp;
-        ocol[sw_p] = sw_xc;
-        sw_c = -1;
-      }
-      if (p != c) {
-        sw_c = d0 + c;
-        sw_p = d0 + p;
-        sw_xc = ocol[sw_c];
-        sw_xp = ocol[sw_p];
-      }
-    }
+    p_last = p;
     const double piv = prow[par][c];
-    pend = piv != 0.0;
+    pend = absbits(piv) != 0;           // (an FP64 comparison takes 64 cycles)
     if (pend) {
       // (4) interchange rows c and p (both current through pivot c-1)
       if (p != c) {
@@ -520,16 +547,14 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
       __syncthreads();
       // (5) multipliers of column c, update of column c+1
       if (tid < rcount && r0 + tid > c) {
-        const double l = fabs(piv) >= 2.2250738585072014e-308 ? P[c * R + tid] * rcp_s : P[c * R + tid] / piv;
+        const double l = absbits(piv) >= 0x0010000000000000ull ? P[c * R + tid] * rcp_s : P[c * R + tid] / piv;
         P[c * R + tid] = l;
         if (c + 1 < w) P[(c + 1) * R + tid] = fma(-l, prow[par][c + 1], P[(c + 1) * R + tid]);
       }
     }
   }
-  if (sw_c >= 0) {
-    ocol[sw_c] = sw_xp;
-    ocol[sw_p] = sw_xc;
-  }
+  if (p_last != w - 1 && p_last >= 0) out.swap(d0 + w - 1, d0 + p_last);
+  out.flush();
   __syncthreads();
   for (int e = tid; e < w * kClusterR; e += blockDim.x) {
     const int lr = e & (kClusterR - 1), c = e / kClusterR;
@@ -1241,8 +1266,9 @@ int launch_leaf(emul_handle_t h, double* A, long lda, int n, int d0, int w, int 
   const int mp = n - d0;
   const int cmax = mp <= kClusterRows ? leaf_cluster_max() : 0;
   if (cmax > 0 && mp <= cmax * kClusterR) {
-    // as many CTAs as keep 32 rows each
-    int cs = 1;
+    // as many CTAs as keep 32 rows each; two at least, for the outside columns'
+    // owners (at most 248 columns, 224 threads a CTA)
+    int cs = 2;
     while (cs < cmax && cs * 32 < mp) cs *= 2;
     const int R = (mp + cs - 1) / cs;
     cudaLaunchConfig_t cfg = {};
