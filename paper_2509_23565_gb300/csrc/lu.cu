@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
                                                                  int pc0, int pc1, int32_t* ipiv, int32_t* info,
                                                                  uint64_t* recs, uint64_t* drec, uint32_t salt,
                                                                  int* status, long long limit) {
-  extern __shared__ double P[];   // P[c*R + lr]
+  extern __shared__ double P[];   // P[c*ld + lr], ld odd: rows are read and written across banks
+  const int ld = R | 1;
   __shared__ double prow[2][kLeaf], crow[kLeaf];
   __shared__ double rcp_s;
   __shared__ uint64_t red_v[kLeafThreads / 32];
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
       for (int j = 0; j < 16; ++j) v[j] = c0 + j < w ? src[static_cast<long>(c0 + j) * lda] : 0.0;
 #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (c0 + j < w) P[(c0 + j) * R + lr] = v[j];
+        if (c0 + j < w) P[(c0 + j) * ld + lr] = v[j];
     }
   }
   __syncthreads();
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
     for (int lr = tid; lr < rcount; lr += blockDim.x) {
       const int pr = r0 + lr;
       if (pr < c) continue;
-      const uint64_t v = absbits(P[c * R + lr]);
+      const uint64_t v = absbits(P[c * ld + lr]);
       if (better(v, pr, bv, br)) {
         bv = v;
         br = pr;
@@ -221,15 +222,15 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
         const int cc = tid >> 1;
         if (pr != 0x7FFFFFFF) {
           const int lr = pr - r0;
-          double v = P[cc * R + lr];
-          if (pend && cc > c) v = fma(-P[(c - 1) * R + lr], pv[cc], v);
+          double v = P[cc * ld + lr];
+          if (pend && cc > c) v = fma(-P[(c - 1) * ld + lr], pv[cc], v);
           const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(v));
           put_word(my + 4 + tid, static_cast<uint32_t>(tid & 1 ? bits >> 32 : bits), ep);
         }
         if (c >= r0 && c < r0 + rcount) {
           const int lr = c - r0;
-          double v = P[cc * R + lr];
-          if (pend && cc > c) v = fma(-P[(c - 1) * R + lr], pv[cc], v);
+          double v = P[cc * ld + lr];
+          if (pend && cc > c) v = fma(-P[(c - 1) * ld + lr], pv[cc], v);
           const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(v));
           put_word(drow + tid, static_cast<uint32_t>(tid & 1 ? bits >> 32 : bits), ep);
         }
@@ -325,7 +326,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
       if (tid == kRcpTid) {
         // the block's candidate is the pivot of the whole panel for one block:
         // its reciprocal is ready when the winner is known
-        const double r = br != 0x7FFFFFFF ? 1.0 / P[c * R + (br - r0)] : 0.0;
+        const double r = br != 0x7FFFFFFF ? 1.0 / P[c * ld + (br - r0)] : 0.0;
         const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(r));
         put_word(my + 4 + 2 * kLeaf, static_cast<uint32_t>(bits), ep);
         put_word(my + 5 + 2 * kLeaf, static_cast<uint32_t>(bits >> 32), ep);
@@ -335,8 +336,8 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
       constexpr int kUpd = kLeafThreads - 64;   // warps 1-6
       for (int lr = tid - 32; lr < rcount; lr += kUpd) {
         if (r0 + lr <= c - 1) continue;
-        const double l = P[(c - 1) * R + lr];
-        for (int cc = c + 1; cc < w; ++cc) P[cc * R + lr] = fma(-l, pv[cc], P[cc * R + lr]);
+        const double l = P[(c - 1) * ld + lr];
+        for (int cc = c + 1; cc < w; ++cc) P[cc * ld + lr] = fma(-l, pv[cc], P[cc * ld + lr]);
       }
       }
     }
@@ -351,9 +352,9 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
       // (4) interchange rows c and p (both current through pivot c-1)
       if (p != c) {
         if (c >= r0 && c < r0 + rcount)
-          for (int cc = tid; cc < w; cc += blockDim.x) P[cc * R + (c - r0)] = prow[par][cc];
+          for (int cc = tid; cc < w; cc += blockDim.x) P[cc * ld + (c - r0)] = prow[par][cc];
         if (p >= r0 && p < r0 + rcount)
-          for (int cc = tid; cc < w; cc += blockDim.x) P[cc * R + (p - r0)] = crow[cc];
+          for (int cc = tid; cc < w; cc += blockDim.x) P[cc * ld + (p - r0)] = crow[cc];
       }
       __syncthreads();
       // (5) multipliers of column c, update of column c+1
@@ -362,9 +363,9 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
       const double u1 = c + 1 < w ? prow[par][c + 1] : 0.0;
       for (int lr = tid; lr < rcount; lr += blockDim.x) {
         if (r0 + lr <= c) continue;
-        const double l = use_rcp ? P[c * R + lr] * rcp : P[c * R + lr] / piv;
-        P[c * R + lr] = l;
-        if (c + 1 < w) P[(c + 1) * R + lr] = fma(-l, u1, P[(c + 1) * R + lr]);
+        const double l = use_rcp ? P[c * ld + lr] * rcp : P[c * ld + lr] / piv;
+        P[c * ld + lr] = l;
+        if (c + 1 < w) P[(c + 1) * ld + lr] = fma(-l, u1, P[(c + 1) * ld + lr]);
       }
     }
     __syncthreads();
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
   if (p_last != w - 1 && p_last >= 0) out.swap(d0 + w - 1, d0 + p_last);
   out.flush();
   for (int c = 0; c < w; ++c)
-    for (int lr = tid; lr < rcount; lr += blockDim.x) A[(d0 + r0 + lr) + static_cast<long>(d0 + c) * lda] = P[c * R + lr];
+    for (int lr = tid; lr < rcount; lr += blockDim.x) A[(d0 + r0 + lr) + static_cast<long>(d0 + c) * lda] = P[c * ld + lr];
 }
 
 // The same leaf on one thread-block cluster, for panels of at most
@@ -398,7 +399,8 @@ constexpr int kPushWarps = 4;
 __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, long lda, int n, int d0, int w, int R,
                                                                     int pc0, int pc1, int32_t* ipiv, int32_t* info,
                                                                     int* status, long long limit) {
-  extern __shared__ double P[];   // P[c*R + lr]
+  extern __shared__ double P[];   // P[c*ld + lr], ld odd: rows are read and written across banks
+  const int ld = R | 1;
   __shared__ double crow[2][kClusterMax][kLeaf], drow[2][kLeaf], prow[2][kLeaf];
   __shared__ uint64_t rec[2][kClusterMax][2];
   __shared__ double rcps[2][kClusterMax];
@@ -435,7 +437,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
     for (int j = 0; j < 16; ++j) v[j] = half * 16 + j < w ? src[static_cast<long>(half * 16 + j) * lda] : 0.0;
 #pragma unroll
     for (int j = 0; j < 16; ++j)
-      if (half * 16 + j < w) P[(half * 16 + j) * R + lr] = v[j];
+      if (half * 16 + j < w) P[(half * 16 + j) * ld + lr] = v[j];
   }
   __syncthreads();
   cluster_sync();               // every CTA's barriers are initialised
@@ -448,7 +450,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
     if (warp < kClusterR / 32) {
       const int pr = r0 + tid;
       const bool in = tid < rcount && pr >= c;
-      const uint64_t v = in ? absbits(P[c * R + tid]) : 0ull;
+      const uint64_t v = in ? absbits(P[c * ld + tid]) : 0ull;
       const uint32_t hi = static_cast<uint32_t>(v >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
       const uint32_t lo = hi == mh ? static_cast<uint32_t>(v) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
       const bool top = in && hi == mh && static_cast<uint32_t>(v) == ml;
@@ -475,12 +477,12 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
       double v = 0.0, dv = 0.0;
       if (lane < w) {
         if (br != 0x7FFFFFFF) {
-          v = P[lane * R + (br - r0)];
-          if (pend && lane > c) v = fma(-P[(c - 1) * R + (br - r0)], pv[lane], v);
+          v = P[lane * ld + (br - r0)];
+          if (pend && lane > c) v = fma(-P[(c - 1) * ld + (br - r0)], pv[lane], v);
         }
         if (own_c) {
-          dv = P[lane * R + (c - r0)];
-          if (pend && lane > c) dv = fma(-P[(c - 1) * R + (c - r0)], pv[lane], dv);
+          dv = P[lane * ld + (c - r0)];
+          if (pend && lane > c) dv = fma(-P[(c - 1) * ld + (c - r0)], pv[lane], dv);
         }
       }
       for (int t = warp; t < G; t += kPushWarps) {
@@ -493,7 +495,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
         if (lane < 2) st_async_b64(to + smem_u32(&rec[par][b][lane]), lane == 0 ? bv : static_cast<uint64_t>(br), bar);
       }
     } else if (warp == kPushWarps) {
-      const double r = br != 0x7FFFFFFF ? 1.0 / P[c * R + (br - r0)] : 0.0;
+      const double r = br != 0x7FFFFFFF ? 1.0 / P[c * ld + (br - r0)] : 0.0;
       if (lane < G) {
         const uint32_t bar = mapa_addr(smem_u32(&full[par]), lane);
         st_async_b64(bar - smem_u32(&full[par]) + smem_u32(&rcps[par][b]),
@@ -528,8 +530,8 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
     } else {
       if (c > 0 && p_last != c - 1) out.swap(d0 + c - 1, d0 + p_last);
       if (pend && doff < cstep && dlr < rcount && r0 + dlr > c - 1) {
-        const double l = P[(c - 1) * R + dlr];
-        for (int cc = c + 1 + doff; cc < w; cc += cstep) P[cc * R + dlr] = fma(-l, pv[cc], P[cc * R + dlr]);
+        const double l = P[(c - 1) * ld + dlr];
+        for (int cc = c + 1 + doff; cc < w; cc += cstep) P[cc * ld + dlr] = fma(-l, pv[cc], P[cc * ld + dlr]);
       }
     }
     __syncthreads();
@@ -541,15 +543,15 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
     if (pend) {
       // (4) interchange rows c and p (both current through pivot c-1)
       if (p != c) {
-        if (tid < w && c >= r0 && c < r0 + rcount) P[tid * R + (c - r0)] = prow[par][tid];
-        if (tid < w && p >= r0 && p < r0 + rcount) P[tid * R + (p - r0)] = drow[par][tid];
+        if (tid < w && c >= r0 && c < r0 + rcount) P[tid * ld + (c - r0)] = prow[par][tid];
+        if (tid < w && p >= r0 && p < r0 + rcount) P[tid * ld + (p - r0)] = drow[par][tid];
       }
       __syncthreads();
       // (5) multipliers of column c, update of column c+1
       if (tid < rcount && r0 + tid > c) {
-        const double l = absbits(piv) >= 0x0010000000000000ull ? P[c * R + tid] * rcp_s : P[c * R + tid] / piv;
-        P[c * R + tid] = l;
-        if (c + 1 < w) P[(c + 1) * R + tid] = fma(-l, prow[par][c + 1], P[(c + 1) * R + tid]);
+        const double l = absbits(piv) >= 0x0010000000000000ull ? P[c * ld + tid] * rcp_s : P[c * ld + tid] / piv;
+        P[c * ld + tid] = l;
+        if (c + 1 < w) P[(c + 1) * ld + tid] = fma(-l, prow[par][c + 1], P[(c + 1) * ld + tid]);
       }
     }
   }
@@ -558,7 +560,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
   __syncthreads();
   for (int e = tid; e < w * kClusterR; e += blockDim.x) {
     const int lr = e & (kClusterR - 1), c = e / kClusterR;
-    if (lr < rcount) A[(d0 + r0 + lr) + static_cast<long>(d0 + c) * lda] = P[c * R + lr];
+    if (lr < rcount) A[(d0 + r0 + lr) + static_cast<long>(d0 + c) * lda] = P[c * ld + lr];
   }
   cluster_sync();               // no CTA leaves while another may still store into it
 }
@@ -1237,7 +1239,7 @@ int leaf_cluster_max() {
   const auto it = cache.find(dev);
   if (it != cache.end()) return it->second;
   int best = 0;
-  const int smem = kClusterR * kLeaf * 8;
+  const int smem = (kClusterR | 1) * kLeaf * 8;
   if (cudaFuncSetAttribute(getf2_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
       cudaFuncSetAttribute(getf2_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
     for (int cs = kClusterMax; cs >= 8 && !best; cs /= 2) {
@@ -1274,7 +1276,7 @@ int launch_leaf(emul_handle_t h, double* A, long lda, int n, int d0, int w, int 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs);
     cfg.blockDim = dim3(kLeafThreads);
-    cfg.dynamicSmemBytes = static_cast<size_t>(R) * w * 8;
+    cfg.dynamicSmemBytes = static_cast<size_t>(R | 1) * w * 8;
     cfg.stream = h->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1295,7 +1297,7 @@ int launch_leaf(emul_handle_t h, double* A, long lda, int n, int d0, int w, int 
   if (G > h->nsm) G = h->nsm;
   if (G > 32 * kMaxRecPerLane) G = 32 * kMaxRecPerLane;
   const int R = (mp + G - 1) / G;
-  const size_t smem = static_cast<size_t>(R) * w * 8;
+  const size_t smem = static_cast<size_t>(R | 1) * w * 8;
   if (smem > 220 * 1024) return set_error(h, EMUL_NOT_SUPPORTED, "panel too tall for the leaf kernel");
   smem_attr(reinterpret_cast<const void*>(getf2_leaf_kernel), 220 * 1024);
   long long limit = h->wait_limit;
