@@ -744,25 +744,29 @@ constexpr int kCholLeaf = 32;
 // j = 4s + q (s = 0..7) in registers, so the FP64 work is spread over the
 // SM's four sub-partitions.  Pivot jj: its owner warp takes r = rsqrt(d) of
 // the pivot d, sets L_jj = d r, scales the column by r and publishes it in
-// shared memory (double-buffered, one 128-thread barrier per pivot); every
-// warp then updates its columns right of jj.  GB300's FP64 latency makes every
-// dependent FP64 step costly, so each pivot takes one reciprocal square root
-// rather than a square root and a division.  A non-positive pivot sets *info
-// (first index) and stops; nothing runs once *info is set.
+// shared memory (double-buffered).  GB300's FP64 latency makes every dependent
+// FP64 step costly (64 cycles a DFMA, 375 an rsqrt), so the chain from pivot to
+// pivot is kept short: the owner of the next pivot updates that column first,
+// scales and publishes it and arrives at the step's barrier before it updates
+// its other columns, and each pivot takes one reciprocal square root rather than
+// a square root and a division.  A non-positive pivot sets *info (first index)
+// and stops; nothing runs once *info is set.
 // It also writes the leaf's inverse L^-1 (lower, w x w) to inv[i + j*ldi]:
-// forward substitution on the identity, all columns at once, each warp on its
-// own columns (row m of X, once final, is broadcast within the warp by
+// forward substitution on the identity, each warp on its own columns from their
+// diagonal on (row m of X, once final, is broadcast within the warp by
 // shuffles; the multipliers L[i][m] come from shared memory), with the
 // diagonal reciprocals formed in parallel up front.
+__device__ __noinline__ double chol_rsqrt(double d) { return rsqrt(d); }
+
 __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int d0, int w, double* inv, int ldi,
                                                        int32_t* info) {
   __shared__ double col[2][kCholLeaf];
   __shared__ double Ls[kCholLeaf][kCholLeaf + 1];
-  __shared__ int fail_s;
+  __shared__ int fail_s;       // pivot that failed
   const int i = threadIdx.x & 31, q = threadIdx.x >> 5;
-  if (threadIdx.x == 0) fail_s = (*info != 0);
+  if (threadIdx.x == 0) fail_s = *info != 0 ? -1 : kCholLeaf;
   __syncthreads();
-  if (fail_s) return;
+  if (fail_s < 0) return;
   double* blk = A + d0 + static_cast<long>(d0) * lda;
   // padding beyond w is the identity, so the inverse below needs no special case
   double d[8];
@@ -771,36 +775,64 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
     const int j = 4 * s + q;
     d[s] = (i < w && j < w) ? (i >= j ? blk[i + static_cast<long>(j) * lda] : 0.0) : (i == j ? 1.0 : 0.0);
   }
+  __syncthreads();               // every thread has read fail_s
+  // pivot jj from its column x (owner warp): scaled and published
+  auto pivot = [&](int jj, double& x) {
+    const double diag = __shfl_sync(0xFFFFFFFFu, x, jj);
+    if (diag > 0.0) {
+      const double r = chol_rsqrt(diag);
+      if (i == jj)
+        x = diag * r;
+      else if (i > jj)
+        x *= r;
+    } else if (i == 0) {
+      atomicCAS(info, 0, d0 + jj + 1);
+      fail_s = jj;
+    }
+    col[jj & 1][i] = i >= jj ? x : 0.0;
+  };
+  if (q == 0) pivot(0, d[0]);
   int done = w;
+  // pivots jj = 4 so + qq; the inner loop stays rolled (32 copies of a step would
+  // run from the instruction cache's misses)
 #pragma unroll
-  for (int jj = 0; jj < kCholLeaf; ++jj) {
-    if (jj >= w) break;                       // uniform over the block
-    const int s0 = jj >> 2;
-    if (q == (jj & 3)) {
-      const double diag = __shfl_sync(0xFFFFFFFFu, d[s0], jj);
-      const bool ok = diag > 0.0;
-      if (ok) {
-        const double r = rsqrt(diag);
-        if (i == jj)
-          d[s0] = diag * r;
-        else if (i > jj)
-          d[s0] *= r;
-      } else if (i == 0) {
-        atomicCAS(info, 0, d0 + jj + 1);
-        fail_s = 1;
+  for (int so = 0; so < kCholLeaf / 4; ++so) {
+#pragma unroll 1
+    for (int qq = 0; qq < 4; ++qq) {
+      const int jj = 4 * so + qq;
+      if (jj >= w || done < w) break;         // uniform over the block
+      // barriers 1 and 2 in turn; the owner has published and does not wait
+      if (q == qq) {
+        __syncwarp();
+        asm volatile("bar.arrive %0, 128;" ::"r"(1 + (jj & 1)) : "memory");
+      } else {
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + (jj & 1)) : "memory");
       }
-      col[jj & 1][i] = i >= jj ? d[s0] : 0.0;
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (fail_s) {
-      done = jj;
-      break;
-    }
-    const double lij = col[jj & 1][i];
+      // a failed pivot stops every warp at its step: the index was stored before
+      // that step's barrier (a later one may already be there: not yet looked at)
+      if (*static_cast<volatile int*>(&fail_s) <= jj) {
+        done = jj;
+        break;
+      }
+      const double lij = col[jj & 1][i];
+      const bool mine = q == ((qq + 1) & 3) && jj + 1 < w;
+      if (mine) {
+        const double ln = col[jj & 1][(jj + 1) & 31];
+        if (qq < 3) {
+          if (i >= jj + 1) d[so] = fma(-lij, ln, d[so]);
+          pivot(jj + 1, d[so]);
+        } else if (so + 1 < kCholLeaf / 4) {
+          double& x = d[so + 1 < kCholLeaf / 4 ? so + 1 : so];
+          if (i >= jj + 1) x = fma(-lij, ln, x);
+          pivot(jj + 1, x);
+        }
+      }
+      const int snext = qq < 3 ? so : so + 1;
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      const int j = 4 * s + q;
-      if (j > jj && i >= j) d[s] = fma(-lij, col[jj & 1][j], d[s]);
+      for (int s = so; s < kCholLeaf / 4; ++s) {
+        const int j = 4 * s + q;
+        if ((s > so || q > qq) && i >= j && !(mine && s == snext)) d[s] = fma(-lij, col[jj & 1][j], d[s]);
+      }
     }
   }
   // write back the columns that were finished (all of them unless a pivot failed)
@@ -818,15 +850,13 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
   double x[8];
 #pragma unroll
   for (int s = 0; s < 8; ++s) x[s] = (i == 4 * s + q) ? 1.0 : 0.0;
-#pragma unroll
+#pragma unroll 1
   for (int m = 0; m < kCholLeaf; ++m) {
-    if (i == m) {
-#pragma unroll
-      for (int s = 0; s < 8; ++s) x[s] *= rcp;   // row m of X is final
-    }
     const double lim = i > m ? Ls[i][m] : 0.0;
 #pragma unroll
     for (int s = 0; s < 8; ++s) {
+      if (m < 4 * s + q) continue;            // rows above a column's diagonal are zero (warp-uniform)
+      if (i == m) x[s] *= rcp;                // row m of X is final
       const double xm = __shfl_sync(0xFFFFFFFFu, x[s], m);
       x[s] = fma(-lim, xm, x[s]);
     }
@@ -840,24 +870,27 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
 
 // C(i, j) = beta C(i, j) + alpha sum_l A(i, l) B(j, l) in FP64, for the m x n
 // C (ldc) with A(i, l) = A[i*ars + l*acs] and B(j, l) = B[j*brs + l*bcs];
-// lower = 1 writes only i >= j.  A block computes a 16 x 32 tile (one entry
+// lower = 1 writes only i >= j.  A block computes an 8 x 32 tile (one entry
 // per thread) over K chunks of 32 staged in shared memory; with n <= 32 and
 // k <= 32 every block reads all its operands before it writes, so C may then
-// alias A's rows of the same block (the in-place triangular solve).
-__global__ void __launch_bounds__(512) dgemm_nt_small_kernel(int m, int n, int k, double alpha, const double* A,
+// alias A's rows of the same block (the in-place triangular solve).  A warp's
+// DFMA holds its sub-partition for 64-76 cycles, so 8 warps take 2 x 32 of them
+// in 2.4 us; tiles of 16 rows took twice that and left most SMs idle.
+constexpr int kNtRows = 8;
+__global__ void __launch_bounds__(32 * kNtRows) dgemm_nt_small_kernel(int m, int n, int k, double alpha, const double* A,
                                                             long ars, long acs, const double* B, long brs,
                                                             long bcs, double beta, double* C, long ldc,
                                                             int lower, const int32_t* info) {
-  __shared__ double As[16][33], Bs[32][33];
+  __shared__ double As[kNtRows][33], Bs[32][33];
   if (*info != 0) return;
-  const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
-  const int i0 = blockIdx.x * 16, j0 = blockIdx.y * 32;
-  if (lower && j0 > i0 + 15) return;          // tile entirely above the diagonal
+  const int ti = threadIdx.x & (kNtRows - 1), tj = threadIdx.x / kNtRows;
+  const int i0 = blockIdx.x * kNtRows, j0 = blockIdx.y * 32;
+  if (lower && j0 > i0 + kNtRows - 1) return;          // tile entirely above the diagonal
   const int i = i0 + ti, j = j0 + tj;
   double acc = 0.0;
   for (int l0 = 0; l0 < k; l0 += 32) {
-    for (int e = threadIdx.x; e < 16 * 32; e += blockDim.x) {
-      const int r = e & 15, l = e >> 4;
+    for (int e = threadIdx.x; e < kNtRows * 32; e += blockDim.x) {
+      const int r = e & (kNtRows - 1), l = e / kNtRows;
       As[r][l] = (i0 + r < m && l0 + l < k) ? A[(i0 + r) * ars + static_cast<long>(l0 + l) * acs] : 0.0;
     }
     for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
@@ -1193,10 +1226,10 @@ int chol_diag(emul_handle_t h, double* A, long lda, int d0, int jb, double* inv,
       double* Lp = A + (d0 + r0) + static_cast<long>(d0 + c0) * lda;   // rows below the leaf, its columns
       const double* ip = inv + c0 + static_cast<long>(c0) * jb;       // the leaf's inverse
       // L(r0.., c0..) = A(r0.., c0..) L_pp^-T, in place (n = k = wp <= 32)
-      dgemm_nt_small_kernel<<<dim3((mr + 15) / 16, 1), 512, 0, h->stream>>>(mr, wp, wp, 1.0, Lp, 1, lda, ip, 1, jb,
+      dgemm_nt_small_kernel<<<dim3((mr + kNtRows - 1) / kNtRows, 1), 32 * kNtRows, 0, h->stream>>>(mr, wp, wp, 1.0, Lp, 1, lda, ip, 1, jb,
                                                                           0.0, Lp, lda, 0, info);
       // A(r0.., r0..) -= L(r0.., c0..) L(r0.., c0..)^T, lower part
-      dgemm_nt_small_kernel<<<dim3((mr + 15) / 16, (mr + 31) / 32), 512, 0, h->stream>>>(
+      dgemm_nt_small_kernel<<<dim3((mr + kNtRows - 1) / kNtRows, (mr + 31) / 32), 32 * kNtRows, 0, h->stream>>>(
           mr, mr, wp, -1.0, Lp, 1, lda, Lp, 1, lda, 1.0, A + (d0 + r0) + static_cast<long>(d0 + r0) * lda, lda, 1,
           info);
       h->launches += 2;

@@ -24,113 +24,155 @@ namespace emul {
 namespace {
 
 constexpr int kNpLeaf = 64;           // widest diagonal block factored in one CTA
-constexpr int kNpThreads = 1024;      // 64 rows x 16 column groups
-constexpr int kNpGroups = kNpThreads / kNpLeaf;
-constexpr int kNpPerThread = kNpLeaf / kNpGroups;
+constexpr int kNpWarps = 8;           // the leaf's warps, columns dealt round
 constexpr int kNpChunk = 1024;        // K of one emulated product in the Schur updates
 constexpr size_t kNpAl = 256;
 
 inline size_t np_al(size_t x) { return (x + kNpAl - 1) / kNpAl * kNpAl; }
 
 // The w x w diagonal block at A[d.., d..] (w <= 64) is factored in place
-// without pivoting, A = L U (L unit lower), in shared memory; then
-// X <- L^-1 (ld ldx, zeros above the diagonal) and Y <- U^-1 (ld w, zeros
-// below).  A zero pivot leaves its column unscaled and records its 1-based
-// index in *info unless an earlier one is there.  Thread (r, g) = (tid % 64,
-// tid / 64) works on row r and the columns g, g + 16, ...; g is uniform in a
-// warp, so the triangular structure is skipped by warp-uniform branches.
-// FP64 runs at a small fraction of the tensor rate on this part, so the
-// divisions are taken once per pivot (a reciprocal in shared memory) and the
-// inverses touch only their nonzero triangles.
-__global__ void __launch_bounds__(kNpThreads, 1) np_leaf_kernel(double* A, long lda, int d, int w, int32_t* info,
-                                                                double* X, long ldx, double* Y) {
-  __shared__ double S[kNpLeaf * (kNpLeaf + 1)];   // w x w, leading dimension w + 1
-  __shared__ double rowbuf[2][kNpLeaf];
-  __shared__ double rdiag[kNpLeaf];                // 1 / U(k,k) (0 for a zero pivot)
-  const int tid = threadIdx.x;
-  const int r = tid & (kNpLeaf - 1);
-  const int g = tid / kNpLeaf;
-  const int ld = w + 1;
+// without pivoting, A = L U (L unit lower).  A zero pivot leaves its column
+// unscaled and records its 1-based index in *info unless an earlier one is
+// there.
+//
+// One CTA: FP64 retires 1.68 FMA per clock per SM, a warp's DFMA occupies its
+// sub-partition for 64-76 cycles and a division takes 560, so what counts is the
+// chain from pivot to pivot and that no FP64 instruction is wasted.  Eight warps
+// hold the block in registers, warp g the columns g, g + 8, ... with rows i and
+// i + 32 in lane i, so a pivot column lies in one warp: its owner updates it
+// first, takes the reciprocal, scales, publishes the multipliers in shared
+// memory and arrives at the step's barrier before it updates its other columns;
+// the other warps meet it there after theirs.  The pivot row comes by shuffles.
+// (64 x 64 with both inverses took 256 us in one CTA of 1024 threads on shared
+// memory with two barriers a step and the division after the update.)
+__device__ __noinline__ double np_recip(double p) { return p != 0.0 ? 1.0 / p : 0.0; }
+
+__global__ void __launch_bounds__(32 * kNpWarps, 1) np_leaf_kernel(double* A, long lda, int d, int w, int32_t* info) {
+  __shared__ double mult[2][kNpLeaf];
+  constexpr int kCols = kNpLeaf / kNpWarps;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   double* D = A + d + static_cast<long>(d) * lda;
-  for (int j = g; j < w; j += kNpGroups)
-    if (r < w) S[r + j * ld] = D[r + static_cast<long>(j) * lda];
-  __syncthreads();
-  if (tid == 0) {
-    const double p = S[0];
-    rdiag[0] = p != 0.0 ? 1.0 / p : 0.0;
-    if (p == 0.0) atomicCAS(info, 0, d + 1);
-  }
-  for (int k = 0; k < w; ++k) {
-    __syncthreads();                               // rdiag[k] and column k final
-    const double rk = rdiag[k];
-    if (g == 0 && r > k && r < w && rk != 0.0) S[r + k * ld] *= rk;
-    __syncthreads();
-    if (r > k && r < w) {
-      const double l = S[r + k * ld];
-      for (int j = k + 1 + g; j < w; j += kNpGroups) S[r + j * ld] = fma(-l, S[k + j * ld], S[r + j * ld]);
-      // the owner of the next pivot publishes its reciprocal
-      if (r == k + 1 && g == 0) {                 // its first column j = k + 1 is the pivot
-        const double p = S[r + r * ld];
-        rdiag[r] = p != 0.0 ? 1.0 / p : 0.0;
-        if (p == 0.0) atomicCAS(info, 0, d + r + 1);
+  // beyond w the block is the identity: nothing there changes or is stored
+  double v[kCols][2];
+#pragma unroll
+  for (int s = 0; s < kCols; ++s)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = lane + 32 * h, j = g + kNpWarps * s;
+      v[s][h] = i < w && j < w ? D[i + static_cast<long>(j) * lda] : (i == j ? 1.0 : 0.0);
+    }
+  // multipliers of pivot k from its column (in registers c0, c1 of the owner)
+  auto scale = [&](int k, double& c0, double& c1) {
+    const double p = __shfl_sync(0xFFFFFFFFu, k < 32 ? c0 : c1, k & 31);
+    const double r = np_recip(p);           // 0 for a zero pivot
+    if (p == 0.0 && lane == 0) atomicCAS(info, 0, d + k + 1);
+    if (r != 0.0) {
+      if (lane > k) c0 *= r;
+      if (lane + 32 > k) c1 *= r;
+    }
+    mult[k & 1][lane] = lane > k ? c0 : 0.0;
+    mult[k & 1][lane + 32] = lane + 32 > k ? c1 : 0.0;
+  };
+  if (g == 0) scale(0, v[0][0], v[0][1]);
+  // pivots k = 8 so + kk; the inner loop stays rolled (64 copies of a step would
+  // run from the instruction cache's misses)
+#pragma unroll
+  for (int so = 0; so < kCols; ++so) {
+#pragma unroll 1
+    for (int kk = 0; kk < kNpWarps; ++kk) {
+      const int k = kNpWarps * so + kk;
+      if (k + 1 >= w) break;
+      // barriers 1 and 2 in turn; the owner has published and does not wait
+      if (g == kk) {
+        __syncwarp();
+        asm volatile("bar.arrive %0, %1;" ::"r"(1 + (k & 1)), "n"(32 * kNpWarps) : "memory");
+      } else {
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + (k & 1)), "n"(32 * kNpWarps) : "memory");
       }
+      const double l0 = mult[k & 1][lane], l1 = mult[k & 1][lane + 32];
+      auto update = [&](double& c0, double& c1) {
+        const double u = __shfl_sync(0xFFFFFFFFu, so < kCols / 2 ? c0 : c1, k & 31);
+        if (so < kCols / 2 && lane > k) c0 = fma(-l0, u, c0);
+        if (lane + 32 > k) c1 = fma(-l1, u, c1);
+      };
+      // the next pivot's column first, and its multipliers
+      const bool mine = g == (kk + 1) % kNpWarps;
+      if (mine) {
+        if (kk + 1 < kNpWarps) {
+          update(v[so][0], v[so][1]);
+          scale(k + 1, v[so][0], v[so][1]);
+        } else if (so + 1 < kCols) {
+          update(v[so + 1 < kCols ? so + 1 : so][0], v[so + 1 < kCols ? so + 1 : so][1]);
+          scale(k + 1, v[so + 1 < kCols ? so + 1 : so][0], v[so + 1 < kCols ? so + 1 : so][1]);
+        }
+      }
+      const int snext = kk + 1 < kNpWarps ? so : so + 1;
+#pragma unroll
+      for (int s = so; s < kCols; ++s)
+        if ((s > so || g > kk) && !(mine && s == snext)) update(v[s][0], v[s][1]);
     }
   }
-  for (int j = g; j < w; j += kNpGroups)
-    if (r < w) D[r + static_cast<long>(j) * lda] = S[r + j * ld];
+#pragma unroll
+  for (int s = 0; s < kCols; ++s)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = lane + 32 * h, j = g + kNpWarps * s;
+      if (i < w && j < w) D[i + static_cast<long>(j) * lda] = v[s][h];
+    }
+}
 
-  // X = L^-1: row r of X is e_r - sum_{k<r} L(r,k) X(k,:); row k of X is
-  // zero right of column k
-  double x[kNpPerThread];
-#pragma unroll
-  for (int t = 0; t < kNpPerThread; ++t) x[t] = (r == g + kNpGroups * t) ? 1.0 : 0.0;
-  for (int k = 0; k + 1 < w; ++k) {
-    double* rb = rowbuf[k & 1];
-    if (r == k) {
-#pragma unroll
-      for (int t = 0; t < kNpPerThread; ++t) rb[g + kNpGroups * t] = x[t];
-    }
-    __syncthreads();
-    if (r > k && r < w) {
-      const double l = S[r + k * ld];
-#pragma unroll
-      for (int t = 0; t < kNpPerThread; ++t)
-        if (g + kNpGroups * t <= k) x[t] = fma(-l, rb[g + kNpGroups * t], x[t]);
-    }
-  }
-  if (r < w) {
-#pragma unroll
-    for (int t = 0; t < kNpPerThread; ++t)
-      if (g + kNpGroups * t < w) X[r + static_cast<long>(g + kNpGroups * t) * ldx] = x[t];
+// Inverses of the leaf's factors: X <- L^-1 (ld ldx, zeros above the diagonal)
+// and Y <- U^-1 (ld w, zeros below; an infinite reciprocal for a zero pivot).
+// One warp per column of X or Y and four columns per block, so every warp has a
+// sub-partition's FP64 unit to itself: a step is a shuffle and two DFMAs
+// (about 200 cycles).  Row k of a column, once final, is broadcast; column j of X
+// starts at row j, of Y at row j and goes up.
+constexpr int kInvCols = 4;
+__global__ void __launch_bounds__(32 * kInvCols) np_inverse_kernel(const double* A, long lda, int d, int w, double* X,
+                                                                  long ldx, double* Y) {
+  __shared__ double S[kNpLeaf][kNpLeaf + 1];      // S[k][i] = (L\U)(i, k)
+  __shared__ double rdiag[kNpLeaf];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double* D = A + d + static_cast<long>(d) * lda;
+  for (int e = threadIdx.x; e < kNpLeaf * kNpLeaf; e += blockDim.x) {
+    const int i = e & (kNpLeaf - 1), k = e / kNpLeaf;
+    S[k][i] = i < w && k < w ? D[i + static_cast<long>(k) * lda] : 0.0;
   }
   __syncthreads();
-
-  // Y = U^-1: row r of Y is (e_r - sum_{k>r} U(r,k) Y(k,:)) / U(r,r), k from
-  // w-1 down; row k of Y is zero left of column k
-#pragma unroll
-  for (int t = 0; t < kNpPerThread; ++t) x[t] = (r == g + kNpGroups * t) ? 1.0 : 0.0;
-  for (int k = w - 1; k >= 0; --k) {
-    double* rb = rowbuf[k & 1];
-    if (r == k) {
-      const double rk = rdiag[k] != 0.0 ? rdiag[k] : __longlong_as_double(0x7FF0000000000000ll);
-#pragma unroll
-      for (int t = 0; t < kNpPerThread; ++t) {
-        if (g + kNpGroups * t >= k) x[t] *= rk;
-        rb[g + kNpGroups * t] = x[t];
-      }
+  const bool lower = blockIdx.y == 0;
+  if (!lower) {
+    if (threadIdx.x < w) {
+      const double p = S[threadIdx.x][threadIdx.x];
+      const double r = p != 0.0 ? 1.0 / p : 0.0;
+      rdiag[threadIdx.x] = r != 0.0 ? r : __longlong_as_double(0x7FF0000000000000ll);
     }
     __syncthreads();
-    if (r < k) {
-      const double l = S[r + k * ld];
-#pragma unroll
-      for (int t = 0; t < kNpPerThread; ++t)
-        if (g + kNpGroups * t >= k) x[t] = fma(-l, rb[g + kNpGroups * t], x[t]);
-    }
   }
-  if (r < w) {
-#pragma unroll
-    for (int t = 0; t < kNpPerThread; ++t)
-      if (g + kNpGroups * t < w) Y[r + static_cast<long>(g + kNpGroups * t) * w] = x[t];
+  const int j = blockIdx.x * kInvCols + warp;
+  if (j >= w) return;
+  double x0 = lane == j ? 1.0 : 0.0, x1 = lane + 32 == j ? 1.0 : 0.0;
+  if (lower) {
+    for (int k = j; k + 1 < w; ++k) {
+      const double xk = __shfl_sync(0xFFFFFFFFu, k < 32 ? x0 : x1, k & 31);
+      if (k < 31 && lane > k) x0 = fma(-S[k][lane], xk, x0);
+      if (lane + 32 > k) x1 = fma(-S[k][lane + 32], xk, x1);
+    }
+    if (lane < w) X[lane + static_cast<long>(j) * ldx] = x0;
+    if (lane + 32 < w) X[lane + 32 + static_cast<long>(j) * ldx] = x1;
+  } else {
+    for (int k = j; k >= 0; --k) {
+      if (lane == (k & 31)) {
+        if (k < 32)
+          x0 *= rdiag[k];
+        else
+          x1 *= rdiag[k];
+      }
+      const double xk = __shfl_sync(0xFFFFFFFFu, k < 32 ? x0 : x1, k & 31);
+      if (lane < k) x0 = fma(-S[k][lane], xk, x0);
+      if (k > 32 && lane + 32 < k) x1 = fma(-S[k][lane + 32], xk, x1);
+    }
+    if (lane < w) Y[lane + static_cast<long>(j) * w] = x0;
+    if (lane + 32 < w) Y[lane + 32 + static_cast<long>(j) * w] = x1;
   }
 }
 
@@ -172,8 +214,10 @@ int np_panel(emul_handle_t h, double* A, long lda, int n, int j0, int d, int w, 
              const NpBufs& B) {
   double* Xd = B.X + (d - j0) + static_cast<long>(d - j0) * B.ldx;
   if (w <= kNpLeaf) {
-    np_leaf_kernel<<<1, kNpThreads, 0, h->stream>>>(A, lda, d, w, info, Xd, B.ldx, B.Y);
-    h->launches++;
+    np_leaf_kernel<<<1, 32 * kNpWarps, 0, h->stream>>>(A, lda, d, w, info);
+    np_inverse_kernel<<<dim3((w + kInvCols - 1) / kInvCols, 2), 32 * kInvCols, 0, h->stream>>>(A, lda, d, w, Xd, B.ldx,
+                                                                                              B.Y);
+    h->launches += 2;
     int rc = check_cuda(h, cudaGetLastError(), "no-pivot leaf");
     if (rc) return rc;
     const int mb = n - d - w;
