@@ -751,24 +751,17 @@ constexpr int kCholLeaf = 32;
 // its other columns, and each pivot takes one reciprocal square root rather than
 // a square root and a division.  A non-positive pivot sets *info (first index)
 // and stops; nothing runs once *info is set.
-// It also writes the leaf's inverse L^-1 (lower, w x w) to inv[i + j*ldi]:
-// forward substitution on the identity, each warp on its own columns from their
-// diagonal on (row m of X, once final, is broadcast within the warp by
-// shuffles; the multipliers L[i][m] come from shared memory), with the
-// diagonal reciprocals formed in parallel up front.
 __device__ __noinline__ double chol_rsqrt(double d) { return rsqrt(d); }
 
-__global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int d0, int w, double* inv, int ldi,
-                                                       int32_t* info) {
+__global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int d0, int w, int32_t* info) {
   __shared__ double col[2][kCholLeaf];
-  __shared__ double Ls[kCholLeaf][kCholLeaf + 1];
   __shared__ int fail_s;       // pivot that failed
   const int i = threadIdx.x & 31, q = threadIdx.x >> 5;
   if (threadIdx.x == 0) fail_s = *info != 0 ? -1 : kCholLeaf;
   __syncthreads();
   if (fail_s < 0) return;
   double* blk = A + d0 + static_cast<long>(d0) * lda;
-  // padding beyond w is the identity, so the inverse below needs no special case
+  // padding beyond w is the identity
   double d[8];
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
@@ -779,17 +772,19 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
   // pivot jj from its column x (owner warp): scaled and published
   auto pivot = [&](int jj, double& x) {
     const double diag = __shfl_sync(0xFFFFFFFFu, x, jj);
-    if (diag > 0.0) {
+    // diag > 0 by the bits (an FP64 comparison would take a DFMA's 64 cycles)
+    const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(diag));
+    if (bits - 1ull < 0x7FF0000000000000ull) {
       const double r = chol_rsqrt(diag);
-      if (i == jj)
-        x = diag * r;
-      else if (i > jj)
-        x *= r;
+      if (i >= jj) x *= r;                    // L_jj = diag r in lane jj
     } else if (i == 0) {
       atomicCAS(info, 0, d0 + jj + 1);
       fail_s = jj;
     }
     col[jj & 1][i] = i >= jj ? x : 0.0;
+    // barriers 1 and 2 in turn; the owner has published and does not wait
+    __syncwarp();
+    asm volatile("bar.arrive %0, 128;" ::"r"(1 + (jj & 1)) : "memory");
   };
   if (q == 0) pivot(0, d[0]);
   int done = w;
@@ -801,13 +796,7 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
     for (int qq = 0; qq < 4; ++qq) {
       const int jj = 4 * so + qq;
       if (jj >= w || done < w) break;         // uniform over the block
-      // barriers 1 and 2 in turn; the owner has published and does not wait
-      if (q == qq) {
-        __syncwarp();
-        asm volatile("bar.arrive %0, 128;" ::"r"(1 + (jj & 1)) : "memory");
-      } else {
-        asm volatile("bar.sync %0, 128;" ::"r"(1 + (jj & 1)) : "memory");
-      }
+      if (q != qq) asm volatile("bar.sync %0, 128;" ::"r"(1 + (jj & 1)) : "memory");
       // a failed pivot stops every warp at its step: the index was stored before
       // that step's barrier (a later one may already be there: not yet looked at)
       if (*static_cast<volatile int*>(&fail_s) <= jj) {
@@ -841,39 +830,39 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
     const int j = 4 * s + q;
     if (i < w && j < done && i >= j) blk[i + static_cast<long>(j) * lda] = d[s];
   }
-  if (done < w) return;
-  // the factor in shared memory for the inverse's multipliers
+}
+
+// The rows below a leaf, X <- X L^-T in place for the w x w (w <= 32) lower L at
+// Lp and the m x w X at Xp: row by row x_j = (x_j - sum_{k<j} x_k L_jk) / L_jj, by
+// one warp per row with column j in lane j, so a step is a shuffle, one
+// multiplication by the reciprocal of the diagonal and one DFMA (a warp has a
+// sub-partition's FP64 unit to itself, rows beside rows).  The leaf's explicit
+// inverse and a product with it took 19 + 7 us.
+constexpr int kCholSolveRows = 4;
+__global__ void __launch_bounds__(32 * kCholSolveRows) chol_solve_kernel(const double* Lp, long lda, int w, double* Xp,
+                                                                        int m, const int32_t* info) {
+  if (*info != 0) return;
+  const int lane = threadIdx.x & 31, r = blockIdx.x * kCholSolveRows + (threadIdx.x >> 5);
+  // lane j holds row j of L: its entries below the diagonal are column k's multipliers
+  double l[kCholLeaf];
 #pragma unroll
-  for (int s = 0; s < 8; ++s) Ls[i][4 * s + q] = d[s];
-  __syncthreads();
-  const double rcp = 1.0 / Ls[i][i];
-  double x[8];
+  for (int k = 0; k < kCholLeaf; ++k) l[k] = k < w && lane < w && lane > k ? Lp[lane + static_cast<long>(k) * lda] : 0.0;
+  const double rcp = lane < w ? 1.0 / Lp[lane + static_cast<long>(lane) * lda] : 0.0;
+  if (r >= m) return;
+  double x = lane < w ? Xp[r + static_cast<long>(lane) * lda] : 0.0;
 #pragma unroll
-  for (int s = 0; s < 8; ++s) x[s] = (i == 4 * s + q) ? 1.0 : 0.0;
-#pragma unroll 1
-  for (int m = 0; m < kCholLeaf; ++m) {
-    const double lim = i > m ? Ls[i][m] : 0.0;
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      if (m < 4 * s + q) continue;            // rows above a column's diagonal are zero (warp-uniform)
-      if (i == m) x[s] *= rcp;                // row m of X is final
-      const double xm = __shfl_sync(0xFFFFFFFFu, x[s], m);
-      x[s] = fma(-lim, xm, x[s]);
-    }
+  for (int j = 0; j < kCholLeaf; ++j) {
+    if (j >= w) break;                     // warp-uniform
+    const double xj = __shfl_sync(0xFFFFFFFFu, x, j) * __shfl_sync(0xFFFFFFFFu, rcp, j);
+    x = lane == j ? xj : fma(-l[j], xj, x);
   }
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int j = 4 * s + q;
-    if (i < w && j < w) inv[i + static_cast<long>(j) * ldi] = x[s];
-  }
+  if (lane < w) Xp[r + static_cast<long>(lane) * lda] = x;
 }
 
 // C(i, j) = beta C(i, j) + alpha sum_l A(i, l) B(j, l) in FP64, for the m x n
 // C (ldc) with A(i, l) = A[i*ars + l*acs] and B(j, l) = B[j*brs + l*bcs];
 // lower = 1 writes only i >= j.  A block computes an 8 x 32 tile (one entry
-// per thread) over K chunks of 32 staged in shared memory; with n <= 32 and
-// k <= 32 every block reads all its operands before it writes, so C may then
-// alias A's rows of the same block (the in-place triangular solve).  A warp's
+// per thread) over K chunks of 32 staged in shared memory.  A warp's
 // DFMA holds its sub-partition for 64-76 cycles, so 8 warps take 2 x 32 of them
 // in 2.4 us; tiles of 16 rows took twice that and left most SMs idle.
 constexpr int kNtRows = 8;
@@ -909,30 +898,32 @@ __global__ void __launch_bounds__(32 * kNtRows) dgemm_nt_small_kernel(int m, int
 }
 
 // inv (nb x nb, ld nb) <- L^-1 for the lower triangular L at A[d0.., d0..]
-// (unit diagonal if `unit`; nb <= 512, one thread per row: launch with
-// trtri_threads(nb) threads): each block solves L x = e_j for the two
-// columns j and nb - 1 - j (balanced work) by column substitution.  Thread i
-// owns row i of both x's in registers and reads row i of L sixteen columns
-// ahead (coalesced along the column); x_k is published through shared
-// memory, one barrier per step.
+// (unit diagonal if `unit`; nb <= 512, one thread per row: launch nb blocks of
+// trtri_threads(nb) threads): each block solves L x = e_j for one column j by
+// column substitution.  Thread i owns row i of x in a register and reads row i
+// of L sixteen columns ahead (coalesced along the column); x_k is published
+// through shared memory, one barrier per step.  A step is a chain of a DFMA (64
+// cycles; another for the non-unit scaling), a store, a barrier and a load; two
+// columns per block put both columns' FP64 work into that chain (40 us at nb =
+// 256, 78 us with the scaling).
 __global__ void __launch_bounds__(512) trtri_cols_kernel(const double* A, long lda, int d0, int nb, int unit,
                                                         double* inv, const int32_t* info) {
-  __shared__ double bc[2][2];
+  __shared__ double bc[2];
   if (info && *info != 0) return;
   const double* L = A + d0 + static_cast<long>(d0) * lda;
   const int i = threadIdx.x;
-  const int j0 = blockIdx.x, j1 = nb - 1 - static_cast<int>(blockIdx.x);
-  double x0 = (i == j0) ? 1.0 : 0.0, x1 = (i == j1) ? 1.0 : 0.0;
+  const int j = blockIdx.x;
+  double x = (i == j) ? 1.0 : 0.0;
   // every row's reciprocal at once: the steps below then multiply (a division
   // on each step's dependent path would cost its full FP64 latency 256 times)
   const double rinv = (!unit && i < nb) ? 1.0 / L[i + static_cast<long>(i) * lda] : 1.0;
   double ln[16];
 #pragma unroll
   for (int q = 0; q < 16; ++q) {
-    const int kk = j0 + q;
+    const int kk = j + q;
     ln[q] = (i < nb && kk < nb && i >= kk + unit) ? L[i + static_cast<long>(kk) * lda] : 0.0;
   }
-  for (int g = j0; g < nb; g += 16) {
+  for (int g = j; g < nb; g += 16) {
     double lv[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) lv[q] = ln[q];
@@ -948,25 +939,14 @@ __global__ void __launch_bounds__(512) trtri_cols_kernel(const double* A, long l
       const int kk = g + q;
       if (kk >= nb) break;
       if (i == kk) {
-        if (!unit) {
-          x0 *= rinv;
-          x1 *= rinv;
-        }
-        bc[kk & 1][0] = x0;
-        bc[kk & 1][1] = x1;
+        if (!unit) x *= rinv;
+        bc[kk & 1] = x;
       }
       __syncthreads();
-      const double b0 = bc[kk & 1][0], b1 = bc[kk & 1][1];
-      if (i > kk && i < nb) {
-        x0 = fma(-lv[q], b0, x0);
-        x1 = fma(-lv[q], b1, x1);
-      }
+      if (i > kk && i < nb) x = fma(-lv[q], bc[kk & 1], x);
     }
   }
-  if (i < nb) {
-    inv[i + static_cast<long>(j0) * nb] = x0;
-    inv[i + static_cast<long>(j1) * nb] = x1;
-  }
+  if (i < nb) inv[i + static_cast<long>(j) * nb] = x;
 }
 
 // One diagonal block of a triangular solve, x <- op(T)^-1 x for the bs x bs
@@ -1218,16 +1198,13 @@ size_t lu_extra_bytes(int nb, int nsm) {
 int chol_diag(emul_handle_t h, double* A, long lda, int d0, int jb, double* inv, int32_t* info, bool want_inv) {
   for (int c0 = 0; c0 < jb; c0 += kCholLeaf) {
     const int wp = kCholLeaf < jb - c0 ? kCholLeaf : jb - c0;
-    chol_leaf_kernel<<<1, 128, 0, h->stream>>>(A, lda, d0 + c0, wp, inv + c0 + static_cast<long>(c0) * jb, jb,
-                                                info);
+    chol_leaf_kernel<<<1, 128, 0, h->stream>>>(A, lda, d0 + c0, wp, info);
     h->launches++;
     const int r0 = c0 + wp, mr = jb - r0;
     if (mr > 0) {
       double* Lp = A + (d0 + r0) + static_cast<long>(d0 + c0) * lda;   // rows below the leaf, its columns
-      const double* ip = inv + c0 + static_cast<long>(c0) * jb;       // the leaf's inverse
-      // L(r0.., c0..) = A(r0.., c0..) L_pp^-T, in place (n = k = wp <= 32)
-      dgemm_nt_small_kernel<<<dim3((mr + kNtRows - 1) / kNtRows, 1), 32 * kNtRows, 0, h->stream>>>(mr, wp, wp, 1.0, Lp, 1, lda, ip, 1, jb,
-                                                                          0.0, Lp, lda, 0, info);
+      chol_solve_kernel<<<(mr + kCholSolveRows - 1) / kCholSolveRows, 32 * kCholSolveRows, 0, h->stream>>>(
+          A + (d0 + c0) + static_cast<long>(d0 + c0) * lda, lda, wp, Lp, mr, info);
       // A(r0.., r0..) -= L(r0.., c0..) L(r0.., c0..)^T, lower part
       dgemm_nt_small_kernel<<<dim3((mr + kNtRows - 1) / kNtRows, (mr + 31) / 32), 32 * kNtRows, 0, h->stream>>>(
           mr, mr, wp, -1.0, Lp, 1, lda, Lp, 1, lda, 1.0, A + (d0 + r0) + static_cast<long>(d0 + r0) * lda, lda, 1,
@@ -1236,7 +1213,7 @@ int chol_diag(emul_handle_t h, double* A, long lda, int d0, int jb, double* inv,
     }
   }
   if (want_inv) {
-    trtri_cols_kernel<<<(jb + 1) / 2, trtri_threads(jb), 0, h->stream>>>(A, lda, d0, jb, 0, inv, info);
+    trtri_cols_kernel<<<jb, trtri_threads(jb), 0, h->stream>>>(A, lda, d0, jb, 0, inv, info);
     h->launches++;
   }
   return check_cuda(h, cudaGetLastError(), "Cholesky diagonal block");
@@ -1425,7 +1402,7 @@ int panel_getrf(emul_handle_t h, double* A, long lda, int n, int j0, int jb, int
   if (rc) return rc;
   rc = laswp(h, A, lda, j0 + w1, j0 + jb, ipiv, j0, j0 + w1, B.map);
   if (rc) return rc;
-  trtri_cols_kernel<<<(w1 + 1) / 2, trtri_threads(w1), 0, h->stream>>>(A, lda, j0, w1, 1, B.inv, nullptr);
+  trtri_cols_kernel<<<w1, trtri_threads(w1), 0, h->stream>>>(A, lda, j0, w1, 1, B.inv, nullptr);
   h->launches++;
   rc = check_cuda(h, cudaGetLastError(), "panel trtri");
   if (rc) return rc;
@@ -1888,7 +1865,7 @@ int emul_dgetrf(emul_handle_t h, int n, double* A, int lda, int32_t* ipiv, int n
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_start, h->stream), "stream events");
       if (!rc) rc = emul::check_cuda(h, cudaStreamWaitEvent(h->aux, h->aux_start, 0), "stream events");
       if (rc) return rc;
-      emul::trtri_cols_kernel<<<(jb + 1) / 2, emul::trtri_threads(jb), 0, h->aux>>>(A, lda, j0, jb, 1, B.inv,
+      emul::trtri_cols_kernel<<<jb, emul::trtri_threads(jb), 0, h->aux>>>(A, lda, j0, jb, 1, B.inv,
                                                                                        nullptr);
       h->launches++;
       rc = emul::check_cuda(h, cudaGetLastError(), "trtri");

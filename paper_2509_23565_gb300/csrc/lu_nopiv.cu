@@ -45,7 +45,11 @@ inline size_t np_al(size_t x) { return (x + kNpAl - 1) / kNpAl * kNpAl; }
 // the other warps meet it there after theirs.  The pivot row comes by shuffles.
 // (64 x 64 with both inverses took 256 us in one CTA of 1024 threads on shared
 // memory with two barriers a step and the division after the update.)
-__device__ __noinline__ double np_recip(double p) { return p != 0.0 ? 1.0 / p : 0.0; }
+__device__ __noinline__ double np_recip(double p) { return 1.0 / p; }
+// x == 0 by the bits (an FP64 comparison would take a DFMA's 64 cycles)
+__device__ __forceinline__ bool np_zero(double x) {
+  return (static_cast<unsigned long long>(__double_as_longlong(x)) << 1) == 0;
+}
 
 __global__ void __launch_bounds__(32 * kNpWarps, 1) np_leaf_kernel(double* A, long lda, int d, int w, int32_t* info) {
   __shared__ double mult[2][kNpLeaf];
@@ -64,14 +68,17 @@ __global__ void __launch_bounds__(32 * kNpWarps, 1) np_leaf_kernel(double* A, lo
   // multipliers of pivot k from its column (in registers c0, c1 of the owner)
   auto scale = [&](int k, double& c0, double& c1) {
     const double p = __shfl_sync(0xFFFFFFFFu, k < 32 ? c0 : c1, k & 31);
-    const double r = np_recip(p);           // 0 for a zero pivot
-    if (p == 0.0 && lane == 0) atomicCAS(info, 0, d + k + 1);
-    if (r != 0.0) {
+    const double r = np_zero(p) ? 0.0 : np_recip(p);
+    if (np_zero(p) && lane == 0) atomicCAS(info, 0, d + k + 1);
+    if (!np_zero(r)) {
       if (lane > k) c0 *= r;
       if (lane + 32 > k) c1 *= r;
     }
     mult[k & 1][lane] = lane > k ? c0 : 0.0;
     mult[k & 1][lane + 32] = lane + 32 > k ? c1 : 0.0;
+    // barriers 1 and 2 in turn; the owner has published and does not wait
+    __syncwarp();
+    if (k + 1 < w) asm volatile("bar.arrive %0, %1;" ::"r"(1 + (k & 1)), "n"(32 * kNpWarps) : "memory");
   };
   if (g == 0) scale(0, v[0][0], v[0][1]);
   // pivots k = 8 so + kk; the inner loop stays rolled (64 copies of a step would
@@ -82,13 +89,7 @@ __global__ void __launch_bounds__(32 * kNpWarps, 1) np_leaf_kernel(double* A, lo
     for (int kk = 0; kk < kNpWarps; ++kk) {
       const int k = kNpWarps * so + kk;
       if (k + 1 >= w) break;
-      // barriers 1 and 2 in turn; the owner has published and does not wait
-      if (g == kk) {
-        __syncwarp();
-        asm volatile("bar.arrive %0, %1;" ::"r"(1 + (k & 1)), "n"(32 * kNpWarps) : "memory");
-      } else {
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + (k & 1)), "n"(32 * kNpWarps) : "memory");
-      }
+      if (g != kk) asm volatile("bar.sync %0, %1;" ::"r"(1 + (k & 1)), "n"(32 * kNpWarps) : "memory");
       const double l0 = mult[k & 1][lane], l1 = mult[k & 1][lane + 32];
       auto update = [&](double& c0, double& c1) {
         const double u = __shfl_sync(0xFFFFFFFFu, so < kCols / 2 ? c0 : c1, k & 31);
