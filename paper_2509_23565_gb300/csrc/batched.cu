@@ -39,8 +39,9 @@ struct BatchSys {
 
 namespace {
 
-constexpr int kBThreads = 256;
+constexpr int kBThreads = 512;
 constexpr int kMaxS = 8;
+constexpr int kMaxN = 4096;       // largest system
 constexpr int kStallIters = 8;   // refinement steps before a system is refactored with 8 slices
 
 struct Scratch {
@@ -50,9 +51,8 @@ struct Scratch {
   int8_t* SB;      // [s][n][nb4] slices of U12 columns
   int* ea;         // n
   int* fb;         // n
-  double* x;       // n
   double* r;       // n
-  float* d;        // n
+  int* perm;       // n: row i of P b is b[perm[i]]
 };
 
 __device__ __forceinline__ int f32_exponent(uint32_t u) {   // smallest e with |x| < 2^e, u = |x| bits (x != 0)
@@ -99,22 +99,6 @@ __device__ void block_argmax(float v, int idx, float* sv, int* si, float& bv, in
   __syncthreads();
 }
 
-__device__ double block_sum_d(double v, double* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kBThreads / 32; ++i) t += red[i];
-    red[0] = t;
-  }
-  __syncthreads();
-  t = red[0];
-  __syncthreads();
-  return t;
-}
-
 __device__ double block_max_d(double v, double* red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
@@ -131,29 +115,63 @@ __device__ double block_max_d(double v, double* red) {
   return t;
 }
 
-// Solve (LU) y = P v in FP32 in place on d (length n): row interchanges, unit
-// lower, upper.  Column-oriented, one barrier per column.
-__device__ void lu_solve_f32(const float* W, int n, const int* piv, float* d) {
-  if (threadIdx.x == 0)
-    for (int k = 0; k < n; ++k) {
-      const int p = piv[k];
-      if (p != k) {
-        const float t = d[k];
-        d[k] = d[p];
-        d[p] = t;
+// Solve (LU) y = d in FP32 in place on d (shared memory, length n, rows already
+// interchanged): unit lower, then upper, by blocks of 32 rows: one warp solves a
+// block (row per lane, values by shuffle), then every thread takes the block's 32
+// columns off its own rows, 32 loads in flight.  Each entry sees the operations
+// of the column-by-column substitution in the same order.
+__device__ void lu_solve_f32(const float* W, int n, float* d) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int nblk = (n + 31) / 32;
+  for (int st = 0; st < 2 * nblk; ++st) {
+    const bool lower = st < nblk;
+    const int k0 = 32 * (lower ? st : 2 * nblk - 1 - st);
+    const int w = n - k0 < 32 ? n - k0 : 32;
+    const float* B = W + k0 + static_cast<long>(k0) * n;      // the diagonal block
+    if (tid < 32) {
+      float v = lane < w ? d[k0 + lane] : 0.f;
+      float l[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) l[k] = k < w && lane < w ? B[lane + static_cast<long>(k) * n] : 0.f;
+      if (lower) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          const float dk = __shfl_sync(0xFFFFFFFFu, v, k);
+          if (lane > k && k < w) v = fmaf(-l[k], dk, v);
+        }
+      } else {
+        const float diag = lane < w ? B[lane + static_cast<long>(lane) * n] : 1.f;
+#pragma unroll
+        for (int k = 31; k >= 0; --k) {
+          if (k >= w) continue;
+          const float dk = __shfl_sync(0xFFFFFFFFu, v / diag, k);
+          if (lane == k)
+            v = dk;
+          else if (lane < k)
+            v = fmaf(-l[k], dk, v);
+        }
       }
+      if (lane < w) d[k0 + lane] = v;
     }
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    const float dk = d[k];
-    for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) d[i] = fmaf(-W[i + static_cast<long>(k) * n], dk, d[i]);
     __syncthreads();
-  }
-  for (int k = n - 1; k >= 0; --k) {
-    if (threadIdx.x == 0) d[k] = d[k] / W[k + static_cast<long>(k) * n];
-    __syncthreads();
-    const float dk = d[k];
-    for (int i = threadIdx.x; i < k; i += blockDim.x) d[i] = fmaf(-W[i + static_cast<long>(k) * n], dk, d[i]);
+    const int lo = lower ? k0 + w : 0, hi = lower ? n : k0;
+    for (int i = lo + tid; i < hi; i += blockDim.x) {
+      const float* p = W + i + static_cast<long>(k0) * n;
+      float l[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) l[k] = k < w ? p[static_cast<long>(k) * n] : 0.f;
+      float v = d[i];
+      if (lower) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+          if (k < w) v = fmaf(-l[k], d[k0 + k], v);
+      } else {
+#pragma unroll
+        for (int k = 31; k >= 0; --k)
+          if (k < w) v = fmaf(-l[k], d[k0 + k], v);
+      }
+      d[i] = v;
+    }
     __syncthreads();
   }
 }
@@ -174,7 +192,9 @@ __device__ __forceinline__ uint32_t ld_s8x4(const int8_t* p, bool ok) {
   return ok ? *reinterpret_cast<const uint32_t*>(p) : 0u;
 }
 
-__device__ void factor_system(const BatchSys& S, int s, Scratch& sc, int* info, float* sv, int* si) {
+// The general factorization: any size, block and slice count, the working copy
+// in global memory throughout.  Serves what factor_fast does not take.
+__device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info, float* sv, int* si) {
   const int n = S.n, nb = S.nb;
   const int nb4 = (nb + 31) / 32 * 32;   // slice row length: whole K steps of 32, zero padded
   float* W = sc.W;
@@ -319,6 +339,552 @@ __device__ void factor_system(const BatchSys& S, int s, Scratch& sc, int* info, 
   }
 }
 
+// ---------------------------------------------------------------- the fast factorization
+// Same arithmetic as factor_general, operation for operation, for n <= kFastN,
+// blocks of 16 or 32 and S = 3, 4 or 8 slices, arranged for one block per SM:
+//  - the panel lives in registers (two rows per thread), a column costs two
+//    barriers: maxima by warp reductions on the bit patterns, the pivot row and
+//    row c through shared memory;
+//  - the interchanges of a panel become one gather map; the columns right of it
+//    are gathered as they are staged for U12 (one warp per column), the L columns
+//    left of it get all later interchanges at the end, composed;
+//  - U12 takes one thread per column with the column in registers;
+//  - digits of L21 (by the threads that hold its rows) and of U12 go to shared
+//    memory (8 planes of L21 to global) as bytes; the level sums take them as FP16
+//    with FP32 accumulation, exact below 2^22 (mma.sync: 1000 multiply-adds per
+//    clock per SM in FP16, 251 in INT8, measured);
+//  - the update W - D keeps one FP64 addition per entry: the conversions around
+//    it are integer operations (FP64 runs at 1.68 lanes per clock per SM, its
+//    conversions below 1).
+// In factor_general every step strides through global memory (U12 by columns
+// apart, full-row interchanges per pivot), and 152 such systems at once overflow
+// L2: 1024 systems of 64..1024 rows took 247 ms.
+constexpr int kFastN = 2 * kBThreads;
+constexpr int kFastNb = 32;
+constexpr int kFastSmem = 200 * 1024;      // digits and staged columns
+
+struct FastShared {
+  float prow[2][kFastNb], crow[kFastNb];
+  uint32_t wk[kBThreads / 32];
+  int wr[kBThreads / 32];
+  int pv[kFastNb];                          // pivot rows, relative to the panel
+  int top[kFastNb];                         // source of row i of the panel's block
+  int ddst[kFastNb], dsrc[kFastNb], dcnt;   // displaced rows
+  float L11[kFastNb][kFastNb + 4];          // L11[k][i]
+  int ea[kFastN], fb[kBThreads];
+};
+
+// Gather map of the panel's jb interchanges (rows relative to the panel): row
+// i < jb receives row top[i], row ddst[q] row dsrc[q].  Run by one warp.
+__device__ void fast_map(FastShared& F, int jb) {
+  const int lane = threadIdx.x & 31;
+  auto sigma = [&](int r) {
+    for (int k = jb - 1; k >= 0; --k) {
+      const int p = F.pv[k];
+      r = r == k ? p : (r == p ? k : r);
+    }
+    return r;
+  };
+  bool disp = false;
+  int p = 0, src = 0;
+  if (lane < jb) {
+    F.top[lane] = sigma(lane);
+    p = F.pv[lane];
+    if (p >= jb) {
+      disp = true;
+      for (int j = 0; j < lane && disp; ++j) disp = F.pv[j] != p;
+      if (disp) {
+        src = sigma(p);
+        disp = src != p;
+      }
+    }
+  }
+  const unsigned m = __ballot_sync(0xFFFFFFFFu, disp);
+  if (disp) {
+    const int q = __popc(m & ((1u << lane) - 1u));
+    F.ddst[q] = p;
+    F.dsrc[q] = src;
+  }
+  if (lane == 0) F.dcnt = __popc(m);
+}
+
+// INT8 digits of a row of up to 32 floats (exponent e), 32 bytes per plane.
+template <int S, int NB>
+__device__ __forceinline__ void fast_digits(const float (&x)[NB], int jb, int e, int8_t* dst, size_t plane) {
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    uint32_t w[S][4];
+#pragma unroll
+    for (int p = 0; p < S; ++p)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[p][i] = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int c = 16 * g + i;
+      if (c >= NB) continue;
+      const uint32_t u = c < jb ? __float_as_uint(x[c < NB ? c : 0]) : 0u;
+      const uint32_t a = u & 0x7FFFFFFFu;
+      const uint64_t mag = a ? f32_scaled(a, e, 7 * S) : 0ull;
+#pragma unroll
+      for (int p = 0; p < S; ++p) {
+        const int dg = static_cast<int>(mag >> (7 * (S - 1 - p))) & 127;
+        w[p][i >> 2] |= (static_cast<uint32_t>(u >> 31 ? -dg : dg) & 255u) << (8 * (i & 3));
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < S; ++p)
+      *reinterpret_cast<uint4*>(dst + p * plane + 16 * g) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+  }
+}
+
+// T 2^sh as a double, exact for |T| < 2^53 and normal results.
+__device__ __forceinline__ double exact_scaled(long long T, int sh) {
+  const unsigned long long sgn = static_cast<unsigned long long>(T >> 63);
+  const unsigned long long a = (static_cast<unsigned long long>(T) ^ sgn) - sgn;
+  const int lz = __clzll(static_cast<long long>(a));
+  const unsigned long long bits = (static_cast<unsigned long long>(63 - lz + sh + 1022) << 52) + ((a << (lz & 63)) >> 11);
+  return a ? __longlong_as_double(static_cast<long long>(bits | (sgn << 63))) : 0.0;
+}
+// An integer-valued float (below 2^24) times 2^sh, exactly.
+__device__ __forceinline__ double float_scaled(float f, int sh) {
+  const uint32_t u = __float_as_uint(f), a = u & 0x7FFFFFFFu;
+  const double d = __hiloint2double(static_cast<int>((u & 0x80000000u) | ((a >> 3) + ((896u + static_cast<uint32_t>(sh)) << 20))),
+                                    static_cast<int>(a << 29));
+  return a ? d : 0.0;
+}
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t u = __float_as_uint(f), a = u & 0x7FFFFFFFu;
+  if (a - 0x00800000u >= 0x7F000000u) return static_cast<double>(f);     // zero, subnormal, Inf, NaN
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | ((a >> 3) + (896u << 20))), static_cast<int>(a << 29));
+}
+__device__ __forceinline__ float narrow(double d) {      // rounded to nearest even
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(d)), lo = static_cast<uint32_t>(__double2loint(d));
+  const uint32_t ah = hi & 0x7FFFFFFFu;
+  if (ah - (897u << 20) >= (254u << 20)) return static_cast<float>(d);   // zero, below or above the normal floats
+  uint32_t v = ((ah - (896u << 20)) << 3) | (lo >> 29);
+  const uint32_t rem = lo & 0x1FFFFFFFu;
+  v += rem > 0x10000000u || (rem == 0x10000000u && (v & 1u)) ? 1u : 0u;
+  return __uint_as_float((hi & 0x80000000u) | v);
+}
+
+// Four signed digits (the bytes of x) as two pairs of FP16, exactly: a digit
+// plus 128 goes under 1024.0's exponent, where one unit is the last place.
+__device__ __forceinline__ void digits_f16(uint32_t x, uint32_t& h0, uint32_t& h1) {
+  x ^= 0x80808080u;
+  const uint32_t m0 = __byte_perm(x, 0x64646464u, 0x4140), m1 = __byte_perm(x, 0x64646464u, 0x4342);
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(h0) : "r"(m0), "r"(0x64806480u));
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(h1) : "r"(m1), "r"(0x64806480u));
+}
+__device__ __forceinline__ void mma_f16_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                                uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// The four words of a plane's 16 x 32 digits of A (rows g and g + 8, K bytes 4 tq
+// and 16 + 4 tq) as the A fragments of two K = 16 MMAs.  Which K a fragment slot
+// stands for is free as long as A and B agree: both take a word's bytes in order.
+__device__ __forceinline__ void a_fragments(const uint32_t (&w)[4], uint32_t (&h)[8]) {
+  digits_f16(w[0], h[0], h[2]);
+  digits_f16(w[1], h[1], h[3]);
+  digits_f16(w[2], h[4], h[6]);
+  digits_f16(w[3], h[5], h[7]);
+}
+
+// D of one entry from its level sums (integer-valued floats below 2^22, levels
+// 2..S+1) at the exponent e = e_i + f_j, as factor_general forms it: for S <= 5
+// the exact sum, converted once; for 8 slices the levels added one after another
+// in FP64, which is exact through level 6 and as long as the sum of the first six
+// stays below 2^53 through level 7.
+template <int S>
+__device__ __forceinline__ double fast_sum(const float (&v)[S], int e) {
+  int c[S];
+#pragma unroll
+  for (int i = 0; i < S; ++i) c[i] = __float_as_int(v[i] + 12582912.0f) - 0x4B400000;   // exact below 2^22
+  if constexpr (S == 3) {
+    return exact_scaled(static_cast<long long>(c[0] * 128 + c[1]) * 128 + c[2], e - 28);
+  } else if constexpr (S == 4) {
+    return exact_scaled((static_cast<long long>(c[0] * 128 + c[1]) << 14) + (c[2] * 128 + c[3]), e - 35);
+  } else {
+    static_assert(S == 8, "slice counts of the fast factorization");
+    const long long s6 = (static_cast<long long>(c[0] * 128 + c[1]) << 21) +
+                         (static_cast<long long>(c[2] * 128 + c[3]) << 7) + c[4];
+    const long long s7 = s6 * 128 + c[5];
+    double d;
+    if (s7 + (1ll << 53) < 0 || s7 > (1ll << 53))
+      d = exact_scaled(s6, e - 42) + float_scaled(v[5], e - 49);
+    else
+      d = exact_scaled(s7, e - 49);
+    d += float_scaled(v[6], e - 56);
+    return d + float_scaled(v[7], e - 63);
+  }
+}
+
+template <int S, int NB>
+__device__ __noinline__ void factor_fast(const BatchSys& sys, Scratch& sc, int* info, FastShared& F, uint8_t* dyn) {
+  const int n = sys.n;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kBThreads / 32;
+  float* W = sc.W;
+  for (int j = warp; j < n; j += kWarps) {
+    const double* src = sys.A + j * sys.lda;
+    float* dst = W + static_cast<long>(j) * n;
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32) dst[i] = static_cast<float>(src[i]);
+  }
+  __syncthreads();
+  for (int j0 = 0; j0 < n; j0 += NB) {
+    const int jb = NB < n - j0 ? NB : n - j0;
+    const int m = n - j0, m2 = m - jb;
+    // ---- panel: thread t holds rows t and t + 512 (relative to j0)
+    float x[2][NB];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = tid + h * kBThreads;
+#pragma unroll
+      for (int c = 0; c < NB; ++c)
+        x[h][c] = r < m && c < jb ? W[(j0 + r) + static_cast<long>(j0 + c) * n] : 0.f;
+    }
+#pragma unroll
+    for (int c = 0; c < NB; ++c) {
+      if (c >= jb) break;
+      // largest |value| (NaN never), then the smallest row; key 0: none
+      uint32_t key[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = tid + h * kBThreads;
+        const uint32_t a = __float_as_uint(x[h][c]) & 0x7FFFFFFFu;
+        key[h] = r >= c && r < m && a <= 0x7F800000u ? a + 1u : 0u;
+      }
+      {
+        const uint32_t mk = __reduce_max_sync(0xFFFFFFFFu, key[0] > key[1] ? key[0] : key[1]);
+        const int mr = __reduce_min_sync(
+            0xFFFFFFFFu, key[0] == mk ? tid : (key[1] == mk ? tid + kBThreads : 0x7FFFFFFF));
+        if (lane == 0) {
+          F.wk[warp] = mk;
+          F.wr[warp] = mr;
+        }
+      }
+      __syncthreads();
+      int p;
+      {
+        const uint32_t k1 = F.wk[lane & (kWarps - 1)];
+        const uint32_t mk = __reduce_max_sync(0xFFFFFFFFu, k1);
+        const int mr = __reduce_min_sync(0xFFFFFFFFu, k1 == mk ? F.wr[lane & (kWarps - 1)] : 0x7FFFFFFF);
+        p = mk ? mr : c;
+      }
+      float* prow = F.prow[c & 1];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (tid + h * kBThreads == p) {
+#pragma unroll
+          for (int q = 0; q < NB; ++q) prow[q] = x[h][q];
+        }
+      if (tid == c && p != c) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) F.crow[q] = x[0][q];
+      }
+      if (tid == 0) F.pv[c] = p;
+      __syncthreads();
+      if (p != c) {
+        if (tid == c) {
+#pragma unroll
+          for (int q = 0; q < NB; ++q) x[0][q] = prow[q];
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (tid + h * kBThreads == p) {
+#pragma unroll
+            for (int q = 0; q < NB; ++q) x[h][q] = F.crow[q];
+          }
+      }
+      const float piv = prow[c];
+      if (piv == 0.f) {
+        if (tid == 0 && *info == 0) *info = j0 + c + 1;
+      } else {
+        float u[NB];
+#pragma unroll
+        for (int q = c + 1; q < NB; ++q) u[q] = prow[q];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (tid + h * kBThreads > c && tid + h * kBThreads < m) {
+            const float l = x[h][c] / piv;
+            x[h][c] = l;
+#pragma unroll
+            for (int q = c + 1; q < NB; ++q) x[h][q] = fmaf(-l, u[q], x[h][q]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = tid + h * kBThreads;
+      if (r < m) {
+#pragma unroll
+        for (int c = 0; c < NB; ++c)
+          if (c < jb) W[(j0 + r) + static_cast<long>(j0 + c) * n] = x[h][c];
+      }
+    }
+    if (tid < jb) sc.piv[j0 + tid] = j0 + F.pv[tid];        // (F.pv was published by the last column's barrier)
+    if (m2 <= 0) break;
+    // ---- gather map; L11 and the digits of L21 into shared memory
+    if (warp == kWarps - 1) fast_map(F, jb);
+    const int m2p = (m2 + 15) / 16 * 16;
+    constexpr bool kSharedA = S <= 4;                       // 8 planes of 1024 rows do not fit
+    int8_t* SA = kSharedA ? reinterpret_cast<int8_t*>(dyn) : sc.SA;   // [S][m2p][32]
+    const size_t pa = static_cast<size_t>(m2p) * 32;
+    const size_t used = kSharedA ? S * pa : 0;
+    uint8_t* rest = dyn + used;
+    int cc = static_cast<int>((kFastSmem - used) / (132 + 32 * S)) / 16 * 16;   // columns staged at a time
+    if (cc > kBThreads) cc = kBThreads;
+    float* Us = reinterpret_cast<float*>(rest + static_cast<size_t>(S) * cc * 32);  // [cc][33]
+    int8_t* SB = reinterpret_cast<int8_t*>(rest);           // [S][cc][32]
+    const size_t pb = static_cast<size_t>(cc) * 32;
+    if (tid < jb) {
+#pragma unroll
+      for (int k = 0; k < NB; ++k) F.L11[k][tid] = x[0][k];
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int q = tid + h * kBThreads - jb;
+      if (q >= 0 && q < m2) {
+        uint32_t mx = 0;
+#pragma unroll
+        for (int c = 0; c < NB; ++c) {
+          const uint32_t a = c < jb ? __float_as_uint(x[h][c]) & 0x7FFFFFFFu : 0u;
+          mx = a > mx ? a : mx;
+        }
+        const int e = mx ? f32_exponent(mx) : 0;
+        F.ea[q] = e;
+        fast_digits<S, NB>(x[h], jb, e, SA + static_cast<size_t>(q) * 32, pa);
+      }
+    }
+    __syncthreads();
+    for (int c0 = 0; c0 < m2; c0 += cc) {
+      const int nc = cc < m2 - c0 ? cc : m2 - c0;
+      // ---- stage the top rows of the columns, interchanged; displaced rows are put in place
+      for (int ci = warp; ci < nc; ci += 4 * kWarps) {
+        float v[4], dv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int cq = ci + q * kWarps;
+          const float* col = W + j0 + static_cast<long>(j0 + jb + c0 + cq) * n;
+          v[q] = cq < nc && lane < jb ? col[F.top[lane]] : 0.f;
+          dv[q] = cq < nc && lane < F.dcnt ? col[F.dsrc[lane]] : 0.f;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int cq = ci + q * kWarps;
+          if (cq >= nc) continue;
+          float* col = W + j0 + static_cast<long>(j0 + jb + c0 + cq) * n;
+          Us[cq * 33 + lane] = v[q];
+          if (lane < F.dcnt) col[F.ddst[lane]] = dv[q];
+        }
+      }
+      __syncthreads();
+      // ---- U12 = L11^-1 A12 and its digits, one thread per column
+      if (tid < nc) {
+        float u[NB];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) u[k] = Us[tid * 33 + k];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+          if (k >= jb) break;
+#pragma unroll
+          for (int i = k + 1; i < NB; ++i)
+            if (i < jb) u[i] = fmaf(-F.L11[k][i], u[k], u[i]);
+        }
+        uint32_t mx = 0;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+          Us[tid * 33 + k] = u[k];
+          const uint32_t a = k < jb ? __float_as_uint(u[k]) & 0x7FFFFFFFu : 0u;
+          mx = a > mx ? a : mx;
+        }
+        const int e = mx ? f32_exponent(mx) : 0;
+        F.fb[tid] = e;
+        fast_digits<S, NB>(u, jb, e, SB + static_cast<size_t>(tid) * 32, pb);
+      }
+      __syncthreads();
+      for (int ci = warp; ci < nc; ci += kWarps)
+        if (lane < jb) W[(j0 + lane) + static_cast<long>(j0 + jb + c0 + ci) * n] = Us[ci * 33 + lane];
+      // ---- A22 -= D (see factor_general): a warp keeps the digits of 16 rows and
+      // goes along its columns, 16 x 8 at a time
+      const int strips = m2p / 16, ct = (nc + 7) / 8;
+      const int cgroups = strips >= kWarps ? 1 : (kWarps + strips - 1) / strips;
+      const int g = lane >> 2, tq = lane & 3;
+      for (int item = warp; item < strips * cgroups; item += kWarps) {
+        const int i0 = (item % strips) * 16;
+        const int ra = i0 + g, rb = ra + 8;
+        uint32_t aw[S][4], ah[S <= 4 ? S : 1][8];
+#pragma unroll
+        for (int p = 0; p < S; ++p) {
+          const int8_t* Ap = SA + p * pa + tq * 4;
+          aw[p][0] = ld_s8x4(Ap + ra * 32, ra < m2);
+          aw[p][1] = ld_s8x4(Ap + rb * 32, rb < m2);
+          aw[p][2] = ld_s8x4(Ap + ra * 32 + 16, ra < m2);
+          aw[p][3] = ld_s8x4(Ap + rb * 32 + 16, rb < m2);
+          if (S <= 4) a_fragments(aw[p], ah[S <= 4 ? p : 0]);
+        }
+        const int e0 = ra < m2 ? F.ea[ra] : 0, e1 = rb < m2 ? F.ea[rb] : 0;
+        float* const w0 = W + (j0 + jb + ra) + static_cast<long>(j0 + jb + c0 + tq * 2) * n;   // (ra, column tq * 2)
+        // the entries of W, one tile ahead
+        auto load_w = [&](int tile, float (&w)[4]) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int j = tile * 8 + (q & 1);
+            w[q] = (q >= 2 ? rb : ra) < m2 && j + tq * 2 < nc ? w0[(q >= 2 ? 8 : 0) + static_cast<long>(j) * n] : 0.f;
+          }
+        };
+        float wn[4] = {0.f, 0.f, 0.f, 0.f};
+        if (item / strips < ct) load_w(item / strips, wn);
+        for (int tile = item / strips; tile < ct; tile += cgroups) {
+          const int cl = tile * 8;                            // columns of the chunk
+          float wv[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) wv[q] = wn[q];
+          if (tile + cgroups < ct) load_w(tile + cgroups, wn);
+          uint32_t bh[S][4];
+#pragma unroll
+          for (int p = 0; p < S; ++p) {
+            const int8_t* Bp = SB + p * pb + static_cast<size_t>(cl + g) * 32 + tq * 4;
+            digits_f16(ld_s8x4(Bp, cl + g < nc), bh[p][0], bh[p][1]);
+            digits_f16(ld_s8x4(Bp + 16, cl + g < nc), bh[p][2], bh[p][3]);
+          }
+          float acc[S][4];
+#pragma unroll
+          for (int i = 0; i < S; ++i)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
+#pragma unroll
+          for (int p = 0; p < S; ++p) {
+            uint32_t h[8];
+            if constexpr (S <= 4) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) h[i] = ah[p][i];
+            } else {
+              a_fragments(aw[p], h);
+            }
+#pragma unroll
+            for (int q = 0; q + p < S; ++q) {                 // planes p + 1 and q + 1: level p + q + 2
+              mma_f16_16x8x16(acc[p + q], h[0], h[1], h[2], h[3], bh[q][0], bh[q][1]);
+              mma_f16_16x8x16(acc[p + q], h[4], h[5], h[6], h[7], bh[q][2], bh[q][3]);
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int j = cl + (q & 1);
+            if ((q >= 2 ? rb : ra) >= m2 || j + tq * 2 >= nc) continue;
+            float v[S];
+#pragma unroll
+            for (int i = 0; i < S; ++i) v[i] = acc[i][q];
+            const double D = fast_sum<S>(v, (q >= 2 ? e1 : e0) + F.fb[j + tq * 2]);
+            w0[(q >= 2 ? 8 : 0) + static_cast<long>(j) * n] = narrow(widen(wv[q]) - D);
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+  __syncthreads();
+  // ---- the L columns of every panel but the last: the later panels'
+  // interchanges, composed from the last panel back; then the whole permutation
+  int* G = reinterpret_cast<int*>(dyn);                     // row r receives row G[r]
+  int* one = G + kFastN;                                    // one panel's map
+  float* buf = reinterpret_cast<float*>(one + kFastN);      // [NB][n]
+  for (int i = tid; i < n; i += blockDim.x) G[i] = i;
+  for (int j0 = (n - 1) / NB * NB; j0 >= 0; j0 -= NB) {
+    const int jb = NB < n - j0 ? NB : n - j0;
+    if (tid < jb) F.pv[tid] = sc.piv[j0 + tid] - j0;
+    for (int i = tid; i < n; i += blockDim.x) one[i] = i;
+    __syncthreads();
+    if (warp == 0) {
+      fast_map(F, jb);
+      __syncwarp();
+      if (lane < jb) one[j0 + lane] = j0 + F.top[lane];
+      if (lane < F.dcnt) one[j0 + F.ddst[lane]] = j0 + F.dsrc[lane];
+    }
+    __syncthreads();
+    for (int i = tid; i < n; i += blockDim.x) G[i] = one[G[i]];
+    __syncthreads();
+    if (j0 == 0) break;
+    // the panel left of j0: columns j0 - NB .. j0 - 1, rows from j0 on
+    for (int e = warp; e < NB; e += kWarps)
+      for (int r = j0 + lane; r < n; r += 32) buf[e * n + r] = W[r + static_cast<long>(j0 - NB + e) * n];
+    __syncthreads();
+    for (int e = warp; e < NB; e += kWarps)
+      for (int r = j0 + lane; r < n; r += 32) W[r + static_cast<long>(j0 - NB + e) * n] = buf[e * n + G[r]];
+    __syncthreads();
+  }
+  for (int i = tid; i < n; i += blockDim.x) sc.perm[i] = G[i];
+  __syncthreads();
+}
+
+// Factor one system and leave its row permutation in sc.perm.
+__device__ __noinline__ void factor_system(const BatchSys& sys, int s, Scratch& sc, int* info, float* sv, int* si, FastShared& F,
+                              uint8_t* dyn) {
+  // the slice counts and blocks the tuner chooses from, and the 8 slices of a
+  // system whose refinement stalls
+  if (sys.n <= kFastN && (s == 3 || s == 4 || s == 8) && (sys.nb == 16 || sys.nb == 32)) {
+    if (sys.nb == 32) {
+      if (s == 3) return factor_fast<3, 32>(sys, sc, info, F, dyn);
+      if (s == 4) return factor_fast<4, 32>(sys, sc, info, F, dyn);
+      return factor_fast<8, 32>(sys, sc, info, F, dyn);
+    }
+    if (s == 3) return factor_fast<3, 16>(sys, sc, info, F, dyn);
+    if (s == 4) return factor_fast<4, 16>(sys, sc, info, F, dyn);
+    return factor_fast<8, 16>(sys, sc, info, F, dyn);
+  }
+  factor_general(sys, s, sc, info, sv, si);
+  __syncthreads();
+  int* G = reinterpret_cast<int*>(dyn);
+  for (int i = threadIdx.x; i < sys.n; i += blockDim.x) G[i] = i;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int k = 0; k < sys.n; ++k) {
+      const int p = sc.piv[k];
+      if (p != k) {
+        const int v = G[k];
+        G[k] = G[p];
+        G[p] = v;
+      }
+    }
+  __syncthreads();
+  for (int i = threadIdx.x; i < sys.n; i += blockDim.x) sc.perm[i] = G[i];
+  __syncthreads();
+}
+
+// acc[h] (h = 0, 1) over the columns of rows i0 and i0 + blockDim.x of A, in
+// column order: acc = f(acc, a, x_j), sixteen loads in flight.
+template <typename Fn>
+__device__ __forceinline__ void row_pass(const double* A, long lda, int n, int i0, double (&acc)[2], Fn f) {
+  const int i1 = i0 + static_cast<int>(blockDim.x);
+  const double* p0 = A + (i0 < n ? i0 : 0);
+  const double* p1 = A + (i1 < n ? i1 : 0);
+  int j = 0;
+  for (; j + 8 <= n; j += 8) {
+    double a0[8], a1[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a0[q] = __ldg(p0 + (j + q) * lda);
+    if (i1 < n) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) a1[q] = __ldg(p1 + (j + q) * lda);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc[0] = f(acc[0], a0[q], j + q);
+    if (i1 < n) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc[1] = f(acc[1], a1[q], j + q);
+    }
+  }
+  for (; j < n; ++j) {
+    acc[0] = f(acc[0], __ldg(p0 + j * lda), j);
+    if (i1 < n) acc[1] = f(acc[1], __ldg(p1 + j * lda), j);
+  }
+}
+
 __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys* sys, int count, unsigned int* queue,
                                                                   uint8_t* scratch, size_t per_block, int nmax,
                                                                   int max_iter, double target, int32_t* info_arr,
@@ -328,6 +894,11 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
   __shared__ double red[kBThreads / 32];
   __shared__ int task_s;
   __shared__ int info_s;
+  __shared__ __align__(16) FastShared F;
+  extern __shared__ __align__(16) uint8_t dyn[];
+  // while solving: the right-hand side and the solution
+  float* ds = reinterpret_cast<float*>(dyn);
+  double* xs = reinterpret_cast<double*>(dyn + kMaxN * sizeof(float));
   uint8_t* base = scratch + per_block * blockIdx.x;
   Scratch sc;
   {
@@ -343,9 +914,8 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
     sc.SB = reinterpret_cast<int8_t*>(take(static_cast<size_t>(kMaxS) * nmax * 64));
     sc.ea = reinterpret_cast<int*>(take(static_cast<size_t>(nmax) * 4));
     sc.fb = reinterpret_cast<int*>(take(static_cast<size_t>(nmax) * 4));
-    sc.x = reinterpret_cast<double*>(take(static_cast<size_t>(nmax) * 8));
     sc.r = reinterpret_cast<double*>(take(static_cast<size_t>(nmax) * 8));
-    sc.d = reinterpret_cast<float*>(take(static_cast<size_t>(nmax) * 4));
+    sc.perm = reinterpret_cast<int*>(take(static_cast<size_t>(nmax) * 4));
   }
   while (true) {
     if (threadIdx.x == 0) task_s = static_cast<int>(atomicAdd(queue, 1u));
@@ -358,21 +928,21 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
     if (threadIdx.x == 0) info_s = 0;
     __syncthreads();
     int s_cur = S.s;
-    factor_system(S, s_cur, sc, &info_s, sv, si);
+    factor_system(S, s_cur, sc, &info_s, sv, si, F, dyn);
     __syncthreads();
     // ||A||_inf in FP64
     double an = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      double rs = 0.0;
-      for (int j = 0; j < n; ++j) rs += fabs(S.A[i + j * S.lda]);
-      an = fmax(an, rs);
+    for (int i = threadIdx.x; i < n; i += 2 * blockDim.x) {
+      double rs[2] = {0.0, 0.0};
+      row_pass(S.A, S.lda, n, i, rs, [](double acc, double a, int) { return acc + fabs(a); });
+      an = fmax(an, fmax(rs[0], rs[1]));
     }
     an = block_max_d(an, red);
     // x0 from the FP32 factors
-    for (int i = threadIdx.x; i < n; i += blockDim.x) sc.d[i] = static_cast<float>(S.b[i]);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(S.b[sc.perm[i]]);
     __syncthreads();
-    lu_solve_f32(sc.W, n, sc.piv, sc.d);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) sc.x[i] = static_cast<double>(sc.d[i]);
+    lu_solve_f32(sc.W, n, ds);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = static_cast<double>(ds[i]);
     __syncthreads();
     double berr = INFINITY;
     int it = 0;
@@ -380,12 +950,18 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
     for (;; ++it, ++since) {
       // r = b - A x (FP64), ||r||, ||x||
       double rmax = 0.0, xmax = 0.0;
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        double acc = S.b[i];
-        for (int j = 0; j < n; ++j) acc = fma(-S.A[i + j * S.lda], sc.x[j], acc);
-        sc.r[i] = acc;
-        rmax = fmax(rmax, fabs(acc));
-        xmax = fmax(xmax, fabs(sc.x[i]));
+      for (int i = threadIdx.x; i < n; i += 2 * blockDim.x) {
+        const int i1 = i + static_cast<int>(blockDim.x);
+        double acc[2] = {S.b[i], i1 < n ? S.b[i1] : 0.0};
+        row_pass(S.A, S.lda, n, i, acc, [&](double v, double a, int j) { return fma(-a, xs[j], v); });
+        sc.r[i] = acc[0];
+        rmax = fmax(rmax, fabs(acc[0]));
+        xmax = fmax(xmax, fabs(xs[i]));
+        if (i1 < n) {
+          sc.r[i1] = acc[1];
+          rmax = fmax(rmax, fabs(acc[1]));
+          xmax = fmax(xmax, fabs(xs[i1]));
+        }
       }
       rmax = block_max_d(rmax, red);
       xmax = block_max_d(xmax, red);
@@ -395,24 +971,24 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
         // the factors are too coarse for this matrix's range: refactor with 8 slices
         s_cur = kMaxS;
         since = 0;
-        factor_system(S, s_cur, sc, &info_s, sv, si);
+        factor_system(S, s_cur, sc, &info_s, sv, si, F, dyn);
         __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) sc.d[i] = static_cast<float>(S.b[i]);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(S.b[sc.perm[i]]);
         __syncthreads();
-        lu_solve_f32(sc.W, n, sc.piv, sc.d);
-        for (int i = threadIdx.x; i < n; i += blockDim.x) sc.x[i] = static_cast<double>(sc.d[i]);
+        lu_solve_f32(sc.W, n, ds);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = static_cast<double>(ds[i]);
         __syncthreads();
         continue;
       }
       // d = (LU)^-1 r, computed on r / ||r|| to stay inside FP32 range
       const double sr = rmax > 0.0 ? rmax : 1.0;
-      for (int i = threadIdx.x; i < n; i += blockDim.x) sc.d[i] = static_cast<float>(sc.r[i] / sr);
+      for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(sc.r[sc.perm[i]] / sr);
       __syncthreads();
-      lu_solve_f32(sc.W, n, sc.piv, sc.d);
-      for (int i = threadIdx.x; i < n; i += blockDim.x) sc.x[i] += static_cast<double>(sc.d[i]) * sr;
+      lu_solve_f32(sc.W, n, ds);
+      for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] += static_cast<double>(ds[i]) * sr;
       __syncthreads();
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) S.b[i] = sc.x[i];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) S.b[i] = xs[i];
     if (threadIdx.x == 0) {
       info_arr[S.index] = info_s;
       berr_arr[S.index] = berr;
@@ -470,7 +1046,7 @@ void pick(const BatchedState* st, int n, int& nb, int& s) {
 size_t per_block_bytes(int nmax) {
   auto a = [](size_t x) { return (x + 255) / 256 * 256; };
   return a((size_t)nmax * nmax * 4) + a((size_t)nmax * 4) + 2 * a((size_t)kMaxS * nmax * 64) + 2 * a((size_t)nmax * 4) +
-         2 * a((size_t)nmax * 8) + a((size_t)nmax * 4) + 256;
+         a((size_t)nmax * 8) + a((size_t)nmax * 4) + 256;
 }
 
 }  // namespace
@@ -478,6 +1054,7 @@ size_t per_block_bytes(int nmax) {
 int batched_run(emul_handle_t h, const std::vector<BatchSys>& sys, int nmax, int32_t* info, double* berr,
                 int32_t* iters, int max_iter, double target) {
   const int count = static_cast<int>(sys.size());
+  smem_attr(reinterpret_cast<const void*>(batched_solve_kernel), kFastSmem);
   const size_t pb = per_block_bytes(nmax);
   const int grid = count < h->nsm ? count : h->nsm;
   const size_t desc_bytes = (count * sizeof(BatchSys) + 255) / 256 * 256;
@@ -501,7 +1078,7 @@ int batched_run(emul_handle_t h, const std::vector<BatchSys>& sys, int nmax, int
   rc = check_cuda(h, cudaStreamBeginCapture(st->capture, cudaStreamCaptureModeThreadLocal), "capture");
   if (rc) return rc;
   cudaMemsetAsync(queue, 0, sizeof(unsigned int), st->capture);
-  batched_solve_kernel<<<grid, kBThreads, 0, st->capture>>>(d_sys, count, queue, scratch, pb, nmax, max_iter, target,
+  batched_solve_kernel<<<grid, kBThreads, kFastSmem, st->capture>>>(d_sys, count, queue, scratch, pb, nmax, max_iter, target,
                                                             info, berr, iters);
   rc = check_cuda(h, cudaStreamEndCapture(st->capture, &graph), "capture");
   if (rc) return rc;
@@ -533,7 +1110,7 @@ int emul_dgesv_batched_ir(emul_handle_t h, int count, const int* n_arr, double* 
   std::vector<emul::BatchSys> sys(count);
   int nmax = 1;
   for (int i = 0; i < count; ++i) {
-    if (n_arr[i] < 1 || n_arr[i] > 4096 || lda_arr[i] < n_arr[i] || !A_arr[i] || !b_arr[i])
+    if (n_arr[i] < 1 || n_arr[i] > emul::kMaxN || lda_arr[i] < n_arr[i] || !A_arr[i] || !b_arr[i])
       return emul::set_error(h, EMUL_INVALID_ARG, "emul_dgesv_batched_ir: invalid system");
     int tnb, ts;
     emul::pick(st, n_arr[i], tnb, ts);
