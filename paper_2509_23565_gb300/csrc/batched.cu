@@ -353,9 +353,8 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
 //    memory (8 planes of L21 to global) as bytes; the level sums take them as FP16
 //    with FP32 accumulation, exact below 2^22 (mma.sync: 1000 multiply-adds per
 //    clock per SM in FP16, 251 in INT8, measured);
-//  - the update W - D keeps one FP64 addition per entry: the conversions around
-//    it are integer operations (FP64 runs at 1.68 lanes per clock per SM, its
-//    conversions below 1).
+//  - the update W - D is formed in FP32 two-sums where they are exact, in FP64
+//    otherwise (FP64 runs at 1.68 lanes per clock per SM, its conversions below 1).
 // In factor_general every step strides through global memory (U12 by columns
 // apart, full-row interchanges per pivot), and 152 such systems at once overflow
 // L2: 1024 systems of 64..1024 rows took 247 ms.
@@ -518,6 +517,69 @@ __device__ __forceinline__ double fast_sum(const float (&v)[S], int e) {
       d = exact_scaled(s7, e - 49);
     d += float_scaled(v[6], e - 56);
     return d + float_scaled(v[7], e - 63);
+  }
+}
+
+// The updated entry, FP32 of (FP64 of W - D), in FP64 arithmetic.
+template <int S>
+__device__ __forceinline__ float update_fp64(float w, const float (&v)[S], int e) {
+  return narrow(widen(w) - fast_sum<S>(v, e));
+}
+__device__ __noinline__ float update_fp64_3(float w, float v0, float v1, float v2, int e) {
+  const float v[3] = {v0, v1, v2};
+  return update_fp64<3>(w, v, e);
+}
+__device__ __noinline__ float update_fp64_4(float w, float v0, float v1, float v2, float v3, int e) {
+  const float v[4] = {v0, v1, v2, v3};
+  return update_fp64<4>(w, v, e);
+}
+
+// a + b = s + e exactly (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// The same entry in FP32 arithmetic for 3 or 4 slices.  D is the sum of the level
+// sums times powers of two, each an exact float, so W - D = s + sum of the
+// two-sums' errors exactly; when the errors add up exactly (E, nothing lost), one
+// last addition rounds the exact value once.  That is also what FP64 first gives:
+// with E below 2^-29 |s| both round to s, otherwise the exact value spans no more
+// bits around a rounding boundary of FP32 than a double holds.  About 40 FP32
+// operations at 118 lanes per clock per SM, where the FP64 form takes an FP64
+// addition (1.68) and 60 integer operations (64): 1.6 cycles per entry.
+// Anything else (errors that do not add up exactly, scales near FP32's ends,
+// Inf, NaN) goes the FP64 way.
+template <int S>
+__device__ __forceinline__ float fast_update(float w, const float (&v)[S], int e) {
+  if constexpr (S <= 4) {
+    float sc = __int_as_float((e + 113) << 23);           // 2^(e - 14), the weight of level 2
+    float s = w, err[S];
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      float sn;
+      two_sum(s, -(v[i] * sc), sn, err[i]);
+      s = sn;
+      sc *= 0.0078125f;
+    }
+    float E = err[0], lost = 0.f;
+#pragma unroll
+    for (int i = 1; i < S; ++i) {
+      float sn, l;
+      two_sum(E, err[i], sn, l);
+      E = sn;
+      lost = fmaxf(lost, fabsf(l));
+    }
+    const float out = __fadd_rn(s, E);
+    // (NaN: the comparison of |out| fails)
+    if (lost == 0.f && fabsf(out) < 1e38f && static_cast<unsigned>(e + 80) <= 160u) return out;
+    if constexpr (S == 3)
+      return update_fp64_3(w, v[0], v[1], v[2], e);
+    else
+      return update_fp64_4(w, v[0], v[1], v[2], v[3], e);
+  } else {
+    return update_fp64<S>(w, v, e);
   }
 }
 
@@ -780,8 +842,8 @@ __device__ __noinline__ void factor_fast(const BatchSys& sys, Scratch& sc, int* 
             float v[S];
 #pragma unroll
             for (int i = 0; i < S; ++i) v[i] = acc[i][q];
-            const double D = fast_sum<S>(v, (q >= 2 ? e1 : e0) + F.fb[j + tq * 2]);
-            w0[(q >= 2 ? 8 : 0) + static_cast<long>(j) * n] = narrow(widen(wv[q]) - D);
+            w0[(q >= 2 ? 8 : 0) + static_cast<long>(j) * n] =
+                fast_update<S>(wv[q], v, (q >= 2 ? e1 : e0) + F.fb[j + tq * 2]);
           }
         }
       }
