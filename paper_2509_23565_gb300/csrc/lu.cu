@@ -82,6 +82,23 @@ __device__ __forceinline__ bool better(uint64_t v1, int r1, uint64_t v2, int r2)
   return v1 > v2 || (v1 == v2 && r1 < r2);
 }
 
+// row[cc ld] -= l pv[cc] for cc = c0, c0 + step, ... < w, four at a time so that
+// their loads do not wait for the stores before them.
+__device__ __forceinline__ void rank1_row(double* row, int ld, double l, const double* pv, int c0, int w, int step) {
+  int cc = c0;
+  for (; cc + 3 * step < w; cc += 4 * step) {
+    double v[4], u[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v[q] = row[(cc + q * step) * ld];
+      u[q] = pv[cc + q * step];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) row[(cc + q * step) * ld] = fma(-l, u[q], v[q]);
+  }
+  for (; cc < w; cc += step) row[cc * ld] = fma(-l, pv[cc], row[cc * ld]);
+}
+
 // A column outside the leaf that follows its interchanges in global memory.  One
 // thread owns it for the whole launch, so successive interchanges of one element
 // stay in program order; the stores of an interchange are put off to the next
@@ -290,14 +307,18 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
         gv = (static_cast<uint64_t>(mh) << 32) | ml;
         gr = mr;
       }
+      // the winner's row and, in flight with it, the reciprocal
+      const uint64_t* rp = rec_all + static_cast<long>(gbk) * kRecWords + 4 + 2 * kLeaf;
+      uint64_t ra = 0, rb = 0;
+      if (ok && lane == 0) get_pair(rp, ra, rb);
       if (ok && lane < w) {
         double pvv = 0.0;
         ok = wait_pair(rec_all + static_cast<long>(gbk) * kRecWords + 4 + 2 * lane, ep, pvv, limit);
         prow[par][lane] = pvv;
       }
       if (ok && lane == 0) {
-        double r = 0.0;
-        ok = wait_pair(rec_all + static_cast<long>(gbk) * kRecWords + 4 + 2 * kLeaf, ep, r, limit);
+        double r = __longlong_as_double(static_cast<long long>((rb << 32) | (ra & 0xFFFFFFFFull)));
+        if (!(has_epoch(ra, ep) && has_epoch(rb, ep))) ok = wait_pair(rp, ep, r, limit);
         rcp_s = r;
       }
       ok = __all_sync(0xFFFFFFFFu, ok);
@@ -336,8 +357,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
       constexpr int kUpd = kLeafThreads - 64;   // warps 1-6
       for (int lr = tid - 32; lr < rcount; lr += kUpd) {
         if (r0 + lr <= c - 1) continue;
-        const double l = P[(c - 1) * ld + lr];
-        for (int cc = c + 1; cc < w; ++cc) P[cc * ld + lr] = fma(-l, pv[cc], P[cc * ld + lr]);
+        rank1_row(P + lr, ld, P[(c - 1) * ld + lr], pv, c + 1, w, 1);
       }
       }
     }
@@ -530,8 +550,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
     } else {
       if (c > 0 && p_last != c - 1) out.swap(d0 + c - 1, d0 + p_last);
       if (pend && doff < cstep && dlr < rcount && r0 + dlr > c - 1) {
-        const double l = P[(c - 1) * ld + dlr];
-        for (int cc = c + 1 + doff; cc < w; cc += cstep) P[cc * ld + dlr] = fma(-l, pv[cc], P[cc * ld + dlr]);
+        rank1_row(P + dlr, ld, P[(c - 1) * ld + dlr], pv, c + 1 + doff, w, cstep);
       }
     }
     __syncthreads();
@@ -949,15 +968,76 @@ __global__ void __launch_bounds__(512) trtri_cols_kernel(const double* A, long l
   if (i < nb) inv[i + static_cast<long>(j) * nb] = x;
 }
 
+// x <- T^-1 x for the bs x bs (bs <= 128) triangle T(i, k) = tb[i + k*ld] in
+// shared memory, by the first 128 threads of a block (thread i holds x_i; x in
+// shared memory, in and out).  `scale`: non-unit diagonal, rcp[k] = 1 / T(k, k).
+// A chain of bs steps, each a shuffle and a DFMA of 64 cycles (and a
+// multiplication with the reciprocal); a warp solves its 32 rows and publishes
+// every 8 values, and the warps behind it take those off their own rows
+// meanwhile, on their own FP64 units (one warp with four rows per lane took four
+// DFMAs, 76 cycles each, into every step).  Each entry takes its updates in the
+// order of the steps.
+template <bool LOWER, bool SCALE>
+__device__ __forceinline__ void diag_solve_t(const double* tb, int ld, const double* rcp, int bs, double* x) {
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
+  double v = i < bs ? x[i] : 0.0;
+  const double r = SCALE && i < bs ? rcp[i] : 1.0;
+  for (int s = 0; s < 16; ++s) {
+    // sub-step s: rows 8 ss .. 8 ss + 7, from the top (LOWER) or the bottom
+    const int ss = LOWER ? s : 15 - s;
+    const int prev = LOWER ? ss - 1 : ss + 1;
+    if (s > 0 && (LOWER ? warp > prev >> 2 : warp < prev >> 2)) {
+      double t[8], y[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int k = 8 * prev + (LOWER ? q : 7 - q);
+        t[q] = k < bs && i < bs ? tb[i + k * ld] : 0.0;
+        y[q] = k < bs ? x[k] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v = fma(-t[q], y[q], v);
+    }
+    if (warp == ss >> 2) {
+      double t[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int k = 8 * ss + (LOWER ? q : 7 - q);
+        t[q] = k < bs && i < bs && (LOWER ? i > k : i < k) ? tb[i + k * ld] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int kl = (8 * ss + (LOWER ? q : 7 - q)) & 31;       // the step's lane; lanes past bs hold zeros
+        if (SCALE) {
+          const double xv = v * r;
+          if (lane == kl) v = xv;
+          v = fma(-t[q], __shfl_sync(0xFFFFFFFFu, xv, kl), v);
+        } else {
+          v = fma(-t[q], __shfl_sync(0xFFFFFFFFu, v, kl), v);
+        }
+      }
+      if (lane >> 3 == (ss & 3) && i < bs) x[i] = v;
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+  }
+}
+__device__ __forceinline__ void diag_solve(const double* tb, int ld, const double* rcp, int bs, bool lower, bool scale,
+                                           double* x) {
+  if (lower)
+    scale ? diag_solve_t<true, true>(tb, ld, rcp, bs, x) : diag_solve_t<true, false>(tb, ld, rcp, bs, x);
+  else
+    scale ? diag_solve_t<false, true>(tb, ld, rcp, bs, x) : diag_solve_t<false, false>(tb, ld, rcp, bs, x);
+}
+
 // One diagonal block of a triangular solve, x <- op(T)^-1 x for the bs x bs
 // block at T[d0.., d0..] (bs <= 128; op = transpose with `trans`).  All
 // threads stage the block (leading dimension bs + 1: conflict-free either
-// way), then warp 0 solves with x in registers (lane l holds rows l, l+32,
-// l+64, l+96), each x_k divided by its diagonal entry (non-unit) and broadcast
-// by shuffle.  blockIdx.x = right-hand side.
+// way, transposed with `trans`), then the first 128 solve (diag_solve, with the
+// reciprocals of the diagonal: a division on the chain takes 560 cycles a step).
+// blockIdx.x = right-hand side.
 __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long ldt, double* X, long ldx, int d0,
                                                           int bs, int lower, int unit, int trans) {
-  extern __shared__ double tb[];   // tb[r + c*(bs+1)] = T(d0+r, d0+c) as stored
+  extern __shared__ double tb[];   // tb[r + c*(bs+1)] = op(T)(d0+r, d0+c)
+  __shared__ double x[128], rcp[128];
   const int ld = bs + 1;
   double* xc = X + static_cast<long>(blockIdx.x) * ldx + d0;
   {
@@ -971,49 +1051,40 @@ __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long 
           v[j] = c < bs ? T[(d0 + r) + static_cast<long>(d0 + c) * ldt] : 0.0;
         }
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (c0 + j * cstep < bs) tb[r + (c0 + j * cstep) * ld] = v[j];
+        for (int j = 0; j < 16; ++j) {
+          const int c = c0 + j * cstep;
+          if (c < bs) tb[trans ? c + r * ld : r + c * ld] = v[j];
+        }
       }
   }
+  if (static_cast<int>(threadIdx.x) < bs) x[threadIdx.x] = xc[threadIdx.x];
   __syncthreads();
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  auto t = [&](int r, int c) -> double { return trans ? tb[c + r * ld] : tb[r + c * ld]; };
-  double x[4];
+  if (threadIdx.x >= 128) return;
+  if (!unit && static_cast<int>(threadIdx.x) < bs) rcp[threadIdx.x] = 1.0 / tb[threadIdx.x + threadIdx.x * ld];
+  asm volatile("bar.sync 1, 128;" ::: "memory");
+  diag_solve(tb, ld, rcp, bs, lower != 0, unit == 0, x);
+  if (static_cast<int>(threadIdx.x) < bs) xc[threadIdx.x] = x[threadIdx.x];
+}
+
+// sum_c t[c ldt] x[c], c ascending, the next sixteen loads in flight during the
+// sixteen FMAs at hand (64 cycles each).
+__device__ __forceinline__ double row_dot(const double* t, long ldt, const double* x, int n) {
+  double acc = 0.0;
+  const int full = n / 16 * 16;
+  double v[16];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) x[q] = lane + 32 * q < bs ? xc[lane + 32 * q] : 0.0;
-  if (lower) {
+  for (int q = 0; q < 16; ++q) v[q] = full ? __ldg(t + q * ldt) : 0.0;
+  for (int c = 0; c < full; c += 16) {
+    double nx[16];
 #pragma unroll
-    for (int q0 = 0; q0 < 4; ++q0)
-      for (int kk = 0; kk < 32; ++kk) {
-        const int k = 32 * q0 + kk;
-        if (k >= bs) break;
-        if (!unit && lane == kk) x[q0] = x[q0] / t(k, k);
-        const double xk = __shfl_sync(0xFFFFFFFFu, x[q0], kk);
+    for (int q = 0; q < 16; ++q) nx[q] = c + 16 < full ? __ldg(t + (c + 16 + q) * ldt) : 0.0;
 #pragma unroll
-        for (int q = q0; q < 4; ++q) {
-          const int i = lane + 32 * q;
-          if (i > k && i < bs) x[q] = fma(-t(i, k), xk, x[q]);
-        }
-      }
-  } else {
+    for (int q = 0; q < 16; ++q) acc = fma(v[q], x[c + q], acc);
 #pragma unroll
-    for (int q0 = 3; q0 >= 0; --q0)
-      for (int kk = 31; kk >= 0; --kk) {
-        const int k = 32 * q0 + kk;
-        if (k >= bs) continue;
-        if (!unit && lane == kk) x[q0] = x[q0] / t(k, k);
-        const double xk = __shfl_sync(0xFFFFFFFFu, x[q0], kk);
-#pragma unroll
-        for (int q = 0; q <= q0; ++q) {
-          const int i = lane + 32 * q;
-          if (i < k) x[q] = fma(-t(i, k), xk, x[q]);
-        }
-      }
+    for (int q = 0; q < 16; ++q) v[q] = nx[q];
   }
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (lane + 32 * q < bs) xc[lane + 32 * q] = x[q];
+  for (int c = full; c < n; ++c) acc = fma(__ldg(t + c * ldt), x[c], acc);
+  return acc;
 }
 
 // x[r] -= sum_{c in [c0, c0+bs)} T(r, c) x[c] for rows r in [r0, r1); T(r, c) =
@@ -1027,9 +1098,7 @@ __global__ void gemv_update_kernel(const double* T, long ldt, double* X, long ld
   if (!trans) {
     const int r = r0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= r1) return;
-    double acc = 0.0;
-    for (int c = 0; c < bs; ++c) acc = fma(T[r + static_cast<long>(c0 + c) * ldt], xs[c], acc);
-    xc[r] -= acc;
+    xc[r] -= row_dot(T + r + static_cast<long>(c0) * ldt, ldt, xs, bs);
   } else {
     // one warp per row: contiguous reads of T[c0.., r]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1489,12 +1558,17 @@ __device__ bool solve_sync(unsigned long long* cnt, unsigned long long target, l
 // Forward (L unit lower) and back (U) substitution with the factors of
 // emul_dgetrf for one right-hand side, in one cooperative launch.  Step s
 // (the 128-row diagonal blocks of L, then those of U from the bottom) is
-// solved by block s % G in one warp (x in registers, broadcast by shuffle,
-// multiplication by the reciprocals of U's diagonal, formed while staging);
-// block (s+1) % G stages the next diagonal block meanwhile.  Then every warp of
-// every block applies the block's column of L (or U) to 32-row groups of the
-// remaining rows.  Two bounded grid barriers per step.  A row's owner changes
-// from step to step, so x is read and written through L2 only.
+// solved by four warps of block s % G (diag_solve, with the reciprocals of U's
+// diagonal, formed while staging), which has staged the diagonal block while the
+// step before was solved.  After one bounded grid barrier every block knows x_s:
+// block (s+1) % G takes it off the rows of the next diagonal block and solves
+// that at once, the others take it off all other remaining rows meanwhile, each
+// warp a group of 32 rows.  So a step costs the update of 128 rows, a diagonal
+// solve and one barrier, whatever n is (two barriers, a one-warp solve and the
+// whole update between them took 38 us a step at n = 12000).  The grid has four
+// groups of rows per block, one per FP64 unit of an SM, if that many SMs exist; a
+// smaller grid makes the barrier cheaper.  A row's owner changes from step to
+// step, so x is read and written through L2 only.
 // Stage the bs x bs diagonal block at d0 for the block solve.  LU factors
 // (chol = false): the block as stored, rcp = 1/diag for the upper (backward)
 // solve.  Cholesky factor (chol = true): the forward solve uses L itself and
@@ -1534,7 +1608,7 @@ template <bool CHOL>
 __global__ void __launch_bounds__(256) getrs1_kernel(const double* LU, long lda, int n, double* x,
                                                      unsigned long long* cnt, int* status, long long limit) {
   extern __shared__ double tb[];   // kSolveBs x (kSolveBs + 1) staging of a diagonal block
-  __shared__ double xs[kSolveBs];
+  __shared__ double xs[kSolveBs], xd[kSolveBs];
   __shared__ double rcp[kSolveBs];
   constexpr int ld = kSolveBs + 1;
   const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1548,69 +1622,37 @@ __global__ void __launch_bounds__(256) getrs1_kernel(const double* LU, long lda,
   };
   unsigned long long target = 0;
   int staged = -1;   // step whose diagonal block this block holds in tb
-  for (int st = 0; st < nsteps; ++st) {
+  auto stage = [&](int st) {
+    if (st >= nsteps || staged == st) return;
     bool lower;
     int d0, bs;
     info(st, lower, d0, bs);
-    const int sb = st % G, nxt = (st + 1) % G;
-    if (b == sb) {
-      if (staged != st) solve_stage(LU, lda, d0, bs, lower, tb, rcp, CHOL);
-      staged = -1;
-      if (tid < 32) {
-        double v[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = lane + 32 * q < bs ? __ldcg(x + d0 + lane + 32 * q) : 0.0;
-        if (lower) {
-#pragma unroll
-          for (int q0 = 0; q0 < 4; ++q0)
-            for (int kk = 0; kk < 32; ++kk) {
-              const int k = 32 * q0 + kk;
-              if (k >= bs) break;
-              if (CHOL && lane == kk) v[q0] = v[q0] * rcp[k];
-              const double xk = __shfl_sync(0xFFFFFFFFu, v[q0], kk);
-#pragma unroll
-              for (int q = q0; q < 4; ++q) {
-                const int i = lane + 32 * q;
-                if (i > k && i < bs) v[q] = fma(-tb[i + k * ld], xk, v[q]);
-              }
-            }
-        } else {
-#pragma unroll
-          for (int q0 = 3; q0 >= 0; --q0)
-            for (int kk = 31; kk >= 0; --kk) {
-              const int k = 32 * q0 + kk;
-              if (k >= bs) continue;
-              if (lane == kk) v[q0] = v[q0] * rcp[k];
-              const double xk = __shfl_sync(0xFFFFFFFFu, v[q0], kk);
-#pragma unroll
-              for (int q = 0; q <= q0; ++q) {
-                const int i = lane + 32 * q;
-                if (i < k) v[q] = fma(-tb[i + k * ld], xk, v[q]);
-              }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (lane + 32 * q < bs) __stcg(x + d0 + lane + 32 * q, v[q]);
-      }
-    } else if (b == nxt && st + 1 < nsteps) {
-      // the next step's solver stages its diagonal block while this one is solved
-      bool l2;
-      int e0, es;
-      info(st + 1, l2, e0, es);
-      solve_stage(LU, lda, e0, es, l2, tb, rcp, CHOL);
-      staged = st + 1;
+    solve_stage(LU, lda, d0, bs, lower, tb, rcp, CHOL);
+    staged = st;
+  };
+  // x_st <- T^-1 x_st, published in x
+  auto solve = [&](int st) {
+    bool lower;
+    int d0, bs;
+    info(st, lower, d0, bs);
+    stage(st);
+    if (tid < kSolveBs) {
+      if (tid < bs) xd[tid] = __ldcg(x + d0 + tid);
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      diag_solve(tb, ld, rcp, bs, lower, CHOL || !lower, xd);
+      if (tid < bs) __stcg(x + d0 + tid, xd[tid]);
     }
-    target += G;
-    if (!solve_sync(cnt, target, limit, status)) return;
-    // rows below (forward) or above (backward) the block, 32-row groups over all warps
-    const int r_lo = lower ? d0 + bs : 0, r_hi = lower ? n : d0;
-    if (CHOL && !lower && r_hi > r_lo) {
+  };
+  // x_r -= (row r of the step's block column) x_st for rows [lo, hi) outside
+  // [skip0, skip1), by the warps first, first + nw, ... (x_st in xs)
+  auto update = [&](int st, int lo, int hi, int skip0, int skip1, int first, int nw) {
+    bool lower;
+    int d0, bs;
+    info(st, lower, d0, bs);
+    if (CHOL && !lower) {
       // x_r -= sum_c L(d0 + c, r) x_c: one warp per row r, lanes along the column
-      for (int c = tid; c < bs; c += blockDim.x) xs[c] = __ldcg(x + d0 + c);
-      __syncthreads();
-      const int wpb = blockDim.x >> 5;
-      for (int r = r_lo + b * wpb + warp; r < r_hi; r += G * wpb) {
+      for (int r = lo + first; r < hi; r += nw) {
+        if (r >= skip0 && r < skip1) continue;
         const double* col = LU + d0 + static_cast<long>(r) * lda;
         double acc = 0.0;
         for (int c = lane; c < bs; c += 32) acc = fma(__ldg(col + c), xs[c], acc);
@@ -1618,25 +1660,54 @@ __global__ void __launch_bounds__(256) getrs1_kernel(const double* LU, long lda,
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
         if (lane == 0) __stcg(x + r, __ldcg(x + r) - acc);
       }
-    } else if (r_hi > r_lo) {
-      for (int c = tid; c < bs; c += blockDim.x) xs[c] = __ldcg(x + d0 + c);
-      __syncthreads();
-      const int wpb = blockDim.x >> 5;
-      for (int rg = b * wpb + warp; r_lo + rg * 32 < r_hi; rg += G * wpb) {
-        const int r = r_lo + rg * 32 + lane;
-        if (r < r_hi) {
-          double acc = 0.0;
-          for (int c = 0; c < bs; ++c) acc = fma(__ldg(LU + r + static_cast<long>(d0 + c) * lda), xs[c], acc);
+    } else {
+      for (int g = first; lo + g * 32 < hi; g += nw) {
+        const int r = lo + g * 32 + lane;
+        if (r < hi && !(r >= skip0 && r < skip1)) {
+          const double acc = row_dot(LU + r + static_cast<long>(d0) * lda, lda, xs, bs);
           __stcg(x + r, __ldcg(x + r) - acc);
         }
       }
     }
+  };
+  const int wpb = blockDim.x >> 5;
+  if (b == 0) solve(0);
+  if (b == 1 % G && G > 1) stage(1);
+  for (int st = 0; st < nsteps; ++st) {
     target += G;
     if (!solve_sync(cnt, target, limit, status)) return;
+    if (st + 1 == nsteps) break;
+    bool lower, l2;
+    int d0, bs, e0, es;
+    info(st, lower, d0, bs);
+    info(st + 1, l2, e0, es);
+    const int nxt = (st + 1) % G;
+    // rows below (forward) or above (backward) the block; the next diagonal
+    // block lies next to it (at the turn it is the same block and has no update)
+    const int lo = lower ? d0 + bs : 0, hi = lower ? n : d0;
+    const bool has_next = e0 >= lo && e0 < hi;
+    for (int c = tid; c < bs; c += blockDim.x) xs[c] = __ldcg(x + d0 + c);
+    __syncthreads();
+    if (b == nxt) {
+      if (has_next) update(st, e0, e0 + es, 0, 0, warp, wpb);
+      if (G == 1) update(st, lo, hi, e0, e0 + es, warp, wpb);
+      __syncthreads();
+      solve(st + 1);
+    } else {
+      const int me = b < nxt ? b : b - 1;   // among the G - 1 others, warps dealt block by block
+      update(st, lo, hi, has_next ? e0 : 0, has_next ? e0 + es : 0, warp * (G - 1) + me, wpb * (G - 1));
+      if (b == (st + 2) % G) stage(st + 2);
+    }
   }
 }
 
 }  // namespace
+
+// Blocks of the one-launch solve: four groups of 32 rows each.
+int solve_blocks(emul_handle_t h, int n) {
+  const int want = (n + 127) / 128;
+  return want < h->nsm ? want : h->nsm;
+}
 
 // Solve with the factors of emul_dgetrf (arguments validated by the caller).
 int getrs_body(emul_handle_t h, int n, int nrhs, const double* LU, int lda, const int32_t* ipiv, double* B,
@@ -1662,7 +1733,7 @@ int getrs_body(emul_handle_t h, int n, int nrhs, const double* LU, int lda, cons
     void* args[] = {const_cast<double**>(&LU), &ldl, &n, &B, &cnt, &status, &limit};
     h->launches++;
     return check_cuda(h,
-                      cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(getrs1_kernel<false>), dim3(h->nsm),
+                      cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(getrs1_kernel<false>), dim3(solve_blocks(h, n)),
                                                   dim3(256), args, kSolveBs * (kSolveBs + 1) * 8, h->stream),
                       "solve");
   }
@@ -2088,7 +2159,7 @@ int emul_dpotrs(emul_handle_t h, char uplo, int n, int nrhs, const double* L, in
     h->launches++;
     rc = emul::check_cuda(h,
                           cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(emul::getrs1_kernel<true>),
-                                                      dim3(h->nsm), dim3(256), args,
+                                                      dim3(emul::solve_blocks(h, n)), dim3(256), args,
                                                       emul::kSolveBs * (emul::kSolveBs + 1) * 8, h->stream),
                           "Cholesky solve");
     emul::phase_end(h, ph);
