@@ -1650,15 +1650,43 @@ __global__ void __launch_bounds__(256) getrs1_kernel(const double* LU, long lda,
     int d0, bs;
     info(st, lower, d0, bs);
     if (CHOL && !lower) {
-      // x_r -= sum_c L(d0 + c, r) x_c: one warp per row r, lanes along the column
-      for (int r = lo + first; r < hi; r += nw) {
-        if (r >= skip0 && r < skip1) continue;
-        const double* col = LU + d0 + static_cast<long>(r) * lda;
-        double acc = 0.0;
-        for (int c = lane; c < bs; c += 32) acc = fma(__ldg(col + c), xs[c], acc);
+      // x_r -= sum_c L(d0 + c, r) x_c: eight rows per warp, lanes along the
+      // columns of L.  The sums over the lanes are those of a butterfly; a lane
+      // keeps half of the rows at each of the first three steps, so eight rows
+      // take 9 additions (76 cycles each) instead of 40.
+      for (int g = first; lo + g * 8 < hi; g += nw) {
+        const int rb = lo + g * 8;
+        double v[8];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-        if (lane == 0) __stcg(x + r, __ldcg(x + r) - acc);
+        for (int q = 0; q < 8; ++q) v[q] = 0.0;
+#pragma unroll
+        for (int cq = 0; cq < kSolveBs / 32; ++cq) {
+          const int c = lane + 32 * cq;
+          double l[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            l[q] = c < bs && rb + q < hi ? __ldg(LU + d0 + c + static_cast<long>(rb + q) * lda) : 0.0;
+          if (c < bs) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = fma(l[q], xs[c], v[q]);
+          }
+        }
+        int mine = 0;                       // row of the group this lane ends up with
+#pragma unroll
+        for (int o = 16, keep = 4; keep >= 1; o >>= 1, keep >>= 1) {
+          const bool upper = lane & o;
+          if (upper) mine += keep;
+#pragma unroll
+          for (int q = 0; q < keep; ++q) {
+            const double send = upper ? v[q] : v[q + keep];
+            const double own = upper ? v[q + keep] : v[q];
+            v[q] = own + __shfl_xor_sync(0xFFFFFFFFu, send, o);
+          }
+        }
+        v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 2);
+        v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 1);
+        const int r = rb + mine;
+        if ((lane & 3) == 0 && r < hi && !(r >= skip0 && r < skip1)) __stcg(x + r, __ldcg(x + r) - v[0]);
       }
     } else {
       for (int g = first; lo + g * 32 < hi; g += nw) {
