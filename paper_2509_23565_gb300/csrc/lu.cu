@@ -82,6 +82,16 @@ __device__ __forceinline__ bool better(uint64_t v1, int r1, uint64_t v2, int r2)
   return v1 > v2 || (v1 == v2 && r1 < r2);
 }
 
+// The best of a warp's (value, row) pairs (better() above), in every lane, by
+// three warp reductions on 32-bit words.
+__device__ __forceinline__ void warp_best(uint64_t& v, int& r) {
+  const uint32_t hi = static_cast<uint32_t>(v >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+  const uint32_t lo = hi == mh ? static_cast<uint32_t>(v) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
+  const bool top = hi == mh && static_cast<uint32_t>(v) == ml;
+  r = __reduce_min_sync(0xFFFFFFFFu, top ? r : 0x7FFFFFFF);
+  v = (static_cast<uint64_t>(mh) << 32) | ml;
+}
+
 // row[cc ld] -= l pv[cc] for cc = c0, c0 + step, ... < w, four at a time so that
 // their loads do not wait for the stores before them.
 __device__ __forceinline__ void rank1_row(double* row, int ld, double l, const double* pv, int c0, int w, int step) {
@@ -208,25 +218,15 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
         br = pr;
       }
     }
-    {
-      const uint32_t hi = static_cast<uint32_t>(bv >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
-      const uint32_t lo = hi == mh ? static_cast<uint32_t>(bv) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
-      const bool top = hi == mh && static_cast<uint32_t>(bv) == ml;
-      const int mr = __reduce_min_sync(0xFFFFFFFFu, top ? br : 0x7FFFFFFF);
-      if (lane == 0) {
-        red_v[warp] = (static_cast<uint64_t>(mh) << 32) | ml;
-        red_r[warp] = mr;
-      }
+    warp_best(bv, br);
+    if (lane == 0) {
+      red_v[warp] = bv;
+      red_r[warp] = br;
     }
     __syncthreads();
-    bv = red_v[0];
-    br = red_r[0];
-#pragma unroll
-    for (int i = 1; i < kLeafThreads / 32; ++i)
-      if (better(red_v[i], red_r[i], bv, br)) {
-        bv = red_v[i];
-        br = red_r[i];
-      }
+    bv = red_v[lane & (kLeafThreads / 32 - 1)];
+    br = red_r[lane & (kLeafThreads / 32 - 1)];
+    warp_best(bv, br);
     if (tid == kRowTid) {
       put_word(my + 0, static_cast<uint32_t>(bv), ep);
       put_word(my + 1, static_cast<uint32_t>(bv >> 32), ep);
@@ -298,14 +298,11 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
         }
       }
       {
-        const uint32_t hi = static_cast<uint32_t>(gv >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
-        const uint32_t lo = hi == mh ? static_cast<uint32_t>(gv) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
-        const bool top = hi == mh && static_cast<uint32_t>(gv) == ml;
-        const int mr = __reduce_min_sync(0xFFFFFFFFu, top ? gr : 0x7FFFFFFF);
-        const int src = __ffs(__ballot_sync(0xFFFFFFFFu, top && gr == mr)) - 1;
+        const uint64_t own_v = gv;
+        const int own_r = gr;
+        warp_best(gv, gr);
+        const int src = __ffs(__ballot_sync(0xFFFFFFFFu, own_v == gv && own_r == gr)) - 1;
         gbk = __shfl_sync(0xFFFFFFFFu, gbk, src);
-        gv = (static_cast<uint64_t>(mh) << 32) | ml;
-        gr = mr;
       }
       // the winner's row and, in flight with it, the reciprocal
       const uint64_t* rp = rec_all + static_cast<long>(gbk) * kRecWords + 4 + 2 * kLeaf;
@@ -369,23 +366,26 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
     const double piv = prow[par][c];
     pend = absbits(piv) != 0;           // (an FP64 comparison takes 64 cycles)
     if (pend) {
-      // (4) interchange rows c and p (both current through pivot c-1)
+      // (4) interchange rows c and p (both current through pivot c-1); columns
+      // c and c+1 of row p are left to the thread that has row p in (5)
       if (p != c) {
         if (c >= r0 && c < r0 + rcount)
           for (int cc = tid; cc < w; cc += blockDim.x) P[cc * ld + (c - r0)] = prow[par][cc];
         if (p >= r0 && p < r0 + rcount)
-          for (int cc = tid; cc < w; cc += blockDim.x) P[cc * ld + (p - r0)] = crow[cc];
+          for (int cc = tid; cc < w; cc += blockDim.x)
+            if (cc != c && cc != c + 1) P[cc * ld + (p - r0)] = crow[cc];
       }
-      __syncthreads();
       // (5) multipliers of column c, update of column c+1
       const bool use_rcp = absbits(piv) >= 0x0010000000000000ull;
       const double rcp = rcp_s;
       const double u1 = c + 1 < w ? prow[par][c + 1] : 0.0;
       for (int lr = tid; lr < rcount; lr += blockDim.x) {
         if (r0 + lr <= c) continue;
-        const double l = use_rcp ? P[c * ld + lr] * rcp : P[c * ld + lr] / piv;
+        const bool swapped = r0 + lr == p;             // (p > c here)
+        const double a0 = swapped ? crow[c] : P[c * ld + lr];
+        const double l = use_rcp ? a0 * rcp : a0 / piv;
         P[c * ld + lr] = l;
-        if (c + 1 < w) P[(c + 1) * ld + lr] = fma(-l, u1, P[(c + 1) * ld + lr]);
+        if (c + 1 < w) P[(c + 1) * ld + lr] = fma(-l, u1, swapped ? crow[c + 1] : P[(c + 1) * ld + lr]);
       }
     }
     __syncthreads();
@@ -470,25 +470,18 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
     if (warp < kClusterR / 32) {
       const int pr = r0 + tid;
       const bool in = tid < rcount && pr >= c;
-      const uint64_t v = in ? absbits(P[c * ld + tid]) : 0ull;
-      const uint32_t hi = static_cast<uint32_t>(v >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
-      const uint32_t lo = hi == mh ? static_cast<uint32_t>(v) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
-      const bool top = in && hi == mh && static_cast<uint32_t>(v) == ml;
-      const int mr = __reduce_min_sync(0xFFFFFFFFu, top ? pr : 0x7FFFFFFF);
+      uint64_t v = in ? absbits(P[c * ld + tid]) : 0ull;
+      int r = in ? pr : 0x7FFFFFFF;
+      warp_best(v, r);
       if (lane == 0) {
-        red_v[warp] = (static_cast<uint64_t>(mh) << 32) | ml;
-        red_r[warp] = mr;
+        red_v[warp] = v;
+        red_r[warp] = r;
       }
     }
     __syncthreads();
-    uint64_t bv = red_v[0];
-    int br = red_r[0];
-#pragma unroll
-    for (int i = 1; i < kClusterR / 32; ++i)
-      if (better(red_v[i], red_r[i], bv, br)) {
-        bv = red_v[i];
-        br = red_r[i];
-      }
+    uint64_t bv = red_v[lane & (kClusterR / 32 - 1)];
+    int br = red_r[lane & (kClusterR / 32 - 1)];
+    warp_best(bv, br);
     // (2) candidate, its row and row c (current through pivot c-1) to every CTA
     // from warps 0-3, one per sub-partition; the candidate's reciprocal, whose
     // division takes as long as the exchange, follows from warp 4
@@ -526,13 +519,12 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
     // (3) winner, its row and the reciprocal (warp 0); deferred update of pivot c-1
     if (warp == 0) {
       const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(&full[par], (c >> 1) & 1, limit));
-      const uint64_t v = lane < G ? rec[par][lane][0] : 0ull;
-      const int r = lane < G ? static_cast<int>(rec[par][lane][1]) : 0x7FFFFFFF;
-      const uint32_t hi = static_cast<uint32_t>(v >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
-      const uint32_t lo = hi == mh ? static_cast<uint32_t>(v) : 0u, ml = __reduce_max_sync(0xFFFFFFFFu, lo);
-      const bool top = lane < G && hi == mh && static_cast<uint32_t>(v) == ml;
-      const int gr = __reduce_min_sync(0xFFFFFFFFu, top ? r : 0x7FFFFFFF);
-      const int src = __ffs(__ballot_sync(0xFFFFFFFFu, top && r == gr)) - 1;
+      const uint64_t own_v = lane < G ? rec[par][lane][0] : 0ull;
+      const int own_r = lane < G ? static_cast<int>(rec[par][lane][1]) : 0x7FFFFFFF;
+      uint64_t gv = own_v;
+      int gr = own_r;
+      warp_best(gv, gr);
+      const int src = __ffs(__ballot_sync(0xFFFFFFFFu, own_v == gv && own_r == gr)) - 1;
       if (lane < w) {
         const double x = crow[par][src][lane];
         prow[par][lane] = x;
@@ -544,7 +536,7 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
         if (!ok) atomicExch(status, kStatusTimeout);
         if (ok && b == 0) {
           ipiv[d0 + c] = d0 + gr + 1;
-          if (mh == 0 && ml == 0) atomicCAS(info, 0, d0 + c + 1);
+          if (gv == 0) atomicCAS(info, 0, d0 + c + 1);
         }
       }
     } else {
@@ -560,17 +552,20 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
     const double piv = prow[par][c];
     pend = absbits(piv) != 0;           // (an FP64 comparison takes 64 cycles)
     if (pend) {
-      // (4) interchange rows c and p (both current through pivot c-1)
+      // (4) interchange rows c and p (both current through pivot c-1); columns
+      // c and c+1 of row p are left to the thread that has row p in (5)
       if (p != c) {
         if (tid < w && c >= r0 && c < r0 + rcount) P[tid * ld + (c - r0)] = prow[par][tid];
-        if (tid < w && p >= r0 && p < r0 + rcount) P[tid * ld + (p - r0)] = drow[par][tid];
+        if (tid < w && tid != c && tid != c + 1 && p >= r0 && p < r0 + rcount) P[tid * ld + (p - r0)] = drow[par][tid];
       }
-      __syncthreads();
       // (5) multipliers of column c, update of column c+1
       if (tid < rcount && r0 + tid > c) {
-        const double l = absbits(piv) >= 0x0010000000000000ull ? P[c * ld + tid] * rcp_s : P[c * ld + tid] / piv;
+        const bool swapped = r0 + tid == p;            // (p > c here)
+        const double a0 = swapped ? drow[par][c] : P[c * ld + tid];
+        const double l = absbits(piv) >= 0x0010000000000000ull ? a0 * rcp_s : a0 / piv;
         P[c * ld + tid] = l;
-        if (c + 1 < w) P[(c + 1) * ld + tid] = fma(-l, prow[par][c + 1], P[(c + 1) * ld + tid]);
+        if (c + 1 < w)
+          P[(c + 1) * ld + tid] = fma(-l, prow[par][c + 1], swapped ? drow[par][c + 1] : P[(c + 1) * ld + tid]);
       }
     }
   }
