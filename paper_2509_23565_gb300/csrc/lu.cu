@@ -581,79 +581,116 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
 
 // Row interchanges ipiv[k1..k2) (1-based global rows, ipiv[k]-1 >= k) resolved
 // into a gather map: after the interchanges, row dst[i] holds the original row
-// src[i], for the *count affected rows (at most 2 (k2-k1)).  Applying
-// transposition k to every row in turn, the content ending at row r is
-// sigma(r) = t_k1(t_k1+1(... t_k2-1(r))): the transpositions taken in reverse
-// order on r alone, so every row is resolved by its own thread (thread i:
-// row k1+i, and row ipiv[k1+i]-1 when it lies beyond the block and no earlier
-// interchange names it).  The map's order is immaterial to its users.
+// src[i], for the *count affected rows (at most 2 (k2-k1)).  The rows are
+// numbered 0..nb-1 for the block's own and kPermMax + i for the row outside it
+// that interchange i names first; the interchanges are taken in eight groups, each
+// applied in order by one thread to an identity map of its own, and a row's source
+// is found by following it through the groups' maps.  (One row after another
+// through all 256 interchanges took 15 us, on the critical path of every panel.)
+// The map's order is immaterial to its users.
 constexpr int kPermMax = 256;          // interchanges per gather map (longer ranges: several maps)
-__global__ void __launch_bounds__(kPermMax) laswp_perm_kernel(const int32_t* ipiv, int k1, int k2,
-                                                             int* map /* [2][2*kPermMax] + count */) {
-  __shared__ int piv_s[kPermMax];
-  __shared__ int cnt_s;
-  const int nb = k2 - k1;
+constexpr int kPermGroups = 8;
+struct PermShared {
+  int piv[kPermMax];                               // global rows, 0-based
+  unsigned short id[kPermMax];                     // number of the row interchange i names
+  unsigned short map[kPermGroups][2 * kPermMax];
+  int dst[2 * kPermMax], src[2 * kPermMax], cnt;
+};
+// Called by all kPermMax threads of a block, S.piv[0..nb) set and visible.
+__device__ void perm_map(PermShared& S, int k1, int nb) {
   const int i = threadIdx.x;
-  if (i < nb) piv_s[i] = ipiv[k1 + i] - 1;
-  if (i == 0) cnt_s = 0;
-  __syncthreads();
-  int* dst = map;
-  int* src = map + 2 * kPermMax;
-  auto sigma = [&](int r) {
-    for (int k = nb - 1; k >= 0; --k) {
-      const int p = piv_s[k], kk = k1 + k;
-      r = r == kk ? p : (r == p ? kk : r);
+  if (i == 0) S.cnt = 0;
+  for (int e = i; e < kPermGroups * 2 * kPermMax; e += kPermMax) S.map[0][e] = static_cast<unsigned short>(e & (2 * kPermMax - 1));
+  int first = i;
+  if (i < nb) {
+    const int p = S.piv[i];
+    if (p >= k1 && p < k1 + nb) {
+      S.id[i] = static_cast<unsigned short>(p - k1);
+    } else {
+      for (int j = 0; j < i; ++j)
+        if (S.piv[j] == p) {
+          first = j;
+          break;
+        }
+      S.id[i] = static_cast<unsigned short>(kPermMax + first);
     }
-    return r;
+  }
+  __syncthreads();
+  const int per = (nb + kPermGroups - 1) / kPermGroups;
+  if (i < kPermGroups) {
+    unsigned short* m = S.map[i];
+    for (int k = i * per; k < (i + 1) * per && k < nb; ++k) {
+      const int p = S.id[k];
+      const unsigned short v = m[k];
+      m[k] = m[p];
+      m[p] = v;
+    }
+  }
+  __syncthreads();
+  // row number e at the end holds map_0(map_1(... map_7(e)))
+  auto source = [&](int e) {
+#pragma unroll
+    for (int g = kPermGroups - 1; g >= 0; --g) e = S.map[g][e];
+    return e;
+  };
+  auto row_of = [&](int e) { return e < kPermMax ? k1 + e : S.piv[e - kPermMax]; };
+  auto put = [&](int e) {
+    const int s = source(e);
+    if (s != e) {
+      const int pos = atomicAdd(&S.cnt, 1);
+      S.dst[pos] = row_of(e);
+      S.src[pos] = row_of(s);
+    }
   };
   if (i < nb) {
-    const int r = k1 + i;
-    const int sr = sigma(r);
-    if (sr != r) {
-      const int pos = atomicAdd(&cnt_s, 1);
-      dst[pos] = r;
-      src[pos] = sr;
-    }
-    const int p = piv_s[i];
-    if (p >= k2) {
-      bool first = true;
-      for (int j = 0; j < i && first; ++j) first = piv_s[j] != p;
-      if (first) {
-        const int sp = sigma(p);
-        if (sp != p) {
-          const int pos = atomicAdd(&cnt_s, 1);
-          dst[pos] = p;
-          src[pos] = sp;
-        }
-      }
-    }
+    put(i);
+    if (S.id[i] == kPermMax + i) put(kPermMax + i);
   }
   __syncthreads();
-  if (i == 0) map[4 * kPermMax] = cnt_s;
 }
 
-// Apply the gather map to columns [c0, c1): each block owns 8 columns, reads
-// every source row into shared memory, then writes the destinations.
+__global__ void __launch_bounds__(kPermMax) laswp_perm_kernel(const int32_t* ipiv, int k1, int k2,
+                                                             int* map /* [2][2*kPermMax] + count */) {
+  __shared__ PermShared S;
+  const int nb = k2 - k1;
+  const int i = threadIdx.x;
+  if (i < nb) S.piv[i] = ipiv[k1 + i] - 1;
+  __syncthreads();
+  perm_map(S, k1, nb);
+  for (int e = i; e < S.cnt; e += kPermMax) {
+    map[e] = S.dst[e];
+    map[2 * kPermMax + e] = S.src[e];
+  }
+  if (i == 0) map[4 * kPermMax] = S.cnt;
+}
+
+// Apply the gather map to columns [c0, c1): each block takes 8 columns, a thread
+// two rows of the map in all of them: sixteen scattered loads in flight, the
+// stores after the whole block has read.
 constexpr int kSwpCols = 8;
 __global__ void __launch_bounds__(256) laswp_apply_kernel(double* A, long lda, int c0, int c1, const int* map) {
-  __shared__ double buf[kSwpCols][2 * kPermMax];
-  __shared__ int dst_s[2 * kPermMax], src_s[2 * kPermMax];
   const int cnt = map[4 * kPermMax];
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-    dst_s[i] = map[i];
-    src_s[i] = map[2 * kPermMax + i];
-  }
-  __syncthreads();
   const int cb = c0 + blockIdx.x * kSwpCols;
   const int ncol = c1 - cb < kSwpCols ? c1 - cb : kSwpCols;
-  for (int j = 0; j < ncol; ++j) {
-    const double* col = A + static_cast<long>(cb + j) * lda;
-    for (int i = threadIdx.x; i < cnt; i += blockDim.x) buf[j][i] = col[src_s[i]];
+  double* base = A + static_cast<long>(cb) * lda;
+  double v[2][kSwpCols];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = threadIdx.x + h * 256;
+    const int s = i < cnt ? map[2 * kPermMax + i] : 0;
+#pragma unroll
+    for (int j = 0; j < kSwpCols; ++j) v[h][j] = i < cnt && j < ncol ? base[s + static_cast<long>(j) * lda] : 0.0;
   }
   __syncthreads();
-  for (int j = 0; j < ncol; ++j) {
-    double* col = A + static_cast<long>(cb + j) * lda;
-    for (int i = threadIdx.x; i < cnt; i += blockDim.x) col[dst_s[i]] = buf[j][i];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = threadIdx.x + h * 256;
+    if (i < cnt) {
+      const int d = map[i];
+#pragma unroll
+      for (int j = 0; j < kSwpCols; ++j)
+        if (j < ncol) base[d + static_cast<long>(j) * lda] = v[h][j];
+    }
   }
 }
 
@@ -1215,21 +1252,43 @@ __global__ void probe_z_kernel(int n, const double* U, long ldu, double* z, doub
   }
 }
 
-// t[i] = sum_q L(r_i, q) z[q], ta[i] = sum_q |L(r_i, q)| za[q]; then the check (one thread per row)
-__global__ void probe_check_kernel(int m, int n, int k, const double* L, long ldl, int R, const double* z,
-                                   const double* za, const double* y0, const double* a0, const double* y1,
-                                   const double* a1, int* flag) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= R) return;
-  const int r = static_cast<int>(static_cast<long>(i) * m / R);
-  double t = 0.0, ta = 0.0;
-  for (int q = 0; q < k; ++q) {
-    const double l = L[r + static_cast<long>(q) * ldl];
-    t = fma(l, z[q], t);
-    ta = fma(fabs(l), za[q], ta);
+// t[i] = sum_q L(r_i, q) z[q], ta[i] = sum_q |L(r_i, q)| za[q]; then the check.
+// One lane per row; even warps form t, odd warps ta, on FP64 units of their own,
+// the next sixteen entries of L in flight.
+__global__ void __launch_bounds__(4 * 32) probe_check_kernel(int m, int n, int k, const double* L, long ldl, int R,
+                                                             const double* z, const double* za, const double* y0,
+                                                             const double* a0, const double* y1, const double* a1,
+                                                             int* flag) {
+  __shared__ double ta_s[kProbeRows];
+  __shared__ double zs[2][128];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = (warp >> 1) * 32 + lane;
+  const bool mag = warp & 1;
+  const int r = i < R ? static_cast<int>(static_cast<long>(i) * m / R) : 0;
+  double t = 0.0;
+  for (int q0 = 0; q0 < k; q0 += 128) {
+    const int kn = k - q0 < 128 ? k - q0 : 128;
+    __syncthreads();
+    if (static_cast<int>(threadIdx.x) < kn) {
+      zs[0][threadIdx.x] = z[q0 + threadIdx.x];
+      zs[1][threadIdx.x] = za[q0 + threadIdx.x];
+    }
+    __syncthreads();
+    const double* row = L + r + static_cast<long>(q0) * ldl;
+    for (int q = 0; q < kn; q += 16) {
+      double l[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) l[j] = q + j < kn ? __ldg(row + static_cast<long>(q + j) * ldl) : 0.0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (q + j < kn) t = fma(mag ? fabs(l[j]) : l[j], zs[mag ? 1 : 0][q + j], t);
+    }
   }
+  if (mag && i < R) ta_s[i] = t;
+  __syncthreads();
+  if (mag || i >= R) return;
   const double u = 1.1102230246251565e-16;
-  const double tol = 6.0 * k * u * ta + 3.0 * n * u * (a0[i] + a1[i]);
+  const double tol = 6.0 * k * u * ta_s[i] + 3.0 * n * u * (a0[i] + a1[i]);
   const double diff = fabs((y0[i] - y1[i]) - t);
   if (!(diff <= tol)) atomicExch(flag, 1);
 }
@@ -1495,34 +1554,35 @@ namespace emul {
 namespace {
 
 constexpr int kSolveBs = 128;      // diagonal block of the persistent solve
-constexpr int kPermSmemMax = 54 * 1024;   // rows whose permutation fits in shared memory (4 B each, + 4 KB)
+constexpr int kPermSmemMax = 52 * 1024;   // rows whose permutation fits in shared memory (4 B each, + 14 KB)
 
 // x <- P x for the interchanges ipiv[0..n) (1-based, applied in order): the
-// composite permutation is built by one thread in shared memory (ipiv staged in
-// chunks), then x is gathered through tmp.  One block.
-__global__ void __launch_bounds__(1024) permute_rhs_kernel(const int32_t* ipiv, int n, double* x, double* tmp) {
+// composite permutation is built in shared memory, 256 interchanges resolved at a
+// time (perm_map), then x is gathered through tmp.  One block.  An entry outside
+// [0, n) leaves its row where it is.
+__global__ void __launch_bounds__(kPermMax) permute_rhs_kernel(const int32_t* ipiv, int n, double* x, double* tmp) {
   extern __shared__ int perm[];
-  __shared__ int chunk[1024];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) perm[i] = i;
-  __syncthreads();
-  for (int k0 = 0; k0 < n; k0 += 1024) {
-    const int m = n - k0 < 1024 ? n - k0 : 1024;
-    if (static_cast<int>(threadIdx.x) < m) chunk[threadIdx.x] = ipiv[k0 + threadIdx.x] - 1;
+  __shared__ PermShared S;
+  const int i = threadIdx.x;
+  for (int e = i; e < n; e += kPermMax) perm[e] = e;
+  for (int k0 = 0; k0 < n; k0 += kPermMax) {
+    const int nb = n - k0 < kPermMax ? n - k0 : kPermMax;
+    if (i < nb) {
+      const int p = ipiv[k0 + i] - 1;
+      S.piv[i] = p >= 0 && p < n ? p : k0 + i;
+    }
     __syncthreads();
-    if (threadIdx.x == 0)
-      for (int j = 0; j < m; ++j) {
-        const int k = k0 + j, p = chunk[j];
-        if (p != k && p >= 0 && p < n) {
-          const int t = perm[k];
-          perm[k] = perm[p];
-          perm[p] = t;
-        }
-      }
+    perm_map(S, k0, nb);
+    int v[2];
+    for (int h = 0; h < 2; ++h) v[h] = i + h * kPermMax < S.cnt ? perm[S.src[i + h * kPermMax]] : 0;
+    __syncthreads();
+    for (int h = 0; h < 2; ++h)
+      if (i + h * kPermMax < S.cnt) perm[S.dst[i + h * kPermMax]] = v[h];
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) tmp[i] = x[perm[i]];
+  for (int e = i; e < n; e += kPermMax) tmp[e] = x[perm[e]];
   __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = tmp[i];
+  for (int e = i; e < n; e += kPermMax) x[e] = tmp[e];
 }
 
 // Bounded grid barrier on a monotonic arrival counter (zeroed before the
@@ -1744,7 +1804,7 @@ int getrs_body(emul_handle_t h, int n, int nrhs, const double* LU, int lda, cons
     double* tmp = reinterpret_cast<double*>(ws + kAl);
     smem_attr(reinterpret_cast<const void*>(permute_rhs_kernel), kPermSmemMax * 4);
     smem_attr(reinterpret_cast<const void*>(getrs1_kernel<false>), kSolveBs * (kSolveBs + 1) * 8);
-    permute_rhs_kernel<<<1, 1024, static_cast<size_t>(n) * 4, h->stream>>>(ipiv, n, B, tmp);
+    permute_rhs_kernel<<<1, kPermMax, static_cast<size_t>(n) * 4, h->stream>>>(ipiv, n, B, tmp);
     h->launches++;
     rc = check_cuda(h, cudaGetLastError(), "rhs permutation");
     if (rc) return rc;
@@ -2033,7 +2093,7 @@ int emul_dgetrf(emul_handle_t h, int n, double* A, int lda, int32_t* ipiv, int n
         double* z = y0 + 4 * emul::kProbeRows;
         double* za = z + nb;
         emul::probe_rows_kernel<<<R, 256, 0, h->stream>>>(m2, m2, A22, lda, R, y1, a1);
-        emul::probe_check_kernel<<<(R + 63) / 64, 64, 0, h->stream>>>(m2, m2, jb, L21, lda, R, z, za, y0, a0, y1,
+        emul::probe_check_kernel<<<1, 4 * 32, 0, h->stream>>>(m2, m2, jb, L21, lda, R, z, za, y0, a0, y1,
                                                                        a1, B.flag);
         h->launches += 2;
         int fl = 0;

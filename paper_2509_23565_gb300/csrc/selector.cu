@@ -43,66 +43,70 @@ __device__ __forceinline__ int entry_exponent(uint64_t u) {   // smallest E with
 }
 
 // Histogram of the rows of a rows x k operand: element (r, c) at X[r*rs + c*cs].
-// One thread per row (rows contiguous) or one warp per row (k contiguous).
-__global__ void hist_kernel(int rows, int k, const double* __restrict__ X, long rs, long cs,
-                            unsigned int* __restrict__ hist) {
-  __shared__ unsigned int h[kBins];
-  for (int i = threadIdx.x; i < kBins; i += blockDim.x) h[i] = 0;
-  __syncthreads();
+// Rows contiguous: a block takes 32 rows, a lane per row, its 8 warps every 8th
+// k; k contiguous: a warp per row, lanes along k.  A lane counts in a column of
+// its own (counters[warp][bin][lane]: no conflicts, no atomics), sixteen loads in
+// flight; most entries fall into a few bins, where shared atomics of a warp
+// queued up, and one thread per row left most SMs idle (107 us for 5744 x 256).
+constexpr int kHistRows = 32, kHistWarps = 8;
+__global__ void __launch_bounds__(32 * kHistWarps) hist_kernel(int rows, int k, const double* __restrict__ X, long rs,
+                                                              long cs, unsigned int* __restrict__ hist) {
+  __shared__ unsigned int h[kHistWarps][kBins][32];
+  __shared__ unsigned long long mx_s[kHistWarps][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint64_t* Xb = reinterpret_cast<const uint64_t*>(X);
-  if (rs == 1) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < rows) {
-      uint64_t mx = 0;
-      for (int c = 0; c < k; ++c) {
-        const uint64_t u = __ldg(Xb + r + static_cast<long>(c) * cs) & 0x7FFFFFFFFFFFFFFFull;
-        mx = u > mx ? u : mx;
-      }
-      if (mx < 0x7FF0000000000000ull) {
-        const int e = mx ? entry_exponent(mx) : 0;
-        for (int c = 0; c < k; ++c) {
-          const uint64_t u = __ldg(Xb + r + static_cast<long>(c) * cs) & 0x7FFFFFFFFFFFFFFFull;
-          int bin = kBins - 1;
-          if (u) {
-            const int off = e - entry_exponent(u);
-            bin = off < kBins - 1 ? off : kBins - 1;
-          }
-          atomicAdd(&h[bin], 1u);
-        }
-      }
-    }
-  } else {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * (blockDim.x / 32) + warp;
-    if (r < rows) {
-      const uint64_t* xr = Xb + static_cast<long>(r) * rs;
-      uint64_t mx = 0;
-      for (int c = lane; c < k; c += 32) {
-        const uint64_t u = __ldg(xr + c) & 0x7FFFFFFFFFFFFFFFull;
-        mx = u > mx ? u : mx;
-      }
+  const bool by_rows = rs == 1;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const uint64_t v = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
-        mx = v > mx ? v : mx;
-      }
-      if (mx < 0x7FF0000000000000ull) {
-        const int e = mx ? entry_exponent(mx) : 0;
-        for (int c = lane; c < k; c += 32) {
-          const uint64_t u = __ldg(xr + c) & 0x7FFFFFFFFFFFFFFFull;
-          int bin = kBins - 1;
-          if (u) {
-            const int off = e - entry_exponent(u);
-            bin = off < kBins - 1 ? off : kBins - 1;
-          }
-          atomicAdd(&h[bin], 1u);
-        }
-      }
+  for (int b = 0; b < kBins; ++b) h[warp][b][lane] = 0;
+  const int r = by_rows ? blockIdx.x * kHistRows + lane : blockIdx.x * kHistWarps + warp;
+  const int c0 = by_rows ? warp : lane, step = by_rows ? kHistWarps : 32;
+  const uint64_t* row = Xb + static_cast<long>(r) * rs;
+  auto pass = [&](auto f) {
+    for (int c = c0; c < k; c += 16 * step) {
+      uint64_t u[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        u[q] = r < rows && c + q * step < k ? __ldg(row + static_cast<long>(c + q * step) * cs) & 0x7FFFFFFFFFFFFFFFull : 0;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) f(u[q], r < rows && c + q * step < k);
+    }
+  };
+  uint64_t mx = 0;
+  pass([&](uint64_t u, bool) { mx = u > mx ? u : mx; });
+  if (by_rows) {
+    mx_s[warp][lane] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kHistWarps; ++w) mx = mx_s[w][lane] > mx ? mx_s[w][lane] : mx;
+  } else {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const uint64_t v = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
+      mx = v > mx ? v : mx;
     }
   }
+  if (mx < 0x7FF0000000000000ull) {
+    const int e = mx ? entry_exponent(mx) : 0;
+    pass([&](uint64_t u, bool in) {
+      int bin = kBins - 1;
+      if (u) {
+        const int off = e - entry_exponent(u);
+        bin = off < kBins - 1 ? off : kBins - 1;
+      }
+      if (in) ++h[warp][bin][lane];
+    });
+  }
   __syncthreads();
-  for (int i = threadIdx.x; i < kBins; i += blockDim.x)
-    if (h[i]) atomicAdd(&hist[i], h[i]);
+  for (int b = warp; b < kBins; b += kHistWarps) {
+    unsigned int s = 0;
+#pragma unroll
+    for (int w = 0; w < kHistWarps; ++w) s += h[w][b][lane];
+    s = __reduce_add_sync(0xFFFFFFFFu, s);
+    if (lane == 0 && s) atomicAdd(&hist[b], s);
+  }
+}
+inline int hist_blocks(int rows, long rs) {
+  return rs == 1 ? (rows + kHistRows - 1) / kHistRows : (rows + kHistWarps - 1) / kHistWarps;
 }
 
 __global__ void hist_finish_kernel(const unsigned int* hist, double na, double nb, float* feat) {
@@ -165,47 +169,65 @@ __global__ void err_finish_kernel(const unsigned long long* bits, double* err) {
 // ------------------------------------------------------------------ MLP
 __device__ __forceinline__ float wbf(const __nv_bfloat16* W, int idx) { return __bfloat162float(W[idx]); }
 
-// Forward pass for kTile samples per block (128 threads).  Z* receive the
-// pre-activations (for the backward pass); H* are kept in shared memory.
+// Output t of a layer for NS samples: bias + sum_i h[s][i] W[t][i], i ascending,
+// the row of W in 16-byte loads, all in flight (one weight at a time, a row per
+// thread and once per sample, a forward pass of one sample took 366 us).
+template <int IN, int NS>
+__device__ __forceinline__ void layer_row(const __nv_bfloat16* W, float bias, const float (*h)[IN], float (&acc)[NS]) {
+  const uint4* w4 = reinterpret_cast<const uint4*>(W);
+  uint4 w[IN / 8];
+#pragma unroll
+  for (int i = 0; i < IN / 8; ++i) w[i] = __ldg(w4 + i);
+#pragma unroll
+  for (int s = 0; s < NS; ++s) acc[s] = bias;
+#pragma unroll
+  for (int i = 0; i < IN / 8; ++i) {
+    const uint32_t p[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float wv = __uint_as_float(q & 1 ? p[q >> 1] & 0xFFFF0000u : p[q >> 1] << 16);
+#pragma unroll
+      for (int s = 0; s < NS; ++s) acc[s] = fmaf(h[s][8 * i + q], wv, acc[s]);
+    }
+  }
+}
+
+// Forward pass for kTile samples per block (128 threads; NS of them computed:
+// all, or the one of a batch of one).  Z* receive the pre-activations (for the
+// backward pass); H* are kept in shared memory.
+template <int NS>
 __device__ void mlp_forward_tile(int b0, int batch, const float* X, const __nv_bfloat16* Wb, const float* P,
                                  float (*h0)[kF], float (*ha)[kH], float (*hb)[kH], float* Z0, float* Z1, float* Z2,
                                  float* Z3) {
+  static_assert(kOffW1 % 8 == 0 && kOffW2 % 8 == 0 && kOffW3 % 8 == 0, "16-byte rows of the BF16 weights");
   const int t = threadIdx.x;
-  for (int idx = t; idx < kTile * kF; idx += blockDim.x) {
+  for (int idx = t; idx < NS * kF; idx += blockDim.x) {
     const int sI = idx / kF, i = idx % kF;
     h0[sI][i] = (b0 + sI < batch) ? X[static_cast<long>(b0 + sI) * kF + i] : 0.f;
   }
   __syncthreads();
-  // layer 0: 64 -> 128
-  for (int sI = 0; sI < kTile; ++sI) {
-    float acc = P[kOffB0 + t];
-    for (int i = 0; i < kF; ++i) acc = fmaf(h0[sI][i], wbf(Wb, kOffW0 + t * kF + i), acc);
-    if (Z0 && b0 + sI < batch) Z0[static_cast<long>(b0 + sI) * kH + t] = acc;
-    ha[sI][t] = fmaxf(acc, 0.f);
-  }
-  __syncthreads();
-  // layer 1
-  for (int sI = 0; sI < kTile; ++sI) {
-    float acc = P[kOffB1 + t];
-    for (int i = 0; i < kH; ++i) acc = fmaf(ha[sI][i], wbf(Wb, kOffW1 + t * kH + i), acc);
-    if (Z1 && b0 + sI < batch) Z1[static_cast<long>(b0 + sI) * kH + t] = acc;
-    hb[sI][t] = fmaxf(acc, 0.f);
-  }
-  __syncthreads();
-  // layer 2
-  for (int sI = 0; sI < kTile; ++sI) {
-    float acc = P[kOffB2 + t];
-    for (int i = 0; i < kH; ++i) acc = fmaf(hb[sI][i], wbf(Wb, kOffW2 + t * kH + i), acc);
-    if (Z2 && b0 + sI < batch) Z2[static_cast<long>(b0 + sI) * kH + t] = acc;
-    ha[sI][t] = fmaxf(acc, 0.f);
-  }
-  __syncthreads();
+  auto store = [&](const float (&acc)[NS], float (*out)[kH], float* Z) {
+#pragma unroll
+    for (int sI = 0; sI < NS; ++sI) {
+      if (Z && b0 + sI < batch) Z[static_cast<long>(b0 + sI) * kH + t] = acc[sI];
+      out[sI][t] = fmaxf(acc[sI], 0.f);
+    }
+    __syncthreads();
+  };
+  float acc[NS];
+  // layers 0 (64 -> 128), 1 and 2
+  layer_row<kF, NS>(Wb + kOffW0 + t * kF, P[kOffB0 + t], h0, acc);
+  store(acc, ha, Z0);
+  layer_row<kH, NS>(Wb + kOffW1 + t * kH, P[kOffB1 + t], ha, acc);
+  store(acc, hb, Z1);
+  layer_row<kH, NS>(Wb + kOffW2 + t * kH, P[kOffB2 + t], hb, acc);
+  store(acc, ha, Z2);
   // layer 3: 128 -> 6 (logits into Z3)
-  for (int idx = t; idx < kTile * kC; idx += blockDim.x) {
+  for (int idx = t; idx < NS * kC; idx += blockDim.x) {
     const int sI = idx / kC, o = idx % kC;
-    float acc = P[kOffB3 + o];
-    for (int i = 0; i < kH; ++i) acc = fmaf(ha[sI][i], wbf(Wb, kOffW3 + o * kH + i), acc);
-    if (b0 + sI < batch) Z3[static_cast<long>(b0 + sI) * kC + o] = acc;
+    float v[1];
+    layer_row<kH, 1>(Wb + kOffW3 + o * kH, P[kOffB3 + o], ha + sI, v);
+    if (b0 + sI < batch) Z3[static_cast<long>(b0 + sI) * kC + o] = v[0];
   }
   __syncthreads();
 }
@@ -213,7 +235,10 @@ __device__ void mlp_forward_tile(int b0, int batch, const float* X, const __nv_b
 __global__ void __launch_bounds__(128) mlp_forward_kernel(int batch, const float* X, const __nv_bfloat16* Wb,
                                                           const float* P, float* Z0, float* Z1, float* Z2, float* Z3) {
   __shared__ float h0[kTile][kF], ha[kTile][kH], hb[kTile][kH];
-  mlp_forward_tile(blockIdx.x * kTile, batch, X, Wb, P, h0, ha, hb, Z0, Z1, Z2, Z3);
+  if (batch == 1)
+    mlp_forward_tile<1>(0, batch, X, Wb, P, h0, ha, hb, Z0, Z1, Z2, Z3);
+  else
+    mlp_forward_tile<kTile>(blockIdx.x * kTile, batch, X, Wb, P, h0, ha, hb, Z0, Z1, Z2, Z3);
 }
 
 __global__ void predict_finish_kernel(int batch, const float* Z3, int32_t* out) {
@@ -398,14 +423,8 @@ int selector_features(emul_handle_t h, int m, int n, int k, Operand A, Operand B
   if (rc) return rc;
   rc = check_cuda(h, cudaMemsetAsync(st->hist, 0, 2 * kBins * 4, h->stream), "features reset");
   if (rc) return rc;
-  if (A.rs == 1)
-    hist_kernel<<<(m + 255) / 256, 256, 0, h->stream>>>(m, k, A.ptr, A.rs, A.cs, st->hist);
-  else
-    hist_kernel<<<(m + 7) / 8, 256, 0, h->stream>>>(m, k, A.ptr, A.rs, A.cs, st->hist);
-  if (B.rs == 1)
-    hist_kernel<<<(n + 255) / 256, 256, 0, h->stream>>>(n, k, B.ptr, B.rs, B.cs, st->hist + kBins);
-  else
-    hist_kernel<<<(n + 7) / 8, 256, 0, h->stream>>>(n, k, B.ptr, B.rs, B.cs, st->hist + kBins);
+  hist_kernel<<<hist_blocks(m, A.rs), 32 * kHistWarps, 0, h->stream>>>(m, k, A.ptr, A.rs, A.cs, st->hist);
+  hist_kernel<<<hist_blocks(n, B.rs), 32 * kHistWarps, 0, h->stream>>>(n, k, B.ptr, B.rs, B.cs, st->hist + kBins);
   hist_finish_kernel<<<1, 32, 0, h->stream>>>(st->hist, static_cast<double>(m) * k, static_cast<double>(n) * k, feat);
   h->launches += 3;
   return check_cuda(h, cudaGetLastError(), "features");
