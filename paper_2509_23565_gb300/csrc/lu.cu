@@ -351,11 +351,15 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
       }
       if (c > 0 && p_last != c - 1) out.swap(d0 + c - 1, d0 + p_last);
       if (pend && c + 1 < w) {
-      constexpr int kUpd = kLeafThreads - 64;   // warps 1-6
-      for (int lr = tid - 32; lr < rcount; lr += kUpd) {
-        if (r0 + lr <= c - 1) continue;
-        rank1_row(P + lr, ld, P[(c - 1) * ld + lr], pv, c + 1, w, 1);
-      }
+        // eight shares of the columns, two for each sub-partition's FP64 unit:
+        // warps 3 and 4, alone beside warps 7 and 0 of the exchange, take two each
+        const int s0 = warp == 3 ? 4 : (warp == 4 ? 6 : (warp < 3 ? warp - 1 : warp - 3));
+        const int s1 = warp == 3 || warp == 4 ? s0 + 2 : s0 + 1;
+        for (int lr = lane; lr < rcount; lr += 32) {
+          if (r0 + lr <= c - 1) continue;
+          const double l = P[(c - 1) * ld + lr];
+          for (int s = s0; s < s1; ++s) rank1_row(P + lr, ld, l, pv, c + 1 + s, w, 8);
+        }
       }
     }
     if ((warp == 0 || warp == kLeafThreads / 32 - 1) && c > 0 && p_last != c - 1) out.swap(d0 + c - 1, d0 + p_last);
@@ -593,6 +597,7 @@ constexpr int kPermGroups = 8;
 struct PermShared {
   int piv[kPermMax];                               // global rows, 0-based
   unsigned short id[kPermMax];                     // number of the row interchange i names
+  int key[4 * kPermMax], first[4 * kPermMax];      // rows outside the block: first interchange naming them
   unsigned short map[kPermGroups][2 * kPermMax];
   int dst[2 * kPermMax], src[2 * kPermMax], cnt;
 };
@@ -601,20 +606,26 @@ __device__ void perm_map(PermShared& S, int k1, int nb) {
   const int i = threadIdx.x;
   if (i == 0) S.cnt = 0;
   for (int e = i; e < kPermGroups * 2 * kPermMax; e += kPermMax) S.map[0][e] = static_cast<unsigned short>(e & (2 * kPermMax - 1));
-  int first = i;
-  if (i < nb) {
-    const int p = S.piv[i];
-    if (p >= k1 && p < k1 + nb) {
-      S.id[i] = static_cast<unsigned short>(p - k1);
-    } else {
-      for (int j = 0; j < i; ++j)
-        if (S.piv[j] == p) {
-          first = j;
-          break;
-        }
-      S.id[i] = static_cast<unsigned short>(kPermMax + first);
-    }
+  for (int e = i; e < 4 * kPermMax; e += kPermMax) {
+    S.key[e] = -1;
+    S.first[e] = kPermMax;
   }
+  __syncthreads();
+  const int p = i < nb ? S.piv[i] : 0;
+  const bool outside = i < nb && (p < k1 || p >= k1 + nb);
+  int slot = 0;
+  if (outside) {
+    // open addressing, at most kPermMax of 4 kPermMax slots taken
+    slot = p & (4 * kPermMax - 1);
+    while (true) {
+      const int was = atomicCAS(&S.key[slot], -1, p);
+      if (was == -1 || was == p) break;
+      slot = (slot + 1) & (4 * kPermMax - 1);
+    }
+    atomicMin(&S.first[slot], i);
+  }
+  __syncthreads();
+  if (i < nb) S.id[i] = static_cast<unsigned short>(outside ? kPermMax + S.first[slot] : p - k1);
   __syncthreads();
   const int per = (nb + kPermGroups - 1) / kPermGroups;
   if (i < kPermGroups) {
@@ -725,60 +736,8 @@ __global__ void gather_rows_kernel(const double* A, long lda, int r0, int n, int
   if (r < n) tmp[(r - r0) + static_cast<long>(c) * (n - r0)] = A[G[r] + static_cast<long>(c0 + c) * lda];
 }
 
-// X (w1 x w2 at A[d0.., c0..]) <- L^-1 X with L unit lower w1 x w1 at A[d0.., d0..]
-// (w1 <= 128).  The strictly lower part of L is staged in shared memory; one
-// warp per column of X (cpb columns per block), lane l holding rows l, l+32,
-// l+64, l+96 in registers, x_k broadcast by shuffle.
 constexpr int kTrsmMax = 128;
 inline int trtri_threads(int nb) { return nb <= 256 ? 256 : 512; }
-__global__ void __launch_bounds__(256) trsm_small_kernel(double* A, long lda, int d0, int w1, int c0, int w2,
-                                                         int cpb) {
-  // all threads stage L; the first cpb warps solve one column of X each
-  extern __shared__ double Ls[];   // Ls[i + k*w1] = L(i, k) for i > k, else 0
-  const int tid = threadIdx.x, lane = tid & 31;
-  {
-    // row i per thread, columns k = tid/128 + 2j, 16 loads in flight before their stores
-    const int i = tid & 127, kstep = blockDim.x >> 7;
-    if (i < w1)
-      for (int k0 = tid >> 7; k0 < w1; k0 += 16 * kstep) {
-        double v[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int k = k0 + j * kstep;
-          v[j] = (k < w1 && i > k) ? A[(d0 + i) + static_cast<long>(d0 + k) * lda] : 0.0;
-        }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int k = k0 + j * kstep;
-          if (k < w1) Ls[i + k * w1] = v[j];
-        }
-      }
-  }
-  __syncthreads();
-  if ((tid >> 5) >= cpb) return;
-  const int j = blockIdx.x * cpb + (tid >> 5);
-  if (j >= w2) return;
-  double* col = A + static_cast<long>(c0 + j) * lda + d0;
-  double x[4];
-#pragma unroll
-  for (int t = 0; t < 4; ++t) x[t] = lane + 32 * t < w1 ? col[lane + 32 * t] : 0.0;
-#pragma unroll
-  for (int t0 = 0; t0 < 4; ++t0) {
-    for (int kk = 0; kk < 32; ++kk) {
-      const int k = 32 * t0 + kk;
-      if (k >= w1) break;
-      const double xk = __shfl_sync(0xFFFFFFFFu, x[t0], kk);
-#pragma unroll
-      for (int t = t0; t < 4; ++t) {
-        const int i = lane + 32 * t;
-        if (i > k && i < w1) x[t] = fma(-Ls[i + k * w1], xk, x[t]);
-      }
-    }
-  }
-#pragma unroll
-  for (int t = 0; t < 4; ++t)
-    if (lane + 32 * t < w1) col[lane + 32 * t] = x[t];
-}
 
 // ---------------------------------------------------------------- Cholesky diagonal block
 // The nb x nb diagonal block of a Cholesky step (nb <= 512) is factored in
@@ -1014,9 +973,10 @@ __device__ __forceinline__ void diag_solve_t(const double* tb, int ld, const dou
   const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
   double v = i < bs ? x[i] : 0.0;
   const double r = SCALE && i < bs ? rcp[i] : 1.0;
-  for (int s = 0; s < 16; ++s) {
+  const int nsub = (bs + 7) / 8;
+  for (int s = 0; s < nsub; ++s) {
     // sub-step s: rows 8 ss .. 8 ss + 7, from the top (LOWER) or the bottom
-    const int ss = LOWER ? s : 15 - s;
+    const int ss = LOWER ? s : nsub - 1 - s;
     const int prev = LOWER ? ss - 1 : ss + 1;
     if (s > 0 && (LOWER ? warp > prev >> 2 : warp < prev >> 2)) {
       double t[8], y[8];
@@ -1058,6 +1018,39 @@ __device__ __forceinline__ void diag_solve(const double* tb, int ld, const doubl
     scale ? diag_solve_t<true, true>(tb, ld, rcp, bs, x) : diag_solve_t<true, false>(tb, ld, rcp, bs, x);
   else
     scale ? diag_solve_t<false, true>(tb, ld, rcp, bs, x) : diag_solve_t<false, false>(tb, ld, rcp, bs, x);
+}
+
+// X (w1 x w2 at A[d0.., c0..]) <- L^-1 X with L unit lower w1 x w1 at A[d0.., d0..]
+// (w1 <= 128), one block per column of X: 256 threads stage L in shared memory,
+// the first 128 solve (diag_solve).
+__global__ void __launch_bounds__(256) trsm_small_kernel(double* A, long lda, int d0, int w1, int c0) {
+  extern __shared__ double Ls[];   // Ls[i + k*ld] = L(i, k), ld odd
+  __shared__ double x[128];
+  const int tid = threadIdx.x, ld = w1 | 1;
+  double* col = A + static_cast<long>(c0 + blockIdx.x) * lda + d0;
+  if (tid < w1) x[tid] = col[tid];
+  {
+    // row i per thread, columns k = tid/128 + 2j, 16 loads in flight before their stores
+    const int i = tid & 127, kstep = blockDim.x >> 7;
+    if (i < w1)
+      for (int k0 = tid >> 7; k0 < w1; k0 += 16 * kstep) {
+        double v[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const int k = k0 + j * kstep;
+          v[j] = (k < w1 && i > k) ? A[(d0 + i) + static_cast<long>(d0 + k) * lda] : 0.0;
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const int k = k0 + j * kstep;
+          if (k < w1) Ls[i + k * ld] = v[j];
+        }
+      }
+  }
+  __syncthreads();
+  if (tid >= 128) return;
+  diag_solve(Ls, ld, nullptr, w1, true, false, x);
+  if (tid < w1) col[tid] = x[tid];
 }
 
 // One diagonal block of a triangular solve, x <- op(T)^-1 x for the bs x bs
@@ -1481,10 +1474,10 @@ int laswp(emul_handle_t h, double* A, long lda, int c0, int c1, const int32_t* i
 int trsm_small(emul_handle_t h, double* A, long lda, int d0, int w1, int c0, int w2) {
   if (w1 <= 0 || w2 <= 0) return EMUL_OK;
   if (w1 > kTrsmMax) return set_error(h, EMUL_NOT_SUPPORTED, "panel trsm wider than 128");
-  smem_attr(reinterpret_cast<const void*>(trsm_small_kernel), kTrsmMax * kTrsmMax * 8);
+  smem_attr(reinterpret_cast<const void*>(trsm_small_kernel), kTrsmMax * (kTrsmMax | 1) * 8);
   // one column per block: the solve is FP64-bound (about 1.6 FMA per clock per
   // SM), so it is spread over as many SMs as columns; 256 threads stage L
-  trsm_small_kernel<<<w2, 256, static_cast<size_t>(w1) * w1 * 8, h->stream>>>(A, lda, d0, w1, c0, w2, 1);
+  trsm_small_kernel<<<w2, 256, static_cast<size_t>(w1) * (w1 | 1) * 8, h->stream>>>(A, lda, d0, w1, c0);
   h->launches++;
   return check_cuda(h, cudaGetLastError(), "panel trsm");
 }
@@ -1554,17 +1547,17 @@ namespace emul {
 namespace {
 
 constexpr int kSolveBs = 128;      // diagonal block of the persistent solve
-constexpr int kPermSmemMax = 52 * 1024;   // rows whose permutation fits in shared memory (4 B each, + 14 KB)
+constexpr int kPermSmemMax = 1 << 16;   // rows whose permutation fits in shared memory (2 B each, + 22 KB)
 
 // x <- P x for the interchanges ipiv[0..n) (1-based, applied in order): the
 // composite permutation is built in shared memory, 256 interchanges resolved at a
 // time (perm_map), then x is gathered through tmp.  One block.  An entry outside
 // [0, n) leaves its row where it is.
 __global__ void __launch_bounds__(kPermMax) permute_rhs_kernel(const int32_t* ipiv, int n, double* x, double* tmp) {
-  extern __shared__ int perm[];
+  extern __shared__ unsigned short perm[];   // n <= kPermSmemMax = 2^16
   __shared__ PermShared S;
   const int i = threadIdx.x;
-  for (int e = i; e < n; e += kPermMax) perm[e] = e;
+  for (int e = i; e < n; e += kPermMax) perm[e] = static_cast<unsigned short>(e);
   for (int k0 = 0; k0 < n; k0 += kPermMax) {
     const int nb = n - k0 < kPermMax ? n - k0 : kPermMax;
     if (i < nb) {
@@ -1573,7 +1566,7 @@ __global__ void __launch_bounds__(kPermMax) permute_rhs_kernel(const int32_t* ip
     }
     __syncthreads();
     perm_map(S, k0, nb);
-    int v[2];
+    unsigned short v[2];
     for (int h = 0; h < 2; ++h) v[h] = i + h * kPermMax < S.cnt ? perm[S.src[i + h * kPermMax]] : 0;
     __syncthreads();
     for (int h = 0; h < 2; ++h)
@@ -1802,9 +1795,9 @@ int getrs_body(emul_handle_t h, int n, int nrhs, const double* LU, int lda, cons
     uint8_t* ws = static_cast<uint8_t*>(h->ws);
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(ws);
     double* tmp = reinterpret_cast<double*>(ws + kAl);
-    smem_attr(reinterpret_cast<const void*>(permute_rhs_kernel), kPermSmemMax * 4);
+    smem_attr(reinterpret_cast<const void*>(permute_rhs_kernel), kPermSmemMax * 2);
     smem_attr(reinterpret_cast<const void*>(getrs1_kernel<false>), kSolveBs * (kSolveBs + 1) * 8);
-    permute_rhs_kernel<<<1, kPermMax, static_cast<size_t>(n) * 4, h->stream>>>(ipiv, n, B, tmp);
+    permute_rhs_kernel<<<1, kPermMax, static_cast<size_t>(n) * 2, h->stream>>>(ipiv, n, B, tmp);
     h->launches++;
     rc = check_cuda(h, cudaGetLastError(), "rhs permutation");
     if (rc) return rc;
