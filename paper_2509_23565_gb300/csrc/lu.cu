@@ -908,55 +908,59 @@ __global__ void __launch_bounds__(32 * kNtRows) dgemm_nt_small_kernel(int m, int
 }
 
 // inv (nb x nb, ld nb) <- L^-1 for the lower triangular L at A[d0.., d0..]
-// (unit diagonal if `unit`; nb <= 512, one thread per row: launch nb blocks of
-// trtri_threads(nb) threads): each block solves L x = e_j for one column j by
-// column substitution.  Thread i owns row i of x in a register and reads row i
-// of L sixteen columns ahead (coalesced along the column); x_k is published
-// through shared memory, one barrier per step.  A step is a chain of a DFMA (64
-// cycles; another for the non-unit scaling), a store, a barrier and a load; two
-// columns per block put both columns' FP64 work into that chain (40 us at nb =
-// 256, 78 us with the scaling).
-__global__ void __launch_bounds__(512) trtri_cols_kernel(const double* A, long lda, int d0, int nb, int unit,
-                                                        double* inv, const int32_t* info) {
-  __shared__ double bc[2];
+// (unit diagonal if UNIT; nb <= 512, one thread per row: launch nb blocks of
+// trtri_threads(nb) threads): block j solves L x = e_j by column substitution,
+// thread i holding row i of x.  As in diag_solve, the warp that holds the rows at
+// hand takes eight steps by shuffles (a DFMA of 64 cycles each, another
+// multiplication for the non-unit scaling) and publishes the eight values, which
+// the warps below take off their rows in the next round; a thread reads row i of
+// the next eight columns of L meanwhile (coalesced along the columns).  (One
+// block-wide barrier per step: 52 us at nb = 256, 54 us with the scaling.)
+template <bool UNIT>
+__global__ void __launch_bounds__(512) trtri_cols_kernel(const double* A, long lda, int d0, int nb, double* inv,
+                                                        const int32_t* info) {
+  __shared__ double xs[512];
   if (info && *info != 0) return;
   const double* L = A + d0 + static_cast<long>(d0) * lda;
-  const int i = threadIdx.x;
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
   const int j = blockIdx.x;
-  double x = (i == j) ? 1.0 : 0.0;
-  // every row's reciprocal at once: the steps below then multiply (a division
-  // on each step's dependent path would cost its full FP64 latency 256 times)
-  const double rinv = (!unit && i < nb) ? 1.0 / L[i + static_cast<long>(i) * lda] : 1.0;
-  double ln[16];
+  double x = (i == j) ? 1.0 : 0.0, res = 0.0;
+  // every row's reciprocal at once: the steps then multiply (a division on the
+  // dependent path would cost its 560 cycles every time)
+  const double rinv = (!UNIT && i < nb) ? 1.0 / L[i + static_cast<long>(i) * lda] : 1.0;
+  auto load = [&](int ss, double (&l)[8]) {
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const int kk = j + q;
-    ln[q] = (i < nb && kk < nb && i >= kk + unit) ? L[i + static_cast<long>(kk) * lda] : 0.0;
-  }
-  for (int g = j; g < nb; g += 16) {
-    double lv[16];
+    for (int q = 0; q < 8; ++q) {
+      const int k = 8 * ss + q;
+      l[q] = (i < nb && k < nb && i > k) ? L[i + static_cast<long>(k) * lda] : 0.0;
+    }
+  };
+  const int nsub = (nb + 7) / 8, first = j / 8;
+  double lp[8], l[8], ln[8];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) lv[q] = ln[q];
-    if (g + 16 < nb) {
+  for (int q = 0; q < 8; ++q) lp[q] = 0.0;
+  load(first, l);
+  for (int ss = first; ss < nsub; ++ss) {
+    load(ss + 1 < nsub ? ss + 1 : ss, ln);
+    if (ss > first && warp > (ss - 1) >> 2) {
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const int kk = g + 16 + q;
-        ln[q] = (i < nb && kk < nb && i >= kk + unit) ? L[i + static_cast<long>(kk) * lda] : 0.0;
+      for (int q = 0; q < 8; ++q) x = fma(-lp[q], xs[8 * (ss - 1) + q], x);
+    }
+    if (warp == ss >> 2) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int kl = (8 * ss + q) & 31;
+        const double xv = UNIT ? x : x * rinv;
+        if (lane == kl) res = xv;              // final; x itself may meet an infinity from here on
+        x = fma(-l[q], __shfl_sync(0xFFFFFFFFu, xv, kl), x);
       }
+      if (lane >> 3 == (ss & 3)) xs[i] = res;
     }
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int kk = g + q;
-      if (kk >= nb) break;
-      if (i == kk) {
-        if (!unit) x *= rinv;
-        bc[kk & 1] = x;
-      }
-      __syncthreads();
-      if (i > kk && i < nb) x = fma(-lv[q], bc[kk & 1], x);
-    }
+    for (int q = 0; q < 8; ++q) lp[q] = l[q], l[q] = ln[q];
+    __syncthreads();
   }
-  if (i < nb) inv[i + static_cast<long>(j) * nb] = x;
+  if (i < nb) inv[i + static_cast<long>(j) * nb] = res;
 }
 
 // x <- T^-1 x for the bs x bs (bs <= 128) triangle T(i, k) = tb[i + k*ld] in
@@ -973,10 +977,12 @@ __device__ __forceinline__ void diag_solve_t(const double* tb, int ld, const dou
   const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
   double v = i < bs ? x[i] : 0.0;
   const double r = SCALE && i < bs ? rcp[i] : 1.0;
-  const int nsub = (bs + 7) / 8;
-  for (int s = 0; s < nsub; ++s) {
+  double res = 0.0;
+#pragma unroll 1
+  for (int s = LOWER ? 0 : 16 - (bs + 7) / 8; s < 16; ++s) {
     // sub-step s: rows 8 ss .. 8 ss + 7, from the top (LOWER) or the bottom
-    const int ss = LOWER ? s : nsub - 1 - s;
+    const int ss = LOWER ? s : 15 - s;
+    if (LOWER && 8 * ss >= bs) break;        // uniform
     const int prev = LOWER ? ss - 1 : ss + 1;
     if (s > 0 && (LOWER ? warp > prev >> 2 : warp < prev >> 2)) {
       double t[8], y[8];
@@ -999,15 +1005,13 @@ __device__ __forceinline__ void diag_solve_t(const double* tb, int ld, const dou
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int kl = (8 * ss + (LOWER ? q : 7 - q)) & 31;       // the step's lane; lanes past bs hold zeros
-        if (SCALE) {
-          const double xv = v * r;
-          if (lane == kl) v = xv;
-          v = fma(-t[q], __shfl_sync(0xFFFFFFFFu, xv, kl), v);
-        } else {
-          v = fma(-t[q], __shfl_sync(0xFFFFFFFFu, v, kl), v);
-        }
+        // the step's row is final: its value is kept aside (v of a finished row,
+        // updated with a zero from here on, may meet an infinity)
+        const double xv = SCALE ? v * r : v;
+        if (lane == kl) res = xv;
+        v = fma(-t[q], __shfl_sync(0xFFFFFFFFu, xv, kl), v);
       }
-      if (lane >> 3 == (ss & 3) && i < bs) x[i] = v;
+      if (lane >> 3 == (ss & 3) && i < bs) x[i] = res;
     }
     asm volatile("bar.sync 1, 128;" ::: "memory");
   }
@@ -1329,7 +1333,7 @@ int chol_diag(emul_handle_t h, double* A, long lda, int d0, int jb, double* inv,
     }
   }
   if (want_inv) {
-    trtri_cols_kernel<<<jb, trtri_threads(jb), 0, h->stream>>>(A, lda, d0, jb, 0, inv, info);
+    trtri_cols_kernel<false><<<jb, trtri_threads(jb), 0, h->stream>>>(A, lda, d0, jb, inv, info);
     h->launches++;
   }
   return check_cuda(h, cudaGetLastError(), "Cholesky diagonal block");
@@ -1518,7 +1522,7 @@ int panel_getrf(emul_handle_t h, double* A, long lda, int n, int j0, int jb, int
   if (rc) return rc;
   rc = laswp(h, A, lda, j0 + w1, j0 + jb, ipiv, j0, j0 + w1, B.map);
   if (rc) return rc;
-  trtri_cols_kernel<<<w1, trtri_threads(w1), 0, h->stream>>>(A, lda, j0, w1, 1, B.inv, nullptr);
+  trtri_cols_kernel<true><<<w1, trtri_threads(w1), 0, h->stream>>>(A, lda, j0, w1, B.inv, nullptr);
   h->launches++;
   rc = check_cuda(h, cudaGetLastError(), "panel trtri");
   if (rc) return rc;
@@ -2012,8 +2016,7 @@ int emul_dgetrf(emul_handle_t h, int n, double* A, int lda, int32_t* ipiv, int n
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_start, h->stream), "stream events");
       if (!rc) rc = emul::check_cuda(h, cudaStreamWaitEvent(h->aux, h->aux_start, 0), "stream events");
       if (rc) return rc;
-      emul::trtri_cols_kernel<<<jb, emul::trtri_threads(jb), 0, h->aux>>>(A, lda, j0, jb, 1, B.inv,
-                                                                                       nullptr);
+      emul::trtri_cols_kernel<true><<<jb, emul::trtri_threads(jb), 0, h->aux>>>(A, lda, j0, jb, B.inv, nullptr);
       h->launches++;
       rc = emul::check_cuda(h, cudaGetLastError(), "trtri");
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_done, h->aux), "stream events");
