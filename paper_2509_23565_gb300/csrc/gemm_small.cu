@@ -181,7 +181,9 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_product_kernel(const Smal
   tc_fence_after();
 
   if (ok) {
-    // T = hi 2^28 + lo: the four highest levels (weights 2^0 .. 2^21) in lo, the others in hi
+    // T = hi 2^28 + lo: the four highest levels (weights 2^0 .. 2^21) in lo, the
+    // others in hi; two adjacent levels in one 32-bit word first.  Below 2^22 a
+    // level sum becomes an integer by an FP32 add (see gemm_kernel.cuh).
     const int quarter = warp & 3, cg = warp >> 2;
     const uint32_t ta = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + (uint32_t)(cg * 8);
     long long lo[8], hi[8];
@@ -197,16 +199,33 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_product_kernel(const Smal
         if (L >= 2) tmem_ld8(ta + (uint32_t)((L - 2) * kSmBN), r[i]);
       }
       tmem_ld_wait();
+      float mx = 0.f;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < 4; ++i)
+        if (s + 1 - 4 * q - i >= 2) {
+#pragma unroll
+          for (int c = 0; c < 8; ++c) mx = fmaxf(mx, fabsf(__uint_as_float(r[i][c])));
+        }
+      const bool quick = mx < 4194304.0f;
+#pragma unroll
+      for (int i = 0; i < 4; i += 2) {
         if (s + 1 - 4 * q - i < 2) continue;
+        const bool two = s + 1 - 4 * q - i - 1 >= 2;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          const long long v = (long long)__float2int_rn(__uint_as_float(r[i][c])) << (7 * i);
+          long long v;
+          if (quick) {
+            int w = __float_as_int(__uint_as_float(r[i][c]) + 12582912.0f) - 0x4B400000;
+            if (two) w += (__float_as_int(__uint_as_float(r[two ? i + 1 : i][c]) + 12582912.0f) - 0x4B400000) * 128;
+            v = w;
+          } else {
+            v = __float2int_rn(__uint_as_float(r[i][c]));
+            if (two) v += (long long)__float2int_rn(__uint_as_float(r[two ? i + 1 : i][c])) * 128;
+          }
           if (q == 0)
-            lo[c] += v;
+            lo[c] += v << (7 * i);
           else
-            hi[c] += v;
+            hi[c] += v << (7 * i);
         }
       }
     }
@@ -227,7 +246,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_product_kernel(const Smal
           const int sh = e + f + sh0;
           if (sh < -1022 || sh > 944) {
             D = rn_scaled(((__int128)hi[c] << 28) + (__int128)lo[c], sh);
-          } else if (S <= 6) {      // |T| <= 6 slices' 2^(14 + 7 + 35): 64 bits hold it
+          } else if (S <= 6 || (S == 7 && a.K <= 64)) {   // |T| < 1.02 2^(14 + 35) k, 2^(14 + 42) k: 64 bits hold it
             D = rn_x64((hi[c] << 28) + lo[c], sh);
           } else {
             D = rn_x80((hi[c] << 12) + (lo[c] >> 16), (uint32_t)lo[c] & 0xFFFFu, sh);

@@ -125,8 +125,7 @@ __global__ void __launch_bounds__(32 * kNpWarps, 1) np_leaf_kernel(double* A, lo
 // Inverses of the leaf's factors: X <- L^-1 (ld ldx, zeros above the diagonal)
 // and Y <- U^-1 (ld w, zeros below; an infinite reciprocal for a zero pivot).
 // One warp per column of X or Y and four columns per block, so every warp has a
-// sub-partition's FP64 unit to itself: a step is a shuffle and two DFMAs
-// (about 200 cycles).  Row k of a column, once final, is broadcast; column j of X
+// sub-partition's FP64 unit to itself: a step is a shuffle and one or two DFMAs.  Row k of a column, once final, is broadcast; column j of X
 // starts at row j, of Y at row j and goes up.
 constexpr int kInvCols = 4;
 __global__ void __launch_bounds__(32 * kInvCols) np_inverse_kernel(const double* A, long lda, int d, int w, double* X,
@@ -135,9 +134,20 @@ __global__ void __launch_bounds__(32 * kInvCols) np_inverse_kernel(const double*
   __shared__ double rdiag[kNpLeaf];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double* D = A + d + static_cast<long>(d) * lda;
-  for (int e = threadIdx.x; e < kNpLeaf * kNpLeaf; e += blockDim.x) {
-    const int i = e & (kNpLeaf - 1), k = e / kNpLeaf;
-    S[k][i] = i < w && k < w ? D[i + static_cast<long>(k) * lda] : 0.0;
+  // sixteen loads in flight per thread
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    double v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int e = threadIdx.x + (16 * h + q) * 32 * kInvCols, i = e & (kNpLeaf - 1), k = e / kNpLeaf;
+      v[q] = i < w && k < w ? D[i + static_cast<long>(k) * lda] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int e = threadIdx.x + (16 * h + q) * 32 * kInvCols;
+      S[e / kNpLeaf][e & (kNpLeaf - 1)] = v[q];
+    }
   }
   __syncthreads();
   const bool lower = blockIdx.y == 0;
@@ -151,29 +161,41 @@ __global__ void __launch_bounds__(32 * kInvCols) np_inverse_kernel(const double*
   }
   const int j = blockIdx.x * kInvCols + warp;
   if (j >= w) return;
-  double x0 = lane == j ? 1.0 : 0.0, x1 = lane + 32 == j ? 1.0 : 0.0;
+  // x0, x1: rows lane and lane + 32 of the column; r0, r1: their final values,
+  // kept aside (a finished row, updated with zeros from then on, may meet an infinity)
+  double x0 = lane == j ? 1.0 : 0.0, x1 = lane + 32 == j ? 1.0 : 0.0, r0 = 0.0, r1 = 0.0;
   if (lower) {
-    for (int k = j; k + 1 < w; ++k) {
-      const double xk = __shfl_sync(0xFFFFFFFFu, k < 32 ? x0 : x1, k & 31);
-      if (k < 31 && lane > k) x0 = fma(-S[k][lane], xk, x0);
-      if (lane + 32 > k) x1 = fma(-S[k][lane + 32], xk, x1);
+    const int n0 = w < 32 ? w : 32;
+    for (int k = j; k < n0; ++k) {
+      const double xk = __shfl_sync(0xFFFFFFFFu, x0, k);
+      if (lane == k) r0 = x0;
+      x0 = fma(lane > k ? -S[k][lane] : 0.0, xk, x0);
+      x1 = fma(-S[k][lane + 32], xk, x1);
     }
-    if (lane < w) X[lane + static_cast<long>(j) * ldx] = x0;
-    if (lane + 32 < w) X[lane + 32 + static_cast<long>(j) * ldx] = x1;
+    for (int k = j > 32 ? j : 32; k < w; ++k) {
+      const double xk = __shfl_sync(0xFFFFFFFFu, x1, k - 32);
+      if (lane == k - 32) r1 = x1;
+      x1 = fma(lane > k - 32 ? -S[k][lane + 32] : 0.0, xk, x1);
+    }
+    if (lane < w) X[lane + static_cast<long>(j) * ldx] = r0;
+    if (lane + 32 < w) X[lane + 32 + static_cast<long>(j) * ldx] = r1;
   } else {
-    for (int k = j; k >= 0; --k) {
-      if (lane == (k & 31)) {
-        if (k < 32)
-          x0 *= rdiag[k];
-        else
-          x1 *= rdiag[k];
-      }
-      const double xk = __shfl_sync(0xFFFFFFFFu, k < 32 ? x0 : x1, k & 31);
-      if (lane < k) x0 = fma(-S[k][lane], xk, x0);
-      if (k > 32 && lane + 32 < k) x1 = fma(-S[k][lane + 32], xk, x1);
+    const double d0 = lane < w ? rdiag[lane] : 1.0, d1 = lane + 32 < w ? rdiag[lane + 32] : 1.0;
+    for (int k = j; k >= 32; --k) {
+      const double xv = x1 * d1;
+      const double xk = __shfl_sync(0xFFFFFFFFu, xv, k - 32);
+      if (lane == k - 32) r1 = xv;
+      x0 = fma(-S[k][lane], xk, x0);
+      x1 = fma(lane < k - 32 ? -S[k][lane + 32] : 0.0, xk, x1);
     }
-    if (lane < w) Y[lane + static_cast<long>(j) * w] = x0;
-    if (lane + 32 < w) Y[lane + 32 + static_cast<long>(j) * w] = x1;
+    for (int k = j < 31 ? j : 31; k >= 0; --k) {
+      const double xv = x0 * d0;
+      const double xk = __shfl_sync(0xFFFFFFFFu, xv, k);
+      if (lane == k) r0 = xv;
+      x0 = fma(lane < k ? -S[k][lane] : 0.0, xk, x0);
+    }
+    if (lane < w) Y[lane + static_cast<long>(j) * w] = r0;
+    if (lane + 32 < w) Y[lane + 32 + static_cast<long>(j) * w] = r1;
   }
 }
 
