@@ -44,6 +44,7 @@
 #include <type_traits>
 
 #include "emul_internal.h"
+#include "launch.h"
 #include "ptx.cuh"
 #include "round.cuh"
 
@@ -315,10 +316,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t rank = PAIR ? cluster_rank() : 0u;
   const int cta0 = (int)blockIdx.x / G, ncta = (int)gridDim.x / G;   // tile loop over CTAs or CTA pairs
 
-  const bool sched_in_smem = a.nsweeps <= kSchedSmem;
-  if (sched_in_smem)
-    for (int i = threadIdx.x; i < a.nsweeps; i += blockDim.x) sched_s[i] = a.sched[i];
-  const Sweep* sched = sched_in_smem ? sched_s : a.sched;
   if (threadIdx.x == 0) {
     for (int i = 0; i < stages; ++i) {
       mbar_init(&stage_full[i], 1);
@@ -338,9 +335,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     else
       tmem_alloc(&tmem_base, Cf::TMEM_COLS);
   }
+  grid_wait();
+  const bool sched_in_smem = a.nsweeps <= kSchedSmem;
+  if (sched_in_smem)
+    for (int i = threadIdx.x; i < a.nsweeps; i += blockDim.x) sched_s[i] = a.sched[i];
+  const Sweep* sched = sched_in_smem ? sched_s : a.sched;
   tc_fence_before();
   __syncthreads();
   if (PAIR) cluster_sync();   // barriers of both CTAs initialised before any copy or arrival
+  grid_launch();              // with the TMEM in hand (ptx.cuh)
   tc_fence_after();
   const uint32_t tmem = tmem_base;
 
@@ -848,22 +851,21 @@ cudaError_t launch_one(cudaStream_t st, const CUtensorMap& tmA, const CUtensorMa
     if (e != cudaSuccess) return e;
     if (dev < kMaxDevices) ready[dev].store(true, std::memory_order_release);
   }
-  if (!PAIR) {
-    kern<<<grid, kThreads, smem_bytes, st>>>(tmA, tmB, args, stages);
-    return cudaGetLastError();
-  }
+  if (!PAIR) return launch_dependent(kern, dim3(grid), dim3(kThreads), smem_bytes, st, tmA, tmB, args, stages);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // launch.h
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   // the persistent grid holds no more pairs than can be resident at once (an
   // SM left without a partner would otherwise run its pair after the others)
   const int pairs = gemm_pair_capacity(smem_bytes);

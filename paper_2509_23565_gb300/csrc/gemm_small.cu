@@ -19,6 +19,7 @@
 #include <cstdint>
 
 #include "emul_internal.h"
+#include "launch.h"
 #include "ptx.cuh"
 #include "round.cuh"
 #include "slice.cuh"
@@ -81,6 +82,12 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_product_kernel(const Smal
   uint8_t* sA = smem;                                       // [s][2 chunks][128 rows x 64 B]
   uint8_t* sB = smem + static_cast<size_t>(s) * 2 * kSmATile;   // [s][2 chunks][32 rows x 64 B]
 
+  if (tid == 0) {
+    mbar_init(&done, 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) tmem_alloc(&tmem_base, kSmTmemCols);
+  grid_wait();
   // operands into registers (all loads in flight together)
   const int ar = tid & 127, ag = tid >> 7;
   const bool b_rows = a.brs == 1;
@@ -90,11 +97,6 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_product_kernel(const Smal
   for (int i = 0; i < 4; ++i) load8(a.A, a.ars, a.acs, m0 + ar, a.M, 8 * (ag + 4 * i), a.K, ua[i]);
   load8(a.B, a.brs, a.bcs, n0 + br, a.N, 8 * bg, a.K, ub);
 
-  if (tid == 0) {
-    mbar_init(&done, 1);
-    fence_mbar_init();
-  }
-  if (warp == 0) tmem_alloc(&tmem_base, kSmTmemCols);
   {
     uint32_t up = 0;
 #pragma unroll
@@ -107,6 +109,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_product_kernel(const Smal
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_launch();
   bool full = false;        // an existing row of zeros and subnormals only
   if (tid < kSmBM) {
     uint32_t up = part_a[0][tid];
@@ -274,8 +277,11 @@ __global__ void __launch_bounds__(kSmThreads, 1) small_product_kernel(const Smal
 }  // namespace
 
 // Whether the one-launch product takes this shape: K and the level sums within
-// its limits, and one block per SM at most.  The line was measured with both
-// sides (us, this kernel / slicing and persistent kernel):
+// its limits, and one block per SM at most.  Both sides of the line in us (this
+// kernel / slicing kernel and persistent kernel, s = 7): 64^3 11.9 / 21.3, 128^3
+// 18.6 / 26.6, 4000 x 64 x 64 12.4 / 16.1, 600 x 960 x 64 (150 tiles) 12.6 / 18.3;
+// with a second block on some SMs 1000 x 1000 x 64 24.3 / 19.0, 8192 x 128 x 128
+// 37.3 / 23.2 (at s = 3 17.4 / 16.5 and 24.0 / 17.2).
 bool small_product_fits(int m, int n, int k, int s, int nsm) {
   const long tiles = static_cast<long>((m + kSmBM - 1) / kSmBM) * ((n + kSmBN - 1) / kSmBN);
   return k >= 1 && k <= kSmMaxK && s * k <= kExactBudget && s <= kMaxSlices && tiles <= nsm;
@@ -294,8 +300,7 @@ cudaError_t launch_small_s(cudaStream_t st, const SmallArgs& a) {
     if (dev < 64) ready[dev].store(true, std::memory_order_release);
   }
   const dim3 grid((a.M + kSmBM - 1) / kSmBM, (a.N + kSmBN - 1) / kSmBN);
-  small_product_kernel<S><<<grid, kSmThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(small_product_kernel<S>, grid, kSmThreads, smem, st, a);
 }
 
 cudaError_t launch_small_product(cudaStream_t st, int m, int n, int k, double alpha, const double* A, long ars,

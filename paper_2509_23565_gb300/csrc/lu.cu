@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include "handle.h"
+#include "launch.h"
 #include "ptx.cuh"
 
 namespace emul {
@@ -453,6 +454,8 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_cluster_kernel(double* A, 
   const int dlr = dgrp * 32 + lane;
   if (tid < 2) mbar_init(&full[tid], 1);
   if (tid == 0) fence_mbar_init();
+  grid_launch();
+  grid_wait();
   for (int lr = tid & (kClusterR - 1), half = tid / kClusterR; lr < rcount; lr += kClusterR) {
     // 16 columns per half of the block, their loads in flight together
     const double* src = A + (d0 + r0 + lr) + static_cast<long>(d0) * lda;
@@ -663,6 +666,8 @@ __device__ void perm_map(PermShared& S, int k1, int nb) {
 __global__ void __launch_bounds__(kPermMax) laswp_perm_kernel(const int32_t* ipiv, int k1, int k2,
                                                              int* map /* [2][2*kPermMax] + count */) {
   __shared__ PermShared S;
+  grid_launch();
+  grid_wait();
   const int nb = k2 - k1;
   const int i = threadIdx.x;
   if (i < nb) S.piv[i] = ipiv[k1 + i] - 1;
@@ -680,6 +685,8 @@ __global__ void __launch_bounds__(kPermMax) laswp_perm_kernel(const int32_t* ipi
 // stores after the whole block has read.
 constexpr int kSwpCols = 8;
 __global__ void __launch_bounds__(256) laswp_apply_kernel(double* A, long lda, int c0, int c1, const int* map) {
+  grid_launch();
+  grid_wait();
   const int cnt = map[4 * kPermMax];
   const int cb = c0 + blockIdx.x * kSwpCols;
   const int ncol = c1 - cb < kSwpCols ? c1 - cb : kSwpCols;
@@ -767,6 +774,8 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
   __shared__ double col[2][kCholLeaf];
   __shared__ int fail_s;       // pivot that failed
   const int i = threadIdx.x & 31, q = threadIdx.x >> 5;
+  grid_launch();
+  grid_wait();
   if (threadIdx.x == 0) fail_s = *info != 0 ? -1 : kCholLeaf;
   __syncthreads();
   if (fail_s < 0) return;
@@ -851,6 +860,8 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
 constexpr int kCholSolveRows = 4;
 __global__ void __launch_bounds__(32 * kCholSolveRows) chol_solve_kernel(const double* Lp, long lda, int w, double* Xp,
                                                                         int m, const int32_t* info) {
+  grid_launch();
+  grid_wait();
   if (*info != 0) return;
   const int lane = threadIdx.x & 31, r = blockIdx.x * kCholSolveRows + (threadIdx.x >> 5);
   // lane j holds row j of L: its entries below the diagonal are column k's multipliers
@@ -881,6 +892,8 @@ __global__ void __launch_bounds__(32 * kNtRows) dgemm_nt_small_kernel(int m, int
                                                             long bcs, double beta, double* C, long ldc,
                                                             int lower, const int32_t* info) {
   __shared__ double As[kNtRows][33], Bs[32][33];
+  grid_launch();
+  grid_wait();
   if (*info != 0) return;
   const int ti = threadIdx.x & (kNtRows - 1), tj = threadIdx.x / kNtRows;
   const int i0 = blockIdx.x * kNtRows, j0 = blockIdx.y * 32;
@@ -920,6 +933,8 @@ template <bool UNIT>
 __global__ void __launch_bounds__(512) trtri_cols_kernel(const double* A, long lda, int d0, int nb, double* inv,
                                                         const int32_t* info) {
   __shared__ double xs[512];
+  grid_launch();
+  grid_wait();
   if (info && *info != 0) return;
   const double* L = A + d0 + static_cast<long>(d0) * lda;
   const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
@@ -1030,6 +1045,8 @@ __device__ __forceinline__ void diag_solve(const double* tb, int ld, const doubl
 __global__ void __launch_bounds__(256) trsm_small_kernel(double* A, long lda, int d0, int w1, int c0) {
   extern __shared__ double Ls[];   // Ls[i + k*ld] = L(i, k), ld odd
   __shared__ double x[128];
+  grid_launch();
+  grid_wait();
   const int tid = threadIdx.x, ld = w1 | 1;
   double* col = A + static_cast<long>(c0 + blockIdx.x) * lda + d0;
   if (tid < w1) x[tid] = col[tid];
@@ -1318,22 +1335,22 @@ size_t lu_extra_bytes(int nb, int nsm) {
 int chol_diag(emul_handle_t h, double* A, long lda, int d0, int jb, double* inv, int32_t* info, bool want_inv) {
   for (int c0 = 0; c0 < jb; c0 += kCholLeaf) {
     const int wp = kCholLeaf < jb - c0 ? kCholLeaf : jb - c0;
-    chol_leaf_kernel<<<1, 128, 0, h->stream>>>(A, lda, d0 + c0, wp, info);
+    launch_dependent(chol_leaf_kernel, dim3(1), dim3(128), 0, h->stream, A, lda, d0 + c0, wp, info);
     h->launches++;
     const int r0 = c0 + wp, mr = jb - r0;
     if (mr > 0) {
       double* Lp = A + (d0 + r0) + static_cast<long>(d0 + c0) * lda;   // rows below the leaf, its columns
-      chol_solve_kernel<<<(mr + kCholSolveRows - 1) / kCholSolveRows, 32 * kCholSolveRows, 0, h->stream>>>(
-          A + (d0 + c0) + static_cast<long>(d0 + c0) * lda, lda, wp, Lp, mr, info);
+      launch_dependent(chol_solve_kernel, dim3((mr + kCholSolveRows - 1) / kCholSolveRows), dim3(32 * kCholSolveRows), 0,
+          h->stream, A + (d0 + c0) + static_cast<long>(d0 + c0) * lda, lda, wp, Lp, mr, info);
       // A(r0.., r0..) -= L(r0.., c0..) L(r0.., c0..)^T, lower part
-      dgemm_nt_small_kernel<<<dim3((mr + kNtRows - 1) / kNtRows, (mr + 31) / 32), 32 * kNtRows, 0, h->stream>>>(
-          mr, mr, wp, -1.0, Lp, 1, lda, Lp, 1, lda, 1.0, A + (d0 + r0) + static_cast<long>(d0 + r0) * lda, lda, 1,
+      launch_dependent(dgemm_nt_small_kernel, dim3((mr + kNtRows - 1) / kNtRows, (mr + 31) / 32), dim3(32 * kNtRows), 0,
+          h->stream, mr, mr, wp, -1.0, Lp, 1, lda, Lp, 1, lda, 1.0, A + (d0 + r0) + static_cast<long>(d0 + r0) * lda, lda, 1,
           info);
       h->launches += 2;
     }
   }
   if (want_inv) {
-    trtri_cols_kernel<false><<<jb, trtri_threads(jb), 0, h->stream>>>(A, lda, d0, jb, inv, info);
+    launch_dependent(trtri_cols_kernel<false>, dim3(jb), dim3(trtri_threads(jb)), 0, h->stream, A, lda, d0, jb, inv, info);
     h->launches++;
   }
   return check_cuda(h, cudaGetLastError(), "Cholesky diagonal block");
@@ -1408,13 +1425,15 @@ int launch_leaf(emul_handle_t h, double* A, long lda, int n, int d0, int w, int 
     cfg.blockDim = dim3(kLeafThreads);
     cfg.dynamicSmemBytes = static_cast<size_t>(R | 1) * w * 8;
     cfg.stream = h->stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // launch.h
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     h->launches++;
     return check_cuda(h, cudaLaunchKernelEx(&cfg, getf2_cluster_kernel, A, lda, n, d0, w, R, pc0, pc1, ipiv, info,
                                             h->d_status, h->wait_limit),
@@ -1449,7 +1468,7 @@ int launch_leaf(emul_handle_t h, double* A, long lda, int n, int d0, int w, int 
 int laswp_prepare(emul_handle_t h, const int32_t* ipiv, int k1, int k2, int* map) {
   if (k2 <= k1) return EMUL_OK;
   if (k2 - k1 > kPermMax) return set_error(h, EMUL_INVALID_ARG, "too many interchanges in one block");
-  laswp_perm_kernel<<<1, kPermMax, 0, h->stream>>>(ipiv, k1, k2, map);
+  launch_dependent(laswp_perm_kernel, dim3(1), dim3(kPermMax), 0, h->stream, ipiv, k1, k2, map);
   h->launches++;
   return check_cuda(h, cudaGetLastError(), "laswp map");
 }
@@ -1457,7 +1476,7 @@ int laswp_prepare(emul_handle_t h, const int32_t* ipiv, int k1, int k2, int* map
 // Apply a prepared gather map to columns [c0, c1).
 int laswp_apply(emul_handle_t h, double* A, long lda, int c0, int c1, const int* map) {
   if (c1 <= c0) return EMUL_OK;
-  laswp_apply_kernel<<<(c1 - c0 + kSwpCols - 1) / kSwpCols, 256, 0, h->stream>>>(A, lda, c0, c1, map);
+  launch_dependent(laswp_apply_kernel, dim3((c1 - c0 + kSwpCols - 1) / kSwpCols), dim3(256), 0, h->stream, A, lda, c0, c1, map);
   h->launches++;
   return check_cuda(h, cudaGetLastError(), "laswp");
 }
@@ -1481,7 +1500,7 @@ int trsm_small(emul_handle_t h, double* A, long lda, int d0, int w1, int c0, int
   smem_attr(reinterpret_cast<const void*>(trsm_small_kernel), kTrsmMax * (kTrsmMax | 1) * 8);
   // one column per block: the solve is FP64-bound (about 1.6 FMA per clock per
   // SM), so it is spread over as many SMs as columns; 256 threads stage L
-  trsm_small_kernel<<<w2, 256, static_cast<size_t>(w1) * (w1 | 1) * 8, h->stream>>>(A, lda, d0, w1, c0);
+  launch_dependent(trsm_small_kernel, dim3(w2), dim3(256), static_cast<size_t>(w1) * (w1 | 1) * 8, h->stream, A, lda, d0, w1, c0);
   h->launches++;
   return check_cuda(h, cudaGetLastError(), "panel trsm");
 }
@@ -1522,7 +1541,7 @@ int panel_getrf(emul_handle_t h, double* A, long lda, int n, int j0, int jb, int
   if (rc) return rc;
   rc = laswp(h, A, lda, j0 + w1, j0 + jb, ipiv, j0, j0 + w1, B.map);
   if (rc) return rc;
-  trtri_cols_kernel<true><<<w1, trtri_threads(w1), 0, h->stream>>>(A, lda, j0, w1, B.inv, nullptr);
+  launch_dependent(trtri_cols_kernel<true>, dim3(w1), dim3(trtri_threads(w1)), 0, h->stream, A, lda, j0, w1, B.inv, nullptr);
   h->launches++;
   rc = check_cuda(h, cudaGetLastError(), "panel trtri");
   if (rc) return rc;
@@ -2016,7 +2035,7 @@ int emul_dgetrf(emul_handle_t h, int n, double* A, int lda, int32_t* ipiv, int n
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_start, h->stream), "stream events");
       if (!rc) rc = emul::check_cuda(h, cudaStreamWaitEvent(h->aux, h->aux_start, 0), "stream events");
       if (rc) return rc;
-      emul::trtri_cols_kernel<true><<<jb, emul::trtri_threads(jb), 0, h->aux>>>(A, lda, j0, jb, B.inv, nullptr);
+      emul::launch_dependent(emul::trtri_cols_kernel<true>, dim3(jb), dim3(emul::trtri_threads(jb)), 0, h->aux, A, lda, j0, jb, B.inv, nullptr);
       h->launches++;
       rc = emul::check_cuda(h, cudaGetLastError(), "trtri");
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_done, h->aux), "stream events");

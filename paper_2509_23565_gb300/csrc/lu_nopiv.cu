@@ -19,6 +19,8 @@
 #include <cuda_runtime.h>
 
 #include "handle.h"
+#include "launch.h"
+#include "ptx.cuh"
 
 namespace emul {
 namespace {
@@ -53,6 +55,8 @@ __device__ __forceinline__ bool np_zero(double x) {
 
 __global__ void __launch_bounds__(32 * kNpWarps, 1) np_leaf_kernel(double* A, long lda, int d, int w, int32_t* info) {
   __shared__ double mult[2][kNpLeaf];
+  grid_launch();
+  grid_wait();
   constexpr int kCols = kNpLeaf / kNpWarps;
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   double* D = A + d + static_cast<long>(d) * lda;
@@ -132,6 +136,8 @@ __global__ void __launch_bounds__(32 * kInvCols) np_inverse_kernel(const double*
                                                                   long ldx, double* Y) {
   __shared__ double S[kNpLeaf][kNpLeaf + 1];      // S[k][i] = (L\U)(i, k)
   __shared__ double rdiag[kNpLeaf];
+  grid_launch();
+  grid_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double* D = A + d + static_cast<long>(d) * lda;
   // sixteen loads in flight per thread
@@ -237,9 +243,9 @@ int np_panel(emul_handle_t h, double* A, long lda, int n, int j0, int d, int w, 
              const NpBufs& B) {
   double* Xd = B.X + (d - j0) + static_cast<long>(d - j0) * B.ldx;
   if (w <= kNpLeaf) {
-    np_leaf_kernel<<<1, 32 * kNpWarps, 0, h->stream>>>(A, lda, d, w, info);
-    np_inverse_kernel<<<dim3((w + kInvCols - 1) / kInvCols, 2), 32 * kInvCols, 0, h->stream>>>(A, lda, d, w, Xd, B.ldx,
-                                                                                              B.Y);
+    launch_dependent(np_leaf_kernel, dim3(1), dim3(32 * kNpWarps), 0, h->stream, A, lda, d, w, info);
+    launch_dependent(np_inverse_kernel, dim3((w + kInvCols - 1) / kInvCols, 2), dim3(32 * kInvCols), 0, h->stream, A,
+                     lda, d, w, Xd, B.ldx, B.Y);
     h->launches += 2;
     int rc = check_cuda(h, cudaGetLastError(), "no-pivot leaf");
     if (rc) return rc;

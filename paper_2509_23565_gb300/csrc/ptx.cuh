@@ -12,6 +12,16 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// ---------------------------------------------------------------- dependent launches
+// A kernel launched with launch_dependent() (launch.h) may start while the one
+// before it in the stream still runs.  grid_wait: until that one has completed
+// and its writes are visible; before any access to memory that others write or
+// read.  grid_launch: lets the next one start (it waits in the same way); a kernel
+// with TMEM calls it once the block's allocation stands, as a block of the next
+// kernel could otherwise take the columns and wait for this one to complete.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));

@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 
 #include "emul_internal.h"
+#include "launch.h"
+#include "ptx.cuh"
 #include "slice.cuh"
 
 namespace emul {
@@ -42,6 +44,8 @@ template <int S, bool KEEP>
 __global__ void __launch_bounds__(kSplitThreads) split_kernel(const SplitArgs a0, const SplitArgs a1) {
   __shared__ uint32_t up_s[kSplitThreads / 32][kSplitRows];
   __shared__ unsigned long long full_s[kSplitRows];
+  grid_launch();
+  grid_wait();
   const bool second = static_cast<int>(blockIdx.x) >= a0.blocks;
   const SplitArgs& a = second ? a1 : a0;
   const int r0 = (static_cast<int>(blockIdx.x) - (second ? a0.blocks : 0)) * kSplitRows;
@@ -58,7 +62,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_kernel(const SplitArgs a0
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int c = 8 * g + j;
-      u[j] = row_ok && c < a.k ? __ldg(row + c * a.cs) : 0ull;
+      u[j] = row_ok && c < a.k ? row[c * a.cs] : 0ull;
     }
   };
   // the maximum over the threads that share a row: lanes 8 and 16 apart, then
@@ -128,10 +132,8 @@ cudaError_t launch_s(cudaStream_t st, const SplitArgs& a, const SplitArgs& b) {
   const int grid = a.blocks + b.blocks;
   const long ldk = a.ldk > b.ldk ? a.ldk : b.ldk;
   if (ldk <= 256)
-    split_kernel<S, true><<<grid, kSplitThreads, 0, st>>>(a, b);
-  else
-    split_kernel<S, false><<<grid, kSplitThreads, 0, st>>>(a, b);
-  return cudaGetLastError();
+    return launch_dependent(split_kernel<S, true>, dim3(grid), dim3(kSplitThreads), 0, st, a, b);
+  return launch_dependent(split_kernel<S, false>, dim3(grid), dim3(kSplitThreads), 0, st, a, b);
 }
 
 SplitArgs make_args(int rows, int k, const double* X, long rs, long cs, int32_t* exps, uint16_t* out, long ldk) {
