@@ -761,7 +761,9 @@ constexpr int kCholLeaf = 32;
 // j = 4s + q (s = 0..7) in registers, so the FP64 work is spread over the
 // SM's four sub-partitions.  Pivot jj: its owner warp takes r = rsqrt(d) of
 // the pivot d, sets L_jj = d r, scales the column by r and publishes it in
-// shared memory (double-buffered).  GB300's FP64 latency makes every dependent
+// shared memory.  A column is published while the owner of the pivot before
+// may still read the column two steps back for its other updates, so the columns
+// go through four buffers in turn.  GB300's FP64 latency makes every dependent
 // FP64 step costly (64 cycles a DFMA, 375 an rsqrt), so the chain from pivot to
 // pivot is kept short: the owner of the next pivot updates that column first,
 // scales and publishes it and arrives at the step's barrier before it updates
@@ -771,7 +773,7 @@ constexpr int kCholLeaf = 32;
 __device__ __noinline__ double chol_rsqrt(double d) { return rsqrt(d); }
 
 __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int d0, int w, int32_t* info) {
-  __shared__ double col[2][kCholLeaf];
+  __shared__ double col[4][kCholLeaf];
   __shared__ int fail_s;       // pivot that failed
   const int i = threadIdx.x & 31, q = threadIdx.x >> 5;
   grid_launch();
@@ -800,7 +802,7 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
       atomicCAS(info, 0, d0 + jj + 1);
       fail_s = jj;
     }
-    col[jj & 1][i] = i >= jj ? x : 0.0;
+    col[jj & 3][i] = i >= jj ? x : 0.0;
     // barriers 1 and 2 in turn; the owner has published and does not wait
     __syncwarp();
     asm volatile("bar.arrive %0, 128;" ::"r"(1 + (jj & 1)) : "memory");
@@ -822,10 +824,10 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
         done = jj;
         break;
       }
-      const double lij = col[jj & 1][i];
+      const double lij = col[jj & 3][i];
       const bool mine = q == ((qq + 1) & 3) && jj + 1 < w;
       if (mine) {
-        const double ln = col[jj & 1][(jj + 1) & 31];
+        const double ln = col[jj & 3][(jj + 1) & 31];
         if (qq < 3) {
           if (i >= jj + 1) d[so] = fma(-lij, ln, d[so]);
           pivot(jj + 1, d[so]);
@@ -839,7 +841,7 @@ __global__ void __launch_bounds__(128) chol_leaf_kernel(double* A, long lda, int
 #pragma unroll
       for (int s = so; s < kCholLeaf / 4; ++s) {
         const int j = 4 * s + q;
-        if ((s > so || q > qq) && i >= j && !(mine && s == snext)) d[s] = fma(-lij, col[jj & 1][j], d[s]);
+        if ((s > so || q > qq) && i >= j && !(mine && s == snext)) d[s] = fma(-lij, col[jj & 3][j], d[s]);
       }
     }
   }

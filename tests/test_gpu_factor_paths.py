@@ -133,6 +133,28 @@ def test_cholesky_failing_pivot(gpu_lib, at):
     assert int(info.item()) == at + 1
 
 
+def test_cholesky_beside_other_work(gpu_lib):
+    """The diagonal blocks' chain on SMs shared with another stream's kernels,
+    which delay its warps against each other: the same bits as alone."""
+    A = inputs.spd(512, 100.0, seed=3)
+    side = torch.cuda.Stream()
+    x = torch.rand((1024, 1024), dtype=torch.float64, device="cuda")
+    want = None
+    for _ in range(8):
+        dA = ColMajor.from_numpy(A)
+        torch.cuda.synchronize()
+        if want is not None:
+            with torch.cuda.stream(side):
+                for _ in range(100):
+                    x.sin_()
+        info = gpu_lib.dpotrf(dA, nb=256, slices=7)
+        torch.cuda.synchronize()
+        assert int(info.item()) == 0
+        got = dA.numpy()
+        want = got if want is None else want
+        assert np.array_equal(got, want)
+
+
 # ---------------------------------------------------------------- no pivoting
 @pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 31, 32, 33, 63, 64, 65, 80, 127, 129, 200])
 @pytest.mark.parametrize("nb", [32, 64, 128])
