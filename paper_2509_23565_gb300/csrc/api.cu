@@ -728,7 +728,8 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
   size_t smem = 0;
   const int stages = gemm_stages(cfg, s, &smem);
   if (stages < 2) return set_error(h, EMUL_NOT_SUPPORTED, "slice tiles do not fit in shared memory");
-  const int units = pair ? h->nsm / 2 : h->nsm;   // CTAs, or CTA pairs
+  const int sms = h->nsm - h->sm_spare;
+  const int units = pair ? sms / 2 : sms;   // CTAs, or CTA pairs
   const int grid = (a.ntiles < units ? a.ntiles : units) * (pair ? 2 : 1);
   emul_handle_s::ProfRec rec{};
   rc = prof_begin(h, &rec, m, n, k, s, t, s_a, s_b, lower, beta, same);
@@ -756,7 +757,7 @@ bool pool_event(emul_handle_t h, cudaEvent_t* ev) {
 }
 }  // namespace
 
-int phase_begin(emul_handle_t h, int kind) {
+int phase_begin(emul_handle_t h, int kind, cudaStream_t st) {
   if (!h->prof) return -1;
   emul_handle_s::PhaseRec r{kind, nullptr, nullptr};
   if (!pool_event(h, &r.e0)) return -1;
@@ -764,14 +765,18 @@ int phase_begin(emul_handle_t h, int kind) {
     h->event_pool.push_back(r.e0);
     return -1;
   }
-  cudaEventRecord(r.e0, h->stream);
+  cudaEventRecord(r.e0, st);
   h->phases.push_back(r);
   return static_cast<int>(h->phases.size()) - 1;
 }
 
-void phase_end(emul_handle_t h, int idx) {
-  if (idx >= 0 && idx < static_cast<int>(h->phases.size())) cudaEventRecord(h->phases[idx].e1, h->stream);
+void phase_end(emul_handle_t h, int idx, cudaStream_t st) {
+  if (idx >= 0 && idx < static_cast<int>(h->phases.size())) cudaEventRecord(h->phases[idx].e1, st);
 }
+
+int phase_begin(emul_handle_t h, int kind) { return phase_begin(h, kind, h->stream); }
+
+void phase_end(emul_handle_t h, int idx) { phase_end(h, idx, h->stream); }
 
 }  // namespace emul
 

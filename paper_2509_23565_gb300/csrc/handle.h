@@ -16,6 +16,7 @@ struct emul_handle_s {
   cudaStream_t stream = nullptr;
   int device = 0;
   int nsm = 0;
+  int sm_spare = 0;                 // SMs the persistent products leave to the second stream
   int* d_status = nullptr;          // device status word written by kernels
   void* ws = nullptr;               // workspace (device)
   size_t ws_bytes = 0;
@@ -46,8 +47,9 @@ struct emul_handle_s {
   std::vector<PhaseRec> phases;
   std::vector<cudaEvent_t> event_pool;
   std::map<uint64_t, int> nb_tuned;  // (kind, n, slices) -> block size chosen by emul_autotune_nb
-  // second stream of the LU step: L11^-1 is formed there while the row
-  // interchanges run on `stream` (created on first use, same device)
+  // second stream (created on first use, same device): an LU step's L11^-1 is
+  // formed there while the row interchanges run on `stream`, a Cholesky step's
+  // next diagonal block is factored there beside the update
   cudaStream_t aux = nullptr;
   cudaEvent_t aux_start = nullptr, aux_done = nullptr;
   void* selector = nullptr;         // emul::SelectorState (selector.cu)
@@ -74,6 +76,8 @@ int reserve_workspace(emul_handle_t h, size_t bytes);
 // event cannot be had), phase_end closes it.
 int phase_begin(emul_handle_t h, int kind);
 void phase_end(emul_handle_t h, int idx);
+int phase_begin(emul_handle_t h, int kind, cudaStream_t st);   // on another stream than the handle's
+void phase_end(emul_handle_t h, int idx, cudaStream_t st);
 // Workspace bytes a product of this shape needs (slices, scales).
 size_t gemm_workspace_bytes(int m, int n, int k, int s, bool same_operand);
 

@@ -15,9 +15,12 @@
 
 namespace emul {
 
+// dependent = false launches the same kernel the plain way: on the second stream,
+// whose kernels with the attribute did not overlap the first stream's (Cholesky at
+// 12000 with its diagonal blocks there 32.8 ms, and 27.3 with plain launches).
 template <typename... Params, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                             Args&&... args) {
+cudaError_t launch_chained(bool dependent, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                           cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -27,8 +30,14 @@ cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, s
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
+template <typename... Params, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             Args&&... args) {
+  return launch_chained(true, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 }  // namespace emul

@@ -1334,27 +1334,31 @@ size_t lu_extra_bytes(int nb, int nsm) {
 // in place, by 32-column panels (chol_leaf_kernel, then the rows below the
 // leaf within the block and the block's trailing lower part by
 // dgemm_nt_small_kernel); with `want_inv`, inv (jb x jb, ld jb) <- L11^-1.
-int chol_diag(emul_handle_t h, double* A, long lda, int d0, int jb, double* inv, int32_t* info, bool want_inv) {
+int chol_diag(emul_handle_t h, double* A, long lda, int d0, int jb, double* inv, int32_t* info, bool want_inv,
+              cudaStream_t st) {
+  const bool dep = st == h->stream;      // launch.h
+  const int ph = phase_begin(h, EMUL_PHASE_PANEL, st);
   for (int c0 = 0; c0 < jb; c0 += kCholLeaf) {
     const int wp = kCholLeaf < jb - c0 ? kCholLeaf : jb - c0;
-    launch_dependent(chol_leaf_kernel, dim3(1), dim3(128), 0, h->stream, A, lda, d0 + c0, wp, info);
+    launch_chained(dep, chol_leaf_kernel, dim3(1), dim3(128), 0, st, A, lda, d0 + c0, wp, info);
     h->launches++;
     const int r0 = c0 + wp, mr = jb - r0;
     if (mr > 0) {
       double* Lp = A + (d0 + r0) + static_cast<long>(d0 + c0) * lda;   // rows below the leaf, its columns
-      launch_dependent(chol_solve_kernel, dim3((mr + kCholSolveRows - 1) / kCholSolveRows), dim3(32 * kCholSolveRows), 0,
-          h->stream, A + (d0 + c0) + static_cast<long>(d0 + c0) * lda, lda, wp, Lp, mr, info);
+      launch_chained(dep, chol_solve_kernel, dim3((mr + kCholSolveRows - 1) / kCholSolveRows), dim3(32 * kCholSolveRows), 0,
+          st, A + (d0 + c0) + static_cast<long>(d0 + c0) * lda, lda, wp, Lp, mr, info);
       // A(r0.., r0..) -= L(r0.., c0..) L(r0.., c0..)^T, lower part
-      launch_dependent(dgemm_nt_small_kernel, dim3((mr + kNtRows - 1) / kNtRows, (mr + 31) / 32), dim3(32 * kNtRows), 0,
-          h->stream, mr, mr, wp, -1.0, Lp, 1, lda, Lp, 1, lda, 1.0, A + (d0 + r0) + static_cast<long>(d0 + r0) * lda, lda, 1,
+      launch_chained(dep, dgemm_nt_small_kernel, dim3((mr + kNtRows - 1) / kNtRows, (mr + 31) / 32), dim3(32 * kNtRows), 0,
+          st, mr, mr, wp, -1.0, Lp, 1, lda, Lp, 1, lda, 1.0, A + (d0 + r0) + static_cast<long>(d0 + r0) * lda, lda, 1,
           info);
       h->launches += 2;
     }
   }
   if (want_inv) {
-    launch_dependent(trtri_cols_kernel<false>, dim3(jb), dim3(trtri_threads(jb)), 0, h->stream, A, lda, d0, jb, inv, info);
+    launch_chained(dep, trtri_cols_kernel<false>, dim3(jb), dim3(trtri_threads(jb)), 0, st, A, lda, d0, jb, inv, info);
     h->launches++;
   }
+  phase_end(h, ph, st);
   return check_cuda(h, cudaGetLastError(), "Cholesky diagonal block");
 }
 
@@ -1904,9 +1908,64 @@ uint64_t nb_key(int kind, int n, int slices) {
 // The LU step's second stream and its two events, created on first use.
 int aux_ready(emul_handle_t h) {
   if (h->aux) return EMUL_OK;
-  int rc = check_cuda(h, cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking), "second stream");
+  int least = 0, greatest = 0;
+  int rc = check_cuda(h, cudaDeviceGetStreamPriorityRange(&least, &greatest), "second stream");
+  if (!rc) rc = check_cuda(h, cudaStreamCreateWithPriority(&h->aux, cudaStreamNonBlocking, greatest), "second stream");
   if (!rc) rc = check_cuda(h, cudaEventCreateWithFlags(&h->aux_start, cudaEventDisableTiming), "stream events");
   if (!rc) rc = check_cuda(h, cudaEventCreateWithFlags(&h->aux_done, cudaEventDisableTiming), "stream events");
+  return rc;
+}
+
+// The columns right of the factored Cholesky block at j0 (jb wide, m2 rows below
+// it): L21 = A21 L11^-T, then A22 -= L21 L21^T on the lower triangle.  With
+// enough left the next diagonal block is updated first and factored on the second
+// stream, while the rest of the update runs on `stream` (*ahead is set; aux_done
+// marks its end): the diagonal block is a chain of small kernels, 330 us at 256
+// columns, that leaves the chip idle.  The persistent products leave it a few SMs.
+// ms of dpotrf without / with it: n = 12000, nb = 256: 30.4 / 27.2; 16384, 512:
+// 64.8 / 59.1; 8192, 128: 17.3 / 15.8; 5000, 256: 8.03 / 7.86.  The lines: with it
+// down to 1024 rows right of the next block 5000, 128 takes 8.38 instead of 8.23
+// and 8192, 256 14.99 instead of 14.91, only above 6000 rows 15.6; at 4000 rows in
+// all 6.05 / 6.2, and with 64 columns, whose updates are bound by memory,
+// 16384 104.2 / 106.4.  Of 8, 16 and 24 SMs: 27.5, 27.5, 27.8 at 12000, 256; 16384,
+// 512 60.2 (8), 59.1 (16); 16384, 128 63.3 (8), 65.2 (16).
+constexpr int kAheadRows = 3072;
+constexpr int kAheadCols = 128;
+int chol_trailing(emul_handle_t h, double* A, long lda, int j0, int jb, int m2, int nb, int s, int32_t* info,
+                  const LuBufs& B, bool* ahead) {
+  auto at = [&](int r, int c) { return A + r + static_cast<long>(c) * lda; };
+  // A(r.., c..) (m x w) -= L21(r..) L21(c..)^T
+  auto update = [&](int r, int c, int m, int w, bool lower) {
+    const int ph = phase_begin(h, EMUL_PHASE_UPDATE);
+    const int rc = gemm_run(h, m, w, jb, -1.0, Operand{at(r, j0), 1, lda}, Operand{at(c, j0), 1, lda}, 1.0, at(r, c),
+                            lda, s, lower, 0, nullptr, 0, 0);
+    phase_end(h, ph);
+    return rc;
+  };
+  const int j1 = j0 + jb, jb1 = nb < m2 ? nb : m2;
+  const int j2 = j1 + jb1, m3 = m2 - jb1;
+  // operand B is (L11^-1)^T, whose row j is row j of L11^-1
+  const int ph = phase_begin(h, EMUL_PHASE_U12);
+  int rc = gemm_run(h, m2, jb, jb, 1.0, Operand{at(j1, j0), 1, lda}, Operand{B.inv, 1, jb}, 0.0, at(j1, j0), lda, s,
+                    false, 0, nullptr, 0, 0);
+  phase_end(h, ph);
+  if (rc) return rc;
+  if (jb < kAheadCols || m3 < kAheadRows) return update(j1, j1, m2, m2, true);
+  rc = aux_ready(h);
+  if (!rc) rc = update(j1, j1, jb1, jb1, true);
+  if (!rc) rc = check_cuda(h, cudaEventRecord(h->aux_start, h->stream), "stream events");
+  if (!rc) rc = check_cuda(h, cudaStreamWaitEvent(h->aux, h->aux_start, 0), "stream events");
+  if (rc) return rc;
+  rc = chol_diag(h, A, lda, j1, jb1, B.inv, info, true, h->aux);
+  const int rc_done = check_cuda(h, cudaEventRecord(h->aux_done, h->aux), "stream events");
+  if (!rc) rc = rc_done;
+  h->sm_spare = jb >= 256 ? 16 : 8;
+  if (!rc) rc = update(j2, j1, m3, jb1, false);
+  if (!rc) rc = update(j2, j2, m3, m3, true);
+  h->sm_spare = 0;
+  // an error here leaves no work of the second stream behind the call
+  if (rc) cudaStreamWaitEvent(h->stream, h->aux_done, 0);
+  *ahead = rc == EMUL_OK;
   return rc;
 }
 
@@ -2037,7 +2096,8 @@ int emul_dgetrf(emul_handle_t h, int n, double* A, int lda, int32_t* ipiv, int n
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_start, h->stream), "stream events");
       if (!rc) rc = emul::check_cuda(h, cudaStreamWaitEvent(h->aux, h->aux_start, 0), "stream events");
       if (rc) return rc;
-      emul::launch_dependent(emul::trtri_cols_kernel<true>, dim3(jb), dim3(emul::trtri_threads(jb)), 0, h->aux, A, lda, j0, jb, B.inv, nullptr);
+      emul::launch_chained(false, emul::trtri_cols_kernel<true>, dim3(jb), dim3(emul::trtri_threads(jb)), 0, h->aux, A, lda,
+                           j0, jb, B.inv, nullptr);
       h->launches++;
       rc = emul::check_cuda(h, cudaGetLastError(), "trtri");
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_done, h->aux), "stream events");
@@ -2208,31 +2268,19 @@ int emul_dpotrf(emul_handle_t h, char uplo, int n, double* A, int lda, int nb, i
   rc = emul::reserve_workspace(h, gw + emul::lu_extra_bytes(nb, h->nsm));
   if (rc) return rc;
   const emul::LuBufs B = emul::carve(h, gw, nb);
-  for (int j0 = 0; j0 < n; j0 += nb) {
+  bool ahead = false;       // block j0 was factored on the second stream
+  for (int j0 = 0; j0 < n && !rc; j0 += nb) {
     const int jb = nb < n - j0 ? nb : n - j0;
     const int m2 = n - j0 - jb;
-    int ph = emul::phase_begin(h, EMUL_PHASE_PANEL);
-    rc = emul::chol_diag(h, A, lda, j0, jb, B.inv, info, m2 > 0);
-    emul::phase_end(h, ph);
-    if (rc) return rc;
-    if (m2 > 0) {
-      double* A21 = A + (j0 + jb) + static_cast<long>(j0) * lda;
-      // L21 = A21 L11^-T: operand B is (L11^-1)^T, whose row j is row j of L11^-1
-      ph = emul::phase_begin(h, EMUL_PHASE_U12);
-      rc = emul::gemm_run(h, m2, jb, jb, 1.0, Operand{A21, 1, lda}, Operand{B.inv, 1, jb}, 0.0, A21, lda, slices,
-                          false, 0, nullptr, 0, 0);
-      emul::phase_end(h, ph);
-      if (rc) return rc;
-      // A22 -= L21 L21^T on the lower triangle; one slice set for both operands
-      ph = emul::phase_begin(h, EMUL_PHASE_UPDATE);
-      rc = emul::gemm_run(h, m2, m2, jb, -1.0, Operand{A21, 1, lda}, Operand{A21, 1, lda}, 1.0,
-                          A + (j0 + jb) + static_cast<long>(j0 + jb) * lda, lda, slices, true, 0, nullptr, 0, 0);
-      emul::phase_end(h, ph);
-      if (rc) return rc;
-    }
+    if (ahead)
+      rc = emul::check_cuda(h, cudaStreamWaitEvent(h->stream, h->aux_done, 0), "stream events");
+    else
+      rc = emul::chol_diag(h, A, lda, j0, jb, B.inv, info, m2 > 0, h->stream);
+    ahead = false;
+    if (!rc && m2 > 0) rc = emul::chol_trailing(h, A, lda, j0, jb, m2, nb, slices, info, B, &ahead);
     if (stats) stats->steps++;
   }
-  return EMUL_OK;
+  return rc;
 }
 
 int emul_dpotrs(emul_handle_t h, char uplo, int n, int nrhs, const double* L, int lda, double* B, int ldb) {

@@ -155,6 +155,23 @@ def test_cholesky_beside_other_work(gpu_lib):
         assert np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("n,nb,k", [(6100, 256, 2816), (5000, 128, 2944), (7000, 512, 3072)])
+def test_cholesky_ahead_agrees(gpu_lib, n, nb, k):
+    """Diagonal blocks factored beside the update (more than 3072 rows right of
+    the next block) against the leading submatrix, which has fewer: the leading
+    columns' blocks, and so their bits, are the same."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    M = torch.rand((n, n), generator=g, dtype=torch.float64, device="cuda")
+    M = M + M.T + 2.0 * n * torch.eye(n, dtype=torch.float64, device="cuda")
+    small = ColMajor(M[:k, :k].clone(), k, k)
+    big = ColMajor(M, n, n)
+    info, sinfo = gpu_lib.dpotrf(big, nb=nb, slices=7), gpu_lib.dpotrf(small, nb=nb, slices=7)
+    gpu_lib.sync_status()
+    assert int(info.item()) == 0 and int(sinfo.item()) == 0
+    assert torch.equal(big.store[:k, :k], small.store)
+
+
 # ---------------------------------------------------------------- no pivoting
 @pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 31, 32, 33, 63, 64, 65, 80, 127, 129, 200])
 @pytest.mark.parametrize("nb", [32, 64, 128])
