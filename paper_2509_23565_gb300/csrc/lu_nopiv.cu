@@ -25,7 +25,7 @@
 namespace emul {
 namespace {
 
-constexpr int kNpLeaf = 64;           // widest diagonal block factored in one CTA
+constexpr int kNpLeaf = 64;           // widest diagonal block factored in one launch
 constexpr int kNpWarps = 8;           // the leaf's warps, columns dealt round
 constexpr int kNpChunk = 1024;        // K of one emulated product in the Schur updates
 constexpr size_t kNpAl = 256;
@@ -37,100 +37,164 @@ inline size_t np_al(size_t x) { return (x + kNpAl - 1) / kNpAl * kNpAl; }
 // unscaled and records its 1-based index in *info unless an earlier one is
 // there.
 //
-// One CTA: FP64 retires 1.68 FMA per clock per SM, a warp's DFMA occupies its
+// FP64 retires 1.68 FMA per clock per SM, a warp's DFMA occupies its
 // sub-partition for 64-76 cycles and a division takes 560, so what counts is the
-// chain from pivot to pivot and that no FP64 instruction is wasted.  Eight warps
-// hold the block in registers, warp g the columns g, g + 8, ... with rows i and
-// i + 32 in lane i, so a pivot column lies in one warp: its owner updates it
-// first, takes the reciprocal, scales, publishes the multipliers in shared
-// memory and arrives at the step's barrier before it updates its other columns;
-// the other warps meet it there after theirs.  The pivot row comes by shuffles.
-// (64 x 64 with both inverses took 256 us in one CTA of 1024 threads on shared
-// memory with two barriers a step and the division after the update.)
+// chain from pivot to pivot and that no FP64 instruction is wasted.  np_factor:
+// eight warps of a CTA hold 32 columns in registers, warp g the columns g, g + 8,
+// ..., rows across the lanes, so a pivot column lies in one warp: its owner
+// updates it first, takes the reciprocal, scales, publishes the multipliers in
+// shared memory (a place of its own for each pivot) and arrives at the step's
+// barrier before it updates its other columns; the other warps meet it there after
+// theirs.  The pivot row comes by shuffles.
+//
+// The left 32 columns and then the lower right 32 x 32 are factored that way by
+// CTA 0 of a cluster.  In between the right 32 columns take the left ones'
+// pivots on all eight CTAs, a warp per column, with the multipliers and the
+// results carried through distributed shared memory: on one SM these updates kept
+// its FP64 units busy for 1000 to 2000 cycles a pivot, twice the chain's length
+// (57 us for 64 x 64 that way, 47 here).  Every entry sees the same operations in the
+// same order as in a plain right-looking elimination.
 __device__ __noinline__ double np_recip(double p) { return 1.0 / p; }
 // x == 0 by the bits (an FP64 comparison would take a DFMA's 64 cycles)
 __device__ __forceinline__ bool np_zero(double x) {
   return (static_cast<unsigned long long>(__double_as_longlong(x)) << 1) == 0;
 }
 
-__global__ void __launch_bounds__(32 * kNpWarps, 1) np_leaf_kernel(double* A, long lda, int d, int w, int32_t* info) {
-  __shared__ double mult[2][kNpLeaf];
-  grid_launch();
-  grid_wait();
-  constexpr int kCols = kNpLeaf / kNpWarps;
-  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-  double* D = A + d + static_cast<long>(d) * lda;
-  // beyond w the block is the identity: nothing there changes or is stored
-  double v[kCols][2];
-#pragma unroll
-  for (int s = 0; s < kCols; ++s)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = lane + 32 * h, j = g + kNpWarps * s;
-      v[s][h] = i < w && j < w ? D[i + static_cast<long>(j) * lda] : (i == j ? 1.0 : 0.0);
-    }
-  // multipliers of pivot k from its column (in registers c0, c1 of the owner)
-  auto scale = [&](int k, double& c0, double& c1) {
-    const double p = __shfl_sync(0xFFFFFFFFu, k < 32 ? c0 : c1, k & 31);
+constexpr int kNpHalf = kNpLeaf / 2;
+constexpr int kNpCluster = 8;                              // CTAs of a leaf
+constexpr int kNpRight = kNpHalf / kNpCluster;             // right columns of each
+constexpr int kNpCols = kNpHalf / kNpWarps;
+
+// Factors the 32 H x 32 columns v (v[s][h]: row lane + 32 h of column g + 8 s), of
+// which the leading w count; pivot k's multipliers go to M[k].  `first` is the
+// global index of the first pivot.
+template <int H>
+__device__ __forceinline__ void np_factor(double (&v)[kNpCols][H], int g, int lane, int w, double (*M)[kNpLeaf],
+                                          int first, int32_t* info) {
+  // multipliers of pivot k from its column (in registers c of the owner)
+  auto scale = [&](int k, double (&c)[H]) {
+    const double p = __shfl_sync(0xFFFFFFFFu, c[0], k);
     const double r = np_zero(p) ? 0.0 : np_recip(p);
-    if (np_zero(p) && lane == 0) atomicCAS(info, 0, d + k + 1);
+    if (np_zero(p) && lane == 0) atomicCAS(info, 0, first + k + 1);
     if (!np_zero(r)) {
-      if (lane > k) c0 *= r;
-      if (lane + 32 > k) c1 *= r;
+      if (lane > k) c[0] *= r;
+      if (H == 2) c[H - 1] *= r;
     }
-    mult[k & 1][lane] = lane > k ? c0 : 0.0;
-    mult[k & 1][lane + 32] = lane + 32 > k ? c1 : 0.0;
+    M[k][lane] = lane > k ? c[0] : 0.0;
+    if (H == 2) M[k][lane + 32] = c[H - 1];
     // barriers 1 and 2 in turn; the owner has published and does not wait
     __syncwarp();
     if (k + 1 < w) asm volatile("bar.arrive %0, %1;" ::"r"(1 + (k & 1)), "n"(32 * kNpWarps) : "memory");
   };
-  if (g == 0) scale(0, v[0][0], v[0][1]);
-  // pivots k = 8 so + kk; the inner loop stays rolled (64 copies of a step would
+  if (g == 0) scale(0, v[0]);
+  // pivots k = 8 so + kk; the inner loop stays rolled (32 copies of a step would
   // run from the instruction cache's misses)
 #pragma unroll
-  for (int so = 0; so < kCols; ++so) {
+  for (int so = 0; so < kNpCols; ++so) {
 #pragma unroll 1
     for (int kk = 0; kk < kNpWarps; ++kk) {
       const int k = kNpWarps * so + kk;
       if (k + 1 >= w) break;
       if (g != kk) asm volatile("bar.sync %0, %1;" ::"r"(1 + (k & 1)), "n"(32 * kNpWarps) : "memory");
-      const double l0 = mult[k & 1][lane], l1 = mult[k & 1][lane + 32];
-      auto update = [&](double& c0, double& c1) {
-        const double u = __shfl_sync(0xFFFFFFFFu, so < kCols / 2 ? c0 : c1, k & 31);
-        if (so < kCols / 2 && lane > k) c0 = fma(-l0, u, c0);
-        if (lane + 32 > k) c1 = fma(-l1, u, c1);
+      const double l0 = M[k][lane], l1 = H == 2 ? M[k][lane + 32] : 0.0;
+      auto update = [&](double (&c)[H]) {
+        const double u = __shfl_sync(0xFFFFFFFFu, c[0], k);
+        if (lane > k) c[0] = fma(-l0, u, c[0]);
+        if (H == 2) c[H - 1] = fma(-l1, u, c[H - 1]);
       };
       // the next pivot's column first, and its multipliers
       const bool mine = g == (kk + 1) % kNpWarps;
       if (mine) {
         if (kk + 1 < kNpWarps) {
-          update(v[so][0], v[so][1]);
-          scale(k + 1, v[so][0], v[so][1]);
-        } else if (so + 1 < kCols) {
-          update(v[so + 1 < kCols ? so + 1 : so][0], v[so + 1 < kCols ? so + 1 : so][1]);
-          scale(k + 1, v[so + 1 < kCols ? so + 1 : so][0], v[so + 1 < kCols ? so + 1 : so][1]);
+          update(v[so]);
+          scale(k + 1, v[so]);
+        } else if (so + 1 < kNpCols) {
+          update(v[so + 1 < kNpCols ? so + 1 : so]);
+          scale(k + 1, v[so + 1 < kNpCols ? so + 1 : so]);
         }
       }
       const int snext = kk + 1 < kNpWarps ? so : so + 1;
 #pragma unroll
-      for (int s = so; s < kCols; ++s)
-        if ((s > so || g > kk) && !(mine && s == snext)) update(v[s][0], v[s][1]);
+      for (int s = so; s < kNpCols; ++s)
+        if ((s > so || g > kk) && !(mine && s == snext)) update(v[s]);
     }
   }
+}
+
+__global__ void __cluster_dims__(kNpCluster, 1, 1) __launch_bounds__(32 * kNpWarps, 1)
+    np_leaf_kernel(double* A, long lda, int d, int w, int32_t* info) {
+  __shared__ double M[kNpHalf][kNpLeaf];       // multipliers of the left columns' pivots
+  __shared__ double S[kNpHalf][kNpHalf];       // CTA 0: S[j][i], the lower right block
+  grid_launch();
+  grid_wait();
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int b = static_cast<int>(cluster_rank());
+  if (w <= kNpHalf && b != 0) return;          // (no cluster barrier then)
+  double* D = A + d + static_cast<long>(d) * lda;
+  // beyond w the block is the identity: nothing there changes or is stored
+  auto load = [&](int i, int j) { return i < w && j < w ? D[i + static_cast<long>(j) * lda] : (i == j ? 1.0 : 0.0); };
+  const int jr = kNpHalf + kNpRight * b + g;   // this warp's right column
+  double c0 = 0.0, c1 = 0.0;
+  if (w > kNpHalf && g < kNpRight) {
+    c0 = load(lane, jr);
+    c1 = load(lane + 32, jr);
+  }
+  if (b == 0) {
+    double v[kNpCols][2];
 #pragma unroll
-  for (int s = 0; s < kCols; ++s)
+    for (int s = 0; s < kNpCols; ++s)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = lane + 32 * h, j = g + kNpWarps * s;
-      if (i < w && j < w) D[i + static_cast<long>(j) * lda] = v[s][h];
+      for (int h = 0; h < 2; ++h) v[s][h] = load(lane + 32 * h, g + kNpWarps * s);
+    np_factor<2>(v, g, lane, w < kNpHalf ? w : kNpHalf, M, d, info);
+#pragma unroll
+    for (int s = 0; s < kNpCols; ++s)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = lane + 32 * h, j = g + kNpWarps * s;
+        if (i < w && j < w) D[i + static_cast<long>(j) * lda] = v[s][h];
+      }
+  }
+  if (w <= kNpHalf) return;
+  cluster_sync();                              // CTA 0's multipliers stand
+  if (b != 0) {
+    const uint32_t from = mapa_addr(smem_u32(&M[0][0]), 0) + 8u * threadIdx.x;
+    constexpr int kEach = kNpHalf * kNpLeaf / (32 * kNpWarps);
+    double x[kEach];
+#pragma unroll
+    for (int q = 0; q < kEach; ++q) x[q] = ld_cluster_f64(from + 8u * 32 * kNpWarps * q);
+#pragma unroll
+    for (int q = 0; q < kEach; ++q) (&M[0][0])[threadIdx.x + 32 * kNpWarps * q] = x[q];
+    __syncthreads();
+  }
+  if (g < kNpRight) {
+#pragma unroll 4
+    for (int k = 0; k < kNpHalf; ++k) {
+      const double u = __shfl_sync(0xFFFFFFFFu, c0, k);
+      if (lane > k) c0 = fma(-M[k][lane], u, c0);
+      c1 = fma(-M[k][lane + 32], u, c1);
     }
+    if (jr < w) D[lane + static_cast<long>(jr) * lda] = c0;
+    st_cluster_f64(mapa_addr(smem_u32(&S[jr - kNpHalf][lane]), 0), c1);
+  }
+  cluster_sync();                              // the lower right block stands in CTA 0
+  if (b != 0) return;
+  double v[kNpCols][1];
+#pragma unroll
+  for (int s = 0; s < kNpCols; ++s) v[s][0] = S[g + kNpWarps * s][lane];
+  np_factor<1>(v, g, lane, w - kNpHalf, M, d + kNpHalf, info);
+#pragma unroll
+  for (int s = 0; s < kNpCols; ++s) {
+    const int i = kNpHalf + lane, j = kNpHalf + g + kNpWarps * s;
+    if (i < w && j < w) D[i + static_cast<long>(j) * lda] = v[s][0];
+  }
 }
 
 // Inverses of the leaf's factors: X <- L^-1 (ld ldx, zeros above the diagonal)
 // and Y <- U^-1 (ld w, zeros below; an infinite reciprocal for a zero pivot).
 // One warp per column of X or Y and four columns per block, so every warp has a
-// sub-partition's FP64 unit to itself: a step is a shuffle and one or two DFMAs.  Row k of a column, once final, is broadcast; column j of X
-// starts at row j, of Y at row j and goes up.
+// sub-partition's FP64 unit to itself: a step is a shuffle and one or two DFMAs.
+// Row k of a column, once final, is broadcast; column j of X starts at row j, of Y
+// at row j and goes up.
 constexpr int kInvCols = 4;
 __global__ void __launch_bounds__(32 * kInvCols) np_inverse_kernel(const double* A, long lda, int d, int w, double* X,
                                                                   long ldx, double* Y) {
@@ -243,7 +307,7 @@ int np_panel(emul_handle_t h, double* A, long lda, int n, int j0, int d, int w, 
              const NpBufs& B) {
   double* Xd = B.X + (d - j0) + static_cast<long>(d - j0) * B.ldx;
   if (w <= kNpLeaf) {
-    launch_dependent(np_leaf_kernel, dim3(1), dim3(32 * kNpWarps), 0, h->stream, A, lda, d, w, info);
+    launch_dependent(np_leaf_kernel, dim3(kNpCluster), dim3(32 * kNpWarps), 0, h->stream, A, lda, d, w, info);
     launch_dependent(np_inverse_kernel, dim3((w + kInvCols - 1) / kInvCols, 2), dim3(32 * kInvCols), 0, h->stream, A,
                      lda, d, w, Xd, B.ldx, B.Y);
     h->launches += 2;

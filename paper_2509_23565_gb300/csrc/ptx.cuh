@@ -184,6 +184,15 @@ __device__ __forceinline__ uint32_t mapa_addr(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
+// Plain accesses to a CTA's shared memory in the cluster (ordered by cluster_sync).
+__device__ __forceinline__ double ld_cluster_f64(uint32_t addr_cl) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr_cl) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_cluster_f64(uint32_t addr_cl, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr_cl), "d"(v) : "memory");
+}
 // Store 8 bytes into a CTA of the cluster and count them on a barrier there.
 __device__ __forceinline__ void st_async_b64(uint32_t addr_cl, uint64_t v, uint32_t bar_cl) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr_cl), "l"(v),
