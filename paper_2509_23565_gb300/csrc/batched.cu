@@ -9,10 +9,10 @@
 //      FP32 panel (pivot = first largest |a|), FP32 triangular solve for U12,
 //      trailing update A22 -= L21 U12 emulated with s INT8 slices: per-row /
 //      per-column power-of-two scales, slices of 7 bits, slice pairs with
-//      p + q <= s + 1 as exact INT8 x INT8 -> INT32 products on the tensor
-//      cores (warp-level mma.sync m16n8k32 tiles: one system per block does
-//      not fill a 128-wide tcgen05 tile), recombination in FP64, then the
-//      FP32 working copy rounded once;
+//      p + q <= s + 1 as exact integer sums on the tensor cores (warp-level
+//      mma.sync tiles, FP16 carriers with FP32 sums or INT8 with INT32: one
+//      system per block does not fill a 128-wide tcgen05 tile), the exact sum
+//      of the levels subtracted and the FP32 working copy rounded once;
 //   2. x0 from the FP32 factors; then until the backward error
 //      ||b - A x|| / (||A|| ||x|| n 2^-53) <= target or max_iter: r = b - A x
 //      in FP64 with the original A, d from the FP32 factors, x += d.
@@ -357,7 +357,8 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
 //    otherwise (FP64 runs at 1.68 lanes per clock per SM, its conversions below 1).
 // In factor_general every step strides through global memory (U12 by columns
 // apart, full-row interchanges per pivot), and 152 such systems at once overflow
-// L2: 1024 systems of 64..1024 rows took 247 ms.
+// L2: 1024 systems of 64..1024 rows took 165 to 297 ms (by how many of the large
+// ones were refactored with 8 slices), and take 37 to 46.
 constexpr int kFastN = 2 * kBThreads;
 constexpr int kFastNb = 32;
 constexpr int kFastSmem = 200 * 1024;      // digits and staged columns
@@ -888,7 +889,10 @@ __device__ __noinline__ void factor_fast(const BatchSys& sys, Scratch& sc, int* 
 __device__ __noinline__ void factor_system(const BatchSys& sys, int s, Scratch& sc, int* info, float* sv, int* si, FastShared& F,
                               uint8_t* dyn) {
   // the slice counts and blocks the tuner chooses from, and the 8 slices of a
-  // system whose refinement stalls
+  // system whose refinement stalls.  152 systems at once, one per SM, without
+  // refinement (ms): n = 1024 14.2 at 3 slices, 15.7 at 4, 29.3 at 8 (20.4 with
+  // blocks of 16); n = 1025, where the panel outgrows two rows per thread and takes
+  // the general path, 128.7, 139.3 and 281.
   if (sys.n <= kFastN && (s == 3 || s == 4 || s == 8) && (sys.nb == 16 || sys.nb == 32)) {
     if (sys.nb == 32) {
       if (s == 3) return factor_fast<3, 32>(sys, sc, info, F, dyn);

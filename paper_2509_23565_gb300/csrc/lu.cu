@@ -5,15 +5,17 @@
 // LU step (right-looking, block nb):
 //   1. panel [A11; A21] factored with partial pivoting: recursive halving; the
 //      inner Schur updates use the emulated product, the leaves (<= 32 columns)
-//      run a cooperative multi-block FP64 kernel (pivot search on the IEEE bit
-//      patterns, one bounded grid barrier per column);
+//      run an FP64 kernel over many blocks (pivot search on the IEEE bit
+//      patterns, one bounded exchange per column: through a cluster's shared
+//      memory, or through L2 above 2048 rows);
 //   2. the panel's row interchanges applied to the columns left and right of it;
 //   3. U12 = L11^-1 A12: L11^-1 formed in FP64 (unit lower, nb x nb), the
 //      product by the emulated GEMM;
 //   4. A22 <- A22 - L21 U12 by the emulated GEMM (alpha = -1, beta = 1).
 // Cholesky step (lower): FP64 diagonal block, L21 = A21 L11^-T through an FP64
 // L11^-1 and the emulated GEMM, then A22 <- A22 - L21 L21^T on lower tiles only,
-// with one slice set serving both operands.
+// with one slice set serving both operands; the next diagonal block is factored
+// beside the update where that is long enough.
 #include <cmath>
 #include <cstdio>
 #include <map>
@@ -414,6 +416,11 @@ __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, lon
 // are spread over up to 16 SMs.  The arithmetic is that of getf2_leaf_kernel,
 // operation for operation.
 //
+// A leaf of 32 columns takes 58 us (26 with few rows, 69 with 2048), the same
+// leaf through L2 93 to 102 at any height.  128 rows per CTA at most: with 256 the
+// rank-1 update of a column (2400 cycles of FP64 on average) would no longer hide
+// behind the exchange.
+//
 // Buffers are double-buffered by column parity: a CTA sends column c + 2 only
 // after it has received column c + 1 from every CTA, which each sends after it
 // has used column c.
@@ -718,6 +725,8 @@ __global__ void __launch_bounds__(256) laswp_apply_kernel(double* A, long lda, i
 // dst[i] receives the original row src[i], a permutation of the touched rows)
 // changes only the rows r = H[dst[i]]: G[r] = src[i], H[src[i]] = r.
 __global__ void iota2_kernel(int n, int* G, int* H) {
+  grid_launch();
+  grid_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     G[i] = i;
     H[i] = i;
@@ -726,6 +735,8 @@ __global__ void iota2_kernel(int n, int* G, int* H) {
 
 __global__ void compose_kernel(const int* map, int* G, int* H) {
   __shared__ int rr[2 * kPermMax];
+  grid_launch();
+  grid_wait();
   const int cnt = map[4 * kPermMax];
   for (int i = threadIdx.x; i < cnt; i += blockDim.x) rr[i] = H[map[i]];
   __syncthreads();
@@ -738,6 +749,8 @@ __global__ void compose_kernel(const int* map, int* G, int* H) {
 
 // tmp[(r - r0) + c (n - r0)] = A[G[r], c0 + c] for r in [r0, n); blockIdx.y = c.
 __global__ void gather_rows_kernel(const double* A, long lda, int r0, int n, int c0, const int* G, double* tmp) {
+  grid_launch();
+  grid_wait();
   const int r = r0 + blockIdx.x * blockDim.x + threadIdx.x;
   const int c = blockIdx.y;
   if (r < n) tmp[(r - r0) + static_cast<long>(c) * (n - r0)] = A[G[r] + static_cast<long>(c0 + c) * lda];
@@ -768,7 +781,8 @@ constexpr int kCholLeaf = 32;
 // pivot is kept short: the owner of the next pivot updates that column first,
 // scales and publishes it and arrives at the step's barrier before it updates
 // its other columns, and each pivot takes one reciprocal square root rather than
-// a square root and a division.  A non-positive pivot sets *info (first index)
+// a square root and a division.  21 us (48 with a barrier for all after the updates
+// and the block's inverse formed as well).  A non-positive pivot sets *info (first index)
 // and stops; nothing runs once *info is set.
 __device__ __noinline__ double chol_rsqrt(double d) { return rsqrt(d); }
 
@@ -929,8 +943,8 @@ __global__ void __launch_bounds__(32 * kNtRows) dgemm_nt_small_kernel(int m, int
 // hand takes eight steps by shuffles (a DFMA of 64 cycles each, another
 // multiplication for the non-unit scaling) and publishes the eight values, which
 // the warps below take off their rows in the next round; a thread reads row i of
-// the next eight columns of L meanwhile (coalesced along the columns).  (One
-// block-wide barrier per step: 52 us at nb = 256, 54 us with the scaling.)
+// the next eight columns of L meanwhile (coalesced along the columns).  30 us at
+// nb = 256, 39 us with the scaling (one block-wide barrier per step: 52 and 54).
 template <bool UNIT>
 __global__ void __launch_bounds__(512) trtri_cols_kernel(const double* A, long lda, int d0, int nb, double* inv,
                                                         const int32_t* info) {
@@ -1086,6 +1100,8 @@ __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long 
                                                           int bs, int lower, int unit, int trans) {
   extern __shared__ double tb[];   // tb[r + c*(bs+1)] = op(T)(d0+r, d0+c)
   __shared__ double x[128], rcp[128];
+  grid_launch();
+  grid_wait();
   const int ld = bs + 1;
   double* xc = X + static_cast<long>(blockIdx.x) * ldx + d0;
   {
@@ -1121,17 +1137,17 @@ __device__ __forceinline__ double row_dot(const double* t, long ldt, const doubl
   const int full = n / 16 * 16;
   double v[16];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) v[q] = full ? __ldg(t + q * ldt) : 0.0;
+  for (int q = 0; q < 16; ++q) v[q] = full ? t[q * ldt] : 0.0;
   for (int c = 0; c < full; c += 16) {
     double nx[16];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) nx[q] = c + 16 < full ? __ldg(t + (c + 16 + q) * ldt) : 0.0;
+    for (int q = 0; q < 16; ++q) nx[q] = c + 16 < full ? t[(c + 16 + q) * ldt] : 0.0;
 #pragma unroll
     for (int q = 0; q < 16; ++q) acc = fma(v[q], x[c + q], acc);
 #pragma unroll
     for (int q = 0; q < 16; ++q) v[q] = nx[q];
   }
-  for (int c = full; c < n; ++c) acc = fma(__ldg(t + c * ldt), x[c], acc);
+  for (int c = full; c < n; ++c) acc = fma(t[c * ldt], x[c], acc);
   return acc;
 }
 
@@ -1140,6 +1156,8 @@ __device__ __forceinline__ double row_dot(const double* t, long ldt, const doubl
 __global__ void gemv_update_kernel(const double* T, long ldt, double* X, long ldx, int r0, int r1, int c0, int bs,
                                    int trans) {
   __shared__ double xs[128];
+  grid_launch();
+  grid_wait();
   double* xc = X + static_cast<long>(blockIdx.y) * ldx;
   if (threadIdx.x < bs) xs[threadIdx.x] = xc[c0 + threadIdx.x];
   __syncthreads();
@@ -1345,17 +1363,19 @@ int chol_diag(emul_handle_t h, double* A, long lda, int d0, int jb, double* inv,
     const int r0 = c0 + wp, mr = jb - r0;
     if (mr > 0) {
       double* Lp = A + (d0 + r0) + static_cast<long>(d0 + c0) * lda;   // rows below the leaf, its columns
-      launch_chained(dep, chol_solve_kernel, dim3((mr + kCholSolveRows - 1) / kCholSolveRows), dim3(32 * kCholSolveRows), 0,
-          st, A + (d0 + c0) + static_cast<long>(d0 + c0) * lda, lda, wp, Lp, mr, info);
+      launch_chained(dep, chol_solve_kernel, dim3((mr + kCholSolveRows - 1) / kCholSolveRows),
+                     dim3(32 * kCholSolveRows), 0, st, A + (d0 + c0) + static_cast<long>(d0 + c0) * lda, lda, wp, Lp,
+                     mr, info);
       // A(r0.., r0..) -= L(r0.., c0..) L(r0.., c0..)^T, lower part
-      launch_chained(dep, dgemm_nt_small_kernel, dim3((mr + kNtRows - 1) / kNtRows, (mr + 31) / 32), dim3(32 * kNtRows), 0,
-          st, mr, mr, wp, -1.0, Lp, 1, lda, Lp, 1, lda, 1.0, A + (d0 + r0) + static_cast<long>(d0 + r0) * lda, lda, 1,
-          info);
+      launch_chained(dep, dgemm_nt_small_kernel, dim3((mr + kNtRows - 1) / kNtRows, (mr + 31) / 32),
+                     dim3(32 * kNtRows), 0, st, mr, mr, wp, -1.0, Lp, 1, lda, Lp, 1, lda, 1.0,
+                     A + (d0 + r0) + static_cast<long>(d0 + r0) * lda, lda, 1, info);
       h->launches += 2;
     }
   }
   if (want_inv) {
-    launch_chained(dep, trtri_cols_kernel<false>, dim3(jb), dim3(trtri_threads(jb)), 0, st, A, lda, d0, jb, inv, info);
+    launch_chained(dep, trtri_cols_kernel<false>, dim3(jb), dim3(trtri_threads(jb)), 0, st, A, lda, d0, jb, inv,
+                   info);
     h->launches++;
   }
   phase_end(h, ph, st);
@@ -1482,7 +1502,8 @@ int laswp_prepare(emul_handle_t h, const int32_t* ipiv, int k1, int k2, int* map
 // Apply a prepared gather map to columns [c0, c1).
 int laswp_apply(emul_handle_t h, double* A, long lda, int c0, int c1, const int* map) {
   if (c1 <= c0) return EMUL_OK;
-  launch_dependent(laswp_apply_kernel, dim3((c1 - c0 + kSwpCols - 1) / kSwpCols), dim3(256), 0, h->stream, A, lda, c0, c1, map);
+  launch_dependent(laswp_apply_kernel, dim3((c1 - c0 + kSwpCols - 1) / kSwpCols), dim3(256), 0, h->stream, A, lda, c0,
+                   c1, map);
   h->launches++;
   return check_cuda(h, cudaGetLastError(), "laswp");
 }
@@ -1506,7 +1527,8 @@ int trsm_small(emul_handle_t h, double* A, long lda, int d0, int w1, int c0, int
   smem_attr(reinterpret_cast<const void*>(trsm_small_kernel), kTrsmMax * (kTrsmMax | 1) * 8);
   // one column per block: the solve is FP64-bound (about 1.6 FMA per clock per
   // SM), so it is spread over as many SMs as columns; 256 threads stage L
-  launch_dependent(trsm_small_kernel, dim3(w2), dim3(256), static_cast<size_t>(w1) * (w1 | 1) * 8, h->stream, A, lda, d0, w1, c0);
+  launch_dependent(trsm_small_kernel, dim3(w2), dim3(256), static_cast<size_t>(w1) * (w1 | 1) * 8, h->stream, A, lda,
+                   d0, w1, c0);
   h->launches++;
   return check_cuda(h, cudaGetLastError(), "panel trsm");
 }
@@ -1547,7 +1569,8 @@ int panel_getrf(emul_handle_t h, double* A, long lda, int n, int j0, int jb, int
   if (rc) return rc;
   rc = laswp(h, A, lda, j0 + w1, j0 + jb, ipiv, j0, j0 + w1, B.map);
   if (rc) return rc;
-  launch_dependent(trtri_cols_kernel<true>, dim3(w1), dim3(trtri_threads(w1)), 0, h->stream, A, lda, j0, w1, B.inv, nullptr);
+  launch_dependent(trtri_cols_kernel<true>, dim3(w1), dim3(trtri_threads(w1)), 0, h->stream, A, lda, j0, w1, B.inv,
+                   nullptr);
   h->launches++;
   rc = check_cuda(h, cudaGetLastError(), "panel trtri");
   if (rc) return rc;
@@ -1853,18 +1876,21 @@ int getrs_body(emul_handle_t h, int n, int nrhs, const double* LU, int lda, cons
   constexpr int bs = 128;  // diagonal blocks of the substitution
   for (int d0 = 0; d0 < n; d0 += bs) {
     const int b = bs < n - d0 ? bs : n - d0;
-    trsv_block_kernel<<<nrhs, 1024, b * (b + 1) * sizeof(double), h->stream>>>(LU, lda, B, ldb, d0, b, 1, 1, 0);
+    launch_dependent(trsv_block_kernel, dim3(nrhs), dim3(1024), b * (b + 1) * sizeof(double), h->stream, LU, lda, B,
+                     ldb, d0, b, 1, 1, 0);
     h->launches += (d0 + b < n) ? 2 : 1;
     if (d0 + b < n)
-      gemv_update_kernel<<<dim3((n - d0 - b + 255) / 256, nrhs), 256, 0, h->stream>>>(LU, lda, B, ldb, d0 + b,
-                                                                                               n, d0, b, 0);
+      launch_dependent(gemv_update_kernel, dim3((n - d0 - b + 255) / 256, nrhs), dim3(256), 0, h->stream, LU, lda, B,
+                       ldb, d0 + b, n, d0, b, 0);
   }
   for (int d0 = ((n - 1) / bs) * bs; d0 >= 0; d0 -= bs) {
     const int b = bs < n - d0 ? bs : n - d0;
-    trsv_block_kernel<<<nrhs, 1024, b * (b + 1) * sizeof(double), h->stream>>>(LU, lda, B, ldb, d0, b, 0, 0, 0);
+    launch_dependent(trsv_block_kernel, dim3(nrhs), dim3(1024), b * (b + 1) * sizeof(double), h->stream, LU, lda, B,
+                     ldb, d0, b, 0, 0, 0);
     h->launches += (d0 > 0) ? 2 : 1;
     if (d0 > 0)
-      gemv_update_kernel<<<dim3((d0 + 255) / 256, nrhs), 256, 0, h->stream>>>(LU, lda, B, ldb, 0, d0, d0, b, 0);
+      launch_dependent(gemv_update_kernel, dim3((d0 + 255) / 256, nrhs), dim3(256), 0, h->stream, LU, lda, B, ldb, 0,
+                       d0, d0, b, 0);
   }
   return check_cuda(h, cudaGetLastError(), "getrs");
 }
@@ -2096,8 +2122,8 @@ int emul_dgetrf(emul_handle_t h, int n, double* A, int lda, int32_t* ipiv, int n
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_start, h->stream), "stream events");
       if (!rc) rc = emul::check_cuda(h, cudaStreamWaitEvent(h->aux, h->aux_start, 0), "stream events");
       if (rc) return rc;
-      emul::launch_chained(false, emul::trtri_cols_kernel<true>, dim3(jb), dim3(emul::trtri_threads(jb)), 0, h->aux, A, lda,
-                           j0, jb, B.inv, nullptr);
+      emul::launch_chained(false, emul::trtri_cols_kernel<true>, dim3(jb), dim3(emul::trtri_threads(jb)), 0, h->aux,
+                           A, lda, j0, jb, B.inv, nullptr);
       h->launches++;
       rc = emul::check_cuda(h, cudaGetLastError(), "trtri");
       if (!rc) rc = emul::check_cuda(h, cudaEventRecord(h->aux_done, h->aux), "stream events");
@@ -2210,18 +2236,19 @@ int emul_dgetrf(emul_handle_t h, int n, double* A, int lda, int32_t* ipiv, int n
     int* G = reinterpret_cast<int*>(static_cast<uint8_t*>(h->ws) + def_off);
     int* H = G + n;
     double* tmp = reinterpret_cast<double*>(static_cast<uint8_t*>(h->ws) + def_off + emul::al(8ull * n));
-    emul::iota2_kernel<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, h->stream>>>(n, G, H);
+    emul::launch_dependent(emul::iota2_kernel, dim3((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024), dim3(256), 0,
+                           h->stream, n, G, H);
     h->launches++;
     for (int k = K - 2; k >= 0; --k) {
       const int r0 = (k + 1) * nb, r1 = r0 + nb < n ? r0 + nb : n;
       // panel k+1's interchanges, composed from its last gather map back
       for (int c = (r1 - r0 - 1) / emul::kPermMax; c >= 0; --c) {
-        emul::compose_kernel<<<1, 512, 0, h->stream>>>(maps + static_cast<size_t>((k + 1) * cpp + c) * emul::kMapInts,
-                                                       G, H);
+        emul::launch_dependent(emul::compose_kernel, dim3(1), dim3(512), 0, h->stream,
+                               maps + static_cast<size_t>((k + 1) * cpp + c) * emul::kMapInts, G, H);
         h->launches++;
       }
-      emul::gather_rows_kernel<<<dim3((n - r0 + 255) / 256, nb), 256, 0, h->stream>>>(A, lda, r0, n, k * nb, G,
-                                                                                         tmp);
+      emul::launch_dependent(emul::gather_rows_kernel, dim3((n - r0 + 255) / 256, nb), dim3(256), 0, h->stream, A,
+                             lda, r0, n, k * nb, G, tmp);
       h->launches++;
       rc = emul::check_cuda(h,
                             cudaMemcpy2DAsync(A + r0 + static_cast<long>(k) * nb * lda, static_cast<size_t>(lda) * 8,
@@ -2316,18 +2343,21 @@ int emul_dpotrs(emul_handle_t h, char uplo, int n, int nrhs, const double* L, in
   constexpr int bs = 128;
   for (int d0 = 0; d0 < n; d0 += bs) {
     const int b = bs < n - d0 ? bs : n - d0;
-    emul::trsv_block_kernel<<<nrhs, 1024, b * (b + 1) * sizeof(double), h->stream>>>(L, lda, B, ldb, d0, b, 1, 0, 0);
+    emul::launch_dependent(emul::trsv_block_kernel, dim3(nrhs), dim3(1024), b * (b + 1) * sizeof(double), h->stream,
+                           L, lda, B, ldb, d0, b, 1, 0, 0);
     h->launches += (d0 + b < n) ? 2 : 1;
     if (d0 + b < n)
-      emul::gemv_update_kernel<<<dim3((n - d0 - b + 255) / 256, nrhs), 256, 0, h->stream>>>(L, lda, B, ldb, d0 + b,
-                                                                                               n, d0, b, 0);
+      emul::launch_dependent(emul::gemv_update_kernel, dim3((n - d0 - b + 255) / 256, nrhs), dim3(256), 0, h->stream,
+                             L, lda, B, ldb, d0 + b, n, d0, b, 0);
   }
   for (int d0 = ((n - 1) / bs) * bs; d0 >= 0; d0 -= bs) {
     const int b = bs < n - d0 ? bs : n - d0;
-    emul::trsv_block_kernel<<<nrhs, 1024, b * (b + 1) * sizeof(double), h->stream>>>(L, lda, B, ldb, d0, b, 0, 0, 1);
+    emul::launch_dependent(emul::trsv_block_kernel, dim3(nrhs), dim3(1024), b * (b + 1) * sizeof(double), h->stream,
+                           L, lda, B, ldb, d0, b, 0, 0, 1);
     h->launches += (d0 > 0) ? 2 : 1;
     if (d0 > 0)
-      emul::gemv_update_kernel<<<dim3((d0 + 7) / 8, nrhs), 256, 0, h->stream>>>(L, lda, B, ldb, 0, d0, d0, b, 1);
+      emul::launch_dependent(emul::gemv_update_kernel, dim3((d0 + 7) / 8, nrhs), dim3(256), 0, h->stream, L, lda, B,
+                             ldb, 0, d0, d0, b, 1);
   }
   emul::phase_end(h, ph);
   return emul::check_cuda(h, cudaGetLastError(), "potrs");
