@@ -115,32 +115,60 @@ __device__ double block_max_d(double v, double* red) {
   return t;
 }
 
+// Values of one thread that are loaded together: none of the loads may be moved
+// down to its value's use.
+__device__ __forceinline__ void loaded(float (&l)[32]) {
+#pragma unroll
+  for (int k = 0; k < 32; k += 8)
+    asm volatile("" : "+f"(l[k]), "+f"(l[k + 1]), "+f"(l[k + 2]), "+f"(l[k + 3]), "+f"(l[k + 4]), "+f"(l[k + 5]),
+                      "+f"(l[k + 6]), "+f"(l[k + 7]));
+}
+
 // Solve (LU) y = d in FP32 in place on d (shared memory, length n, rows already
 // interchanged): unit lower, then upper, by blocks of 32 rows: one warp solves a
 // block (row per lane, values by shuffle), then every thread takes the block's 32
 // columns off its own rows, 32 loads in flight.  Each entry sees the operations
-// of the column-by-column substitution in the same order.
-__device__ void lu_solve_f32(const float* W, int n, float* d) {
+// of the column-by-column substitution in the same order.  All threads fetch the
+// next diagonal block meanwhile (dg: two of 32 x 32 in shared memory, by columns).
+// With the solving warp loading it, each load came just before its use or its
+// spill, 32 trips to L2 in a row: 2.1 million cycles for n = 1000, 0.81 now.
+__device__ __noinline__ void lu_solve_f32(const float* W, int n, float* d, float* dg) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int nblk = (n + 31) / 32;
+  auto first_row = [&](int st) { return 32 * (st < nblk ? st : 2 * nblk - 1 - st); };
+  constexpr int kEach = 32 * 32 / kBThreads;
+  float nx[kEach];                            // this thread's part of the next diagonal block
+  auto load_diag = [&](int st) {
+    const int k0 = first_row(st), w = n - k0 < 32 ? n - k0 : 32;
+#pragma unroll
+    for (int q = 0; q < kEach; ++q) {
+      const int e = tid + q * kBThreads, r = e & 31, k = e >> 5;
+      nx[q] = r < w && k < w ? W[(k0 + r) + static_cast<long>(k0 + k) * n] : 0.f;
+    }
+  };
+  auto store_diag = [&](int st) {
+#pragma unroll
+    for (int q = 0; q < kEach; ++q) dg[(st & 1) * 1024 + tid + q * kBThreads] = nx[q];
+  };
+  load_diag(0);
+  store_diag(0);
+  __syncthreads();
   for (int st = 0; st < 2 * nblk; ++st) {
     const bool lower = st < nblk;
-    const int k0 = 32 * (lower ? st : 2 * nblk - 1 - st);
+    const int k0 = first_row(st);
     const int w = n - k0 < 32 ? n - k0 : 32;
-    const float* B = W + k0 + static_cast<long>(k0) * n;      // the diagonal block
+    if (st + 1 < 2 * nblk) load_diag(st + 1);
     if (tid < 32) {
+      const float* B = dg + (st & 1) * 1024 + lane;          // B[32 k]: column k of row k0 + lane
       float v = lane < w ? d[k0 + lane] : 0.f;
-      float l[32];
-#pragma unroll
-      for (int k = 0; k < 32; ++k) l[k] = k < w && lane < w ? B[lane + static_cast<long>(k) * n] : 0.f;
       if (lower) {
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
           const float dk = __shfl_sync(0xFFFFFFFFu, v, k);
-          if (lane > k && k < w) v = fmaf(-l[k], dk, v);
+          if (lane > k && k < w) v = fmaf(-B[32 * k], dk, v);
         }
       } else {
-        const float diag = lane < w ? B[lane + static_cast<long>(lane) * n] : 1.f;
+        const float diag = lane < w ? B[32 * lane] : 1.f;
 #pragma unroll
         for (int k = 31; k >= 0; --k) {
           if (k >= w) continue;
@@ -148,7 +176,7 @@ __device__ void lu_solve_f32(const float* W, int n, float* d) {
           if (lane == k)
             v = dk;
           else if (lane < k)
-            v = fmaf(-l[k], dk, v);
+            v = fmaf(-B[32 * k], dk, v);
         }
       }
       if (lane < w) d[k0 + lane] = v;
@@ -160,6 +188,7 @@ __device__ void lu_solve_f32(const float* W, int n, float* d) {
       float l[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) l[k] = k < w ? p[static_cast<long>(k) * n] : 0.f;
+      loaded(l);
       float v = d[i];
       if (lower) {
 #pragma unroll
@@ -172,6 +201,7 @@ __device__ void lu_solve_f32(const float* W, int n, float* d) {
       }
       d[i] = v;
     }
+    if (st + 1 < 2 * nblk) store_diag(st + 1);
     __syncthreads();
   }
 }
@@ -358,7 +388,7 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
 // In factor_general every step strides through global memory (U12 by columns
 // apart, full-row interchanges per pivot), and 152 such systems at once overflow
 // L2: 1024 systems of 64..1024 rows took 165 to 297 ms (by how many of the large
-// ones were refactored with 8 slices), and take 37 to 46.
+// ones were refactored with 8 slices), and take 24 to 41.
 constexpr int kFastN = 2 * kBThreads;
 constexpr int kFastNb = 32;
 constexpr int kFastSmem = 200 * 1024;      // digits and staged columns
@@ -477,7 +507,7 @@ __device__ __forceinline__ void digits_f16(uint32_t x, uint32_t& h0, uint32_t& h
 }
 __device__ __forceinline__ void mma_f16_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                 uint32_t b0, uint32_t b1) {
-  asm volatile(
+  asm(
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
@@ -535,6 +565,12 @@ __device__ __noinline__ float update_fp64_4(float w, float v0, float v1, float v
   return update_fp64<4>(w, v, e);
 }
 
+__device__ __noinline__ float update_fp64_8(float w, float v0, float v1, float v2, float v3, float v4, float v5, float v6,
+                                            float v7, int e) {
+  const float v[8] = {v0, v1, v2, v3, v4, v5, v6, v7};
+  return update_fp64<8>(w, v, e);
+}
+
 // a + b = s + e exactly (Knuth's two-sum).
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
@@ -552,6 +588,15 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // addition (1.68) and 60 integer operations (64): 1.6 cycles per entry.
 // Anything else (errors that do not add up exactly, scales near FP32's ends,
 // Inf, NaN) goes the FP64 way.
+//
+// With 8 slices W - D spans too many bits to be exact in two floats, but FP32
+// only has to find the float that the FP64 form rounds to.  With M the largest
+// |partial sum|, the two-sums' errors are at most 2^-24 M each, so adding the
+// eight of them in FP32 is wrong by less than 56 2^-48 M; the FP64 form's own four
+// roundings are below 2^-50 M.  Where s + E rounds to the same float with 2^-41 M
+// added and taken off, that float is the answer (rounding is monotonic); the rest,
+// results near a midpoint or small beside M, goes the FP64 way, one entry in 2^17
+// without cancellation.
 template <int S>
 __device__ __forceinline__ float fast_update(float w, const float (&v)[S], int e) {
   if constexpr (S <= 4) {
@@ -580,7 +625,22 @@ __device__ __forceinline__ float fast_update(float w, const float (&v)[S], int e
     else
       return update_fp64_4(w, v[0], v[1], v[2], v[3], e);
   } else {
-    return update_fp64<S>(w, v, e);
+    static_assert(S == 8, "slice counts of the fast factorization");
+    float sc = __int_as_float((e + 113) << 23);
+    float s = w, E = 0.f, M = fabsf(w);
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      float sn, err;
+      two_sum(s, -(v[i] * sc), sn, err);
+      s = sn;
+      E += err;
+      M = fmaxf(M, fabsf(s));
+      sc *= 0.0078125f;
+    }
+    const float d = M * 4.5474735e-13f;                   // 2^-41
+    const float lo = __fadd_rn(s, E - d), hi = __fadd_rn(s, E + d);
+    if (lo == hi && lo != 0.f && fabsf(lo) < 1e38f && M > 1e-30f && static_cast<unsigned>(e + 80) <= 160u) return lo;
+    return update_fp64_8(w, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], e);
   }
 }
 
@@ -831,10 +891,11 @@ __device__ __noinline__ void factor_fast(const BatchSys& sys, Scratch& sc, int* 
               a_fragments(aw[p], h);
             }
 #pragma unroll
-            for (int q = 0; q + p < S; ++q) {                 // planes p + 1 and q + 1: level p + q + 2
+            for (int q = 0; q + p < S; ++q)                   // planes p + 1 and q + 1: level p + q + 2
               mma_f16_16x8x16(acc[p + q], h[0], h[1], h[2], h[3], bh[q][0], bh[q][1]);
+#pragma unroll
+            for (int q = 0; q + p < S; ++q)                   // (one accumulator's MMAs apart)
               mma_f16_16x8x16(acc[p + q], h[4], h[5], h[6], h[7], bh[q][2], bh[q][3]);
-            }
           }
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
@@ -962,9 +1023,11 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
   __shared__ int info_s;
   __shared__ __align__(16) FastShared F;
   extern __shared__ __align__(16) uint8_t dyn[];
-  // while solving: the right-hand side and the solution
+  // while solving: the right-hand side, the solution, diagonal blocks
   float* ds = reinterpret_cast<float*>(dyn);
   double* xs = reinterpret_cast<double*>(dyn + kMaxN * sizeof(float));
+  float* dg = reinterpret_cast<float*>(dyn + kMaxN * (sizeof(float) + sizeof(double)));   // two diagonal blocks
+  static_assert(kMaxN * 12 + 2 * 32 * 32 * 4 <= kFastSmem, "shared memory of the solve");
   uint8_t* base = scratch + per_block * blockIdx.x;
   Scratch sc;
   {
@@ -1007,7 +1070,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
     // x0 from the FP32 factors
     for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(S.b[sc.perm[i]]);
     __syncthreads();
-    lu_solve_f32(sc.W, n, ds);
+    lu_solve_f32(sc.W, n, ds, dg);
     for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = static_cast<double>(ds[i]);
     __syncthreads();
     double berr = INFINITY;
@@ -1041,7 +1104,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
         __syncthreads();
         for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(S.b[sc.perm[i]]);
         __syncthreads();
-        lu_solve_f32(sc.W, n, ds);
+        lu_solve_f32(sc.W, n, ds, dg);
         for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = static_cast<double>(ds[i]);
         __syncthreads();
         continue;
@@ -1050,7 +1113,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
       const double sr = rmax > 0.0 ? rmax : 1.0;
       for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(sc.r[sc.perm[i]] / sr);
       __syncthreads();
-      lu_solve_f32(sc.W, n, ds);
+      lu_solve_f32(sc.W, n, ds, dg);
       for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] += static_cast<double>(ds[i]) * sr;
       __syncthreads();
     }
