@@ -358,7 +358,8 @@ typedef struct emul_profile {
  * UPDATE the trailing update A22 - L21 U12 (slicing, product, selector probe),
  * SOLVE  emul_dgetrs.
  * emul_dpotrf / emul_dpotrs use the same slots: PANEL the diagonal block
- * (L11 and L11^-1), U12 the product L21 = A21 L11^-T, UPDATE the lower
+ * (L11 and L11^-1; beside the update where that is long, so the phases may
+ * overlap), U12 the product L21 = A21 L11^-T, UPDATE the lower
  * trailing update A22 - L21 L21^T, SOLVE emul_dpotrs. */
 #define EMUL_PHASE_PANEL 0
 #define EMUL_PHASE_SWAP 1

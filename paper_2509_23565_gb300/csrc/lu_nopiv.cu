@@ -278,11 +278,9 @@ struct NpBufs {
 };
 
 // C <- beta C + alpha A B as consecutive emulated products over K chunks of at
-// most kNpChunk (each rounded once; C must not overlap A or B).  A wider K
-// would need level 2 in more than one accumulator job (1040 products of
-// 127^2 per FP32 accumulator), which the 128-column product cannot take: it
-// would fall back to 64-column tiles at half the rate; C is read and written
-// once per chunk instead.
+// most kNpChunk (each rounded once, which is part of the result; C must not overlap
+// A or B).  Up to 1024 level 2 is one accumulator job (1040 products of 127^2 per
+// FP32 accumulator); C is read and written once per chunk.
 int gemm_kchunks(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Operand B, double beta, double* C,
                  long ldc, int s) {
   for (int c0 = 0; c0 < k; c0 += kNpChunk) {
