@@ -388,7 +388,7 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
 // In factor_general every step strides through global memory (U12 by columns
 // apart, full-row interchanges per pivot), and 152 such systems at once overflow
 // L2: 1024 systems of 64..1024 rows took 165 to 297 ms (by how many of the large
-// ones were refactored with 8 slices), and take 24 to 41.
+// ones were refactored with 8 slices), and take 20 to 42.
 constexpr int kFastN = 2 * kBThreads;
 constexpr int kFastNb = 32;
 constexpr int kFastSmem = 200 * 1024;      // digits and staged columns
