@@ -249,6 +249,7 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
       float gv;
       int p;
       block_argmax(bv, bi, sv, si, gv, p);
+      if (p == 0x7FFFFFFF) p = c;             // NaN in every row: no candidate, no interchange
       if (threadIdx.x == 0) sc.piv[c] = p;
       if (p != c)
         for (int j = threadIdx.x; j < n; j += blockDim.x) {
