@@ -99,14 +99,22 @@ __device__ void block_argmax(float v, int idx, float* sv, int* si, float& bv, in
   __syncthreads();
 }
 
+// The larger in magnitude; NaN if either is NaN (fmax would drop it, and a
+// residual of NaN would pass for zero).  Without their signs the bit patterns
+// are ordered like the magnitudes, NaN above all.
+__device__ __forceinline__ double max_mag(double a, double b) {
+  const uint64_t x = static_cast<uint64_t>(__double_as_longlong(a)), y = static_cast<uint64_t>(__double_as_longlong(b));
+  return x << 1 > y << 1 ? a : b;
+}
+
 __device__ double block_max_d(double v, double* red) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+  for (int o = 16; o > 0; o >>= 1) v = max_mag(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kBThreads / 32; ++i) t = fmax(t, red[i]);
+    for (int i = 0; i < kBThreads / 32; ++i) t = max_mag(t, red[i]);
     red[0] = t;
   }
   __syncthreads();
@@ -1065,7 +1073,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
     for (int i = threadIdx.x; i < n; i += 2 * blockDim.x) {
       double rs[2] = {0.0, 0.0};
       row_pass(S.A, S.lda, n, i, rs, [](double acc, double a, int) { return acc + fabs(a); });
-      an = fmax(an, fmax(rs[0], rs[1]));
+      an = max_mag(an, max_mag(rs[0], rs[1]));
     }
     an = block_max_d(an, red);
     // x0 from the FP32 factors
@@ -1085,12 +1093,12 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
         double acc[2] = {S.b[i], i1 < n ? S.b[i1] : 0.0};
         row_pass(S.A, S.lda, n, i, acc, [&](double v, double a, int j) { return fma(-a, xs[j], v); });
         sc.r[i] = acc[0];
-        rmax = fmax(rmax, fabs(acc[0]));
-        xmax = fmax(xmax, fabs(xs[i]));
+        rmax = max_mag(rmax, fabs(acc[0]));
+        xmax = max_mag(xmax, fabs(xs[i]));
         if (i1 < n) {
           sc.r[i1] = acc[1];
-          rmax = fmax(rmax, fabs(acc[1]));
-          xmax = fmax(xmax, fabs(xs[i1]));
+          rmax = max_mag(rmax, fabs(acc[1]));
+          xmax = max_mag(xmax, fabs(xs[i1]));
         }
       }
       rmax = block_max_d(rmax, red);

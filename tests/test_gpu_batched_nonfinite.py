@@ -46,3 +46,17 @@ def test_no_pivot_candidate(gpu_lib, n, nb, slices, what):
     torch.cuda.synchronize()
     assert np.array_equal(beside.numpy(), alone.numpy())
     assert int(info[1].item()) == 0 and float(berr[1].item()) <= 1.0
+
+
+@pytest.mark.parametrize("n,nb,slices", [(40, 32, 3), (100, 64, 3), (1040, 32, 3), (700, 16, 4)])
+def test_nan_solution_has_no_backward_error(gpu_lib, n, nb, slices):
+    """NaN in the top right corner of a triangular matrix reaches the first entries
+    of x only, and through them every residual: the backward error is NaN, not
+    that of the finite entries."""
+    A = np.triu(inputs.uniform(n, n, seed=n)) / n + 4.0 * np.eye(n)
+    A[0, n - 1] = np.nan
+    x = ColMajor.from_numpy(inputs.vector(n, seed=3))
+    _, berr, _ = gpu_lib.dgesv_batched_ir([ColMajor.from_numpy(A)], [x], nb=nb, slices=slices)
+    torch.cuda.synchronize()
+    assert np.isnan(x.numpy()[0, 0]) and np.isfinite(x.numpy()[n - 1, 0])
+    assert np.isnan(float(berr[0].item()))
