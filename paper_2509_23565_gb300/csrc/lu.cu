@@ -994,21 +994,45 @@ __global__ void __launch_bounds__(512) trtri_cols_kernel(const double* A, long l
   if (i < nb) inv[i + static_cast<long>(j) * nb] = res;
 }
 
+// How diag_solve forms x_k = v / d from its row's value v and the diagonal entry d.
+enum Diag {
+  kUnit = 0,    // d = 1
+  kRecip = 1,   // v r with r = RN(1 / d): two roundings
+  kQuot = 2     // v r + v (1 / d - r): one rounding
+};
+// 2^lo <= |x| < 2^hi, by the upper word alone (lo >= -1022).
+__device__ __forceinline__ bool in_window(double x, int lo, int hi) {
+  const uint32_t h = static_cast<uint32_t>(__double2hiint(x)) & 0x7FFFFFFFu;
+  return h - (static_cast<uint32_t>(lo + 1023) << 20) < (static_cast<uint32_t>(hi - lo) << 20);
+}
+// Diagonal entries whose reciprocal is normal (kRecip).  Outside, 1 / d is infinite,
+// or subnormal and short of bits, where v / d may be an ordinary number.
+__device__ __forceinline__ bool recip_ok(double d) { return in_window(d, -1022, 1022); }
+// Diagonal entries and values of kQuot: every product is then normal.
+__device__ __forceinline__ bool quot_ok(double x) { return in_window(x, -400, 400); }
+__device__ __forceinline__ bool is_zero(double x) { return ((__double2hiint(x) & 0x7FFFFFFF) | __double2loint(x)) == 0; }
+
 // x <- T^-1 x for the bs x bs (bs <= 128) triangle T(i, k) = tb[i + k*ld] in
 // shared memory, by the first 128 threads of a block (thread i holds x_i; x in
-// shared memory, in and out).  `scale`: non-unit diagonal, rcp[k] = 1 / T(k, k).
-// A chain of bs steps, each a shuffle and a DFMA of 64 cycles (and a
-// multiplication with the reciprocal); a warp solves its 32 rows and publishes
+// shared memory, in and out).  rcp[k] = RN(1 / T(k, k)), rest[k] (kQuot) what it
+// leaves of 1 / T(k, k).  False in a thread whose value lies outside the window of
+// kQuot: x is then to be solved again by diag_solve_divide.
+// A chain of bs steps, each a shuffle and a DFMA of 64 cycles, and one or two more
+// for kRecip and kQuot (a division takes 560); a warp solves its 32 rows and publishes
 // every 8 values, and the warps behind it take those off their own rows
 // meanwhile, on their own FP64 units (one warp with four rows per lane took four
 // DFMAs, 76 cycles each, into every step).  Each entry takes its updates in the
-// order of the steps.
-template <bool LOWER, bool SCALE>
-__device__ __forceinline__ void diag_solve_t(const double* tb, int ld, const double* rcp, int bs, double* x) {
+// order of the steps.  kQuot: r and its rest together are 1 / d to 2^-105, so the
+// quotient is that of a division unless it lies within 2^-104 of the middle of two
+// doubles.
+template <bool LOWER, int DIAG>
+__device__ __forceinline__ bool diag_solve(const double* tb, int ld, const double* rcp, const double* rest, int bs,
+                                             double* x) {
   const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
   double v = i < bs ? x[i] : 0.0;
-  const double r = SCALE && i < bs ? rcp[i] : 1.0;
-  double res = 0.0;
+  const double r = (DIAG == kRecip || DIAG == kQuot) && i < bs ? rcp[i] : 1.0;
+  const double rl = DIAG == kQuot && i < bs ? rest[i] : 0.0;
+  double res = 0.0, last = 0.0;        // x_i, and the value it was formed from
 #pragma unroll 1
   for (int s = LOWER ? 0 : 16 - (bs + 7) / 8; s < 16; ++s) {
     // sub-step s: rows 8 ss .. 8 ss + 7, from the top (LOWER) or the bottom
@@ -1038,21 +1062,36 @@ __device__ __forceinline__ void diag_solve_t(const double* tb, int ld, const dou
         const int kl = (8 * ss + (LOWER ? q : 7 - q)) & 31;       // the step's lane; lanes past bs hold zeros
         // the step's row is final: its value is kept aside (v of a finished row,
         // updated with a zero from here on, may meet an infinity)
-        const double xv = SCALE ? v * r : v;
-        if (lane == kl) res = xv;
+        const double xv = DIAG == kUnit ? v : DIAG == kRecip ? v * r : fma(v, r, v * rl);
+        if (lane == kl) {
+          res = xv;
+          if (DIAG == kQuot) last = v;
+        }
         v = fma(-t[q], __shfl_sync(0xFFFFFFFFu, xv, kl), v);
       }
-      if (lane >> 3 == (ss & 3) && i < bs) x[i] = res;
+      if (lane >> 3 == (ss & 3) && i < bs) {
+        // (v r + v rest would be +0 for terms of unlike signs)
+        if (DIAG == kQuot && is_zero(last))
+          res = __hiloint2double((__double2hiint(last) ^ __double2hiint(r)) & 0x80000000, 0);
+        x[i] = res;
+      }
     }
     asm volatile("bar.sync 1, 128;" ::: "memory");
   }
+  return DIAG != kQuot || i >= bs || is_zero(last) || quot_ok(last);
 }
-__device__ __forceinline__ void diag_solve(const double* tb, int ld, const double* rcp, int bs, bool lower, bool scale,
-                                           double* x) {
-  if (lower)
-    scale ? diag_solve_t<true, true>(tb, ld, rcp, bs, x) : diag_solve_t<true, false>(tb, ld, rcp, bs, x);
-  else
-    scale ? diag_solve_t<false, true>(tb, ld, rcp, bs, x) : diag_solve_t<false, false>(tb, ld, rcp, bs, x);
+// The same by a division per step, for the few blocks that need it: little
+// code, as what is beside the other variants in a kernel costs them registers.
+__device__ __forceinline__ void diag_solve_divide(const double* tb, int ld, int bs, bool lower, double* x) {
+  const int i = threadIdx.x;
+  double v = i < bs ? x[i] : 0.0;
+#pragma unroll 1
+  for (int s = 0; s < bs; ++s) {
+    const int k = lower ? s : bs - 1 - s;
+    if (i == k) x[k] = v / tb[k + k * ld];
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (i < bs && (lower ? i > k : i < k)) v = fma(-tb[i + k * ld], x[k], v);
+  }
 }
 
 // X (w1 x w2 at A[d0.., c0..]) <- L^-1 X with L unit lower w1 x w1 at A[d0.., d0..]
@@ -1086,20 +1125,26 @@ __global__ void __launch_bounds__(256) trsm_small_kernel(double* A, long lda, in
   }
   __syncthreads();
   if (tid >= 128) return;
-  diag_solve(Ls, ld, nullptr, w1, true, false, x);
+  diag_solve<true, kUnit>(Ls, ld, nullptr, nullptr, w1, x);
   if (tid < w1) col[tid] = x[tid];
 }
 
 // One diagonal block of a triangular solve, x <- op(T)^-1 x for the bs x bs
 // block at T[d0.., d0..] (bs <= 128; op = transpose with `trans`).  All
 // threads stage the block (leading dimension bs + 1: conflict-free either
-// way, transposed with `trans`), then the first 128 solve (diag_solve, with the
-// reciprocals of the diagonal: a division on the chain takes 560 cycles a step).
+// way, transposed with `trans`), then the first 128 solve (diag_solve: quotients
+// by the diagonal's reciprocals in two parts, or by divisions throughout where an
+// entry of the block's diagonal or a value lies outside their window).  dpotrs
+// with two right-hand sides at n = 128 (two blocks) takes 59 us, 136 with divisions
+// throughout and 47 with x_k = v RN(1 / d), whose second rounding shows: the error of
+// a substitution with 200 rows is then 1 to 7 % larger.
 // blockIdx.x = right-hand side.
 __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long ldt, double* X, long ldx, int d0,
                                                           int bs, int lower, int unit, int trans) {
   extern __shared__ double tb[];   // tb[r + c*(bs+1)] = op(T)(d0+r, d0+c)
-  __shared__ double x[128], rcp[128];
+  __shared__ double x[128], rcp[128], rest[128];
+  __shared__ int odd_s;            // a value outside the window of kQuot
+  if (threadIdx.x == 0) odd_s = 0;
   grid_launch();
   grid_wait();
   const int ld = bs + 1;
@@ -1123,10 +1168,31 @@ __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long 
   }
   if (static_cast<int>(threadIdx.x) < bs) x[threadIdx.x] = xc[threadIdx.x];
   __syncthreads();
+  bool odd = false;
+  if (!unit && static_cast<int>(threadIdx.x) < bs) {
+    const double d = tb[threadIdx.x + threadIdx.x * ld], r = 1.0 / d;
+    rcp[threadIdx.x] = r;
+    rest[threadIdx.x] = fma(-d, r, 1.0) * r;
+    odd = !quot_ok(d);
+  }
+  odd = __syncthreads_or(odd);
   if (threadIdx.x >= 128) return;
-  if (!unit && static_cast<int>(threadIdx.x) < bs) rcp[threadIdx.x] = 1.0 / tb[threadIdx.x + threadIdx.x * ld];
-  asm volatile("bar.sync 1, 128;" ::: "memory");
-  diag_solve(tb, ld, rcp, bs, lower != 0, unit == 0, x);
+  if (unit) {                        // (a lower triangle)
+    diag_solve<true, kUnit>(tb, ld, nullptr, nullptr, bs, x);
+  } else {
+    if (!odd) {
+      odd = !(lower ? diag_solve<true, kQuot>(tb, ld, rcp, rest, bs, x)
+                    : diag_solve<false, kQuot>(tb, ld, rcp, rest, bs, x));
+      if (odd) odd_s = 1;
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      odd = odd_s;
+      if (odd) {
+        if (static_cast<int>(threadIdx.x) < bs) x[threadIdx.x] = xc[threadIdx.x];
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+      }
+    }
+    if (odd) diag_solve_divide(tb, ld, bs, lower != 0, x);
+  }
   if (static_cast<int>(threadIdx.x) < bs) xc[threadIdx.x] = x[threadIdx.x];
 }
 
@@ -1673,8 +1739,9 @@ __device__ bool solve_sync(unsigned long long* cnt, unsigned long long target, l
 // (chol = false): the block as stored, rcp = 1/diag for the upper (backward)
 // solve.  Cholesky factor (chol = true): the forward solve uses L itself and
 // the backward solve L^T, so the block is staged transposed there; rcp = 1/diag
-// for both.
-__device__ void solve_stage(const double* LU, long lda, int d0, int bs, bool lower, double* tb, double* rcp,
+// for both.  True (in every thread) if some reciprocal is not normal: the block is
+// then solved with divisions.
+__device__ bool solve_stage(const double* LU, long lda, int d0, int bs, bool lower, double* tb, double* rcp,
                             bool chol) {
   constexpr int ld = kSolveBs + 1;
   const int tid = threadIdx.x;
@@ -1695,17 +1762,24 @@ __device__ void solve_stage(const double* LU, long lda, int d0, int bs, bool low
       }
     }
   __syncthreads();
-  if ((chol || !lower) && tid < bs) rcp[tid] = 1.0 / tb[tid + tid * ld];
-  __syncthreads();
+  bool odd = false;
+  if ((chol || !lower) && tid < bs) {
+    const double d = tb[tid + tid * ld];
+    rcp[tid] = 1.0 / d;
+    odd = !recip_ok(d);
+  }
+  return __syncthreads_or(odd);
 }
 
 // CHOL = false: A = L U from the LU (unit L below the diagonal, U on and
 // above it).  CHOL = true: A = L L^T from the lower Cholesky factor, forward
 // with L (non-unit diagonal) and backward with L^T, whose rows are columns of
 // L: the update of the rows above a block then reads each column of L
-// contiguously, one warp per row of L^T.
+// contiguously, one warp per row of L^T.  (One block per SM by its shared memory;
+// without the bound's 1 the LU solve is compiled for 64 registers, with spills:
+// n = 4001 1.66 ms instead of 1.55.)
 template <bool CHOL>
-__global__ void __launch_bounds__(256) getrs1_kernel(const double* LU, long lda, int n, double* x,
+__global__ void __launch_bounds__(256, 1) getrs1_kernel(const double* LU, long lda, int n, double* x,
                                                      unsigned long long* cnt, int* status, long long limit) {
   extern __shared__ double tb[];   // kSolveBs x (kSolveBs + 1) staging of a diagonal block
   __shared__ double xs[kSolveBs], xd[kSolveBs];
@@ -1722,12 +1796,13 @@ __global__ void __launch_bounds__(256) getrs1_kernel(const double* LU, long lda,
   };
   unsigned long long target = 0;
   int staged = -1;   // step whose diagonal block this block holds in tb
+  bool odd = false;  // it is solved with divisions
   auto stage = [&](int st) {
     if (st >= nsteps || staged == st) return;
     bool lower;
     int d0, bs;
     info(st, lower, d0, bs);
-    solve_stage(LU, lda, d0, bs, lower, tb, rcp, CHOL);
+    odd = solve_stage(LU, lda, d0, bs, lower, tb, rcp, CHOL);
     staged = st;
   };
   // x_st <- T^-1 x_st, published in x
@@ -1739,7 +1814,12 @@ __global__ void __launch_bounds__(256) getrs1_kernel(const double* LU, long lda,
     if (tid < kSolveBs) {
       if (tid < bs) xd[tid] = __ldcg(x + d0 + tid);
       asm volatile("bar.sync 1, 128;" ::: "memory");
-      diag_solve(tb, ld, rcp, bs, lower, CHOL || !lower, xd);
+      if (odd)
+        diag_solve_divide(tb, ld, bs, lower, xd);
+      else if (!lower)
+        diag_solve<false, kRecip>(tb, ld, rcp, nullptr, bs, xd);
+      else
+        diag_solve<true, CHOL ? kRecip : kUnit>(tb, ld, rcp, nullptr, bs, xd);
       if (tid < bs) __stcg(x + d0 + tid, xd[tid]);
     }
   };
