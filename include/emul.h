@@ -65,17 +65,21 @@ size_t emul_workspace_bytes(emul_handle_t handle);
 
 /* Host-only introspection of the product kernel's schedule (the order in
  * which the level sums I_L of Sec. 2 are accumulated; the paper fixes only
- * their values, not this order): the sweeps and the TMEM slot plan the kernel
- * would use for `slices` slices and inner dimension k.  wide = 1 selects the
- * 64-column variant, level_sums = 1 the emul_level_sums mode; threshold is
+ * their values, not this order): the sweeps and the TMEM slots of the variants with
+ * one CTA per tile (at most 128 rows, or what emul_schedule_pair has no schedule for)
+ * for `slices` slices and inner dimension k.  wide = 1 selects the 64-column variant;
+ * level_sums = 1 (the emul_level_sums mode) takes the same schedule; threshold is
  * the last level kept (0: slices + 1; else 2..2*slices).  Needs no GPU.
  *   sweeps     out, cap_sweeps rows of EMUL_SWEEP_INTS ints:
  *              k0c, k1c (K chunks of 32), L[2], pb[2], pe[2], flags[2],
  *              nplanes, kcs (L[1] = 0: one job; flags: 1 final, the job
  *              whose term completes the exact sum that is rounded)
  *   table      out, cap_table bytes: slot (bits 0-1) and barrier parity
- *              (bit 2) of job j in tile phase ph at ph * njobs + j
- *   meta       out, 5 ints: nsweeps, njobs, t0, period, table bytes
+ *              (bit 2) of job j in tile phase ph at ph * njobs + j.  The kernel
+ *              counts: job i of all its tiles takes slot i % 4, parity (i / 4) & 1;
+ *              the i-th tile is in phase i % period
+ *   meta       out, 5 ints: nsweeps, njobs, 0 (tiles before the first phase),
+ *              period, table bytes
  * Returns EMUL_OK, EMUL_INVALID_ARG (no schedule for these arguments, or a
  * capacity too small; meta is still filled when a schedule exists). */
 #define EMUL_SWEEP_INTS 12
@@ -324,8 +328,8 @@ int emul_selector_load(emul_handle_t h, const char* path);
  * lives in one 16 MiB static device array that every GPU which loads this
  * library holds until the process exits.  Limit: with kp = k rounded up to a
  * multiple of 8, 2 * slices * kp * (m + n) + 4 * (m + n) + about 17 KB must
- * fit in 16 MiB, else the call returns EMUL_NO_WORKSPACE and enqueues
- * nothing.  The first call on a device sets up that device (it looks up the
+ * fit in 16 MiB, and the schedule in 16 KB (k up to about 59000 at 7 slices, 51000 at
+ * 8), else the call returns EMUL_NO_WORKSPACE and enqueues nothing.  The first call on a device sets up that device (it looks up the
  * device address of the array); make that first call before any stream
  * capture.  Every call reuses the same array and keeps the previous call's
  * contents: calls that overlap on the GPU (other streams, other threads)

@@ -174,56 +174,6 @@ bool build_levelwise(const PairSet& ps, int t, int nch, bool wide, std::vector<S
   return true;
 }
 
-// TMEM slot of every job.  The MMA issuer and the epilogue follow one rule:
-// a job takes the slot whose current job is drained earliest (ties: lowest
-// slot); the epilogue releases a slot when it has drained its job (in
-// level-sum mode every job is drained the same way).  The rule is simulated
-// tile by tile until the slot state (release points relative to the tile,
-// use-count parities) repeats; the table holds the transient tiles and one
-// period.  A sweep may only take slots released by jobs before it, otherwise
-// the schedule is rejected.
-bool plan_slots(const std::vector<Sweep>& sw, std::vector<uint8_t>& tab, int& njobs, int& t0, int& period) {
-  std::vector<int> first_of_job;
-  for (const Sweep& w : sw) {
-    const int first = static_cast<int>(first_of_job.size());
-    for (int j = 0; j < w.njobs; ++j) first_of_job.push_back(first);
-  }
-  njobs = static_cast<int>(first_of_job.size());
-  if (njobs == 0) return false;
-  constexpr int kS = 4, kMaxTiles = 64;
-  constexpr long long kFree = -(1ll << 40);
-  long long rel[kS];
-  int cnt[kS];
-  for (int i = 0; i < kS; ++i) rel[i] = kFree, cnt[i] = 0;
-  std::vector<std::vector<long long>> states;
-  tab.clear();
-  for (int tile = 0; tile < kMaxTiles; ++tile) {
-    const long long base = static_cast<long long>(tile) * njobs;
-    std::vector<long long> key;
-    for (int i = 0; i < kS; ++i) {
-      key.push_back(rel[i] == kFree ? kFree : rel[i] - base);
-      key.push_back(cnt[i] & 1);
-    }
-    for (size_t i0 = 0; i0 < states.size(); ++i0)
-      if (states[i0] == key) {
-        t0 = static_cast<int>(i0);
-        period = tile - t0;
-        return true;
-      }
-    states.push_back(key);
-    for (int j = 0; j < njobs; ++j) {
-      int b = 0;
-      for (int i = 1; i < kS; ++i)
-        if (rel[i] < rel[b]) b = i;
-      if (rel[b] >= base + first_of_job[j]) return false;
-      tab.push_back(static_cast<uint8_t>(b | ((cnt[b] & 1) << 2)));
-      rel[b] = base + j;
-      cnt[b]++;
-    }
-  }
-  return false;
-}
-
 // K chunks per stage: a stage holds s tiles of A and s of B, so a sweep that
 // stages fewer planes packs several chunks into one stage (one barrier phase
 // for more bytes; the copy engine's rate grows with the bytes per phase).
@@ -236,31 +186,29 @@ void set_chunks_per_stage(int s, std::vector<Sweep>& out) {
   }
 }
 
-// Schedule and slot plan for the levels 2..t (t = 0: the default threshold
-// s + 1 of the method): the banded schedule when it exists and plans, else the
-// level-ordered one.  The level-sum mode (mode1) drains every job the same
-// way and uses the same schedule.
+// Schedule of the one-CTA variants for the levels 2..t (t = 0: the default
+// threshold s + 1 of the method): the banded one when it exists, else the
+// level-ordered one.  The level-sum mode drains every job the same way and uses the
+// same schedule.
 // sa, sb: slices of A and of B whose pairs are kept (0: s); s = max(sa, sb)
 // is the split both operands get and the number of planes a stage holds.
-bool build_schedule(int s, int nch, bool wide, bool mode1, std::vector<Sweep>& out, std::vector<uint8_t>& tab,
-                    int& njobs, int& t0, int& period, int t = 0, int sa = 0, int sb = 0) {
-  (void)mode1;
+bool build_schedule(int s, int nch, bool wide, std::vector<Sweep>& out, int t = 0, int sa = 0, int sb = 0) {
   if (sa == 0) sa = s;
   if (sb == 0) sb = s;
   if (t == 0) t = s + 1;
   if (t < 2 || t > sa + sb || (sa > sb ? sa : sb) != s) return false;
   const PairSet ps{sa, sb};
-  if (!(build_banded(ps, t, nch, wide, out) && plan_slots(out, tab, njobs, t0, period)) &&
-      !(build_levelwise(ps, t, nch, wide, out) && plan_slots(out, tab, njobs, t0, period)))
-    return false;
+  if (!build_banded(ps, t, nch, wide, out) && !build_levelwise(ps, t, nch, wide, out)) return false;
   set_chunks_per_stage(s, out);
-  return true;
+  return !out.empty();
 }
 
-// Schedule of the CTA-pair kernel.  Its single issuing warp takes a job's slot
-// only before the job's own first MMA, so a sweep may hold as many jobs as
-// there are slots: bands of up to four adjacent levels share every staged
-// chunk.  At s = 7 the bands {8,7,6,5} and {4,3,2} stage 10 planes per chunk,
+// Schedule of the CTA-pair kernel: bands of up to four adjacent levels share every
+// staged chunk.  A sweep may hold as many jobs as there are slots: the two issuing
+// warps take its jobs alternately, each waits for a job's slot only before that
+// job's own first MMA, and the slot's job before it belongs to an earlier sweep,
+// whose MMAs are all issued; both warps commit every stage, so a stage is freed also
+// when one of them has no job in the sweep.  At s = 7 the bands {8,7,6,5} and {4,3,2} stage 10 planes per chunk,
 // bands of two levels 16, and the staged bytes set the pace (12 KB per plane
 // and chunk against 64 cycles per MMA: with 16 planes the copies alone need
 // 1.0 of the MMAs' time at 54 bytes per clock, with 10 planes 0.65).  The bands
@@ -399,9 +347,7 @@ bool narrow_ok(int s, int k, int t = 0, int sa = 0, int sb = 0) {
   if (s > 7) return false;
   const int nch = (k + kBK - 1) / kBK;
   std::vector<Sweep> tmp;
-  std::vector<uint8_t> tab;
-  int nj, t0, per;
-  if (!build_schedule(s, nch, false, false, tmp, tab, nj, t0, per, t, sa, sb)) return false;
+  if (!build_schedule(s, nch, false, tmp, t, sa, sb)) return false;
   // R, the sum of the levels 3..t with their weights, stays below 2^61, so
   // that R + I_2 2^(7(t-2)) fits in 64 bits whenever |I_2| 2^(7(t-2)) <= 2^62
   // (the epilogue's test; otherwise it adds the term in 128 bits).
@@ -418,12 +364,12 @@ bool wide_ok(int s, int t, int k, int sa = 0, int sb = 0) {
   return exact_sum_bound_per_k(PairSet{sa ? sa : s, sb ? sb : s}, t) * static_cast<long double>(nch * kBK) < 8.5e37L;
 }
 
-int get_schedule(emul_handle_t h, int s, int t, int nch, bool wide, bool pair, bool mode1, Sweep** dptr, int* count,
+int get_schedule(emul_handle_t h, int s, int t, int nch, bool wide, bool pair, Sweep** dptr, int* count,
                  DrainConstants* drains, int sa, int sb) {
   const uint64_t key = (static_cast<uint64_t>(pair) << 48) | (static_cast<uint64_t>(sa) << 40) |
                        (static_cast<uint64_t>(sb) << 32) | (static_cast<uint64_t>(s) << 24) |
-                       (static_cast<uint64_t>(wide) << 23) | (static_cast<uint64_t>(mode1) << 22) |
-                       (static_cast<uint64_t>(t) << 13) | static_cast<uint64_t>(nch);   // nch < 2^13 (k <= 65536)
+                       (static_cast<uint64_t>(wide) << 23) | (static_cast<uint64_t>(t) << 13) |
+                       static_cast<uint64_t>(nch);   // nch < 2^13 (k <= 65536)
   auto it = h->sched_cache.find(key);
   if (it != h->sched_cache.end()) {
     *dptr = it->second.sched;
@@ -432,10 +378,8 @@ int get_schedule(emul_handle_t h, int s, int t, int nch, bool wide, bool pair, b
     return EMUL_OK;
   }
   std::vector<Sweep> v;
-  std::vector<uint8_t> tab;
-  int njobs, t0, period, stash = -1;
-  if (pair ? pair_plan(s, t, nch, sa, sb, &v, &stash) == 0
-           : !build_schedule(s, nch, wide, mode1, v, tab, njobs, t0, period, t, sa, sb))
+  int stash = -1;
+  if (pair ? pair_plan(s, t, nch, sa, sb, &v, &stash) == 0 : !build_schedule(s, nch, wide, v, t, sa, sb))
     return set_error(h, EMUL_INVALID_ARG, "no schedule for this slice count / k");
   const DrainConstants dc = drained_constants(v, t, stash);
   Sweep* d = nullptr;
@@ -682,7 +626,7 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
   Sweep* sched = nullptr;
   int nsweeps = 0;
   DrainConstants drains{};
-  rc = get_schedule(h, s, t, nch, wide, pair, mode == 1, &sched, &nsweeps, &drains, s_a, s_b);
+  rc = get_schedule(h, s, t, nch, wide, pair, &sched, &nsweeps, &drains, s_a, s_b);
   if (rc) return rc;
   const int BN = cfg.bn;
   CUtensorMap tmA, tmB;
@@ -899,15 +843,19 @@ int emul_schedule(int slices, int k, int wide, int level_sums, int threshold, in
   using namespace emul;
   if (slices < 1 || slices > kMaxSlices || k < 1 || !meta) return EMUL_INVALID_ARG;
   if (threshold != 0 && (threshold < 2 || threshold > 2 * slices)) return EMUL_INVALID_ARG;
+  (void)level_sums;                  // both modes take the same schedule
   const int nch = (k + kBK - 1) / kBK;
   std::vector<Sweep> v;
-  std::vector<uint8_t> tab;
-  int njobs = 0, t0 = 0, period = 0;
-  if (!build_schedule(slices, nch, wide != 0, level_sums != 0, v, tab, njobs, t0, period, threshold))
-    return EMUL_INVALID_ARG;
+  if (!build_schedule(slices, nch, wide != 0, v, threshold)) return EMUL_INVALID_ARG;
+  int njobs = 0, period = 1;
+  for (const Sweep& w : v) njobs += w.njobs;
+  // jobs counted over all tiles take the slots in turn: 8 jobs until slot and parity repeat
+  while (period * njobs % (2 * kTmemSlots) != 0) ++period;
+  std::vector<uint8_t> tab(static_cast<size_t>(period) * njobs);
+  for (size_t j = 0; j < tab.size(); ++j) tab[j] = static_cast<uint8_t>(j % kTmemSlots | (j / kTmemSlots & 1) << 2);
   meta[0] = static_cast<int>(v.size());
   meta[1] = njobs;
-  meta[2] = t0;
+  meta[2] = 0;
   meta[3] = period;
   meta[4] = static_cast<int>(tab.size());
   if (!sweeps || !table || cap_sweeps < static_cast<int>(v.size()) || cap_table < static_cast<int>(tab.size()))
@@ -1028,7 +976,7 @@ namespace emul {
 namespace {
 
 constexpr size_t kNoAllocScratchBytes = size_t(16) << 20;   // 16 MiB
-constexpr size_t kNoAllocSchedBytes = 16384;                // sweeps (16 B each); the slot plan counts towards the limit
+constexpr size_t kNoAllocSchedBytes = 16384;                // 1024 sweeps
 constexpr int kNoAllocMaxDevices = 64;
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
@@ -1121,10 +1069,8 @@ extern "C" int emul_dgemm_noalloc(void* stream, int m, int n, int k, double alph
   const bool wide = !narrow_ok(slices, k);
   const int nch = (k + kBK - 1) / kBK;
   std::vector<Sweep> v;
-  std::vector<uint8_t> tab;
-  int njobs, t0, period;
-  if (!build_schedule(slices, nch, wide, false, v, tab, njobs, t0, period)) return EMUL_INVALID_ARG;
-  if (v.size() * sizeof(Sweep) + tab.size() > kNoAllocSchedBytes) return EMUL_NO_WORKSPACE;
+  if (!build_schedule(slices, nch, wide, v)) return EMUL_INVALID_ARG;
+  if (v.size() * sizeof(Sweep) > kNoAllocSchedBytes) return EMUL_NO_WORKSPACE;
   const DrainConstants drains = drained_constants(v, slices + 1, -1);
   // the status word must start at zero; the rest is fully rewritten by this call
   if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return EMUL_CUDA_ERROR;

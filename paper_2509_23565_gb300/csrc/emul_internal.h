@@ -20,6 +20,9 @@ constexpr int kExactBudget = 1040;       // k * pairs per accumulator: 1040 * 12
 // job of the 64-bit variants) completes T = R + I 2^(7(t-L)), rounds it and
 // updates C.
 constexpr int kSweepJobs = 4;
+// TMEM accumulator slots.  Job j, counted over all tiles of a CTA or CTA pair, takes
+// slot j % 4; its barriers' phase is the parity of j / 4.
+constexpr int kTmemSlots = 4;
 struct Sweep {
   int16_t k0c, k1c;       // chunk range
   int8_t L[kSweepJobs];   // job levels (0: no job)

@@ -57,7 +57,7 @@ constexpr int kMmaWarps = 2;           // warps 1 .. kMmaWarps issue MMAs
 constexpr int kLaunchRegs = 96;         // 640 x 96 = 61440 registers at launch
 constexpr int kLowRegs = 32;            // producer warpgroup after setmaxnreg.dec
 constexpr int kHighRegs = 112;          // epilogue warpgroups: 128*32 + 512*112 = 61440
-constexpr int kSlots = 4;
+constexpr int kSlots = kTmemSlots;
 constexpr int kEpiWarps = 16;
 constexpr int kStashBits = 16;         // low bits of the exact sum put aside (STASH)
 constexpr int kSchedSmem = 64;
