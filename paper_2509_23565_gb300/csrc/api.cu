@@ -601,11 +601,19 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
   // the variant tests plan a schedule; they are made once per (s, t, K chunks)
   const uint64_t nkey = (static_cast<uint64_t>(s_a) << 48) | (static_cast<uint64_t>(s_b) << 40) |
                         (static_cast<uint64_t>(s) << 32) | (static_cast<uint64_t>(t) << 16) | static_cast<uint64_t>(nch);
+  Sweep* sched = nullptr;
+  int nsweeps = 0;
+  DrainConstants drains{};
   auto nit = h->narrow_cache.find(nkey);
   if (nit == h->narrow_cache.end()) {
     const int kinds = (narrow_ok(s, k, t, s_a, s_b) ? 4 : 0) |
                       pair_plan(s, t, nch, s_a, s_b, nullptr, nullptr);
     nit = h->narrow_cache.emplace(nkey, kinds).first;
+    // the schedules of both shapes of tile now: the first product with this k and
+    // slice count is then the only one that allocates, whatever the others' m and n
+    // (a later one may be captured); one that this call needs is asked for again below
+    get_schedule(h, s, t, nch, !(kinds & 4), false, &sched, &nsweeps, &drains, s_a, s_b);
+    if (kinds & 3) get_schedule(h, s, t, nch, false, true, &sched, &nsweeps, &drains, s_a, s_b);
   }
   // CTA pairs (cta_group::2) once there are two 128-row tiles: each SM stages
   // half of B, a quarter less than alone
@@ -623,9 +631,6 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
   const bool wide = cfg.var == Variant::kWide;
   if (wide && mode == 0 && !wide_ok(s, t, k, s_a, s_b))
     return set_error(h, EMUL_NOT_SUPPORTED, "threshold too high for this k: the 128-bit exact sum could overflow");
-  Sweep* sched = nullptr;
-  int nsweeps = 0;
-  DrainConstants drains{};
   rc = get_schedule(h, s, t, nch, wide, pair, &sched, &nsweeps, &drains, s_a, s_b);
   if (rc) return rc;
   const int BN = cfg.bn;

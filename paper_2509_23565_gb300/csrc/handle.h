@@ -25,7 +25,7 @@ struct emul_handle_s {
     int nsweeps;
     emul::DrainConstants drains;
   };
-  std::map<uint64_t, SchedEntry> sched_cache;   // (slices of A / B, s, wide, level-sum mode, threshold, chunks) -> device schedule
+  std::map<uint64_t, SchedEntry> sched_cache;   // (pair, slices of A / B, s, wide, threshold, chunks) -> device schedule
   std::map<uint64_t, int> narrow_cache;         // (s, t, chunks) -> variants that apply: bit 2 one CTA per
                                                 // 128-column tile, bits 0-1 CTA pairs (1, or 2 with low bits aside)
   std::string last_error;
