@@ -616,13 +616,19 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
     if (kinds & 3) get_schedule(h, s, t, nch, false, true, &sched, &nsweeps, &drains, s_a, s_b);
   }
   // CTA pairs (cta_group::2) once there are two 128-row tiles: each SM stages
-  // half of B, a quarter less than alone
+  // half of B, a quarter less than alone.  64-column tiles where the pairs take them
+  // all at once: a wave of them costs 0.7 of a wave of 128-column tiles, so they gain
+  // only while they are one wave too.  us, 64 / 128 columns, s = 7, 76 pairs: 1024 x
+  // 1024 x 256 (64 tiles of 64 columns) 31 / 38, 4864 x 256 x 256 (76) 34 / 41, with k
+  // = 1024 120 / 152, at s = 8 37 / 50, at s = 3 28 / 30; just past the line 2560 x
+  // 512 x 256 (80) 49 / 39, k = 1024 167 / 130, s = 8 55 / 49, s = 3 38 / 31, and
+  // 2048 x 1152 x 256 (144) 49 / 40
   GemmConfig cfg{Variant::kWide, 64, false};
   const int pair_kind = nit->second & 3;
   if (pair_kind && m > 128 && h->nsm >= 2) {
     GemmConfig c{Variant::kPair, 128, pair_kind == 2};
-    const long tiles = static_cast<long>((m + 255) / 256) * ((n + 127) / 128);
-    if (!lower && tiles < h->nsm / 2) c.bn = 64;
+    const long tiles64 = static_cast<long>((m + 255) / 256) * ((n + 63) / 64);
+    if (!lower && tiles64 <= (h->nsm - h->sm_spare) / 2) c.bn = 64;
     size_t smem_pair = 0;
     if (gemm_stages(c, s, &smem_pair) >= 2 && gemm_pair_capacity(smem_pair) >= 1) cfg = c;   // else one CTA per tile
   }
