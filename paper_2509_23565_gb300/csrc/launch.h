@@ -6,8 +6,8 @@
 // (every chain of 4 to 120 us kernels measured here took a multiple of 2.048 us
 // per kernel), and the panels of the factorizations are chains of such kernels:
 // a product of 64 x 64 x 64 in a loop took 14.3 us that way and takes 11.8, LU at
-// n = 4001 17.8 ms and 17.2, Cholesky at 12000 36.6 and 35.8, LU without pivoting
-// at 6144 23.9 and 23.0.  Cooperative kernels are launched the plain way.
+// n = 4001 17.8 ms and 17.2, Cholesky at 12000 36.6 and 35.9, LU without pivoting
+// at 6144 23.9 and 22.5.  Cooperative kernels are launched the plain way.
 #pragma once
 #include <utility>
 

@@ -155,13 +155,14 @@ struct OutsideColumn {
 //
 // Every interchange is also applied to the columns [pc0, d0) and [d0+w, pc1) of
 // the enclosing panel, which live in global memory: the outside column q
-// (0-based over both ranges) belongs to block q % G for the whole launch, to
-// the (q / G)-th of its threads other than thread 0 (it publishes the block's
-// candidate) and the row-c reader (first lane of the last warp), so successive
-// interchanges of one element stay in program order.  Its loads are issued
-// when the pivot is known, its stores when the next pivot is known, off the
-// critical path.  At most 248 outside columns exist (panel <= 256 wide, leaf
-// >= 8 wide); 254 owners per block are available.
+// (0-based over both ranges) belongs to one thread of block q % G for the whole
+// launch, so successive interchanges of one element stay in program order: to the
+// (q / G)-th of the block's 256 threads, counted from warp 1 to warp 6 first, then
+// warps 0 and 7, which run the exchange and interchange after it.  A column's loads
+// are issued when the pivot is known, its stores when the next pivot is known, off
+// the critical path.  At most 248 outside columns exist (panel <= 256 wide, leaf
+// >= 8 wide).  The candidate's value and row are published by the first lane of
+// warp 7, its reciprocal by the first lane of warp 6.
 __global__ void __launch_bounds__(kLeafThreads) getf2_leaf_kernel(double* A, long lda, int n, int d0, int w, int R,
                                                                  int pc0, int pc1, int32_t* ipiv, int32_t* info,
                                                                  uint64_t* recs, uint64_t* drec, uint32_t salt,

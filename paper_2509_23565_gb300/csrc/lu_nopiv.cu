@@ -4,16 +4,16 @@
 //
 // Step j0 (right-looking, block nb):
 //   1. the panel A[j0:n, j0:j0+jb] is factored by recursive halving.  A leaf
-//      (<= 64 columns) factors its diagonal block in FP64 inside one CTA and
-//      forms the inverses of both triangular factors there; its rows below
-//      become L21 = A21 U11^-1 through the emulated product.  An inner node
+//      (<= 64 columns) factors its diagonal block in FP64 on one cluster of eight
+//      CTAs and forms the inverses of both triangular factors, a warp per column;
+//      its rows below become L21 = A21 U11^-1 through the emulated product.  An inner node
 //      forms U12 = L11^-1 A12 and the Schur update of the rows below with the
 //      emulated product, recurses into its right half, and joins the two
 //      halves' unit-lower inverses, X21 = -X22 (L21 X11);
 //   2. U12 = X A12 with X = L11^-1 of the whole block (emulated product);
 //   3. A22 <- A22 - L21 U12 (emulated product, alpha = -1, beta = 1).
-// The Schur updates and U12 run as products over K chunks of at most 1024, so
-// every product at s <= 7 keeps the 128-column tile (see gemm_kchunks).
+// The Schur updates and U12 run as products over K chunks of at most 1024
+// (see gemm_kchunks).
 // No row is ever exchanged, so the factorization is stable only for matrices
 // that need no pivoting (diagonally dominant, SPD).
 #include <cuda_runtime.h>
@@ -278,9 +278,11 @@ struct NpBufs {
 };
 
 // C <- beta C + alpha A B as consecutive emulated products over K chunks of at
-// most kNpChunk (each rounded once, which is part of the result; C must not overlap
-// A or B).  Up to 1024 level 2 is one accumulator job (1040 products of 127^2 per
-// FP32 accumulator); C is read and written once per chunk.
+// most kNpChunk; C must not overlap A or B, and is read and written once per chunk.
+// Each chunk is rounded once, and these roundings are part of the result, so the
+// chunks are the same for every m.  The one-CTA variants (at most 128 rows) need them
+// for speed: up to 1024 level 2 is one accumulator job (1040 products of 127^2 per
+// FP32 accumulator); the CTA pairs would take any K at s <= 7.
 int gemm_kchunks(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Operand B, double beta, double* C,
                  long ldc, int s) {
   for (int c0 = 0; c0 < k; c0 += kNpChunk) {
