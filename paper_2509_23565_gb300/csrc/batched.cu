@@ -27,6 +27,8 @@
 #include <vector>
 
 #include "handle.h"
+#include "launch.h"
+#include "ptx.cuh"
 
 namespace emul {
 
@@ -35,6 +37,7 @@ struct BatchSys {
   double* b;
   long lda;
   int n, nb, s, index;
+  int it;          // refinement steps taken before (a system handed over)
 };
 
 namespace {
@@ -140,7 +143,7 @@ __device__ __forceinline__ void loaded(float (&l)[32]) {
 // next diagonal block meanwhile (dg: two of 32 x 32 in shared memory, by columns).
 // With the solving warp loading it, each load came just before its use or its
 // spill, 32 trips to L2 in a row: 2.1 million cycles for n = 1000, 0.81 now.
-__device__ __noinline__ void lu_solve_f32(const float* W, int n, float* d, float* dg) {
+__device__ __noinline__ void lu_solve_f32(const float* W, int ld, int n, float* d, float* dg) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int nblk = (n + 31) / 32;
   auto first_row = [&](int st) { return 32 * (st < nblk ? st : 2 * nblk - 1 - st); };
@@ -151,7 +154,7 @@ __device__ __noinline__ void lu_solve_f32(const float* W, int n, float* d, float
 #pragma unroll
     for (int q = 0; q < kEach; ++q) {
       const int e = tid + q * kBThreads, r = e & 31, k = e >> 5;
-      nx[q] = r < w && k < w ? W[(k0 + r) + static_cast<long>(k0 + k) * n] : 0.f;
+      nx[q] = r < w && k < w ? W[(k0 + r) + static_cast<long>(k0 + k) * ld] : 0.f;
     }
   };
   auto store_diag = [&](int st) {
@@ -192,10 +195,10 @@ __device__ __noinline__ void lu_solve_f32(const float* W, int n, float* d, float
     __syncthreads();
     const int lo = lower ? k0 + w : 0, hi = lower ? n : k0;
     for (int i = lo + tid; i < hi; i += blockDim.x) {
-      const float* p = W + i + static_cast<long>(k0) * n;
+      const float* p = W + i + static_cast<long>(k0) * ld;
       float l[32];
 #pragma unroll
-      for (int k = 0; k < 32; ++k) l[k] = k < w ? p[static_cast<long>(k) * n] : 0.f;
+      for (int k = 0; k < 32; ++k) l[k] = k < w ? p[static_cast<long>(k) * ld] : 0.f;
       loaded(l);
       float v = d[i];
       if (lower) {
@@ -232,13 +235,15 @@ __device__ __forceinline__ uint32_t ld_s8x4(const int8_t* p, bool ok) {
 
 // The general factorization: any size, block and slice count, the working copy
 // in global memory throughout.  Serves what factor_fast does not take.
-__device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info, float* sv, int* si) {
+__device__ __forceinline__ void factor_general(const BatchSys& S, int s, const Scratch& sc, int* info, float* sv,
+                                               int* si) {
   const int n = S.n, nb = S.nb;
   const int nb4 = (nb + 31) / 32 * 32;   // slice row length: whole K steps of 32, zero padded
   float* W = sc.W;
+  const long ld = n;
   for (long idx = threadIdx.x; idx < static_cast<long>(n) * n; idx += blockDim.x) {
     const int i = static_cast<int>(idx % n), j = static_cast<int>(idx / n);
-    W[idx] = static_cast<float>(S.A[i + j * S.lda]);
+    W[i + j * ld] = static_cast<float>(S.A[i + j * S.lda]);
   }
   __syncthreads();
   for (int j0 = 0; j0 < n; j0 += nb) {
@@ -248,7 +253,7 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
       float bv = -1.f;
       int bi = 0x7FFFFFFF;
       for (int r = c + threadIdx.x; r < n; r += blockDim.x) {
-        const float v = fabsf(W[r + static_cast<long>(c) * n]);
+        const float v = fabsf(W[r + static_cast<long>(c) * ld]);
         if (v > bv || (v == bv && r < bi)) {
           bv = v;
           bi = r;
@@ -261,22 +266,22 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
       if (threadIdx.x == 0) sc.piv[c] = p;
       if (p != c)
         for (int j = threadIdx.x; j < n; j += blockDim.x) {
-          const float t = W[c + static_cast<long>(j) * n];
-          W[c + static_cast<long>(j) * n] = W[p + static_cast<long>(j) * n];
-          W[p + static_cast<long>(j) * n] = t;
+          const float t = W[c + static_cast<long>(j) * ld];
+          W[c + static_cast<long>(j) * ld] = W[p + static_cast<long>(j) * ld];
+          W[p + static_cast<long>(j) * ld] = t;
         }
       __syncthreads();
-      const float piv = W[c + static_cast<long>(c) * n];
+      const float piv = W[c + static_cast<long>(c) * ld];
       if (piv == 0.f) {
         if (threadIdx.x == 0 && *info == 0) *info = c + 1;
         __syncthreads();
         continue;
       }
       for (int r = c + 1 + threadIdx.x; r < n; r += blockDim.x) {
-        const float l = W[r + static_cast<long>(c) * n] / piv;
-        W[r + static_cast<long>(c) * n] = l;
+        const float l = W[r + static_cast<long>(c) * ld] / piv;
+        W[r + static_cast<long>(c) * ld] = l;
         for (int cc = c + 1; cc < j0 + jb; ++cc)
-          W[r + static_cast<long>(cc) * n] = fmaf(-l, W[c + static_cast<long>(cc) * n], W[r + static_cast<long>(cc) * n]);
+          W[r + static_cast<long>(cc) * ld] = fmaf(-l, W[c + static_cast<long>(cc) * ld], W[r + static_cast<long>(cc) * ld]);
       }
       __syncthreads();
     }
@@ -285,9 +290,9 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
     // ---- U12 = L11^-1 A12 (one thread per column)
     for (int j = j0 + jb + threadIdx.x; j < n; j += blockDim.x)
       for (int k = j0; k < j0 + jb; ++k) {
-        const float ukj = W[k + static_cast<long>(j) * n];
+        const float ukj = W[k + static_cast<long>(j) * ld];
         for (int i = k + 1; i < j0 + jb; ++i)
-          W[i + static_cast<long>(j) * n] = fmaf(-W[i + static_cast<long>(k) * n], ukj, W[i + static_cast<long>(j) * n]);
+          W[i + static_cast<long>(j) * ld] = fmaf(-W[i + static_cast<long>(k) * ld], ukj, W[i + static_cast<long>(j) * ld]);
       }
     __syncthreads();
     // ---- scales and slices of L21 (by rows) and U12 (by columns)
@@ -297,7 +302,7 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
       const int q = isA ? t : t - m2;
       uint32_t mx = 0;
       for (int k = 0; k < jb; ++k) {
-        const float v = isA ? W[(j0 + jb + q) + static_cast<long>(j0 + k) * n] : W[(j0 + k) + static_cast<long>(j0 + jb + q) * n];
+        const float v = isA ? W[(j0 + jb + q) + static_cast<long>(j0 + k) * ld] : W[(j0 + k) + static_cast<long>(j0 + jb + q) * ld];
         const uint32_t u = __float_as_uint(v) & 0x7FFFFFFFu;
         mx = u > mx ? u : mx;
       }
@@ -307,7 +312,7 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
       for (int k = 0; k < nb4; ++k) {
         uint32_t u = 0, neg = 0;
         if (k < jb) {
-          const float v = isA ? W[(j0 + jb + q) + static_cast<long>(j0 + k) * n] : W[(j0 + k) + static_cast<long>(j0 + jb + q) * n];
+          const float v = isA ? W[(j0 + jb + q) + static_cast<long>(j0 + k) * ld] : W[(j0 + k) + static_cast<long>(j0 + jb + q) * ld];
           u = __float_as_uint(v);
           neg = u >> 31;
           u &= 0x7FFFFFFFu;
@@ -370,7 +375,7 @@ __device__ void factor_general(const BatchSys& S, int s, Scratch& sc, int* info,
         const int i = i0 + g + (q >= 2 ? 8 : 0), j = c0 + tq * 2 + (q & 1);
         if (i >= m2 || j >= m2) continue;
         const double D = s <= 5 ? ldexp(static_cast<double>(T[q]), sc.ea[i] + sc.fb[j] - 7 * t) : Dd[q];
-        float* cp = W + (j0 + jb + i) + static_cast<long>(j0 + jb + j) * n;
+        float* cp = W + (j0 + jb + i) + static_cast<long>(j0 + jb + j) * ld;
         *cp = static_cast<float>(static_cast<double>(*cp) - D);
       }
     }
@@ -955,41 +960,48 @@ __device__ __noinline__ void factor_fast(const BatchSys& sys, Scratch& sc, int* 
   __syncthreads();
 }
 
-// Factor one system and leave its row permutation in sc.perm.
-__device__ __noinline__ void factor_system(const BatchSys& sys, int s, Scratch& sc, int* info, float* sv, int* si, FastShared& F,
-                              uint8_t* dyn) {
-  // the slice counts and blocks the tuner chooses from, and the 8 slices of a
-  // system whose refinement stalls.  152 systems at once, one per SM, without
-  // refinement (ms): n = 1024 14.2 at 3 slices, 15.7 at 4, 29.3 at 8 (20.4 with
-  // blocks of 16); n = 1025, where the panel outgrows two rows per thread and takes
-  // the general path, 128.7, 139.3 and 281.
-  if (sys.n <= kFastN && (s == 3 || s == 4 || s == 8) && (sys.nb == 16 || sys.nb == 32)) {
+// What factor_fast takes: the slice counts and blocks the tuner chooses from, and
+// the 8 slices of a system whose refinement stalls.  152 systems at once, one per SM,
+// without refinement (ms): n = 1024 14.2 at 3 slices, 15.7 at 4, 29.3 at 8 (20.4 with
+// blocks of 16); n = 1025, where the panel outgrows two rows per thread and takes the
+// general path, 115 at 3 and 234 at 8.
+__host__ __device__ __forceinline__ bool fast_takes(int n, int nb, int s) {
+  return n <= kFastN && (s == 3 || s == 4 || s == 8) && (nb == 16 || nb == 32);
+}
+
+// Factor one system and leave its row permutation in sc.perm.  (By value: out of
+// line, a reference would put the pointers into local memory.)
+template <bool FAST>
+__device__ __noinline__ void factor_system(const BatchSys sys, int s, Scratch sc, int* info, float* sv, int* si,
+                                           FastShared* F, uint8_t* dyn) {
+  if constexpr (FAST) {
     if (sys.nb == 32) {
-      if (s == 3) return factor_fast<3, 32>(sys, sc, info, F, dyn);
-      if (s == 4) return factor_fast<4, 32>(sys, sc, info, F, dyn);
-      return factor_fast<8, 32>(sys, sc, info, F, dyn);
+      if (s == 3) return factor_fast<3, 32>(sys, sc, info, *F, dyn);
+      if (s == 4) return factor_fast<4, 32>(sys, sc, info, *F, dyn);
+      return factor_fast<8, 32>(sys, sc, info, *F, dyn);
     }
-    if (s == 3) return factor_fast<3, 16>(sys, sc, info, F, dyn);
-    if (s == 4) return factor_fast<4, 16>(sys, sc, info, F, dyn);
-    return factor_fast<8, 16>(sys, sc, info, F, dyn);
-  }
-  factor_general(sys, s, sc, info, sv, si);
-  __syncthreads();
-  int* G = reinterpret_cast<int*>(dyn);
-  for (int i = threadIdx.x; i < sys.n; i += blockDim.x) G[i] = i;
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 0; k < sys.n; ++k) {
-      const int p = sc.piv[k];
-      if (p != k) {
-        const int v = G[k];
-        G[k] = G[p];
-        G[p] = v;
+    if (s == 3) return factor_fast<3, 16>(sys, sc, info, *F, dyn);
+    if (s == 4) return factor_fast<4, 16>(sys, sc, info, *F, dyn);
+    return factor_fast<8, 16>(sys, sc, info, *F, dyn);
+  } else {
+    factor_general(sys, s, sc, info, sv, si);
+    __syncthreads();
+    int* G = reinterpret_cast<int*>(dyn);
+    for (int i = threadIdx.x; i < sys.n; i += blockDim.x) G[i] = i;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int k = 0; k < sys.n; ++k) {
+        const int p = sc.piv[k];
+        if (p != k) {
+          const int v = G[k];
+          G[k] = G[p];
+          G[p] = v;
+        }
       }
-    }
-  __syncthreads();
-  for (int i = threadIdx.x; i < sys.n; i += blockDim.x) sc.perm[i] = G[i];
-  __syncthreads();
+    __syncthreads();
+    for (int i = threadIdx.x; i < sys.n; i += blockDim.x) sc.perm[i] = G[i];
+    __syncthreads();
+  }
 }
 
 // acc[h] (h = 0, 1) over the columns of rows i0 and i0 + blockDim.x of A, in
@@ -1021,23 +1033,50 @@ __device__ __forceinline__ void row_pass(const double* A, long lda, int n, int i
   }
 }
 
-__global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys* sys, int count, unsigned int* queue,
-                                                                  uint8_t* scratch, size_t per_block, int nmax,
-                                                                  int max_iter, double target, int32_t* info_arr,
-                                                                  double* berr_arr, int32_t* iters_arr) {
+struct BatchedArgs {
+  const BatchSys* sys;
+  int count;                 // systems, or
+  const unsigned* dcount;    // where their number stands (unless null)
+  unsigned* queue;
+  uint8_t* scratch;          // per_block bytes per block, for systems of up to nmax rows
+  size_t per_block;
+  int nmax, cap;             // cap: rows that the shared vectors hold, a multiple of 64
+  int max_iter;
+  double target;
+  int32_t* info;
+  double* berr;
+  int32_t* iters;
+  BatchSys* stalled;         // general path: systems handed to the fast one, and their number
+  unsigned* nstalled;
+};
+// While solving, shared memory holds the right-hand side (float), the solution
+// (double) and two diagonal blocks of 32 x 32 floats.
+constexpr size_t kDiagBytes = 2 * 32 * 32 * sizeof(float);
+constexpr size_t solve_smem(int cap) { return static_cast<size_t>(cap) * 12 + kDiagBytes; }
+static_assert(solve_smem(kFastN) <= kFastSmem, "shared memory of the solve");
+
+// FAST: the systems that factor_fast takes.  The others run in a kernel of their own
+// with little shared memory: factor_general works in global memory and lives off L1,
+// which 200 KB of shared memory leave no room for (100 systems of 300 rows at 7 slices
+// 11.2 ms, 5.9 so; 20 of 700 with blocks of 64 40.6 and 20.0).  A system of theirs that has to be
+// refactored with 8 slices and can be in the fast way is handed over.
+template <bool FAST>
+__global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchedArgs a) {
   __shared__ float sv[kBThreads / 32];
   __shared__ int si[kBThreads / 32];
   __shared__ double red[kBThreads / 32];
   __shared__ int task_s;
   __shared__ int info_s;
-  __shared__ __align__(16) FastShared F;
+  __shared__ __align__(16) uint8_t f_s[FAST ? sizeof(FastShared) : 16];
+  FastShared* F = reinterpret_cast<FastShared*>(f_s);
   extern __shared__ __align__(16) uint8_t dyn[];
-  // while solving: the right-hand side, the solution, diagonal blocks
   float* ds = reinterpret_cast<float*>(dyn);
-  double* xs = reinterpret_cast<double*>(dyn + kMaxN * sizeof(float));
-  float* dg = reinterpret_cast<float*>(dyn + kMaxN * (sizeof(float) + sizeof(double)));   // two diagonal blocks
-  static_assert(kMaxN * 12 + 2 * 32 * 32 * 4 <= kFastSmem, "shared memory of the solve");
-  uint8_t* base = scratch + per_block * blockIdx.x;
+  double* xs = reinterpret_cast<double*>(dyn + static_cast<size_t>(a.cap) * sizeof(float));
+  float* dg = reinterpret_cast<float*>(dyn + static_cast<size_t>(a.cap) * (sizeof(float) + sizeof(double)));
+  if (!FAST) grid_launch();       // the fast systems' kernel takes the SMs that this one leaves
+  const int nmax = a.nmax, max_iter = a.max_iter;
+  const int count = a.dcount ? static_cast<int>(*a.dcount) : a.count;
+  uint8_t* base = a.scratch + a.per_block * blockIdx.x;
   Scratch sc;
   {
     size_t o = 0;
@@ -1056,17 +1095,17 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
     sc.perm = reinterpret_cast<int*>(take(static_cast<size_t>(nmax) * 4));
   }
   while (true) {
-    if (threadIdx.x == 0) task_s = static_cast<int>(atomicAdd(queue, 1u));
+    if (threadIdx.x == 0) task_s = static_cast<int>(atomicAdd(a.queue, 1u));
     __syncthreads();
     const int t = task_s;
     __syncthreads();
     if (t >= count) break;
-    const BatchSys S = sys[t];
+    const BatchSys S = a.sys[t];
     const int n = S.n;
     if (threadIdx.x == 0) info_s = 0;
     __syncthreads();
     int s_cur = S.s;
-    factor_system(S, s_cur, sc, &info_s, sv, si, F, dyn);
+    factor_system<FAST>(S, s_cur, sc, &info_s, sv, si, F, dyn);
     __syncthreads();
     // ||A||_inf in FP64
     double an = 0.0;
@@ -1079,12 +1118,13 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
     // x0 from the FP32 factors
     for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(S.b[sc.perm[i]]);
     __syncthreads();
-    lu_solve_f32(sc.W, n, ds, dg);
+    lu_solve_f32(sc.W, n, n, ds, dg);
     for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = static_cast<double>(ds[i]);
     __syncthreads();
     double berr = INFINITY;
-    int it = 0;
+    int it = S.it;
     int since = 0;
+    bool handed = false;
     for (;; ++it, ++since) {
       // r = b - A x (FP64), ||r||, ||x||
       double rmax = 0.0, xmax = 0.0;
@@ -1104,16 +1144,26 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
       rmax = block_max_d(rmax, red);
       xmax = block_max_d(xmax, red);
       berr = rmax / (an * xmax * n * 1.1102230246251565e-16);
-      if (!(berr > target) || it >= max_iter || info_s != 0) break;
+      if (!(berr > a.target) || it >= max_iter || info_s != 0) break;
       if (since >= kStallIters && s_cur < kMaxS) {
         // the factors are too coarse for this matrix's range: refactor with 8 slices
+        if (!FAST && fast_takes(n, S.nb, kMaxS)) {
+          if (threadIdx.x == 0) {
+            BatchSys h = S;
+            h.s = kMaxS;
+            h.it = it + 1;
+            a.stalled[atomicAdd(a.nstalled, 1u)] = h;
+          }
+          handed = true;
+          break;
+        }
         s_cur = kMaxS;
         since = 0;
-        factor_system(S, s_cur, sc, &info_s, sv, si, F, dyn);
+        factor_system<FAST>(S, s_cur, sc, &info_s, sv, si, F, dyn);
         __syncthreads();
         for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(S.b[sc.perm[i]]);
         __syncthreads();
-        lu_solve_f32(sc.W, n, ds, dg);
+        lu_solve_f32(sc.W, n, n, ds, dg);
         for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = static_cast<double>(ds[i]);
         __syncthreads();
         continue;
@@ -1122,18 +1172,21 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchSys
       const double sr = rmax > 0.0 ? rmax : 1.0;
       for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(sc.r[sc.perm[i]] / sr);
       __syncthreads();
-      lu_solve_f32(sc.W, n, ds, dg);
+      lu_solve_f32(sc.W, n, n, ds, dg);
       for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] += static_cast<double>(ds[i]) * sr;
       __syncthreads();
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) S.b[i] = xs[i];
-    if (threadIdx.x == 0) {
-      info_arr[S.index] = info_s;
-      berr_arr[S.index] = berr;
-      iters_arr[S.index] = it;
+    if (!handed) {
+      for (int i = threadIdx.x; i < n; i += blockDim.x) S.b[i] = xs[i];
+      if (threadIdx.x == 0) {
+        a.info[S.index] = info_s;
+        a.berr[S.index] = berr;
+        a.iters[S.index] = it;
+      }
     }
     __syncthreads();
   }
+  if (FAST) grid_wait();          // this kernel's end is also the end of the general one beside it
 }
 
 // --------------------------------------------------------------- autotuning
@@ -1189,23 +1242,68 @@ size_t per_block_bytes(int nmax) {
 
 }  // namespace
 
-int batched_run(emul_handle_t h, const std::vector<BatchSys>& sys, int nmax, int32_t* info, double* berr,
-                int32_t* iters, int max_iter, double target) {
+// `sys`: the general systems first, each kind from the largest down.
+int batched_run(emul_handle_t h, const std::vector<BatchSys>& sys, int32_t* info, double* berr, int32_t* iters,
+                int max_iter, double target) {
   const int count = static_cast<int>(sys.size());
-  smem_attr(reinterpret_cast<const void*>(batched_solve_kernel), kFastSmem);
-  const size_t pb = per_block_bytes(nmax);
-  const int grid = count < h->nsm ? count : h->nsm;
-  const size_t desc_bytes = (count * sizeof(BatchSys) + 255) / 256 * 256;
-  int rc = reserve_workspace(h, desc_bytes + 256 + pb * grid);
+  int ngen = 0, nelig = 0, nelig_max = 1;       // general systems, those that may be handed over
+  while (ngen < count && !fast_takes(sys[ngen].n, sys[ngen].nb, sys[ngen].s)) {
+    if (fast_takes(sys[ngen].n, sys[ngen].nb, kMaxS)) {
+      ++nelig;
+      nelig_max = sys[ngen].n > nelig_max ? sys[ngen].n : nelig_max;
+    }
+    ++ngen;
+  }
+  const int nfast = count - ngen;
+  auto blocks = [&](int n) { return n < h->nsm ? n : h->nsm; };
+  const int gen_max = ngen ? sys[0].n : 1, fast_max = nfast ? sys[ngen].n : 1;
+  auto al = [](size_t x) { return (x + 255) / 256 * 256; };
+  const size_t desc = al(count * sizeof(BatchSys)), stalled = al(nelig * sizeof(BatchSys));
+  const size_t gen_scratch = al(per_block_bytes(gen_max) * blocks(ngen));
+  // [systems | systems handed over | counters | scratch of the general blocks, then of
+  // those that take what they hand over | scratch of the fast blocks]
+  int rc = reserve_workspace(h, desc + stalled + 256 + gen_scratch + per_block_bytes(fast_max) * blocks(nfast));
   if (rc) return rc;
   uint8_t* w = static_cast<uint8_t*>(h->ws);
   BatchSys* d_sys = reinterpret_cast<BatchSys*>(w);
-  unsigned int* queue = reinterpret_cast<unsigned int*>(w + desc_bytes);
-  uint8_t* scratch = w + desc_bytes + 256;
+  unsigned* counters = reinterpret_cast<unsigned*>(w + desc + stalled);
   rc = check_cuda(h, cudaMemcpyAsync(d_sys, sys.data(), count * sizeof(BatchSys), cudaMemcpyHostToDevice, h->stream),
                   "batch descriptors");
   if (rc) return rc;
-  // one persistent launch, recorded into a CUDA graph together with the queue
+  BatchedArgs gen{};
+  gen.sys = d_sys;
+  gen.count = ngen;
+  gen.queue = counters;
+  gen.scratch = w + desc + stalled + 256;
+  gen.per_block = per_block_bytes(gen_max);
+  gen.nmax = gen_max;
+  gen.cap = (gen_max + 63) / 64 * 64;
+  gen.max_iter = max_iter;
+  gen.target = target;
+  gen.info = info;
+  gen.berr = berr;
+  gen.iters = iters;
+  gen.stalled = reinterpret_cast<BatchSys*>(w + desc);
+  gen.nstalled = counters + 3;
+  BatchedArgs fast = gen;
+  fast.sys = d_sys + ngen;
+  fast.count = nfast;
+  fast.queue = counters + 1;
+  fast.scratch = gen.scratch + gen_scratch;
+  fast.per_block = per_block_bytes(fast_max);
+  fast.nmax = fast_max;
+  fast.cap = kFastN;
+  BatchedArgs late = fast;       // what the general systems hand over, on their scratch
+  late.sys = gen.stalled;
+  late.dcount = gen.nstalled;
+  late.queue = counters + 2;
+  late.scratch = gen.scratch;
+  late.per_block = per_block_bytes(nelig_max);
+  late.nmax = nelig_max;
+  smem_attr(reinterpret_cast<const void*>(batched_solve_kernel<true>), kFastSmem);
+  smem_attr(reinterpret_cast<const void*>(batched_solve_kernel<false>), static_cast<int>(solve_smem(kMaxN)));
+  prefer_l1(reinterpret_cast<const void*>(batched_solve_kernel<false>));
+  // persistent launches, recorded into a CUDA graph together with the queue
   // reset (on a private stream), then launched on the handle's stream
   BatchedState* st = bstate(h);
   if (!st->capture) {
@@ -1215,9 +1313,20 @@ int batched_run(emul_handle_t h, const std::vector<BatchSys>& sys, int nmax, int
   cudaGraph_t graph;
   rc = check_cuda(h, cudaStreamBeginCapture(st->capture, cudaStreamCaptureModeThreadLocal), "capture");
   if (rc) return rc;
-  cudaMemsetAsync(queue, 0, sizeof(unsigned int), st->capture);
-  batched_solve_kernel<<<grid, kBThreads, kFastSmem, st->capture>>>(d_sys, count, queue, scratch, pb, nmax, max_iter, target,
-                                                            info, berr, iters);
+  cudaMemsetAsync(counters, 0, 4 * sizeof(unsigned), st->capture);
+  if (ngen) {
+    batched_solve_kernel<false><<<blocks(ngen), kBThreads, solve_smem(gen.cap), st->capture>>>(gen);
+    h->launches++;
+  }
+  if (nfast) {
+    // beside the general kernel, once all of that one's blocks run (launch.h)
+    launch_chained(ngen > 0, batched_solve_kernel<true>, dim3(blocks(nfast)), dim3(kBThreads), kFastSmem, st->capture, fast);
+    h->launches++;
+  }
+  if (nelig) {
+    batched_solve_kernel<true><<<blocks(nelig), kBThreads, kFastSmem, st->capture>>>(late);
+    h->launches++;
+  }
   rc = check_cuda(h, cudaStreamEndCapture(st->capture, &graph), "capture");
   if (rc) return rc;
   if (st->exec) {
@@ -1227,7 +1336,6 @@ int batched_run(emul_handle_t h, const std::vector<BatchSys>& sys, int nmax, int
   rc = check_cuda(h, cudaGraphInstantiate(&st->exec, graph, 0), "graph instantiate");
   cudaGraphDestroy(graph);
   if (rc) return rc;
-  h->launches++;
   return check_cuda(h, cudaGraphLaunch(st->exec, h->stream), "graph launch");
 }
 
@@ -1246,18 +1354,19 @@ int emul_dgesv_batched_ir(emul_handle_t h, int count, const int* n_arr, double* 
   if (count == 0) return EMUL_OK;
   emul::BatchedState* st = emul::bstate(h);
   std::vector<emul::BatchSys> sys(count);
-  int nmax = 1;
   for (int i = 0; i < count; ++i) {
     if (n_arr[i] < 1 || n_arr[i] > emul::kMaxN || lda_arr[i] < n_arr[i] || !A_arr[i] || !b_arr[i])
       return emul::set_error(h, EMUL_INVALID_ARG, "emul_dgesv_batched_ir: invalid system");
     int tnb, ts;
     emul::pick(st, n_arr[i], tnb, ts);
-    sys[i] = emul::BatchSys{A_arr[i], b_arr[i], lda_arr[i], n_arr[i], nb ? nb : tnb, slices ? slices : ts, i};
-    nmax = n_arr[i] > nmax ? n_arr[i] : nmax;
+    sys[i] = emul::BatchSys{A_arr[i], b_arr[i], lda_arr[i], n_arr[i], nb ? nb : tnb, slices ? slices : ts, i, 0};
   }
-  // largest systems first so the queue ends with short tasks
-  std::stable_sort(sys.begin(), sys.end(), [](const emul::BatchSys& a, const emul::BatchSys& b) { return a.n > b.n; });
-  return emul::batched_run(h, sys, nmax, info_arr, berr_arr, iters_arr, max_iter, 1.0);
+  // the general systems, then the fast ones, the largest first so that the queues end with short tasks
+  std::stable_sort(sys.begin(), sys.end(), [](const emul::BatchSys& a, const emul::BatchSys& b) {
+    const bool fa = emul::fast_takes(a.n, a.nb, a.s), fb = emul::fast_takes(b.n, b.nb, b.s);
+    return fa != fb ? fb : a.n > b.n;
+  });
+  return emul::batched_run(h, sys, info_arr, berr_arr, iters_arr, max_iter, 1.0);
 }
 
 int emul_autotune(emul_handle_t h, const char* cache_path) {

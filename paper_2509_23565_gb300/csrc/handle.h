@@ -67,6 +67,8 @@ struct Operand {
 int set_error(emul_handle_t h, int code, const std::string& msg);
 // Raise a kernel's dynamic shared-memory limit to `bytes`, once per device.
 void smem_attr(const void* fn, int bytes);
+// No more of L1 for shared memory than the launch asks for (set once per device).
+void prefer_l1(const void* fn);
 int check_cuda(emul_handle_t h, cudaError_t e, const char* what);
 
 // Grow the workspace to at least `bytes` (synchronises the device when it grows).
