@@ -47,8 +47,16 @@ constexpr int kMaxS = 8;
 constexpr int kMaxN = 4096;       // largest system
 constexpr int kStallIters = 8;   // refinement steps before a system is refactored with 8 slices
 
+// Leading dimension of the general factorization's working copy: a multiple of four
+// and not of eight.  U12 takes a thread per column, so a warp's access goes to 32
+// columns: they then lie in eight banks of L1, and the columns are 16-byte aligned.
+// ms for 152 systems (64-wide blocks up to 700 rows), ld = n / a multiple of 32 / this:
+// n = 300 5.3 / 6.1 / 5.3, 513 41 / 12.2 / 9.4, 700 21.8 / 26.1 / 21.9, 1025 115 / 56 /
+// 50; any odd ld is as slow as 513 and 1025 are (700: 85).
+__host__ __device__ __forceinline__ int general_ld(int n) { return (n + 3) / 8 * 8 + 4; }
+
 struct Scratch {
-  float* W;        // n x n (ld n), the FP32 factors
+  float* W;        // the FP32 factors, ld n (fast) or general_ld(n)
   int* piv;        // n
   int8_t* SA;      // [s][n][nb4] slices of L21 rows
   int8_t* SB;      // [s][n][nb4] slices of U12 columns
@@ -234,13 +242,14 @@ __device__ __forceinline__ uint32_t ld_s8x4(const int8_t* p, bool ok) {
 }
 
 // The general factorization: any size, block and slice count, the working copy
-// in global memory throughout.  Serves what factor_fast does not take.
+// in global memory throughout (leading dimension general_ld).  Serves what
+// factor_fast does not take.
 __device__ __forceinline__ void factor_general(const BatchSys& S, int s, const Scratch& sc, int* info, float* sv,
                                                int* si) {
   const int n = S.n, nb = S.nb;
   const int nb4 = (nb + 31) / 32 * 32;   // slice row length: whole K steps of 32, zero padded
   float* W = sc.W;
-  const long ld = n;
+  const long ld = general_ld(n);
   for (long idx = threadIdx.x; idx < static_cast<long>(n) * n; idx += blockDim.x) {
     const int i = static_cast<int>(idx % n), j = static_cast<int>(idx / n);
     W[i + j * ld] = static_cast<float>(S.A[i + j * S.lda]);
@@ -964,7 +973,7 @@ __device__ __noinline__ void factor_fast(const BatchSys& sys, Scratch& sc, int* 
 // the 8 slices of a system whose refinement stalls.  152 systems at once, one per SM,
 // without refinement (ms): n = 1024 14.2 at 3 slices, 15.7 at 4, 29.3 at 8 (20.4 with
 // blocks of 16); n = 1025, where the panel outgrows two rows per thread and takes the
-// general path, 115 at 3 and 234 at 8.
+// general path, 50.4 at 3 and 199 at 8.
 __host__ __device__ __forceinline__ bool fast_takes(int n, int nb, int s) {
   return n <= kFastN && (s == 3 || s == 4 || s == 8) && (nb == 16 || nb == 32);
 }
@@ -1085,7 +1094,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchedA
       o += (bytes + 255) / 256 * 256;
       return p;
     };
-    sc.W = reinterpret_cast<float*>(take(static_cast<size_t>(nmax) * nmax * 4));
+    sc.W = reinterpret_cast<float*>(take(static_cast<size_t>(nmax) * general_ld(nmax) * 4));
     sc.piv = reinterpret_cast<int*>(take(static_cast<size_t>(nmax) * 4));
     sc.SA = reinterpret_cast<int8_t*>(take(static_cast<size_t>(kMaxS) * nmax * 64));
     sc.SB = reinterpret_cast<int8_t*>(take(static_cast<size_t>(kMaxS) * nmax * 64));
@@ -1102,6 +1111,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchedA
     if (t >= count) break;
     const BatchSys S = a.sys[t];
     const int n = S.n;
+    const int ldw = FAST ? n : general_ld(n);
     if (threadIdx.x == 0) info_s = 0;
     __syncthreads();
     int s_cur = S.s;
@@ -1118,7 +1128,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchedA
     // x0 from the FP32 factors
     for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(S.b[sc.perm[i]]);
     __syncthreads();
-    lu_solve_f32(sc.W, n, n, ds, dg);
+    lu_solve_f32(sc.W, ldw, n, ds, dg);
     for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = static_cast<double>(ds[i]);
     __syncthreads();
     double berr = INFINITY;
@@ -1163,7 +1173,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchedA
         __syncthreads();
         for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(S.b[sc.perm[i]]);
         __syncthreads();
-        lu_solve_f32(sc.W, n, n, ds, dg);
+        lu_solve_f32(sc.W, ldw, n, ds, dg);
         for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = static_cast<double>(ds[i]);
         __syncthreads();
         continue;
@@ -1172,7 +1182,7 @@ __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchedA
       const double sr = rmax > 0.0 ? rmax : 1.0;
       for (int i = threadIdx.x; i < n; i += blockDim.x) ds[i] = static_cast<float>(sc.r[sc.perm[i]] / sr);
       __syncthreads();
-      lu_solve_f32(sc.W, n, n, ds, dg);
+      lu_solve_f32(sc.W, ldw, n, ds, dg);
       for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] += static_cast<double>(ds[i]) * sr;
       __syncthreads();
     }
@@ -1236,7 +1246,7 @@ void pick(const BatchedState* st, int n, int& nb, int& s) {
 
 size_t per_block_bytes(int nmax) {
   auto a = [](size_t x) { return (x + 255) / 256 * 256; };
-  return a((size_t)nmax * nmax * 4) + a((size_t)nmax * 4) + 2 * a((size_t)kMaxS * nmax * 64) + 2 * a((size_t)nmax * 4) +
+  return a((size_t)nmax * general_ld(nmax) * 4) + a((size_t)nmax * 4) + 2 * a((size_t)kMaxS * nmax * 64) + 2 * a((size_t)nmax * 4) +
          a((size_t)nmax * 8) + a((size_t)nmax * 4) + 256;
 }
 
