@@ -143,6 +143,30 @@ __device__ __forceinline__ void loaded(float (&l)[32]) {
                       "+f"(l[k + 6]), "+f"(l[k + 7]));
 }
 
+// One block of the solve below by one warp, row per lane: w rows, of which lane's
+// entry (k) is B[32 k].
+template <bool LOWER, int UNROLL>
+__device__ __forceinline__ float diag_f32(const float* B, int lane, int w, float v) {
+  if (LOWER) {
+#pragma unroll UNROLL
+    for (int k = 0; k < w; ++k) {
+      const float dk = __shfl_sync(0xFFFFFFFFu, v, k);
+      if (lane > k) v = fmaf(-B[32 * k], dk, v);
+    }
+  } else {
+    const float diag = lane < w ? B[32 * lane] : 1.f;
+#pragma unroll UNROLL
+    for (int k = w - 1; k >= 0; --k) {
+      const float dk = __shfl_sync(0xFFFFFFFFu, v / diag, k);
+      if (lane == k)
+        v = dk;
+      else if (lane < k)
+        v = fmaf(-B[32 * k], dk, v);
+    }
+  }
+  return v;
+}
+
 // Solve (LU) y = d in FP32 in place on d (shared memory, length n, rows already
 // interchanged): unit lower, then upper, by blocks of 32 rows: one warp solves a
 // block (row per lane, values by shuffle), then every thread takes the block's 32
@@ -180,24 +204,12 @@ __device__ __noinline__ void lu_solve_f32(const float* W, int ld, int n, float* 
     if (tid < 32) {
       const float* B = dg + (st & 1) * 1024 + lane;          // B[32 k]: column k of row k0 + lane
       float v = lane < w ? d[k0 + lane] : 0.f;
-      if (lower) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          const float dk = __shfl_sync(0xFFFFFFFFu, v, k);
-          if (lane > k && k < w) v = fmaf(-B[32 * k], dk, v);
-        }
-      } else {
-        const float diag = lane < w ? B[32 * lane] : 1.f;
-#pragma unroll
-        for (int k = 31; k >= 0; --k) {
-          if (k >= w) continue;
-          const float dk = __shfl_sync(0xFFFFFFFFu, v / diag, k);
-          if (lane == k)
-            v = dk;
-          else if (lane < k)
-            v = fmaf(-B[32 * k], dk, v);
-        }
-      }
+      // a whole block in straight code, a ragged one in loops: a system of a few rows
+      // otherwise ran from the instruction cache's misses (5 us a step more at 4 rows)
+      if (w == 32)
+        v = lower ? diag_f32<true, 32>(B, lane, 32, v) : diag_f32<false, 32>(B, lane, 32, v);
+      else
+        v = lower ? diag_f32<true, 1>(B, lane, w, v) : diag_f32<false, 1>(B, lane, w, v);
       if (lane < w) d[k0 + lane] = v;
     }
     __syncthreads();
