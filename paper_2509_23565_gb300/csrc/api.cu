@@ -639,8 +639,14 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
     GemmConfig c{Variant::kPair, 128, pair_kind == 2};
     const long tiles64 = static_cast<long>((m + 255) / 256) * ((n + 63) / 64);
     if (!lower && tiles64 <= (h->nsm - h->sm_spare) / 2) c.bn = 64;
+    // level sums read and write their planes once per job, and bands of two levels
+    // have fewer jobs: one CTA per tile, and 128-column pair tiles (us): 2000 x 2500 x 200,
+    // s = 8 572 / 698, with k = 1000 1238 / 1823, at s = 7 1235 / 1565; 5000 x 5000 x 256, s =
+    // 7 2427 / 2531.  In one wave of small tiles pairs gain (512 x 512 x 256 79, 105 before)
+    const bool fewer_jobs = mode == 1 && c.bn == 128;
     size_t smem_pair = 0;
-    if (gemm_stages(c, s, &smem_pair) >= 2 && gemm_pair_capacity(smem_pair) >= 1) cfg = c;   // else one CTA per tile
+    if (!fewer_jobs && gemm_stages(c, s, &smem_pair) >= 2 && gemm_pair_capacity(smem_pair) >= 1)
+      cfg = c;   // else one CTA per tile
   }
   const bool pair = cfg.var == Variant::kPair;
   if (!pair && (nit->second & 4)) cfg = GemmConfig{Variant::kNarrow, 128, false};

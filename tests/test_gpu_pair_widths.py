@@ -32,3 +32,15 @@ def test_widths_agree(gpu_lib, m, n, k, s, one_sign):
             gpu_lib.dgemm(ColMajor(A, m, k), ColMajor(B[c:e], k, e - c), ColMajor(D[c:e], m, e - c), s, alpha, beta)
         gpu_lib.sync_status()
         assert torch.equal(C, D)
+
+
+@pytest.mark.parametrize("k,s", [(100, 8), (300, 8), (1100, 7), (256, 7)])
+def test_level_sums_widths_agree(gpu_lib, k, s):
+    """Level sums of a product too large for one wave of CTA pairs against those of
+    its column blocks."""
+    m, n = 2100, 700
+    A, B = _entries(m, k, 1, False), _entries(k, n, 2, False)
+    whole = gpu_lib.level_sums(ColMajor(A, m, k), ColMajor(B, k, n), s)
+    for c in range(0, n, 256):
+        e = min(n, c + 256)
+        assert torch.equal(whole[:, c:e], gpu_lib.level_sums(ColMajor(A, m, k), ColMajor(B[c:e], k, e - c), s))
