@@ -302,19 +302,21 @@ inline int np_split(int w) {
 }
 
 // Factor the panel A[d:n, d:d+w] (no pivoting) and leave L^-1 of its diagonal
-// block in X at (d - j0, d - j0).
+// block in X at (d - j0, d - j0), unless the panel is the matrix's last.
 int np_panel(emul_handle_t h, double* A, long lda, int n, int j0, int d, int w, int s, int32_t* info,
              const NpBufs& B) {
   double* Xd = B.X + (d - j0) + static_cast<long>(d - j0) * B.ldx;
   if (w <= kNpLeaf) {
     launch_dependent(np_leaf_kernel, dim3(kNpCluster), dim3(32 * kNpWarps), 0, h->stream, A, lda, d, w, info);
-    launch_dependent(np_inverse_kernel, dim3((w + kInvCols - 1) / kInvCols, 2), dim3(32 * kInvCols), 0, h->stream, A,
-                     lda, d, w, Xd, B.ldx, B.Y);
-    h->launches += 2;
-    int rc = check_cuda(h, cudaGetLastError(), "no-pivot leaf");
-    if (rc) return rc;
+    h->launches++;
     const int mb = n - d - w;
-    if (mb <= 0) return EMUL_OK;
+    if (mb > 0) {                 // (no row and no column is left to use the last leaf's inverses)
+      launch_dependent(np_inverse_kernel, dim3((w + kInvCols - 1) / kInvCols, 2), dim3(32 * kInvCols), 0, h->stream,
+                       A, lda, d, w, Xd, B.ldx, B.Y);
+      h->launches++;
+    }
+    int rc = check_cuda(h, cudaGetLastError(), "no-pivot leaf");
+    if (rc || mb <= 0) return rc;
     double* A21 = A + (d + w) + static_cast<long>(d) * lda;
     // L21 = A21 U11^-1, written over A21 (both operands are sliced before the product writes)
     return gemm_run(h, mb, w, w, 1.0, Operand{A21, 1, lda}, Operand{B.Y, w, 1}, 0.0, A21, lda, s, false, 0,
@@ -334,7 +336,7 @@ int np_panel(emul_handle_t h, double* A, long lda, int n, int j0, int d, int w, 
   rc = gemm_kchunks(h, n - d - w1, w2, w1, -1.0, Operand{L21, 1, lda}, Operand{A12, lda, 1}, 1.0, A22, lda, s);
   if (rc) return rc;
   rc = np_panel(h, A, lda, n, j0, d + w1, w2, s, info, B);
-  if (rc) return rc;
+  if (rc || d + w == n) return rc;
   // join the inverses: X21 = -X22 (L21 X11), L21 the w2 x w1 block below the left diagonal block
   double* X22 = Xd + w1 + static_cast<long>(w1) * B.ldx;
   double* X21 = Xd + w1;
