@@ -632,13 +632,19 @@ int gemm_run(emul_handle_t h, int m, int n, int k, double alpha, Operand A, Oper
   // 1024 x 256 (64 tiles of 64 columns) 31 / 38, 4864 x 256 x 256 (76) 34 / 41, with k
   // = 1024 120 / 152, at s = 8 37 / 50, at s = 3 28 / 30; just past the line 2560 x
   // 512 x 256 (80) 49 / 39, k = 1024 167 / 130, s = 8 55 / 49, s = 3 38 / 31, and
-  // 2048 x 1152 x 256 (144) 49 / 40
+  // 2048 x 1152 x 256 (144) 49 / 40.  With a short K what a wave waits for is a ragged
+  // tile's rounding with its checks, half as long with 64 columns: up to short_k they
+  // gain as long as 128-column tiles are one wave.  2262 x 691, s = 7: k = 79 30.1 / 33.3,
+  // 128 32.9 / 34.7, 256 50.8 / 46.9; s = 8: 128 38.5 / 43.0, 256 57.3 / 56.9; s = 3: 128
+  // 23.7 / 27.5, 256 32.3 / 32.7; whole tiles, 2304 x 1024 x 64 at s = 7: 25.0 / 23.1
   GemmConfig cfg{Variant::kWide, 64, false};
   const int pair_kind = nit->second & 3;
   if (pair_kind && m > 128 && h->nsm >= 2) {
     GemmConfig c{Variant::kPair, 128, pair_kind == 2};
-    const long tiles64 = static_cast<long>((m + 255) / 256) * ((n + 63) / 64);
-    if (!lower && tiles64 <= (h->nsm - h->sm_spare) / 2) c.bn = 64;
+    const long rows = (m + 255) / 256, tiles64 = rows * ((n + 63) / 64), tiles128 = rows * ((n + 127) / 128);
+    const int pairs = (h->nsm - h->sm_spare) / 2, short_k = s == 8 ? 224 : s <= 3 ? 256 : 160;
+    const bool ragged = m % 256 != 0 || n % 128 != 0;
+    if (!lower && (tiles64 <= pairs || (ragged && k <= short_k && tiles128 < pairs))) c.bn = 64;
     // level sums read and write their planes once per job, and bands of two levels
     // have fewer jobs: one CTA per tile, and 128-column pair tiles (us): 2000 x 2500 x 200,
     // s = 8 572 / 698, with k = 1000 1238 / 1823, at s = 7 1235 / 1565; 5000 x 5000 x 256, s =
