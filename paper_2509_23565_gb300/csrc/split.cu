@@ -19,7 +19,9 @@ namespace emul {
 namespace {
 
 constexpr int kSplitThreads = 256;
-constexpr int kSplitRows = 8;            // rows per block
+constexpr int kSplitRows = 8;            // rows per block, with 32 groups of eight k at a time
+constexpr int kSplitTall = 32;           // the same with 8 groups, for k <= 64 and
+constexpr int kSplitTallRows = 4096;     // at least so many rows in the launch
 
 struct SplitArgs {
   const double* X;
@@ -31,29 +33,32 @@ struct SplitArgs {
   int blocks;       // blocks of this operand
 };
 
-// One block slices eight rows.  Rows contiguous in memory (rs = 1): a warp
-// covers the 8 rows x 4 groups of eight k, so a column of the tile is one 64-byte
-// piece and the four groups of a row are 64 bytes of a plane; k contiguous: a
-// warp takes one row, 32 groups at a time.  KEEP: all of K fits in one pass, the elements
-// stay in registers between the maximum and the digits; otherwise the second
-// pass reads them again (from L2).  Bound by memory for tall operands
-// (8 B read, 2s B written per element), by latency for small ones; the blocks
-// are small so that a 256-row operand already fills 32 SMs, and both operands
-// of a product go in one launch.
-template <int S, bool KEEP>
+// One block slices eight rows (R; 32 of a tall operand with k <= 64, where a row has
+// at most 8 groups of eight k for its threads: 100000 x 8 at s = 3 7.3 us, 23.7 with
+// eight, 16384 x 64 at s = 7 7.1 and 8.4; 256 x 64 3.0 and 2.2).  Rows contiguous in
+// memory (rs = 1): a warp covers the 8 rows x 4 groups, so a column of the tile is one
+// 64-byte piece and the four groups of a row are 64 bytes of a plane (R = 32: 32
+// rows of one group); k contiguous: a warp takes one row, 32 groups at a time (R =
+// 32: four rows).  KEEP: all of K fits in one pass, the elements stay in registers
+// between the maximum and the digits; otherwise the second pass reads them again
+// (from L2).  Bound by memory for tall operands (8 B read, 2s B written per
+// element), by latency for small ones; the blocks are small so that a 256-row
+// operand already fills 32 SMs, and both operands of a product go in one launch.
+template <int S, bool KEEP, int R>
 __global__ void __launch_bounds__(kSplitThreads) split_kernel(const SplitArgs a0, const SplitArgs a1) {
-  __shared__ uint32_t up_s[kSplitThreads / 32][kSplitRows];
-  __shared__ unsigned long long full_s[kSplitRows];
+  constexpr int gstep = kSplitThreads / R;      // groups of a row taken at once
+  __shared__ uint32_t up_s[kSplitThreads / 32][R];
+  __shared__ unsigned long long full_s[R];
   grid_launch();
   grid_wait();
   const bool second = static_cast<int>(blockIdx.x) >= a0.blocks;
   const SplitArgs& a = second ? a1 : a0;
-  const int r0 = (static_cast<int>(blockIdx.x) - (second ? a0.blocks : 0)) * kSplitRows;
+  const int r0 = (static_cast<int>(blockIdx.x) - (second ? a0.blocks : 0)) * R;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool by_rows = a.rs == 1;
-  const int rl = by_rows ? lane & 7 : warp;                       // row within the block
-  const int g0 = by_rows ? warp * 4 + (lane >> 3) : lane;         // first K group of this thread
-  constexpr int gstep = 32;
+  const int tid = threadIdx.x;
+  const int rl = by_rows ? tid % R : tid / gstep;                 // row within the block
+  const int g0 = by_rows ? tid / R : tid % gstep;                 // first K group of this thread
   const int groups = static_cast<int>(a.ldk >> 3);
   const int r = r0 + rl;
   const bool row_ok = r < a.rows;
@@ -65,8 +70,8 @@ __global__ void __launch_bounds__(kSplitThreads) split_kernel(const SplitArgs a0
       u[j] = row_ok && c < a.k ? row[c * a.cs] : 0ull;
     }
   };
-  // the maximum over the threads that share a row: lanes 8 and 16 apart, then
-  // the warps (rows contiguous), or the warp (k contiguous)
+  // the maximum over the threads that share a row: lanes R apart, then the warps
+  // (rows contiguous), or gstep neighbouring lanes (k contiguous)
   uint64_t u[8];
   uint32_t up = 0;
   if (KEEP) {
@@ -79,13 +84,16 @@ __global__ void __launch_bounds__(kSplitThreads) split_kernel(const SplitArgs a0
     }
   }
   if (by_rows) {
-    up = max(up, __shfl_xor_sync(0xFFFFFFFFu, up, 8));
-    up = max(up, __shfl_xor_sync(0xFFFFFFFFu, up, 16));
-    if (lane < kSplitRows) up_s[warp][lane] = up;
-  } else {
+#pragma unroll
+    for (int o = R; o < 32; o *= 2) up = max(up, __shfl_xor_sync(0xFFFFFFFFu, up, o));
+    if (lane < R) up_s[warp][lane] = up;
+  } else if (gstep == 32) {
     up = __reduce_max_sync(0xFFFFFFFFu, up);
+  } else {
+#pragma unroll
+    for (int o = 1; o < gstep; o *= 2) up = max(up, __shfl_xor_sync(0xFFFFFFFFu, up, o));
   }
-  if (threadIdx.x < kSplitRows) full_s[threadIdx.x] = 0;
+  if (tid < R) full_s[tid] = 0;
   __syncthreads();
   if (by_rows) {
 #pragma unroll
@@ -128,20 +136,24 @@ __global__ void __launch_bounds__(kSplitThreads) split_kernel(const SplitArgs a0
 }
 
 template <int S>
-cudaError_t launch_s(cudaStream_t st, const SplitArgs& a, const SplitArgs& b) {
-  const int grid = a.blocks + b.blocks;
+cudaError_t launch_s(cudaStream_t st, SplitArgs a, SplitArgs b) {
   const long ldk = a.ldk > b.ldk ? a.ldk : b.ldk;
-  if (ldk <= 256)
-    return launch_dependent(split_kernel<S, true>, dim3(grid), dim3(kSplitThreads), 0, st, a, b);
-  return launch_dependent(split_kernel<S, false>, dim3(grid), dim3(kSplitThreads), 0, st, a, b);
+  const bool tall = ldk <= kSplitThreads / kSplitTall * 8 && a.rows + b.rows >= kSplitTallRows;
+  const int R = tall ? kSplitTall : kSplitRows;
+  a.blocks = (a.rows + R - 1) / R;
+  b.blocks = (b.rows + R - 1) / R;
+  const dim3 grid(a.blocks + b.blocks), block(kSplitThreads);
+  if (tall) return launch_dependent(split_kernel<S, true, kSplitTall>, grid, block, 0, st, a, b);
+  if (ldk <= 256) return launch_dependent(split_kernel<S, true, kSplitRows>, grid, block, 0, st, a, b);
+  return launch_dependent(split_kernel<S, false, kSplitRows>, grid, block, 0, st, a, b);
 }
 
 SplitArgs make_args(int rows, int k, const double* X, long rs, long cs, int32_t* exps, uint16_t* out, long ldk) {
-  return SplitArgs{X, rs, cs, rows, k, exps, out, ldk, rows > 0 ? (rows + kSplitRows - 1) / kSplitRows : 0};
+  return SplitArgs{X, rs, cs, rows > 0 ? rows : 0, k, exps, out, ldk, 0};
 }
 
 cudaError_t dispatch(cudaStream_t st, int s, const SplitArgs& a, const SplitArgs& b) {
-  if (a.blocks + b.blocks == 0) return cudaSuccess;
+  if (a.rows + b.rows == 0) return cudaSuccess;
   switch (s) {
     case 1: return launch_s<1>(st, a, b);
     case 2: return launch_s<2>(st, a, b);
