@@ -1136,18 +1136,22 @@ __global__ void __launch_bounds__(256) trsm_small_kernel(double* A, long lda, in
 // way, transposed with `trans`), then the first 128 solve (diag_solve: quotients
 // by the diagonal's reciprocals in two parts, or by divisions throughout where an
 // entry of the block's diagonal or a value lies outside their window).  dpotrs
-// with two right-hand sides at n = 128 (two blocks) takes 59 us, 136 with divisions
+// with two right-hand sides at n = 128 (two blocks) takes 55 us, 136 with divisions
 // throughout and 47 with x_k = v RN(1 / d), whose second rounding shows: the error of
 // a substitution with 200 rows is then 1 to 7 % larger.
+//
+// early: a kernel of this solve came before.  It lets the next kernels start only
+// once it has waited itself, so T stood complete before this kernel began, and the
+// block of T is staged (past L1) while the kernel ahead still works on X (dgetrs n =
+// 4001, 8 right-hand sides 2.03 ms, 2.39 otherwise).
 // blockIdx.x = right-hand side.
 __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long ldt, double* X, long ldx, int d0,
-                                                          int bs, int lower, int unit, int trans) {
+                                                          int bs, int lower, int unit, int trans, int early) {
   extern __shared__ double tb[];   // tb[r + c*(bs+1)] = op(T)(d0+r, d0+c)
   __shared__ double x[128], rcp[128], rest[128];
   __shared__ int odd_s;            // a value outside the window of kQuot
   if (threadIdx.x == 0) odd_s = 0;
-  grid_launch();
-  grid_wait();
+  if (!early) grid_wait();
   const int ld = bs + 1;
   double* xc = X + static_cast<long>(blockIdx.x) * ldx + d0;
   {
@@ -1158,7 +1162,7 @@ __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long 
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const int c = c0 + j * cstep;
-          v[j] = c < bs ? T[(d0 + r) + static_cast<long>(d0 + c) * ldt] : 0.0;
+          v[j] = c < bs ? __ldcg(T + (d0 + r) + static_cast<long>(d0 + c) * ldt) : 0.0;
         }
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
@@ -1167,7 +1171,6 @@ __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long 
         }
       }
   }
-  if (static_cast<int>(threadIdx.x) < bs) x[threadIdx.x] = xc[threadIdx.x];
   __syncthreads();
   bool odd = false;
   if (!unit && static_cast<int>(threadIdx.x) < bs) {
@@ -1177,7 +1180,11 @@ __global__ void __launch_bounds__(1024) trsv_block_kernel(const double* T, long 
     odd = !quot_ok(d);
   }
   odd = __syncthreads_or(odd);
+  grid_wait();
+  grid_launch();
   if (threadIdx.x >= 128) return;
+  if (static_cast<int>(threadIdx.x) < bs) x[threadIdx.x] = xc[threadIdx.x];
+  asm volatile("bar.sync 1, 128;" ::: "memory");
   if (unit) {                        // (a lower triangle)
     diag_solve<true, kUnit>(tb, ld, nullptr, nullptr, bs, x);
   } else {
@@ -1958,7 +1965,7 @@ int getrs_body(emul_handle_t h, int n, int nrhs, const double* LU, int lda, cons
   for (int d0 = 0; d0 < n; d0 += bs) {
     const int b = bs < n - d0 ? bs : n - d0;
     launch_dependent(trsv_block_kernel, dim3(nrhs), dim3(1024), b * (b + 1) * sizeof(double), h->stream, LU, lda, B,
-                     ldb, d0, b, 1, 1, 0);
+                     ldb, d0, b, 1, 1, 0, d0 > 0);
     h->launches += (d0 + b < n) ? 2 : 1;
     if (d0 + b < n)
       launch_dependent(gemv_update_kernel, dim3((n - d0 - b + 255) / 256, nrhs), dim3(256), 0, h->stream, LU, lda, B,
@@ -1967,7 +1974,7 @@ int getrs_body(emul_handle_t h, int n, int nrhs, const double* LU, int lda, cons
   for (int d0 = ((n - 1) / bs) * bs; d0 >= 0; d0 -= bs) {
     const int b = bs < n - d0 ? bs : n - d0;
     launch_dependent(trsv_block_kernel, dim3(nrhs), dim3(1024), b * (b + 1) * sizeof(double), h->stream, LU, lda, B,
-                     ldb, d0, b, 0, 0, 0);
+                     ldb, d0, b, 0, 0, 0, 1);
     h->launches += (d0 > 0) ? 2 : 1;
     if (d0 > 0)
       launch_dependent(gemv_update_kernel, dim3((d0 + 255) / 256, nrhs), dim3(256), 0, h->stream, LU, lda, B, ldb, 0,
@@ -2425,7 +2432,7 @@ int emul_dpotrs(emul_handle_t h, char uplo, int n, int nrhs, const double* L, in
   for (int d0 = 0; d0 < n; d0 += bs) {
     const int b = bs < n - d0 ? bs : n - d0;
     emul::launch_dependent(emul::trsv_block_kernel, dim3(nrhs), dim3(1024), b * (b + 1) * sizeof(double), h->stream,
-                           L, lda, B, ldb, d0, b, 1, 0, 0);
+                           L, lda, B, ldb, d0, b, 1, 0, 0, d0 > 0);
     h->launches += (d0 + b < n) ? 2 : 1;
     if (d0 + b < n)
       emul::launch_dependent(emul::gemv_update_kernel, dim3((n - d0 - b + 255) / 256, nrhs), dim3(256), 0, h->stream,
@@ -2434,7 +2441,7 @@ int emul_dpotrs(emul_handle_t h, char uplo, int n, int nrhs, const double* L, in
   for (int d0 = ((n - 1) / bs) * bs; d0 >= 0; d0 -= bs) {
     const int b = bs < n - d0 ? bs : n - d0;
     emul::launch_dependent(emul::trsv_block_kernel, dim3(nrhs), dim3(1024), b * (b + 1) * sizeof(double), h->stream,
-                           L, lda, B, ldb, d0, b, 0, 0, 1);
+                           L, lda, B, ldb, d0, b, 0, 0, 1, 1);
     h->launches += (d0 > 0) ? 2 : 1;
     if (d0 > 0)
       emul::launch_dependent(emul::gemv_update_kernel, dim3((d0 + 7) / 8, nrhs), dim3(256), 0, h->stream, L, lda, B,
