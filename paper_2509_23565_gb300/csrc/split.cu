@@ -21,7 +21,7 @@ namespace {
 constexpr int kSplitThreads = 256;
 constexpr int kSplitRows = 8;            // rows per block, with 32 groups of eight k at a time
 constexpr int kSplitTall = 32;           // the same with 8 groups, for k <= 64 and
-constexpr int kSplitTallRows = 4096;     // at least so many rows in the launch
+constexpr int kSplitTallRows = 32768;    // at least so many rows in the launch
 
 struct SplitArgs {
   const double* X;
@@ -35,15 +35,18 @@ struct SplitArgs {
 
 // One block slices eight rows (R; 32 of a tall operand with k <= 64, where a row has
 // at most 8 groups of eight k for its threads: 100000 x 8 at s = 3 7.3 us, 23.7 with
-// eight, 16384 x 64 at s = 7 7.1 and 8.4; 256 x 64 3.0 and 2.2).  Rows contiguous in
-// memory (rs = 1): a warp covers the 8 rows x 4 groups, so a column of the tile is one
-// 64-byte piece and the four groups of a row are 64 bytes of a plane (R = 32: 32
-// rows of one group); k contiguous: a warp takes one row, 32 groups at a time (R =
-// 32: four rows).  KEEP: all of K fits in one pass, the elements stay in registers
-// between the maximum and the digits; otherwise the second pass reads them again
-// (from L2).  Bound by memory for tall operands (8 B read, 2s B written per
-// element), by latency for small ones; the blocks are small so that a 256-row
-// operand already fills 32 SMs, and both operands of a product go in one launch.
+// eight, 50000 x 64 at s = 7 16.8 and 21.1; 256 x 64 3.0 and 2.2; between, where the
+// slicing alone gains a microsecond or two, the product that follows loses as much as
+// often as not: 2421 x 8184 x 54 at s = 3 237 and 234, 16384 x 16384 x 64 2728 and 2736).
+// Rows contiguous in memory (rs = 1): a warp covers the 8 rows x 4 groups, so a
+// column of the tile is one 64-byte piece and the four groups of a row are 64 bytes of
+// a plane (R = 32: 32 rows of one group); k contiguous: a warp takes one row, 32
+// groups at a time (R = 32: four rows).  KEEP: all of K fits in one pass, the elements
+// stay in registers between the maximum and the digits; otherwise the second pass
+// reads them again (from L2).  Bound by memory for tall operands (8 B read, 2s B
+// written per element), by latency for small ones; the blocks are small so that a
+// 256-row operand already fills 32 SMs, and both operands of a product go in one
+// launch.
 template <int S, bool KEEP, int R>
 __global__ void __launch_bounds__(kSplitThreads) split_kernel(const SplitArgs a0, const SplitArgs a1) {
   constexpr int gstep = kSplitThreads / R;      // groups of a row taken at once
