@@ -328,9 +328,10 @@ int emul_selector_load(emul_handle_t h, const char* path);
  * lives in one 16 MiB static device array that every GPU which loads this
  * library holds until the process exits.  Limit: with kp = k rounded up to a
  * multiple of 8, 2 * slices * kp * (m + n) + 4 * (m + n) + about 17 KB must
- * fit in 16 MiB, and the schedule in 16 KB (k up to about 59000 at 7 slices, 51000 at
- * 8), else the call returns EMUL_NO_WORKSPACE and enqueues nothing.  The first call on a device sets up that device (it looks up the
- * device address of the array); make that first call before any stream
+ * fit in 16 MiB, and the schedule in 16 KB (k up to about 59000 at 7 slices,
+ * 51000 at 8), else the call returns EMUL_NO_WORKSPACE and enqueues nothing.
+ * The first call on a device sets up that device (it looks up the device
+ * address of the array); make that first call before any stream
  * capture.  Every call reuses the same array and keeps the previous call's
  * contents: calls that overlap on the GPU (other streams, other threads)
  * race and give unspecified results.  A device-side wait that gives up is

@@ -1,5 +1,5 @@
-// Batched solves of many independent, uneven systems A_i x_i = b_i in one
-// persistent launch, with the split-integer product of
+// Batched solves of many independent, uneven systems A_i x_i = b_i in
+// persistent launches, with the split-integer product of
 // arXiv 2509.23565 (Sec. 2, Eq. 2) at a reduced slice count in the LU
 // factorization and FP64 iterative refinement on the residual of Eq. 8.
 //
@@ -1079,8 +1079,8 @@ static_assert(solve_smem(kFastN) <= kFastSmem, "shared memory of the solve");
 // FAST: the systems that factor_fast takes.  The others run in a kernel of their own
 // with little shared memory: factor_general works in global memory and lives off L1,
 // which 200 KB of shared memory leave no room for (100 systems of 300 rows at 7 slices
-// 11.2 ms, 5.9 so; 20 of 700 with blocks of 64 40.6 and 20.0).  A system of theirs that has to be
-// refactored with 8 slices and can be in the fast way is handed over.
+// 11.2 ms, 5.9 so; 20 of 700 with blocks of 64 40.6 and 20.0).  A system of theirs
+// that has to be refactored with 8 slices and can be in the fast way is handed over.
 template <bool FAST>
 __global__ void __launch_bounds__(kBThreads) batched_solve_kernel(const BatchedArgs a) {
   __shared__ float sv[kBThreads / 32];
